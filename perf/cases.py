@@ -21,7 +21,7 @@ PHYS = {
     "batch2d": dict(h=5.0, dt=0.5e-3, f=25.0, v_min=1500.0, v_max=4000.0, v_lo=1500.0, v_hi=4000.0, cap=4000.0),
     "shot3d": dict(h=10.0, dt=1e-3, f=15.0, v_min=1500.0, v_max=4500.0, v_lo=1500.0, v_hi=4500.0, cap=4500.0),
 }
-EPS_REL = 1e-3                 # water level of the image ratio
+EPS_REL = 1e-2                 # water level of the image ratio
 C = (1.6, -0.2, 8.0 / 315.0, -1.0 / 560.0)   # 8th-order second-derivative weights c1..c4
 C0 = -2.0 * sum(C)
 
