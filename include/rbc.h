@@ -132,6 +132,16 @@ int rbc_destroy(rbc_ctx *ctx);
 int rbc_set_coef(rbc_ctx *ctx, const float *a_dev, int check, void *stream);
 
 /*
+ * rbc_set_share -- tell a context that `contexts` contexts of its kind run at
+ * the same time on their own streams (1 at creation): its 2-D time loops then
+ * take that share of the device each, so that the contexts' loops run side by
+ * side instead of one after the other.  Results do not depend on it.
+ * Synchronises the device when the number changes.
+ * Errors: RBC_EINVAL (NULL, contexts < 1), RBC_ENOMEM, RBC_ECUDA.
+ */
+int rbc_set_share(rbc_ctx *ctx, int contexts);
+
+/*
  * rbc_model -- Algorithm 1 (seismic modeling) for one shot.
  *   src_host: (x, y, z) padded node of the point source.
  *   wavelet_dev: f[0..nt-1] fp32 (f[n] drives step n -> n+1).

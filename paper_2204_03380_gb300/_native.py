@@ -72,6 +72,8 @@ def _load():
     lib.rbc_destroy.argtypes = [P]
     lib.rbc_set_coef.argtypes = [P, P, I, P]
     lib.rbc_set_coef.restype = I
+    lib.rbc_set_share.argtypes = [P, I]
+    lib.rbc_set_share.restype = I
     lib.rbc_model.argtypes = [P, P, P, I, P, P, P]
     lib.rbc_rtm_shot.argtypes = [P, P, P, I, P, P, I, P, P, P]
     lib.rbc_image_stack.argtypes = [G, P, P, F, I, I, G, P, P]
@@ -126,7 +128,7 @@ EXPORTED = ("rbc_build_velocity", "rbc_create", "rbc_destroy", "rbc_model", "rbc
             "rbc_cnn_param_count", "rbc_cnn_workspace_bytes", "rbc_cnn_forward", "rbc_cnn_infer", "rbc_cnn_backward",
             "rbc_cnn_mse", "rbc_cnn_adam", "rbc_inject_fault", "rbc_last_error",
             "rbc_launch_count", "rbc_nyquist_stride", "rbc_storage_bytes", "rbc_rtm_storage",
-            "rbc_set_coef")
+            "rbc_set_coef", "rbc_set_share")
 
 
 def _check(code):
@@ -178,6 +180,11 @@ def rbc_destroy(ctx):
 def rbc_set_coef(ctx, grid, a, check=True, stream=None):
     """Replace the context's padded coefficient a (grid.padded fp32 CUDA)."""
     _check(_lib.rbc_set_coef(C.c_void_p(ctx), _dev(a, grid.padded, "a"), int(bool(check)), _stream(stream)))
+
+
+def rbc_set_share(ctx, contexts):
+    """Contexts of this kind in flight at once (a scheduling hint; results do not depend on it)."""
+    _check(_lib.rbc_set_share(C.c_void_p(ctx), int(contexts)))
 
 
 def rbc_model(ctx, src, wavelet, rec, seis, stream=None):

@@ -13,6 +13,7 @@
 
 #include "../../include/rbc.h"
 #include "rbc_internal.cuh"
+#include "rbc_resident.cuh"
 
 using namespace rbc;
 
@@ -126,6 +127,14 @@ struct rbc_ctx {
   int *err_host = nullptr;
   int *err_dev = nullptr;
   int fault = 0;  // rbc_inject_fault: applies to the next call only
+  // 2-D grids that fit on the chip: the whole time loop as one launch
+  // (rbc_resident.cu), 0 forward, 1 reverse (variant -1: one launch per step)
+  ResPlan res[2];
+  ResTile *res_tiles[2] = {nullptr, nullptr};
+  unsigned long long *res_ll = nullptr;
+  char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, receiver cells
+  size_t res_blob_cap = 0;
+  int share = 1;             // contexts in flight at once (rbc_set_share)
 };
 
 namespace {
@@ -173,10 +182,7 @@ int node_ok(const rbc_ctx *c, const int *r) {
   return y >= 0 && y < L.NY;
 }
 
-// Upload the per-shot tables: source offset and scales, receiver offsets and
-// the receiver list of every reverse-kernel tile (counting sort by tile).
-int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinject,
-                cudaStream_t s) {
+int check_nodes(const rbc_ctx *c, const int *src, int nrec, const int *rec) {
   if (!src) return fail(RBC_EINVAL, "src is NULL");
   if (!node_ok(c, src)) return fail(RBC_EINVAL, "source node (%d,%d,%d) outside the padded grid", src[0], src[1], src[2]);
   if (nrec < 0 || (nrec > 0 && !rec)) return fail(RBC_EINVAL, "bad receiver list");
@@ -184,18 +190,32 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
     if (!node_ok(c, rec + 3 * r))
       return fail(RBC_EINVAL, "receiver %d node (%d,%d,%d) outside the padded grid", r, rec[3 * r],
                   rec[3 * r + 1], rec[3 * r + 2]);
-  int rc = ensure_receivers(c, std::max(nrec, 1));
-  if (rc) return rc;
-  const Lay &L = c->L;
-  const double ps = (L.ndim == 3) ? 1.0 / c->g.h : 1.0;  // h^(2-d)
+  return RBC_OK;
+}
+
+ShotInfo shot_info(rbc_ctx *c, const int *src, int nrec, int reinject) {
+  const double ps = (c->L.ndim == 3) ? 1.0 / c->g.h : 1.0;  // h^(2-d)
   ShotInfo info{};
-  info.src_off = lay_off(L, src[0], src[1], src[2]);
+  info.src_off = lay_off(c->L, src[0], src[1], src[2]);
   info.nrec = nrec;
   info.src_fwd = (float)ps;
   info.src_rev = reinject ? (float)ps : 0.f;
   info.rec_scale = (float)ps;
   info.fault = c->fault;
   c->fault = 0;
+  return info;
+}
+
+// Upload the per-shot tables: source offset and scales, receiver offsets and
+// the receiver list of every reverse-kernel tile (counting sort by tile).
+int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinject,
+                cudaStream_t s) {
+  int rc = check_nodes(c, src, nrec, rec);
+  if (rc) return rc;
+  rc = ensure_receivers(c, std::max(nrec, 1));
+  if (rc) return rc;
+  const Lay &L = c->L;
+  const ShotInfo info = shot_info(c, src, nrec, reinject);
   int gx, gy, gz, t;
   rev_tiling(L, c->zc_r, &gx, &gy, &gz, &t);
   std::vector<int> off(std::max(nrec, 1)), tile(std::max(nrec, 1)), ptr(c->ntiles + 1, 0),
@@ -218,6 +238,85 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
     CK(cudaMemcpyAsync(c->tile_rec, order.data(), sizeof(int) * nrec, cudaMemcpyHostToDevice, s));
   }
   CK(cudaMemcpyAsync(c->tile_ptr, ptr.data(), sizeof(int) * (c->ntiles + 1), cudaMemcpyHostToDevice, s));
+  return RBC_OK;
+}
+
+// Whether this call's loop (0 forward, 1 reverse) runs as one resident launch.
+bool resident(const rbc_ctx *c, int dir) {
+  return c->res[dir].variant >= 0 && c->snap.empty() && (dir == 1 || c->levels_per_launch == 1);
+}
+
+// Tables of a resident loop (one copy to the device) and its launch.  The
+// receivers are sorted by the warp that owns their rows; num / den are the
+// reverse loop's outputs.
+int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, int reinject, int sample, int grad,
+                 int overwrite, int dense, float *num, float *den, cudaStream_t s) {
+  const ResPlan &P = c->res[dir];
+  const Lay &L = c->L;
+  const int cells = P.blocks * P.warps;
+  auto up = [](size_t n) { return (n + 63) / 64 * 64; };
+  const size_t o_shot = 64, o_ptr = o_shot + up(sizeof(ResShot)), o_rec = o_ptr + up(sizeof(int) * (cells + 1)),
+               need = o_rec + up(sizeof(int2) * nrec);
+  static_assert(sizeof(ShotInfo) <= 64, "the shot's info precedes its table");
+  if (need > c->res_blob_cap) {
+    cudaFree(c->res_blob);  // waits for the work that reads it
+    c->res_blob = nullptr;
+    c->res_blob_cap = 0;
+    CK(cudaMalloc(&c->res_blob, 2 * need));
+    c->res_blob_cap = 2 * need;
+  }
+  std::vector<char> blob(need, 0);
+  const ShotInfo info = shot_info(c, src, nrec, reinject);
+  std::memcpy(blob.data(), &info, sizeof info);
+  int *ptr = reinterpret_cast<int *>(blob.data() + o_ptr);
+  int2 *cr = reinterpret_cast<int2 *>(blob.data() + o_rec);
+  std::vector<int> cell(nrec), loc(nrec);
+  for (int r = 0; r < nrec; ++r) {
+    res_cell(P, L, rec[3 * r], rec[3 * r + 2], &cell[r], &loc[r]);
+    ++ptr[cell[r] + 1];
+  }
+  for (int k = 0; k < cells; ++k) ptr[k + 1] += ptr[k];
+  std::vector<int> fill(ptr, ptr + cells);
+  for (int r = 0; r < nrec; ++r) cr[fill[cell[r]]++] = make_int2(loc[r], r);
+  ResShot S{};
+  S.L = L;
+  S.a = c->a;
+  S.p[0] = c->p[0];
+  S.p[1] = c->p[1];
+  S.info = reinterpret_cast<const ShotInfo *>(c->res_blob);
+  S.seis_t = c->seis_t;
+  S.cell_ptr = reinterpret_cast<const int *>(c->res_blob + o_ptr);
+  S.cell_rec = reinterpret_cast<const int2 *>(c->res_blob + o_rec);
+  S.num = num;
+  S.den = den;
+  S.ix0 = c->g.nb;
+  S.ix1 = c->g.nb + c->g.nx;
+  S.iz0 = top_rows(&c->g);
+  S.iz1 = S.iz0 + c->g.nz;
+  std::memcpy(blob.data() + o_shot, &S, sizeof S);
+  CK(cudaMemcpyAsync(c->res_blob, blob.data(), need, cudaMemcpyHostToDevice, s));
+  ResArgs A{};
+  A.tiles = c->res_tiles[dir];
+  A.shots = reinterpret_cast<const ResShot *>(c->res_blob + o_shot);
+  A.ll = c->res_ll;
+  A.wav = c->wav;
+  A.nt = c->g.nt;
+  A.sample = sample;
+  A.grad = grad;
+  A.overwrite = overwrite;
+  A.dense = dense;
+  A.err = c->err_dev;
+  CK(res_launch(P, dir == 0, A, s));
+  ++g_launches;
+  return RBC_OK;
+}
+
+// A capturing stream is refused before anything is queued (the time loops'
+// tables are copied from memory that does not outlive the call).
+int check_capture(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(s, &st));
+  if (st != cudaStreamCaptureStatusNone) return fail(RBC_ECUDA, "the stream is capturing");
   return RBC_OK;
 }
 
@@ -387,6 +486,26 @@ int enqueue_reverse(rbc_ctx *c, cudaStream_t s) {
     ++g_launches;
   }
   CKL();
+  return RBC_OK;
+}
+
+// Plans and tables of the resident loops of a 2-D context.
+int create_resident(rbc_ctx *c) {
+  if (c->L.ndim != 2) return RBC_OK;
+  size_t ll = 0;
+  cudaFree(c->res_ll);
+  c->res_ll = nullptr;
+  for (int dir = 0; dir < 2; ++dir) {
+    cudaFree(c->res_tiles[dir]);
+    c->res_tiles[dir] = nullptr;
+    ResPlan &P = c->res[dir];
+    if (!res_plan(&c->L, 1, dir == 0, c->share, &P)) continue;
+    const size_t tb = sizeof(ResTile) * P.tiles.size();
+    CK(cudaMalloc(&c->res_tiles[dir], tb));
+    CK(cudaMemcpy(c->res_tiles[dir], P.tiles.data(), tb, cudaMemcpyHostToDevice));
+    ll = std::max(ll, res_ll_bytes(P, dir == 0));
+  }
+  if (ll) CK(cudaMalloc(&c->res_ll, ll));
   return RBC_OK;
 }
 
@@ -573,6 +692,17 @@ int run_loop(rbc_ctx *c, int kind, enqueue_fn fn, cudaStream_t s) {
   return RBC_OK;
 }
 
+// Algorithm 1 with the record at the receivers (time-major, in c->seis_t).
+int run_model(rbc_ctx *c, const int *src, int nrec, const int *rec, const float *wavelet, cudaStream_t s) {
+  const bool res = resident(c, 0);
+  int rc = res ? check_nodes(c, src, nrec, rec) : upload_shot(c, src, nrec, rec, 1, s);
+  if (rc) return rc;
+  if (res && ((rc = check_capture(s)) || (rc = ensure_receivers(c, std::max(nrec, 1))))) return rc;
+  CK(cudaMemcpyAsync(c->wav, wavelet, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
+  if (res) return run_resident(c, 0, src, nrec, rec, 1, 1, 0, 0, 0, nullptr, nullptr, s);
+  return run_loop(c, 0, enq_model, s);
+}
+
 } // namespace
 
 // ===================================================================== ABI ==
@@ -682,6 +812,11 @@ int rbc_create(const rbc_grid *g, const float *a_dev, rbc_ctx **out) {
   }
   launch_copy_in(L, a_dev, c->a, 0);
   ++g_launches;
+  rc = create_resident(c);
+  if (rc) {
+    rbc_destroy(c);
+    return rc;
+  }
   rc = ensure_receivers(c, 64);
   if (rc) {
     rbc_destroy(c);
@@ -721,6 +856,14 @@ int rbc_set_coef(rbc_ctx *c, const float *a_dev, int check, void *stream) {
   return RBC_OK;
 }
 
+int rbc_set_share(rbc_ctx *c, int contexts) {
+  if (!c || contexts < 1) return fail(RBC_EINVAL, "ctx is NULL or contexts < 1");
+  if (contexts == c->share) return RBC_OK;
+  CK(cudaDeviceSynchronize());
+  c->share = contexts;
+  return create_resident(c);
+}
+
 int rbc_destroy(rbc_ctx *c) {
   if (!c) return RBC_OK;
   cudaDeviceSynchronize();
@@ -734,6 +877,9 @@ int rbc_destroy(rbc_ctx *c) {
   cudaFree(c->tile_ptr);
   cudaFree(c->seis_t);
   cudaFree(c->dmax);
+  for (ResTile *t : c->res_tiles) cudaFree(t);
+  cudaFree(c->res_ll);
+  cudaFree(c->res_blob);
   if (c->cap) cudaStreamDestroy(c->cap);
   if (c->err_host) cudaFreeHost(c->err_host);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -749,10 +895,7 @@ int rbc_model(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int nre
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  rc = upload_shot(c, src_host, nrec, rec_host, 1, s);
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(c->wav, wavelet_dev, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
-  rc = run_loop(c, 0, enq_model, s);
+  rc = run_model(c, src_host, nrec, rec_host, wavelet_dev, s);
   if (rc) return rc;
   if (nrec > 0) {
     launch_transpose(c->seis_t, seis_dev, c->g.nt + 1, nrec, s);
@@ -772,7 +915,12 @@ int rbc_rtm_shot(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int 
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  rc = upload_shot(c, src_host, nrec, rec_host, flags & RBC_REINJECT_SOURCE, s);
+  const int rein = flags & RBC_REINJECT_SOURCE, ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
+  const bool resf = resident(c, 0), resr = resident(c, 1);
+  rc = check_nodes(c, src_host, nrec, rec_host);
+  if (rc) return rc;
+  if ((resf || resr) && (rc = check_capture(s))) return rc;
+  rc = resf && resr ? ensure_receivers(c, std::max(nrec, 1)) : upload_shot(c, src_host, nrec, rec_host, rein, s);
   if (rc) return rc;
   CK(cudaMemcpyAsync(c->wav, wavelet_dev, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
   if (nrec > 0) {
@@ -780,18 +928,23 @@ int rbc_rtm_shot(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int 
     ++g_launches;
   }
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = run_loop(c, 1, enq_rtm_fwd, s);
+  rc = resf ? run_resident(c, 0, src_host, 0, nullptr, rein, 0, 0, 0, 0, nullptr, nullptr, s)
+            : run_loop(c, 1, enq_rtm_fwd, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = run_loop(c, 2, enq_rtm_rev, s);
+  rc = resr ? run_resident(c, 1, src_host, nrec, rec_host, rein, 0, 0, ow, 1, num_dev, den_dev, s)
+            : run_loop(c, 2, enq_rtm_rev, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
-  const int ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
+  c->have_panels = 0;  // the reverse pass consumed the panels
+  if (resr) {
+    CKL();
+    return RBC_OK;
+  }
   launch_accum_interior(c->L, c->num, num_dev, c->g.nb, top_rows(&c->g), c->g.nx, c->g.ny, c->g.nz, ow, s);
   launch_accum_interior(c->L, c->den, den_dev, c->g.nb, top_rows(&c->g), c->g.nx, c->g.ny, c->g.nz, ow, s);
   g_launches += 2;
   CKL();
-  c->have_panels = 0;  // the reverse pass consumed the panels
   return RBC_OK;
 }
 
@@ -897,10 +1050,7 @@ int rbc_fwi_forward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  rc = upload_shot(c, src_host, nrec, rec_host, 1, s);
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(c->wav, wavelet_dev, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
-  rc = run_loop(c, 0, enq_model, s);
+  rc = run_model(c, src_host, nrec, rec_host, wavelet_dev, s);
   if (rc) return rc;
   launch_fwi_residual(c->seis_t, dobs_dev, resid_dev, misfit_dev, nrec, c->g.nt, s);
   ++g_launches;
@@ -926,8 +1076,10 @@ int rbc_fwi_backward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, 
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  rc = upload_shot(c, src_host, nrec, rec_host, 1, s);
+  const bool res = resident(c, 1);
+  rc = res ? check_nodes(c, src_host, nrec, rec_host) : upload_shot(c, src_host, nrec, rec_host, 1, s);
   if (rc) return rc;
+  if (res && ((rc = check_capture(s)) || (rc = ensure_receivers(c, std::max(nrec, 1))))) return rc;
   CK(cudaMemcpyAsync(c->wav, wavelet_dev, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
   const int nt = c->g.nt;
   if (panels_dev) {
@@ -938,7 +1090,8 @@ int rbc_fwi_backward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, 
   // adjoint record: row m = -resid[.][m-1] / h^(2-d), injected as + h^(2-d) a row
   launch_fwi_adjoint_source(resid_dev, c->seis_t, nrec, nt, -1.0f, s);
   ++g_launches;
-  rc = run_loop(c, 3, enq_fwi_adj, s);
+  rc = res ? run_resident(c, 1, src_host, nrec, rec_host, 1, 0, 1, 1, 0, c->num, nullptr, s)
+           : run_loop(c, 3, enq_fwi_adj, s);
   if (rc) return rc;
   launch_fwi_finalize(c->L, c->num, c->a, grad_dev, c->g.nb, c->g.nx, c->g.nz, c->g.dt, c->g.h, s);
   ++g_launches;

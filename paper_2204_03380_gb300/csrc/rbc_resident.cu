@@ -1,0 +1,787 @@
+// rbc_resident.cu -- 2-D time loops that stay on the chip.
+//
+// A launch per time step moves every field through L2 at every step (forward
+// 16 bytes per node, fused reverse 60) and pays a launch's latency.  A grid of
+// up to about 2.1 M padded nodes (the 2421 x 871 survey grid, at 7 fields) has
+// room on the chip: 152 SMs hold 34 MB of shared memory and 39 MB of tensor
+// memory.  Here one cooperative launch runs a whole loop.  Each block keeps a
+// tile of 128 columns x H rows for all its steps: the two levels of each field
+// in shared memory; a and the imaging sums in registers and shared memory
+// (tiles of one or two rows per warp) or in tensor memory, which serves as a
+// thread-private store (32 lanes of a quarter x 512 columns; no MMA runs) and
+// leaves shared memory to the fields.  Only the tile's four edge rows and
+// columns leave the SM: they go to the neighbouring tiles as 8-byte words of
+// {value, level} through L2, so that a reader that finds the level it waits
+// for has the value with it -- no fence, no flag, one L2 round trip.  A word's
+// place alternates between even and odd levels: a writer is at most one level
+// ahead of its reader, because it needs the reader's own words to get there.
+// All blocks are resident (the launch is cooperative) and every wait is bounded.
+//
+// What bounds it: on the survey grid the fp32 pipes (59 packed operations per
+// four nodes and field, 1.6 us a step of the 3.9 us) and the exchange, about
+// 1.5 us from a tile's last row to its neighbours' first; on small grids the
+// exchange alone.  Measured (us per step; before, one launch per step): survey
+// forward 3.9 (6.1), forward + reverse 12.2 (18.8); 300 x 300 forward 1.5
+// (2.7), forward + reverse 4.5 (6.7).  Tensor memory for a and the sums: 8 us
+// per reverse step against 12.4 with the sums in registers (spilled) and a
+// read from L2 twice.  Tried and not kept: a warp-to-warp order (mbarriers)
+// instead of the block barrier at each step -- the warps drift apart and their
+// unrolled rows no longer fit the instruction cache (18 us per reverse step);
+// the same with the rows rolled up into a loop of two (9.8 us).
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <type_traits>
+
+#include "rbc_resident.cuh"
+#include "rbc_tile2d.cuh"
+
+namespace rbc {
+
+namespace {
+
+typedef unsigned long long u64;
+constexpr long long kResWait = 2000000000LL;  // about a second
+constexpr int kEdge = 4 * kTileX;             // words of a top or bottom halo (4 rows)
+
+__device__ __forceinline__ void ll_ld(const u64 *p, u64 &a, u64 &b) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void ll_st(u64 *p, float x, float y, uint32_t tag) {
+  u64 a, b;
+  asm volatile("mov.b64 %0, {%1, %2};" : "=l"(a) : "r"(__float_as_uint(x)), "r"(tag));
+  asm volatile("mov.b64 %0, {%1, %2};" : "=l"(b) : "r"(__float_as_uint(y)), "r"(tag));
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+__device__ __forceinline__ float ll_val(u64 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ bool ll_ok(u64 v, uint32_t tag) { return (uint32_t)(v >> 32) == tag; }
+
+// Four consecutive halo values of one lane: two 16-byte loads.
+struct Ll4 {
+  u64 v[4];
+  __device__ __forceinline__ void load(const u64 *p0, const u64 *p1) {
+    ll_ld(p0, v[0], v[1]);
+    ll_ld(p1, v[2], v[3]);
+  }
+  __device__ __forceinline__ bool ok(uint32_t tag) const {
+    return ll_ok(v[0], tag) && ll_ok(v[1], tag) && ll_ok(v[2], tag) && ll_ok(v[3], tag);
+  }
+  __device__ __forceinline__ float4 value() const {
+    return make_float4(ll_val(v[0]), ll_val(v[1]), ll_val(v[2]), ll_val(v[3]));
+  }
+  // Bounded wait for the values of `tag`; false if it gave up.
+  __device__ __forceinline__ bool wait(const u64 *p0, const u64 *p1, uint32_t tag) {
+    if (ok(tag)) return true;
+    const long long t0 = clock64();
+    do {
+      load(p0, p1);
+      if (ok(tag)) return true;
+    } while (clock64() - t0 < kResWait);
+    return false;
+  }
+};
+
+// Halo words of one tile, field and parity: rows above [4][2][32][2], rows
+// below [4][2][32][2], columns to the left [H][4], columns to the right [H][4].
+__host__ __device__ __forceinline__ int ll_words(int H) { return 2 * kEdge + 8 * H; }
+
+__device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// A warp's place in its tile (rows r0 .. r0 + RZ - 1) and this lane's ends of
+// the halo words (offsets from the exchange buffer, field 0, even levels).
+struct Place {
+  int lane, r0, rows, H;
+  bool up, dn, lr;            // rows above / below come from another tile; this lane moves a column halo
+  bool right;                 // ... of the right-hand side
+  u64 *in_lr, *in_tb;         // own tile: column halo of this lane's row; rows above (below: + kEdge)
+  u64 *out_lr, *out_up, *out_dn;
+};
+
+template <int RZ>
+__device__ __forceinline__ Place place_of(const ResArgs &A, const ResTile &T, int w, int lane, int H, int nf) {
+  Place W;
+  W.lane = lane;
+  W.r0 = w * RZ;
+  W.rows = T.rows;
+  W.H = H;
+  W.up = T.up >= 0;
+  W.dn = T.dn >= 0;
+  const size_t tw = (size_t)ll_words(H) * 2 * nf;
+  const int j = lane & 15;   // lane j: the left of row j, lane 16 + j: the right
+  W.right = lane >= 16;
+  const int side = W.right ? T.rt : T.lf;
+  W.lr = j < RZ && W.r0 + j < T.rows && side >= 0;
+  const int col = 4 * (W.r0 + (j < RZ ? j : 0));
+  W.in_lr = A.ll + blockIdx.x * tw + 2 * kEdge + (W.right ? 4 * H : 0) + col;
+  W.out_lr = A.ll + max(side, 0) * tw + 2 * kEdge + (W.right ? 0 : 4 * H) + col;
+  W.in_tb = A.ll + blockIdx.x * tw + 2 * lane;
+  W.out_up = A.ll + max(T.up, 0) * tw + kEdge + 2 * lane;
+  W.out_dn = A.ll + max(T.dn, 0) * tw + 2 * lane;
+  return W;
+}
+
+// Offset of a field's words of level `tag`, opaque so that the addresses
+// formed from it are not all kept in registers across the time loop.
+__device__ __forceinline__ int ll_off(int f, uint32_t tag, int H) {
+  int o = (2 * f + (int)(tag & 1)) * ll_words(H);
+  asm volatile("" : "+r"(o));
+  return o;
+}
+
+// Halo of level `tag` for this warp: the columns beside its rows into s_lr
+// ([H][2][4]); where its stencil reaches over the tile's edge, the rows above
+// into s_up[4][128] (or, for TIGHT, into the row queue's first four entries)
+// and the rows below into s_dn[4][128].
+template <int RZ, bool TIGHT>
+__device__ __forceinline__ bool halo_in(const Place &W, int f, uint32_t tag, float *s_lr, float *s_up, float *s_dn,
+                                        float4 *qa) {
+  const int o = ll_off(f, tag, W.H);
+  Ll4 c;
+  if (W.lr) c.load(W.in_lr + o, W.in_lr + o + 2);
+  bool ok = true;
+  // With fewer than four rows per warp, a warp reads only the halo rows its
+  // own rows reach (the others' next level may already be on its way): the
+  // rest of its four loads repeat the nearest of those.
+  if (W.up && W.r0 < 4) {  // rows r0 .. 3 of the four above
+    const u64 *b = W.in_tb + o;
+    Ll4 t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const u64 *p = b + (RZ < 4 ? max(k, W.r0) : k) * kTileX;
+      t[k].load(p, p + 64);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int kk = RZ < 4 ? max(k, W.r0) : k;
+      ok = t[k].wait(b + kk * kTileX, b + kk * kTileX + 64, tag) && ok;
+      if (TIGHT) qa[k] = t[k].value();
+      else *reinterpret_cast<float4 *>(s_up + kk * kTileX + 4 * W.lane) = t[k].value();
+    }
+  }
+  if (W.dn && W.r0 + RZ + 3 >= W.H) {  // rows 0 .. r0 + RZ + 3 - H of the four below
+    const u64 *b = W.in_tb + o + kEdge;
+    const int k1 = W.r0 + RZ + 3 - W.H;
+    Ll4 t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const u64 *p = b + (RZ < 4 ? min(k, k1) : k) * kTileX;
+      t[k].load(p, p + 64);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int kk = RZ < 4 ? min(k, k1) : k;
+      ok = t[k].wait(b + kk * kTileX, b + kk * kTileX + 64, tag) && ok;
+      *reinterpret_cast<float4 *>(s_dn + kk * kTileX + 4 * W.lane) = t[k].value();
+    }
+  }
+  if (W.lr) {
+    ok = c.wait(W.in_lr + o, W.in_lr + o + 2, tag) && ok;
+    *reinterpret_cast<float4 *>(s_lr + ((W.r0 + (W.lane & 15)) * 2 + (W.right ? 1 : 0)) * 4) = c.value();
+  }
+  __syncwarp();
+  return ok;
+}
+
+// This warp's edge rows and columns of a finished level, from shared memory,
+// to the neighbours' halo words.
+template <int RZ>
+__device__ __forceinline__ void halo_out(const Place &W, int f, uint32_t tag, const float *s) {
+  const int o = ll_off(f, tag, W.H);
+  if (W.lr) {
+    const float4 v = lds4(s + (W.r0 + (W.lane & 15)) * kTileX + (W.right ? kTileX - 4 : 0));
+    ll_st(W.out_lr + o, v.x, v.y, tag);
+    ll_st(W.out_lr + o + 2, v.z, v.w, tag);
+  }
+  if (W.up && W.r0 < 4) {
+#pragma unroll
+    for (int i = 0; i < (RZ < 4 ? RZ : 4); ++i) {
+      const int r = W.r0 + i;
+      if (RZ >= 4 || r < 4) {  // rows past a short last tile are zero in its buffer, and are sent
+        const float4 v = lds4(s + r * kTileX + 4 * W.lane);
+        u64 *b = W.out_up + o + r * kTileX;
+        ll_st(b, v.x, v.y, tag);
+        ll_st(b + 64, v.z, v.w, tag);
+      }
+    }
+  }
+  if (W.dn && W.r0 + RZ > W.H - 4) {
+#pragma unroll
+    for (int i = 0; i < (RZ < 4 ? RZ : 4); ++i) {
+      const int r = W.r0 + (RZ < 4 ? i : RZ - 4 + i), k = r - (W.H - 4);
+      if (RZ >= 4 || k >= 0) {
+        const float4 v = lds4(s + r * kTileX + 4 * W.lane);
+        u64 *b = W.out_dn + o + k * kTileX;
+        ll_st(b, v.x, v.y, tag);
+        ll_st(b + 64, v.z, v.w, tag);
+      }
+    }
+  }
+}
+
+// One level of one field over this warp's rows: pre(j) starts the loads of
+// what is kept elsewhere (a, the imaging sums), body(j, c, old, lap) finishes
+// row j and stores it.  The z differences D_k (rbc_stencil.cuh) march down the
+// rows in registers.  c0 / n0: the level's / the overwritten level's tile rows
+// in shared memory; up / dn: the four rows above / below the warp's rows.
+template <int RZ, bool TIGHT, typename Pre, typename Body>
+__device__ __forceinline__ void sweep(const Place &W, const float *smem, int c0, int n0, const float *up,
+                                      const float *dn, bool have_up, const float4 *qa, int lofs, int lstep, int rofs,
+                                      int rstep, Pre pre, Body body) {
+  const int lane = W.lane;
+  const float *own = smem + c0 + W.r0 * kTileX + 4 * lane;
+  const float *lp = smem + lofs + (lane == 0 ? 0 : c0), *rp = smem + rofs + (lane == 31 ? 0 : c0);
+  const float *np = smem + n0 + W.r0 * kTileX + 4 * lane;
+  auto row = [&](int i) {  // row i - 4 of the warp
+    return i < 4 ? (TIGHT && have_up ? qa[i < 4 ? i : 0] : lds4(up + i * kTileX + 4 * lane))
+                 : i < RZ + 4 ? lds4(own + (i - 4) * kTileX) : lds4(dn + (i - RZ - 4) * kTileX + 4 * lane);
+  };
+  float4 q[RZ + 8], D[4][RZ + 4];  // D[k - 1][i] = D_k at row i - 4 (of each k, the last k rows are live)
+#pragma unroll
+  for (int i = 0; i < 8; ++i) q[i] = row(i);
+#pragma unroll
+  for (int k = 1; k <= 4; ++k)
+#pragma unroll
+    for (int i = 4 - k; i < 4; ++i) D[k - 1][i] = sub4(q[i + k], q[i]);
+#pragma unroll
+  for (int j = 0; j < RZ; ++j) {
+    if (W.r0 + j >= W.rows) break;
+    pre(j);
+    const float4 lf = lds4(lp + j * lstep), rt = lds4(rp + j * rstep), po = lds4(np + j * kTileX);
+    q[j + 8] = row(j + 8);
+    float4 z[4];
+#pragma unroll
+    for (int k = 1; k <= 4; ++k) {
+      D[k - 1][j + 4] = sub4(q[j + 4 + k], q[j + 4]);
+      z[k - 1] = sub4(D[k - 1][j + 4], D[k - 1][j + 4 - k]);
+    }
+    body(j, q[j + 4], po, lap_shared(lf, q[j + 4], rt, z));
+  }
+}
+
+// This warp's receivers: the first K * 32 in registers (node's place in the
+// tile, receiver), the rest read from the table at every step.
+template <int K>
+struct Recs {
+  int beg, end, loc[K], id[K];
+  __device__ __forceinline__ void load(const int *ptr, const int2 *rec, int cell, int lane, bool any) {
+    beg = any ? ptr[cell] : 0;
+    end = any ? ptr[cell + 1] : 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const int k = beg + lane + 32 * i;
+      const int2 c = k < end ? __ldg(rec + k) : make_int2(0, -1);
+      loc[i] = c.x;
+      id[i] = c.y;
+    }
+  }
+};
+
+// Shared memory of one field's buffer: H rows, and unless TIGHT four rows
+// above and below that the halo is received into.
+template <bool TIGHT>
+__host__ __device__ __forceinline__ int buf_floats(int H) { return (H + (TIGHT ? 0 : 8)) * kTileX; }
+
+// ------------------------------------------------------------- forward ----
+template <int RZ, int MAXW, int MINB>
+__global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, const int H) {
+  extern __shared__ __align__(16) float smem[];
+  const int fl = buf_floats<false>(H), h4 = 4 * kTileX;
+  float *s_a = smem + 2 * fl;
+  float *s_lr = s_a + H * kTileX;       // [H][2][4]
+  const ResTile T = A.tiles[blockIdx.x];
+  const ResShot &S = A.shots[T.shot];
+  const int lane = threadIdx.x, w = threadIdx.y, nthr = 32 * blockDim.y, tid = 32 * w + lane;
+  const int origin = S.L.origin, pitch = S.L.pitch, NX4 = S.L.NX4;
+  const Place W = place_of<RZ>(A, T, w, lane, H, 1);
+  for (int i = tid; i < (2 * fl + H * kTileX + 8 * H) / 4; i += nthr) *reinterpret_cast<float4 *>(smem + 4 * i) = zero4();
+  __syncthreads();
+  for (int i = tid; i < T.rows * 32; i += nthr) {
+    const int r = i >> 5, x = T.x0 + 4 * (i & 31);
+    if (x < NX4) *reinterpret_cast<float4 *>(s_a + 4 * i) = ldg4(S.a + origin + (T.z0 + r) * pitch + x);
+  }
+  const int x0 = T.x0 + 4 * lane;
+  const bool xok = x0 < NX4;
+  const int nrec = S.info->nrec;
+  const int src = S.info->src_off;
+  const float fsc = S.info->src_fwd;
+  const int2 *cell_rec = S.cell_rec;
+  float *seis_t = S.seis_t;
+  const int cell = (blockIdx.x - S.tile0) * blockDim.y + w;
+  constexpr int K = RZ < 10 ? 4 : 2;
+  Recs<K> rec;
+  rec.load(S.cell_ptr, cell_rec, cell, lane, A.sample != 0);
+  auto record = [&](int n, const float *p) {  // p^n at this warp's receivers
+    float *row = seis_t + (long long)n * nrec;
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      if (rec.id[i] >= 0) row[rec.id[i]] = p[rec.loc[i]];
+    for (int k = rec.beg + 32 * K + lane; k < rec.end; k += 32) {
+      const int2 c = __ldg(cell_rec + k);
+      row[c.y] = p[c.x];
+    }
+  };
+  const int row0 = origin + (T.z0 + W.r0) * pitch;  // this warp's first row
+  const bool has_src = src >= row0 + T.x0 && src < row0 + T.x0 + RZ * pitch;
+  // left / right neighbours of the lane's four columns: the tile's own row, or the halo columns
+  const int lstep = lane == 0 ? 8 : kTileX, rstep = lane == 31 ? 8 : kTileX;
+  const int lofs = lane == 0 ? (int)(s_lr - smem) + W.r0 * 8 : W.r0 * kTileX + 4 * lane - 4;
+  const int rofs = lane == 31 ? (int)(s_lr - smem) + W.r0 * 8 + 4 : W.r0 * kTileX + 4 * lane + 4;
+  const float *pa = s_a + W.r0 * kTileX + 4 * lane;
+  __syncthreads();
+  const int nt = A.nt;
+  bool ok = true;
+  float f = has_src ? A.wav[0] * fsc : 0.f, f_next = 0.f;
+  for (int n = 0; n < nt; ++n) {
+    if (has_src && n + 1 < nt) f_next = A.wav[n + 1];  // in flight during this step
+    const int c0 = (n & 1 ? fl : 0) + h4, n0 = (n & 1 ? 0 : fl) + h4;
+    float *cur = smem + c0, *np = smem + n0 + W.r0 * kTileX + 4 * lane;
+    if (n > 0) ok = halo_in<RZ, false>(W, 0, (uint32_t)n, s_lr, cur - h4, cur + H * kTileX, nullptr);
+    sweep<RZ, false>(W, smem, c0, n0, cur + W.r0 * kTileX - h4, cur + (W.r0 + RZ) * kTileX, false, nullptr, lofs, lstep,
+                     rofs, rstep, [](int) {},
+                     [&](int j, const float4 c, const float4 po, const float4 lap) {
+                       const float4 av = lds4(pa + j * kTileX);
+                       float4 v = leap_fin<false>(c, po, av, lap, nullptr);
+                       if (has_src) {
+                         const int d = src - (row0 + j * pitch + x0);
+                         if ((unsigned)d < 4u) point_sub(v, d, cmp(av, d) * f);
+                       }
+                       if (xok) st4(np + j * kTileX, v);
+                     });
+    __syncwarp();
+    if (n + 1 < nt) halo_out<RZ>(W, 0, (uint32_t)n + 1, smem + n0);
+    record(n, cur);
+    f = f_next * fsc;
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicOr_system(A.err, 1);
+      return;
+    }
+  }
+  record(nt, smem + (nt & 1 ? fl : 0) + h4);
+  // the last two levels, for the reverse loop and rbc_get_panels
+  for (int j = 0; j < RZ; ++j) {
+    const int r = W.r0 + j;
+    if (r < W.rows && xok) {
+      const int o = row0 + j * pitch + x0;
+      st4(S.p[0] + o, lds4(smem + h4 + r * kTileX + 4 * lane));
+      st4(S.p[1] + o, lds4(smem + fl + h4 + r * kTileX + 4 * lane));
+    }
+  }
+}
+
+// ------------------------------------------------------------- reverse ----
+// acc + a b with both roundings, as the one-launch-per-step kernels add up
+__device__ __forceinline__ float4 madd4(const float4 a, const float4 b, const float4 c) {
+  const float2 l = __fadd2_rn(__fmul2_rn(lo2(a), lo2(b)), lo2(c)), h = __fadd2_rn(__fmul2_rn(hi2(a), hi2(b)), hi2(c));
+  return make_float4(l.x, l.y, h.x, h.y);
+}
+
+// What a thread keeps of its own nodes besides the fields: a and the imaging
+// sums (FWI: the gradient sum in num).  Small tiles: a in shared memory, the
+// sums in registers.
+template <int RZ, bool kGrad>
+struct KeepReg {
+  const float *pa;
+  float4 num[RZ], den[kGrad ? 1 : RZ];
+  __device__ __forceinline__ void init(float *s_a, const Place &W) {
+    pa = s_a + W.r0 * kTileX + 4 * W.lane;
+#pragma unroll
+    for (int j = 0; j < RZ; ++j) {
+      num[j] = zero4();
+      if (!kGrad) den[j] = zero4();
+    }
+  }
+  __device__ __forceinline__ void pre_a(int) {}
+  __device__ __forceinline__ void pre_all(int) {}
+  __device__ __forceinline__ float4 a(int j) { return lds4(pa + j * kTileX); }
+  __device__ __forceinline__ void add(int j, const float4 c, const float4 b) {
+    num[j] = madd4(c, b, num[j]);
+    if (!kGrad) den[j] = madd4(c, c, den[j]);
+  }
+  __device__ __forceinline__ void flush() {}
+  __device__ __forceinline__ void sums(int j, float4 &n, float4 &d) {
+    n = num[j];
+    if (!kGrad) d = den[j];
+  }
+};
+
+__device__ __forceinline__ void tm_ld4(uint32_t ta, float4 &v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(ta));
+}
+__device__ __forceinline__ void tm_st4(uint32_t ta, const float4 v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ta), "f"(v.x), "f"(v.y), "f"(v.z),
+               "f"(v.w)
+               : "memory");
+}
+// Wait for this thread's tensor-memory loads; the loaded values are used after it only.
+__device__ __forceinline__ void tm_wait(float4 &a) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(a.x), "+f"(a.y), "+f"(a.z), "+f"(a.w)::"memory");
+}
+__device__ __forceinline__ void tm_tie(float4 &a) { asm volatile("" : "+f"(a.x), "+f"(a.y), "+f"(a.z), "+f"(a.w)); }
+
+// Large tiles: a and the sums in tensor memory, used as a thread-private store
+// (a warp reaches the 32 lanes of its quarter; 12 columns per row: a, num, den).
+template <int RZ, bool kGrad>
+struct KeepTm {
+  uint32_t ta;
+  float4 av, nv, dv;
+  __device__ __forceinline__ void pre_a(int j) { tm_ld4(ta + 12 * j, av); }
+  __device__ __forceinline__ void pre_all(int j) {
+    tm_ld4(ta + 12 * j, av);
+    tm_ld4(ta + 12 * j + 4, nv);
+    if (!kGrad) tm_ld4(ta + 12 * j + 8, dv);
+  }
+  __device__ __forceinline__ float4 a(int) {
+    tm_wait(av);
+    return av;
+  }
+  __device__ __forceinline__ void add(int j, const float4 c, const float4 b) {
+    tm_tie(nv);
+    nv = madd4(c, b, nv);
+    if (!kGrad) {
+      tm_tie(dv);
+      dv = madd4(c, c, dv);
+    }
+    __syncwarp();
+    tm_st4(ta + 12 * j + 4, nv);
+    if (!kGrad) tm_st4(ta + 12 * j + 8, dv);
+  }
+  __device__ __forceinline__ void flush() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+  __device__ __forceinline__ void sums(int j, float4 &n, float4 &d) {
+    tm_ld4(ta + 12 * j + 4, nv);
+    if (!kGrad) tm_ld4(ta + 12 * j + 8, dv);
+    tm_wait(nv);
+    n = nv;
+    if (!kGrad) {
+      tm_tie(dv);
+      d = dv;
+    }
+  }
+};
+constexpr int tm_cols(int rz, int warps) {
+  const int c = (warps + 3) / 4 * rz * 12;
+  return c <= 128 ? 128 : c <= 256 ? 256 : 512;
+}
+
+template <int RZ, int MAXW, int MINB, bool TIGHT, bool TM, bool kGrad>
+__global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, const int H) {
+  extern __shared__ __align__(16) float smem[];
+  const int fl = buf_floats<TIGHT>(H), h4 = TIGHT ? 0 : 4 * kTileX;
+  float *s_lr = smem + 4 * fl;        // [H][2][4], the warp's own rows: both fields in turn
+  // TIGHT: [4][128] rows below, read by the last warp, both fields in turn; without TM: a [H][128]
+  float *s_x = s_lr + 8 * H;
+  const int xfl = ((TIGHT ? 4 : 0) + (TM ? 0 : H)) * kTileX;
+  uint32_t *s_tm = reinterpret_cast<uint32_t *>(s_x + xfl);  // TM: the tensor memory's address
+  static_assert(TM || !TIGHT, "the tight layout leaves no shared memory for a");
+  const ResTile T = A.tiles[blockIdx.x];
+  const ResShot &S = A.shots[T.shot];
+  const int lane = threadIdx.x, w = threadIdx.y, nthr = 32 * blockDim.y, tid = 32 * w + lane;
+  const int origin = S.L.origin, pitch = S.L.pitch, NX4 = S.L.NX4;
+  const Place W = place_of<RZ>(A, T, w, lane, H, 2);
+  const int nt = A.nt;
+  constexpr int TC = tm_cols(RZ, MAXW);
+  if (TM && w == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+        (uint32_t)__cvta_generic_to_shared(s_tm)), "r"(TC));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  for (int i = tid; i < (4 * fl + 8 * H + xfl) / 4; i += nthr)
+    *reinterpret_cast<float4 *>(smem + 4 * i) = zero4();
+  if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (TM) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  for (int i = tid; i < T.rows * 32; i += nthr) {
+    const int r = i >> 5, x = T.x0 + 4 * (i & 31), o = origin + (T.z0 + r) * pitch + x;
+    if (x < NX4) {
+      st4(smem + h4 + 4 * i, ld4(S.p[0] + o));
+      st4(smem + fl + h4 + 4 * i, ld4(S.p[1] + o));
+      if (!TM) st4(s_x + 4 * i, ldg4(S.a + o));
+    }
+  }
+  const int x0 = T.x0 + 4 * lane;
+  const bool xok = x0 < NX4;
+  const int nrec = S.info->nrec;
+  const int src = S.info->src_off;
+  const float fsc = S.info->src_rev, rsc = S.info->rec_scale;
+  const int2 *cell_rec = S.cell_rec;
+  const float *seis_t = S.seis_t, *sa = S.a + origin + T.z0 * pitch + T.x0;
+  const int cell = (blockIdx.x - S.tile0) * blockDim.y + w;
+  constexpr int K = 4;
+  Recs<K> rec;
+  rec.load(S.cell_ptr, cell_rec, cell, lane, true);
+  float rec_a[K], rec_s[K];  // scale * a at the receivers; the record's values, loaded a step ahead
+  auto load_s = [&](int row) {
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      if (rec.id[i] >= 0) rec_s[i] = seis_t[(long long)row * nrec + rec.id[i]];
+  };
+#pragma unroll
+  for (int i = 0; i < K; ++i)
+    rec_a[i] = rec.id[i] >= 0 ? rsc * __ldg(sa + (rec.loc[i] / kTileX) * pitch + rec.loc[i] % kTileX) : 0.f;
+  load_s(kGrad ? A.nt + 1 : A.nt);
+  const int row0 = origin + (T.z0 + W.r0) * pitch;
+  const bool has_src = src >= row0 + T.x0 && src < row0 + T.x0 + RZ * pitch;
+  const int lstep = lane == 0 ? 8 : kTileX, rstep = lane == 31 ? 8 : kTileX;
+  const int lofs = lane == 0 ? (int)(s_lr - smem) + W.r0 * 8 : W.r0 * kTileX + 4 * lane - 4;
+  const int rofs = lane == 31 ? (int)(s_lr - smem) + W.r0 * 8 + 4 : W.r0 * kTileX + 4 * lane + 4;
+  const int own = W.r0 * kTileX + 4 * lane;
+  const bool top = W.r0 == 0, last = W.r0 + RZ == H;  // TIGHT: the warps at the tile's edges
+  uint32_t tmem = 0;
+  std::conditional_t<TM, KeepTm<RZ, kGrad>, KeepReg<RZ, kGrad>> keep;
+  if constexpr (TM) {
+    tmem = *s_tm;
+    keep.ta = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * RZ * 12);
+#pragma unroll 1
+    for (int j = 0; j < RZ; ++j) {
+      const float4 av = W.r0 + j < T.rows && xok ? ldg4(S.a + row0 + j * pitch + x0) : zero4();
+      __syncwarp();
+      tm_st4(keep.ta + 12 * j, av);
+      tm_st4(keep.ta + 12 * j + 4, zero4());
+      tm_st4(keep.ta + 12 * j + 8, zero4());
+    }
+    keep.flush();
+  } else {
+    keep.init(s_x, W);
+  }
+  __syncthreads();
+  bool ok = true;
+  float f_next = 0.f;
+  for (int t = 0; t <= nt; ++t) {
+    const float f = f_next * fsc;
+    if (has_src && t < nt) f_next = A.wav[nt - 1 - t];  // in flight during this step
+    // p^R level n; pbar level n (FWI: adjoint level n + 1)
+    const int n = nt - t, pr = n & 1, pb = kGrad ? pr ^ 1 : pr;
+    const int rc0 = pr * fl + h4, rn0 = (pr ^ 1) * fl + h4, bc0 = (2 + pb) * fl + h4, bn0 = (2 + (pb ^ 1)) * fl + h4;
+    const bool do_r = t > 0 && (kGrad || n > 0), do_b = kGrad || n > 0;
+    float4 qa[4];
+    if (TIGHT) qa[0] = qa[1] = qa[2] = qa[3] = zero4();
+    if (do_r) {
+      float *rc = smem + rc0;
+      ok = halo_in<RZ, TIGHT>(W, 0, (uint32_t)t, s_lr, rc - h4, TIGHT ? s_x : rc + H * kTileX, qa) && ok;
+      sweep<RZ, TIGHT>(W, smem, rc0, rn0, rc + W.r0 * kTileX - 4 * kTileX,
+                       TIGHT && last ? s_x : rc + (W.r0 + RZ) * kTileX, top, qa, lofs, lstep, rofs, rstep,
+                       [&](int j) { keep.pre_all(j); },
+                       [&](int j, const float4 c, const float4 po, const float4 lap) {
+                         const float4 cb = lds4(smem + bc0 + own + j * kTileX), av = keep.a(j);
+                         float4 inc, v = leap_fin<kGrad>(c, po, av, lap, &inc);
+                         if (has_src) {
+                           const int d = src - (row0 + j * pitch + x0);
+                           if ((unsigned)d < 4u) {
+                             point_sub(v, d, cmp(av, d) * f);
+                             if (kGrad) point_sub(inc, d, cmp(av, d) * f);
+                           }
+                         }
+                         keep.add(j, kGrad ? inc : c, cb);
+                         if (xok) st4(smem + rn0 + own + j * kTileX, v);
+                       });
+      keep.flush();
+    } else if (!kGrad) {
+#pragma unroll
+      for (int j = 0; j < RZ; ++j) {
+        if (W.r0 + j >= W.rows) break;
+        keep.pre_all(j);
+        keep.a(j);
+        keep.add(j, lds4(smem + rc0 + own + j * kTileX), lds4(smem + bc0 + own + j * kTileX));
+      }
+      keep.flush();
+    }
+    __syncwarp();
+    if (t < nt) halo_out<RZ>(W, 0, (uint32_t)t + 1, smem + rn0);
+    if (do_b) {
+      float *bc = smem + bc0, *bn = smem + bn0;
+      if (t > 0)  // level nt is zero everywhere
+        ok = halo_in<RZ, TIGHT>(W, 1, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
+      sweep<RZ, TIGHT>(W, smem, bc0, bn0, bc + W.r0 * kTileX - 4 * kTileX,
+                       TIGHT && last ? s_x : bc + (W.r0 + RZ) * kTileX, top, qa, lofs, lstep, rofs, rstep,
+                       [&](int j) { keep.pre_a(j); },
+                       [&](int j, const float4 c, const float4 po, const float4 lap) {
+                         const float4 v = leap_fin<false>(c, po, keep.a(j), lap, nullptr);
+                         if (xok) st4(bn + own + j * kTileX, v);
+                       });
+      __syncwarp();
+      if (rec.end > rec.beg) {
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+          if (rec.id[i] >= 0) atomicAdd(bn + rec.loc[i], rec_a[i] * rec_s[i]);
+        const int r = kGrad ? n + 1 : n;  // row of the record
+        for (int k = rec.beg + 32 * K + lane; k < rec.end; k += 32) {
+          const int2 c = __ldg(cell_rec + k);
+          const float av = __ldg(sa + (c.x / kTileX) * pitch + c.x % kTileX);
+          atomicAdd(bn + c.x, rsc * av * __ldg(seis_t + (long long)r * nrec + c.y));
+        }
+        load_s(r - 1);
+        __syncwarp();
+      }
+      if (t < nt) halo_out<RZ>(W, 1, (uint32_t)t + 1, bn);
+    }
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicOr_system(A.err, 1);
+      break;
+    }
+  }
+  // outputs (not after a wait that gave up)
+#pragma unroll
+  for (int j = 0; j < RZ; ++j) {
+    const int z = T.z0 + W.r0 + j;
+    float4 n4, d4;
+    keep.sums(j, n4, d4);
+    if (!ok || W.r0 + j >= W.rows || z < S.iz0 || z >= S.iz1) continue;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int x = x0 + e;
+      if (x < S.ix0 || x >= S.ix1) continue;
+      const long long o = A.dense ? (long long)(z - S.iz0) * (S.ix1 - S.ix0) + x - S.ix0
+                                  : (long long)(row0 + j * pitch + x);
+      S.num[o] = A.overwrite ? cmp(n4, e) : S.num[o] + cmp(n4, e);
+      if (!kGrad) S.den[o] = A.overwrite ? cmp(d4, e) : S.den[o] + cmp(d4, e);
+    }
+  }
+  if (TM) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC));
+  }
+}
+
+// ----------------------------------------------------------- host side ----
+inline int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+struct Variant {
+  int rz, maxw, minb;
+  bool tight, tm;
+  const void *fwd, *rev, *grad;
+};
+#define RBC_RES_VARIANT(RZ, MAXW, MINB, TIGHT, TM)                           \
+  {RZ, MAXW, MINB, TIGHT, TM, (const void *)k_res_fwd<RZ, MAXW, MINB>,       \
+   (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, false>,                \
+   (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, true>}
+// Rows per warp, most warps per block, blocks per SM, layout.  res_plan takes
+// the first that holds the grid: with few rows per warp a step is short (300 x
+// 300 forward: 1.6 / 1.9 / 2.5 / 2.8 / 3.1 us with 1 / 2 / 4 / 7 / 10 rows).
+// One or two rows per warp run 8 warps (two blocks to an SM); the others,
+// whose kernels allocate tensor memory and so run one block per SM, as few
+// warps as fit, which spreads the grid over the SMs (1500 x 800 forward +
+// reverse: 9.3 us with 10 warps of 7 rows, 11.2 with 15).  The last is the
+// tallest tile whose four buffers fit 227 KB: TIGHT keeps no halo rows in them.
+const Variant kVariants[] = {
+    RBC_RES_VARIANT(1, 8, 2, false, false), RBC_RES_VARIANT(2, 8, 2, false, false),
+    RBC_RES_VARIANT(4, 16, 1, false, true), RBC_RES_VARIANT(7, 15, 1, true, true),
+    RBC_RES_VARIANT(10, 11, 1, true, true),
+};
+
+size_t res_smem(bool fwd, int H, const Variant &V) {
+  const size_t rows = fwd ? 3 * H + 16 : V.tight ? 4 * H + 4 : 4 * (H + 8) + (V.tm ? 0 : H);
+  return sizeof(float) * (rows * kTileX + 8 * (size_t)H) + (!fwd && V.tm ? 16 : 0);
+}
+
+} // namespace
+
+bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out) {
+  out->variant = -1;
+  const char *env = getenv("RBC_RESIDENT");  // 0: one launch per step
+  if (env && env[0] == '0') return false;
+  int dev = 0, sms = 0, maxsm = 0, coop = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+    cudaGetLastError();
+    return false;
+  }
+  int force_v = -1, force_w = -1;
+  if (const char *e = getenv("RBC_RES_TILE")) sscanf(e, "%d,%d", &force_v, &force_w);
+  int best_v = -1, best_w = 0;
+  for (int v = 0; best_v < 0 && v < (int)(sizeof kVariants / sizeof kVariants[0]); ++v) {
+    const Variant &V = kVariants[v];
+    int nzmax = 1;
+    for (int s = 0; s < nshots; ++s) nzmax = std::max(nzmax, L[s].NZ);
+    // one or two rows per warp: the tallest tiles (two blocks to an SM); more: the lowest that fit (one)
+    const int top = std::min(V.maxw, std::max(cdiv(nzmax, V.rz), cdiv(4, V.rz)));
+    for (int i = 1; best_v < 0 && i <= top; ++i) {
+      const int nw = V.rz < 4 ? top + 1 - i : i;
+      if (force_v >= 0 && (v != force_v || (force_w > 0 && nw != force_w))) continue;
+      const int H = nw * V.rz;
+      if (H < 4) continue;
+      const size_t sm = res_smem(fwd, H, V);
+      if (sm > (size_t)maxsm) continue;
+      long long blocks = 0;
+      for (int s = 0; s < nshots; ++s) blocks += (long long)cdiv(L[s].NX, kTileX) * cdiv(L[s].NZ, H);
+      int per = 1 << 20;
+      for (const void *fn : {fwd ? V.fwd : V.rev, fwd ? V.fwd : V.grad}) {
+        int k = 0;
+        // the limit is raised to the device's for every plan alike: contexts on other threads share it
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, 32 * nw, sm) != cudaSuccess)
+          k = 0;
+        per = std::min(per, k);
+      }
+      if (blocks * share <= (long long)per * sms) best_v = v, best_w = nw;
+    }
+  }
+  cudaGetLastError();
+  if (best_v < 0) return false;
+  const Variant &V = kVariants[best_v];
+  out->variant = best_v;
+  out->rz = V.rz;
+  out->warps = best_w;
+  out->H = best_w * V.rz;
+  out->smem = res_smem(fwd, out->H, V);
+  out->tiles.clear();
+  out->tile0.assign(1, 0);
+  for (int s = 0; s < nshots; ++s) {
+    const int gx = cdiv(L[s].NX, kTileX), gz = cdiv(L[s].NZ, out->H), t0 = (int)out->tiles.size();
+    for (int bz = 0; bz < gz; ++bz)
+      for (int bx = 0; bx < gx; ++bx) {
+        const int i = t0 + bz * gx + bx;
+        ResTile T;
+        T.shot = s;
+        T.x0 = bx * kTileX;
+        T.z0 = bz * out->H;
+        T.rows = std::min(out->H, L[s].NZ - T.z0);
+        T.up = bz > 0 ? i - gx : -1;
+        T.dn = bz + 1 < gz ? i + gx : -1;
+        T.lf = bx > 0 ? i - 1 : -1;
+        T.rt = bx + 1 < gx ? i + 1 : -1;
+        out->tiles.push_back(T);
+      }
+    out->tile0.push_back((int)out->tiles.size());
+  }
+  out->blocks = (int)out->tiles.size();
+  return true;
+}
+
+size_t res_ll_bytes(const ResPlan &P, bool fwd) {
+  return sizeof(u64) * (size_t)P.blocks * (fwd ? 1 : 2) * 2 * ll_words(P.H);
+}
+
+void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc) {
+  const int t = (z / P.H) * cdiv(L.NX, kTileX) + x / kTileX, r = z % P.H;
+  *cell = t * P.warps + r / P.rz;
+  *loc = r * kTileX + x % kTileX;
+}
+
+cudaError_t res_launch(const ResPlan &P, bool fwd, const ResArgs &A, cudaStream_t s) {
+  const Variant &V = kVariants[P.variant];
+  const void *fn = fwd ? V.fwd : (A.grad ? V.grad : V.rev);
+  cudaError_t e = cudaMemsetAsync(A.ll, 0, res_ll_bytes(P, fwd), s);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(P.blocks);
+  cfg.blockDim = dim3(32, P.warps);
+  cfg.dynamicSmemBytes = P.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ResArgs a = A;
+  int H = P.H;
+  void *args[2] = {&a, &H};
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+} // namespace rbc

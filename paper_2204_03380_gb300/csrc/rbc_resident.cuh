@@ -1,0 +1,67 @@
+// rbc_resident.cuh -- tables of the resident 2-D time loops (rbc_resident.cu),
+// shared by the single-shot contexts (rbc_abi.cu) and the batches (rbc_batch.cu).
+#pragma once
+
+#include <vector>
+
+#include "rbc_internal.cuh"
+
+namespace rbc {
+
+// One block's tile: 128 columns x `rows` rows of one shot's padded grid.
+struct ResTile {
+  int shot;
+  int x0, z0;
+  int rows;       // rows of the grid in this tile (the last tile of a column may have fewer than H)
+  int up, dn, lf, rt;  // neighbouring tiles (index into the tile table), or -1
+};
+
+// One shot: its fields in the pitched layout and the per-call tables.
+struct ResShot {
+  Lay L;
+  const float *a;
+  float *p[2];              // level m in p[m & 1]: written by the forward loop, read by the reverse loop
+  const ShotInfo *info;
+  float *seis_t;            // [levels][nrec] time-major record
+  const int *cell_ptr;      // receivers of each (tile, warp) of this shot's tile range (CSR)
+  const int2 *cell_rec;     // {node's place in the tile (row * 128 + column), receiver index}
+  float *num, *den;         // outputs of the reverse loop (see ResArgs)
+  int tile0;                // this shot's first tile
+  int ix0, ix1, iz0, iz1;   // interior box in padded nodes
+};
+
+struct ResArgs {
+  const ResTile *tiles;
+  const ResShot *shots;
+  unsigned long long *ll;   // halo exchange words, zeroed before the launch
+  const float *wav;         // f[0..nt-1]
+  int nt;
+  int sample;               // forward: record every level at the receivers
+  int grad;                 // reverse: 1 = FWI gradient (num += mu p_tt), 0 = imaging integrals
+  int overwrite;            // reverse: outputs are set, not added to
+  int dense;                // reverse: num / den are dense interior arrays (else pitched)
+  int *err;
+};
+
+// Tiling of a resident loop over one or several grids: `warps` warps of `rz`
+// rows per block (H = warps * rz rows per tile), `blocks` blocks, all resident.
+struct ResPlan {
+  int variant = -1;         // index into the kernel variants, -1: does not fit
+  int rz = 0, warps = 0, H = 0;
+  int blocks = 0;
+  size_t smem = 0;
+  std::vector<ResTile> tiles;
+  std::vector<int> tile0;   // first tile of each shot, then the tile count
+};
+
+// Plan for the forward / reverse loop of the given layouts (variant -1 when
+// they do not fit on this device at once); share: the device is shared by that
+// many such loops.
+bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out);
+size_t res_ll_bytes(const ResPlan &P, bool fwd);
+// The (tile, warp) cell that owns a node, within its shot's tiles, and the
+// node's place in the tile.
+void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc);
+cudaError_t res_launch(const ResPlan &P, bool fwd, const ResArgs &A, cudaStream_t s);
+
+} // namespace rbc

@@ -51,6 +51,8 @@ def _pool(grid, a, n, device):
     pool = _POOL.setdefault(key, [])
     while len(pool) < n:
         pool.append((N.rbc_create(grid, a), torch.cuda.Stream(device)))
+    for ctx, _ in pool[:n]:
+        N.rbc_set_share(ctx, n)   # (nothing to do unless the number of shots in flight changed)
     return pool[:n]
 
 
