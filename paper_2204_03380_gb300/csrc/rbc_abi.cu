@@ -128,9 +128,9 @@ struct rbc_ctx {
   int *err_dev = nullptr;
   int fault = 0;  // rbc_inject_fault: applies to the next call only
   // 2-D grids that fit on the chip: the whole time loop as one launch
-  // (rbc_resident.cu), 0 forward, 1 reverse (variant -1: one launch per step)
-  ResPlan res[2];
-  ResTile *res_tiles[2] = {nullptr, nullptr};
+  // (rbc_resident.cu), by kResFwd .. kResStore (variant -1: one launch per step)
+  ResPlan res[3];
+  ResTile *res_tiles[3] = {nullptr, nullptr, nullptr};
   unsigned long long *res_ll = nullptr;
   char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, receiver cells
   size_t res_blob_cap = 0;
@@ -241,16 +241,16 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
   return RBC_OK;
 }
 
-// Whether this call's loop (0 forward, 1 reverse) runs as one resident launch.
+// Whether this call's loop (kResFwd ..) runs as one resident launch.
 bool resident(const rbc_ctx *c, int dir) {
-  return c->res[dir].variant >= 0 && c->snap.empty() && (dir == 1 || c->levels_per_launch == 1);
+  return c->res[dir].variant >= 0 && c->snap.empty() && (dir != kResFwd || c->levels_per_launch == 1);
 }
 
 // Tables of a resident loop (one copy to the device) and its launch.  The
 // receivers are sorted by the warp that owns their rows; num / den are the
 // reverse loop's outputs.
 int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, int reinject, int sample, int grad,
-                 int overwrite, int dense, float *num, float *den, cudaStream_t s) {
+                 int overwrite, int dense, float *num, float *den, cudaStream_t s, int stride = 0) {
   const ResPlan &P = c->res[dir];
   const Lay &L = c->L;
   const int cells = P.blocks * P.warps;
@@ -270,14 +270,7 @@ int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, 
   std::memcpy(blob.data(), &info, sizeof info);
   int *ptr = reinterpret_cast<int *>(blob.data() + o_ptr);
   int2 *cr = reinterpret_cast<int2 *>(blob.data() + o_rec);
-  std::vector<int> cell(nrec), loc(nrec);
-  for (int r = 0; r < nrec; ++r) {
-    res_cell(P, L, rec[3 * r], rec[3 * r + 2], &cell[r], &loc[r]);
-    ++ptr[cell[r] + 1];
-  }
-  for (int k = 0; k < cells; ++k) ptr[k + 1] += ptr[k];
-  std::vector<int> fill(ptr, ptr + cells);
-  for (int r = 0; r < nrec; ++r) cr[fill[cell[r]]++] = make_int2(loc[r], r);
+  res_cells(P, L, cells, nrec, rec, 0, ptr, cr);
   ResShot S{};
   S.L = L;
   S.a = c->a;
@@ -305,8 +298,10 @@ int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, 
   A.grad = grad;
   A.overwrite = overwrite;
   A.dense = dense;
+  A.store = c->store;
+  A.stride = stride;
   A.err = c->err_dev;
-  CK(res_launch(P, dir == 0, A, s));
+  CK(res_launch(P, dir, A, s));
   ++g_launches;
   return RBC_OK;
 }
@@ -495,15 +490,15 @@ int create_resident(rbc_ctx *c) {
   size_t ll = 0;
   cudaFree(c->res_ll);
   c->res_ll = nullptr;
-  for (int dir = 0; dir < 2; ++dir) {
+  for (int dir = 0; dir < 3; ++dir) {
     cudaFree(c->res_tiles[dir]);
     c->res_tiles[dir] = nullptr;
     ResPlan &P = c->res[dir];
-    if (!res_plan(&c->L, 1, dir == 0, c->share, &P)) continue;
+    if (!res_plan(&c->L, 1, dir, c->share, &P)) continue;
     const size_t tb = sizeof(ResTile) * P.tiles.size();
     CK(cudaMalloc(&c->res_tiles[dir], tb));
     CK(cudaMemcpy(c->res_tiles[dir], P.tiles.data(), tb, cudaMemcpyHostToDevice));
-    ll = std::max(ll, res_ll_bytes(P, dir == 0));
+    ll = std::max(ll, res_ll_bytes(P, dir));
   }
   if (ll) CK(cudaMalloc(&c->res_ll, ll));
   return RBC_OK;
@@ -982,7 +977,13 @@ int rbc_rtm_storage(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  rc = upload_shot(c, src_host, nrec, rec_host, 0, s);
+  // both loops resident, or both by steps (the forward step path keeps a level with a launch of its own, whatever
+  // the temporal-blocking option)
+  const bool res = c->res[kResFwd].variant >= 0 && c->res[kResStore].variant >= 0 && c->snap.empty();
+  rc = check_nodes(c, src_host, nrec, rec_host);
+  if (rc) return rc;
+  if (res && (rc = check_capture(s))) return rc;
+  rc = res ? ensure_receivers(c, std::max(nrec, 1)) : upload_shot(c, src_host, nrec, rec_host, 0, s);
   if (rc) return rc;
   if (c->store != store_dev || c->stride != stride) {  // the storage graphs bake both in
     for (int k = 4; k < 6; ++k) {
@@ -998,13 +999,20 @@ int rbc_rtm_storage(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
     ++g_launches;
   }
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = run_loop(c, 4, enq_store_fwd, s);
-  if (rc) return rc;
-  if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = run_loop(c, 5, enq_store_rev, s);
-  if (rc) return rc;
-  if (c->timing && (rc = record_event(c, s))) return rc;
   const int ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
+  rc = res ? run_resident(c, kResFwd, src_host, 0, nullptr, 0, 0, 0, 0, 0, nullptr, nullptr, s, stride)
+           : run_loop(c, 4, enq_store_fwd, s);
+  if (rc) return rc;
+  if (c->timing && (rc = record_event(c, s))) return rc;
+  rc = res ? run_resident(c, kResStore, src_host, nrec, rec_host, 0, 0, 0, ow, 1, num_dev, den_dev, s, stride)
+           : run_loop(c, 5, enq_store_rev, s);
+  if (rc) return rc;
+  if (c->timing && (rc = record_event(c, s))) return rc;
+  if (res) {
+    CKL();
+    c->have_panels = 1;
+    return RBC_OK;
+  }
   launch_accum_interior(c->L, c->num, num_dev, c->g.nb, top_rows(&c->g), c->g.nx, c->g.ny, c->g.nz, ow, s);
   launch_accum_interior(c->L, c->den, den_dev, c->g.nb, top_rows(&c->g), c->g.nx, c->g.ny, c->g.nz, ow, s);
   g_launches += 2;

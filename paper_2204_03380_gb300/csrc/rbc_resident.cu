@@ -282,6 +282,25 @@ struct Recs {
 template <bool TIGHT>
 __host__ __device__ __forceinline__ int buf_floats(int H) { return (H + (TIGHT ? 0 : 8)) * kTileX; }
 
+// The interior nodes of this warp's rows of level n to its slot of the store
+// (lane l writes columns l, l + 32, ...: whole sectors).
+template <int RZ>
+__device__ __forceinline__ void keep_level(const ResArgs &A, const ResShot &S, const ResTile &T, const Place &W, int n,
+                                           const float *cur) {
+  const int nx = S.ix1 - S.ix0;
+  float *slot = A.store + (long long)(n / A.stride) * nx * (S.iz1 - S.iz0);
+#pragma unroll 1
+  for (int j = 0; j < RZ; ++j) {
+    const int r = W.r0 + j, z = T.z0 + r;
+    if (r >= W.rows || z < S.iz0 || z >= S.iz1) continue;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int c = W.lane + 32 * e, x = T.x0 + c;
+      if (x >= S.ix0 && x < S.ix1) slot[(long long)(z - S.iz0) * nx + x - S.ix0] = cur[r * kTileX + c];
+    }
+  }
+}
+
 // ------------------------------------------------------------- forward ----
 template <int RZ, int MAXW, int MINB>
 __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, const int H) {
@@ -350,6 +369,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, co
                      });
     __syncwarp();
     if (n + 1 < nt) halo_out<RZ>(W, 0, (uint32_t)n + 1, smem + n0);
+    if (A.stride > 0 && n % A.stride == 0) keep_level<RZ>(A, S, T, W, n, cur);
     record(n, cur);
     f = f_next * fsc;
     if (__syncthreads_or(!ok)) {
@@ -358,6 +378,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, co
     }
   }
   record(nt, smem + (nt & 1 ? fl : 0) + h4);
+  if (A.stride > 0 && nt % A.stride == 0) keep_level<RZ>(A, S, T, W, nt, smem + (nt & 1 ? fl : 0) + h4);
   // the last two levels, for the reverse loop and rbc_get_panels
   for (int j = 0; j < RZ; ++j) {
     const int r = W.r0 + j;
@@ -370,17 +391,27 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, co
 }
 
 // ------------------------------------------------------------- reverse ----
-// acc + a b with both roundings, as the one-launch-per-step kernels add up
-__device__ __forceinline__ float4 madd4(const float4 a, const float4 b, const float4 c) {
-  const float2 l = __fadd2_rn(__fmul2_rn(lo2(a), lo2(b)), lo2(c)), h = __fadd2_rn(__fmul2_rn(hi2(a), hi2(b)), hi2(c));
+// acc + a b, rounded as the one-launch-per-step kernels round it: product and
+// sum (their products are masked), or once (k_store_image)
+template <int MODE>
+__device__ __forceinline__ float4 add_prod(const float4 a, const float4 b, const float4 c) {
+  float2 l, h;
+  if (MODE == 2) {
+    l = __ffma2_rn(lo2(a), lo2(b), lo2(c));
+    h = __ffma2_rn(hi2(a), hi2(b), hi2(c));
+  } else {
+    l = __fadd2_rn(__fmul2_rn(lo2(a), lo2(b)), lo2(c));
+    h = __fadd2_rn(__fmul2_rn(hi2(a), hi2(b)), hi2(c));
+  }
   return make_float4(l.x, l.y, h.x, h.y);
 }
 
 // What a thread keeps of its own nodes besides the fields: a and the imaging
 // sums (FWI: the gradient sum in num).  Small tiles: a in shared memory, the
 // sums in registers.
-template <int RZ, bool kGrad>
+template <int RZ, int MODE>
 struct KeepReg {
+  static constexpr bool kGrad = MODE == 1;
   const float *pa;
   float4 num[RZ], den[kGrad ? 1 : RZ];
   __device__ __forceinline__ void init(float *s_a, const Place &W) {
@@ -395,8 +426,8 @@ struct KeepReg {
   __device__ __forceinline__ void pre_all(int) {}
   __device__ __forceinline__ float4 a(int j) { return lds4(pa + j * kTileX); }
   __device__ __forceinline__ void add(int j, const float4 c, const float4 b) {
-    num[j] = madd4(c, b, num[j]);
-    if (!kGrad) den[j] = madd4(c, c, den[j]);
+    num[j] = add_prod<MODE>(c, b, num[j]);
+    if (!kGrad) den[j] = add_prod<MODE>(c, c, den[j]);
   }
   __device__ __forceinline__ void flush() {}
   __device__ __forceinline__ void sums(int j, float4 &n, float4 &d) {
@@ -423,8 +454,9 @@ __device__ __forceinline__ void tm_tie(float4 &a) { asm volatile("" : "+f"(a.x),
 
 // Large tiles: a and the sums in tensor memory, used as a thread-private store
 // (a warp reaches the 32 lanes of its quarter; 12 columns per row: a, num, den).
-template <int RZ, bool kGrad>
+template <int RZ, int MODE>
 struct KeepTm {
+  static constexpr bool kGrad = MODE == 1;
   uint32_t ta;
   float4 av, nv, dv;
   __device__ __forceinline__ void pre_a(int j) { tm_ld4(ta + 12 * j, av); }
@@ -439,10 +471,10 @@ struct KeepTm {
   }
   __device__ __forceinline__ void add(int j, const float4 c, const float4 b) {
     tm_tie(nv);
-    nv = madd4(c, b, nv);
+    nv = add_prod<MODE>(c, b, nv);
     if (!kGrad) {
       tm_tie(dv);
-      dv = madd4(c, c, dv);
+      dv = add_prod<MODE>(c, c, dv);
     }
     __syncwarp();
     tm_st4(ta + 12 * j + 4, nv);
@@ -465,11 +497,15 @@ constexpr int tm_cols(int rz, int warps) {
   return c <= 128 ? 128 : c <= 256 ? 256 : 512;
 }
 
-template <int RZ, int MAXW, int MINB, bool TIGHT, bool TM, bool kGrad>
+// MODE 0: imaging integrals (Eq. 3); 1: FWI gradient; 2: RTM with wavefield storage (Algorithm 2: only pbar is
+// stepped, and the integrals are formed at the kept levels, with p^n read from the store)
+template <int RZ, int MAXW, int MINB, bool TIGHT, bool TM, int MODE>
 __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, const int H) {
+  constexpr bool kGrad = MODE == 1, kStore = MODE == 2;
+  constexpr int NB = kStore ? 2 : 4, B0 = kStore ? 0 : 2, FB = kStore ? 0 : 1;  // buffers; pbar's first, its exchange field
   extern __shared__ __align__(16) float smem[];
   const int fl = buf_floats<TIGHT>(H), h4 = TIGHT ? 0 : 4 * kTileX;
-  float *s_lr = smem + 4 * fl;        // [H][2][4], the warp's own rows: both fields in turn
+  float *s_lr = smem + NB * fl;        // [H][2][4], the warp's own rows: both fields in turn
   // TIGHT: [4][128] rows below, read by the last warp, both fields in turn; without TM: a [H][128]
   float *s_x = s_lr + 8 * H;
   const int xfl = ((TIGHT ? 4 : 0) + (TM ? 0 : H)) * kTileX;
@@ -479,7 +515,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
   const ResShot &S = A.shots[T.shot];
   const int lane = threadIdx.x, w = threadIdx.y, nthr = 32 * blockDim.y, tid = 32 * w + lane;
   const int origin = S.L.origin, pitch = S.L.pitch, NX4 = S.L.NX4;
-  const Place W = place_of<RZ>(A, T, w, lane, H, 2);
+  const Place W = place_of<RZ>(A, T, w, lane, H, kStore ? 1 : 2);
   const int nt = A.nt;
   constexpr int TC = tm_cols(RZ, MAXW);
   if (TM && w == 0) {
@@ -487,7 +523,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
         (uint32_t)__cvta_generic_to_shared(s_tm)), "r"(TC));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  for (int i = tid; i < (4 * fl + 8 * H + xfl) / 4; i += nthr)
+  for (int i = tid; i < (NB * fl + 8 * H + xfl) / 4; i += nthr)
     *reinterpret_cast<float4 *>(smem + 4 * i) = zero4();
   if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -495,8 +531,10 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
   for (int i = tid; i < T.rows * 32; i += nthr) {
     const int r = i >> 5, x = T.x0 + 4 * (i & 31), o = origin + (T.z0 + r) * pitch + x;
     if (x < NX4) {
-      st4(smem + h4 + 4 * i, ld4(S.p[0] + o));
-      st4(smem + fl + h4 + 4 * i, ld4(S.p[1] + o));
+      if (!kStore) {
+        st4(smem + h4 + 4 * i, ld4(S.p[0] + o));
+        st4(smem + fl + h4 + 4 * i, ld4(S.p[1] + o));
+      }
       if (!TM) st4(s_x + 4 * i, ldg4(S.a + o));
     }
   }
@@ -529,7 +567,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
   const int own = W.r0 * kTileX + 4 * lane;
   const bool top = W.r0 == 0, last = W.r0 + RZ == H;  // TIGHT: the warps at the tile's edges
   uint32_t tmem = 0;
-  std::conditional_t<TM, KeepTm<RZ, kGrad>, KeepReg<RZ, kGrad>> keep;
+  std::conditional_t<TM, KeepTm<RZ, MODE>, KeepReg<RZ, MODE>> keep;
   if constexpr (TM) {
     tmem = *s_tm;
     keep.ta = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * RZ * 12);
@@ -553,8 +591,8 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
     if (has_src && t < nt) f_next = A.wav[nt - 1 - t];  // in flight during this step
     // p^R level n; pbar level n (FWI: adjoint level n + 1)
     const int n = nt - t, pr = n & 1, pb = kGrad ? pr ^ 1 : pr;
-    const int rc0 = pr * fl + h4, rn0 = (pr ^ 1) * fl + h4, bc0 = (2 + pb) * fl + h4, bn0 = (2 + (pb ^ 1)) * fl + h4;
-    const bool do_r = t > 0 && (kGrad || n > 0), do_b = kGrad || n > 0;
+    const int rc0 = pr * fl + h4, rn0 = (pr ^ 1) * fl + h4, bc0 = (B0 + pb) * fl + h4, bn0 = (B0 + (pb ^ 1)) * fl + h4;
+    const bool do_r = !kStore && t > 0 && (kGrad || n > 0), do_b = kGrad || n > 0;
     float4 qa[4];
     if (TIGHT) qa[0] = qa[1] = qa[2] = qa[3] = zero4();
     if (do_r) {
@@ -577,6 +615,26 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
                          if (xok) st4(smem + rn0 + own + j * kTileX, v);
                        });
       keep.flush();
+    } else if (kStore) {
+      if (n % A.stride == 0) {  // Eq. 3 at a kept level
+        const int nx = S.ix1 - S.ix0;
+        const float *slot = A.store + (long long)(n / A.stride) * nx * (S.iz1 - S.iz0);
+#pragma unroll
+        for (int j = 0; j < RZ; ++j) {
+          if (W.r0 + j >= W.rows) break;
+          const int z = T.z0 + W.r0 + j;
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            v[e] = z >= S.iz0 && z < S.iz1 && x0 + e >= S.ix0 && x0 + e < S.ix1
+                       ? slot[(long long)(z - S.iz0) * nx + x0 + e - S.ix0] : 0.f;
+          __syncwarp();
+          keep.pre_all(j);
+          keep.a(j);
+          keep.add(j, make_float4(v[0], v[1], v[2], v[3]), lds4(smem + bc0 + own + j * kTileX));
+        }
+        keep.flush();
+      }
     } else if (!kGrad) {
 #pragma unroll
       for (int j = 0; j < RZ; ++j) {
@@ -588,11 +646,11 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
       keep.flush();
     }
     __syncwarp();
-    if (t < nt) halo_out<RZ>(W, 0, (uint32_t)t + 1, smem + rn0);
+    if (!kStore && t < nt) halo_out<RZ>(W, 0, (uint32_t)t + 1, smem + rn0);
     if (do_b) {
       float *bc = smem + bc0, *bn = smem + bn0;
       if (t > 0)  // level nt is zero everywhere
-        ok = halo_in<RZ, TIGHT>(W, 1, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
+        ok = halo_in<RZ, TIGHT>(W, FB, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
       sweep<RZ, TIGHT>(W, smem, bc0, bn0, bc + W.r0 * kTileX - 4 * kTileX,
                        TIGHT && last ? s_x : bc + (W.r0 + RZ) * kTileX, top, qa, lofs, lstep, rofs, rstep,
                        [&](int j) { keep.pre_a(j); },
@@ -614,7 +672,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
         load_s(r - 1);
         __syncwarp();
       }
-      if (t < nt) halo_out<RZ>(W, 1, (uint32_t)t + 1, bn);
+      if (t < nt) halo_out<RZ>(W, FB, (uint32_t)t + 1, bn);
     }
     if (__syncthreads_or(!ok)) {
       if (tid == 0) atomicOr_system(A.err, 1);
@@ -652,12 +710,12 @@ inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 struct Variant {
   int rz, maxw, minb;
   bool tight, tm;
-  const void *fwd, *rev, *grad;
+  const void *fn[4];  // forward, imaging, FWI gradient, storage
 };
-#define RBC_RES_VARIANT(RZ, MAXW, MINB, TIGHT, TM)                           \
-  {RZ, MAXW, MINB, TIGHT, TM, (const void *)k_res_fwd<RZ, MAXW, MINB>,       \
-   (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, false>,                \
-   (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, true>}
+#define RBC_RES_VARIANT(RZ, MAXW, MINB, TIGHT, TM)                                                                 \
+  {RZ, MAXW, MINB, TIGHT, TM,                                                                                      \
+   {(const void *)k_res_fwd<RZ, MAXW, MINB>, (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 0>,                \
+    (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 1>, (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 2>}}
 // Rows per warp, most warps per block, blocks per SM, layout.  res_plan takes
 // the first that holds the grid: with few rows per warp a step is short (300 x
 // 300 forward: 1.6 / 1.9 / 2.5 / 2.8 / 3.1 us with 1 / 2 / 4 / 7 / 10 rows).
@@ -672,14 +730,17 @@ const Variant kVariants[] = {
     RBC_RES_VARIANT(10, 11, 1, true, true),
 };
 
-size_t res_smem(bool fwd, int H, const Variant &V) {
-  const size_t rows = fwd ? 3 * H + 16 : V.tight ? 4 * H + 4 : 4 * (H + 8) + (V.tm ? 0 : H);
-  return sizeof(float) * (rows * kTileX + 8 * (size_t)H) + (!fwd && V.tm ? 16 : 0);
+size_t res_smem(int dir, int H, const Variant &V) {
+  const int nb = dir == kResRev ? 4 : 2;  // field buffers
+  size_t rows;
+  if (dir == kResFwd) rows = 2 * (H + 8) + H;
+  else rows = V.tight ? nb * H + 4 : nb * (H + 8) + (V.tm ? 0 : H);
+  return sizeof(float) * (rows * kTileX + 8 * (size_t)H) + (dir != kResFwd && V.tm ? 16 : 0);
 }
 
 } // namespace
 
-bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out) {
+bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
   out->variant = -1;
   const char *env = getenv("RBC_RESIDENT");  // 0: one launch per step
   if (env && env[0] == '0') return false;
@@ -705,12 +766,15 @@ bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out) {
       if (force_v >= 0 && (v != force_v || (force_w > 0 && nw != force_w))) continue;
       const int H = nw * V.rz;
       if (H < 4) continue;
-      const size_t sm = res_smem(fwd, H, V);
+      const size_t sm = res_smem(dir, H, V);
       if (sm > (size_t)maxsm) continue;
       long long blocks = 0;
       for (int s = 0; s < nshots; ++s) blocks += (long long)cdiv(L[s].NX, kTileX) * cdiv(L[s].NZ, H);
+      // (more blocks than the variant's registers allow: no need to ask the runtime)
+      if (blocks * share > (long long)(V.maxw * V.minb / nw) * sms) continue;
       int per = 1 << 20;
-      for (const void *fn : {fwd ? V.fwd : V.rev, fwd ? V.fwd : V.grad}) {
+      for (int f = dir == kResStore ? 3 : dir; f <= (dir == kResRev ? 2 : dir == kResStore ? 3 : 0); ++f) {
+        const void *fn = V.fn[f];
         int k = 0;
         // the limit is raised to the device's for every plan alike: contexts on other threads share it
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm) != cudaSuccess ||
@@ -728,7 +792,7 @@ bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out) {
   out->rz = V.rz;
   out->warps = best_w;
   out->H = best_w * V.rz;
-  out->smem = res_smem(fwd, out->H, V);
+  out->smem = res_smem(dir, out->H, V);
   out->tiles.clear();
   out->tile0.assign(1, 0);
   for (int s = 0; s < nshots; ++s) {
@@ -753,8 +817,8 @@ bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out) {
   return true;
 }
 
-size_t res_ll_bytes(const ResPlan &P, bool fwd) {
-  return sizeof(u64) * (size_t)P.blocks * (fwd ? 1 : 2) * 2 * ll_words(P.H);
+size_t res_ll_bytes(const ResPlan &P, int dir) {
+  return sizeof(u64) * (size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H);
 }
 
 void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc) {
@@ -763,10 +827,68 @@ void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc)
   *loc = r * kTileX + x % kTileX;
 }
 
-cudaError_t res_launch(const ResPlan &P, bool fwd, const ResArgs &A, cudaStream_t s) {
+void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *rec, int base, int *ptr, int2 *out) {
+  std::vector<int> cell(nrec), loc(nrec), fill(cells + 1, 0);
+  for (int r = 0; r < nrec; ++r) {
+    res_cell(P, L, rec[3 * r], rec[3 * r + 2], &cell[r], &loc[r]);
+    ++fill[cell[r] + 1];
+  }
+  for (int k = 0; k < cells; ++k) fill[k + 1] += fill[k];
+  for (int k = 0; k <= cells; ++k) ptr[k] = base + fill[k];
+  for (int r = 0; r < nrec; ++r) out[fill[cell[r]]++] = make_int2(loc[r], r);
+}
+
+// Every variant's tiles, first-fit by falling tile count; the variant whose
+// groups take the least time in all is kept.  Time of a forward and a reverse
+// step by rows per warp, measured on grids that fill the device (us).
+std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
+  const double step_us[] = {4.4, 5.5, 7.3, 9.4, 11.0};
+  int dev = 0, sms = 0;
+  std::vector<std::vector<int>> best;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return best;
+  std::vector<int> order(nshots);
+  for (int i = 0; i < nshots; ++i) {
+    ResPlan f, r;
+    if (!res_plan(L + i, 1, kResFwd, 1, &f) || !res_plan(L + i, 1, kResRev, 1, &r)) return best;
+    order[i] = i;
+  }
+  double best_us = 1e30;
+  for (int v = 0; v < (int)(sizeof kVariants / sizeof kVariants[0]); ++v) {
+    const Variant &V = kVariants[v];
+    const int cap = V.minb * sms;
+    int hmax = V.maxw * V.rz;
+    while (hmax > V.rz && res_smem(kResRev, hmax, V) > 227 * 1024 / V.minb) hmax -= V.rz;
+    std::vector<int> tiles(nshots);
+    bool fits = true;
+    for (int i = 0; i < nshots; ++i) {
+      tiles[i] = cdiv(L[i].NX, kTileX) * cdiv(L[i].NZ, hmax);
+      fits = fits && tiles[i] <= cap;
+    }
+    if (!fits) continue;
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return tiles[a] != tiles[b] ? tiles[a] > tiles[b] : a < b; });
+    std::vector<std::vector<int>> g;
+    std::vector<int> room;
+    for (int i : order) {
+      size_t k = 0;
+      while (k < g.size() && room[k] < tiles[i]) ++k;
+      if (k == g.size()) {
+        g.push_back({});
+        room.push_back(cap);
+      }
+      g[k].push_back(i);
+      room[k] -= tiles[i];
+    }
+    if (g.size() * step_us[v] < best_us) best_us = g.size() * step_us[v], best = g;
+  }
+  return best;
+}
+
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s) {
   const Variant &V = kVariants[P.variant];
-  const void *fn = fwd ? V.fwd : (A.grad ? V.grad : V.rev);
-  cudaError_t e = cudaMemsetAsync(A.ll, 0, res_ll_bytes(P, fwd), s);
+  const void *fn = V.fn[dir == kResStore ? 3 : dir == kResRev && A.grad ? 2 : dir];
+  cudaError_t e = cudaMemsetAsync(A.ll, 0, res_ll_bytes(P, dir), s);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.blocks);

@@ -8,6 +8,8 @@
 
 namespace rbc {
 
+enum { kResFwd = 0, kResRev = 1, kResStore = 2 };  // the loops: forward, reverse (imaging, FWI), storage-RTM reverse
+
 // One block's tile: 128 columns x `rows` rows of one shot's padded grid.
 struct ResTile {
   int shot;
@@ -40,6 +42,8 @@ struct ResArgs {
   int grad;                 // reverse: 1 = FWI gradient (num += mu p_tt), 0 = imaging integrals
   int overwrite;            // reverse: outputs are set, not added to
   int dense;                // reverse: num / den are dense interior arrays (else pitched)
+  float *store;             // storage RTM: the kept levels, every `stride` steps (0: none kept)
+  int stride;
   int *err;
 };
 
@@ -54,14 +58,20 @@ struct ResPlan {
   std::vector<int> tile0;   // first tile of each shot, then the tile count
 };
 
-// Plan for the forward / reverse loop of the given layouts (variant -1 when
+// Plan for one loop (dir) of the given layouts (variant -1 when
 // they do not fit on this device at once); share: the device is shared by that
 // many such loops.
-bool res_plan(const Lay *L, int nshots, bool fwd, int share, ResPlan *out);
-size_t res_ll_bytes(const ResPlan &P, bool fwd);
+bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out);
+// Shots of a batch sorted into groups whose loops run at once: groups of shot
+// indices, or none when a shot does not fit.
+std::vector<std::vector<int>> res_groups(const Lay *L, int nshots);
+size_t res_ll_bytes(const ResPlan &P, int dir);
 // The (tile, warp) cell that owns a node, within its shot's tiles, and the
 // node's place in the tile.
 void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc);
-cudaError_t res_launch(const ResPlan &P, bool fwd, const ResArgs &A, cudaStream_t s);
+// Receiver cells of one shot (its tiles * warps cells): CSR pointers and
+// {place in the tile, receiver}, positions offset by `base`.
+void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *rec, int base, int *ptr, int2 *out);
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s);
 
 } // namespace rbc
