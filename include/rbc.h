@@ -298,7 +298,9 @@ int rbc_batch_destroy(rbc_batch *b);
  * work list of (shot, tile) items; then, per shot, I = num / (den + eps_rel
  * max den) (Eq. 3) is stacked into image_dev (nz, survey_nx) at column off_x
  * (+=, shots may overlap).  shots: nshots descriptors (host); flags must be
- * RBC_REINJECT_SOURCE.  The shots run in groups of consecutive shots whose
+ * RBC_REINJECT_SOURCE.  When every shot fits on the chip (about 2.1 M padded
+ * nodes), the shots run in groups that fill it, one launch per phase and
+ * group.  Otherwise they run in groups of consecutive shots whose
  * seven fields fit an L2 budget (environment RBC_BATCH_L2MB, megabytes,
  * default 96; 0 = one group), each group's forward then reverse phase, so
  * that a group's fields stay in L2 through its time loops.  Each phase of
@@ -325,7 +327,8 @@ int rbc_batch_timing(rbc_batch *b, int enable, double *out);
  * per-launch time in microseconds of every candidate on the first shot
  * group: forward streaming / 1 / 2 / 4 rows, reverse 1 / 2 rows / streaming /
  * tiles (0 where a candidate was not timed), then the number of shot groups.
- * Host only. */
+ * All of this describes the one-launch-per-step kernels; a batch whose shots
+ * fit on the chip does not time them and does not run them.  Host only. */
 int rbc_batch_info(const rbc_batch *b, int *out);
 
 /* ------------------------------------------------------------------------
