@@ -17,17 +17,21 @@
 // ahead of its reader, because it needs the reader's own words to get there.
 // All blocks are resident (the launch is cooperative) and every wait is bounded.
 //
-// What bounds it: on the survey grid the fp32 pipes (59 packed operations per
-// four nodes and field, 1.6 us a step of the 3.9 us) and the exchange, about
-// 1.5 us from a tile's last row to its neighbours' first; on small grids the
-// exchange alone.  Measured (us per step; before, one launch per step): survey
-// forward 3.9 (6.1), forward + reverse 12.2 (18.8); 300 x 300 forward 1.5
-// (2.7), forward + reverse 4.5 (6.7).  Tensor memory for a and the sums: 8 us
-// per reverse step against 12.4 with the sums in registers (spilled) and a
-// read from L2 twice.  Tried and not kept: a warp-to-warp order (mbarriers)
-// instead of the block barrier at each step -- the warps drift apart and their
-// unrolled rows no longer fit the instruction cache (18 us per reverse step);
-// the same with the rows rolled up into a loop of two (9.8 us).
+// What bounds it: one block by itself takes 0.9 us per level and field plus
+// 0.69 us for every ten-row warp on a scheduler (143 clocks per row; 59 packed
+// operations take 118), so a survey tile (11 warps) 2.9 us, and the exchange
+// adds 0.5 us; on small grids the fixed part and the exchange are all there
+// is.  Measured (us per step; before, one launch per step): survey forward 3.6
+// (6.1), forward + reverse 11.2 (18.8); 300 x 300 forward 1.5 (2.7), forward +
+// reverse 4.5 (6.7).  Tensor memory for a and the sums: 8 us per reverse step
+// against 12.4 with the sums in registers (spilled) and a read from L2 twice.
+// Tried and not kept: a warp-to-warp order (mbarriers) instead of the block
+// barrier at each step -- the warps drift apart and their unrolled rows no
+// longer fit the instruction cache (18 us per reverse step); the same with the
+// rows rolled up into a loop of two (9.8 us); the tile's outer columns updated
+// last, so that nothing else waits for the words beside it (forward 3.8 us
+// against 3.4: the wait is not what bounds a step); 16 warps of 7 rows instead
+// of 11 of 10 (the same).
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -42,7 +46,7 @@ namespace rbc {
 namespace {
 
 typedef unsigned long long u64;
-constexpr long long kResWait = 2000000000LL;  // about a second
+constexpr int kSpins = 2000000;               // polls of a wait before it gives up (each an L2 round trip: about a second)
 constexpr int kEdge = 4 * kTileX;             // words of a top or bottom halo (4 rows)
 
 __device__ __forceinline__ void ll_ld(const u64 *p, u64 &a, u64 &b) {
@@ -70,15 +74,14 @@ struct Ll4 {
   __device__ __forceinline__ float4 value() const {
     return make_float4(ll_val(v[0]), ll_val(v[1]), ll_val(v[2]), ll_val(v[3]));
   }
-  // Bounded wait for the values of `tag`; false if it gave up.
+  // Poll, from a first load, until the values are those of `tag`; false if it gave up.
   __device__ __forceinline__ bool wait(const u64 *p0, const u64 *p1, uint32_t tag) {
-    if (ok(tag)) return true;
-    const long long t0 = clock64();
-    do {
+#pragma unroll 1
+    for (int i = 0; !ok(tag); ++i) {
+      if (i == kSpins) return false;
       load(p0, p1);
-      if (ok(tag)) return true;
-    } while (clock64() - t0 < kResWait);
-    return false;
+    }
+    return true;
   }
 };
 
@@ -140,41 +143,39 @@ __device__ __forceinline__ bool halo_in(const Place &W, int f, uint32_t tag, flo
   Ll4 c;
   if (W.lr) c.load(W.in_lr + o, W.in_lr + o + 2);
   bool ok = true;
-  // With fewer than four rows per warp, a warp reads only the halo rows its
-  // own rows reach (the others' next level may already be on its way): the
-  // rest of its four loads repeat the nearest of those.
-  if (W.up && W.r0 < 4) {  // rows r0 .. 3 of the four above
-    const u64 *b = W.in_tb + o;
+  // Rows k0 .. k1 of the four of a side, polled together.  With fewer than
+  // four rows per warp, a warp reads only the halo rows its own rows reach
+  // (the others' next level may already be on its way): the rest of its four
+  // loads repeat the nearest of those.  (One short loop per side: with a wait
+  // of its own behind every load the code a warp jumps over costs more
+  // instruction fetches than it saves polls.)
+  auto rows_in = [&](const u64 *b, int k0, int k1, auto put) {
     Ll4 t[4];
+    bool all;
+    int i = 0;
+#pragma unroll 1
+    do {
+      all = true;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const u64 *p = b + (RZ < 4 ? max(k, W.r0) : k) * kTileX;
-      t[k].load(p, p + 64);
-    }
+      for (int k = 0; k < 4; ++k) {
+        const u64 *p = b + (RZ < 4 ? min(max(k, k0), k1) : k) * kTileX;
+        t[k].load(p, p + 64);
+      }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int kk = RZ < 4 ? max(k, W.r0) : k;
-      ok = t[k].wait(b + kk * kTileX, b + kk * kTileX + 64, tag) && ok;
-      if (TIGHT) qa[k] = t[k].value();
-      else *reinterpret_cast<float4 *>(s_up + kk * kTileX + 4 * W.lane) = t[k].value();
-    }
-  }
-  if (W.dn && W.r0 + RZ + 3 >= W.H) {  // rows 0 .. r0 + RZ + 3 - H of the four below
-    const u64 *b = W.in_tb + o + kEdge;
-    const int k1 = W.r0 + RZ + 3 - W.H;
-    Ll4 t[4];
+      for (int k = 0; k < 4; ++k) all = all && t[k].ok(tag);
+    } while (!all && ++i < kSpins);
+    ok = ok && all;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const u64 *p = b + (RZ < 4 ? min(k, k1) : k) * kTileX;
-      t[k].load(p, p + 64);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int kk = RZ < 4 ? min(k, k1) : k;
-      ok = t[k].wait(b + kk * kTileX, b + kk * kTileX + 64, tag) && ok;
-      *reinterpret_cast<float4 *>(s_dn + kk * kTileX + 4 * W.lane) = t[k].value();
-    }
-  }
+    for (int k = 0; k < 4; ++k) put(RZ < 4 ? min(max(k, k0), k1) : k, k, t[k].value());
+  };
+  if (W.up && W.r0 < 4)  // rows r0 .. 3 of the four above
+    rows_in(W.in_tb + o, W.r0, 3, [&](int kk, int k, float4 v) {
+      if (TIGHT) qa[k] = v;
+      else st4(s_up + kk * kTileX + 4 * W.lane, v);
+    });
+  if (W.dn && W.r0 + RZ + 3 >= W.H)  // rows 0 .. r0 + RZ + 3 - H of the four below
+    rows_in(W.in_tb + o + kEdge, 0, W.r0 + RZ + 3 - W.H,
+            [&](int kk, int, float4 v) { st4(s_dn + kk * kTileX + 4 * W.lane, v); });
   if (W.lr) {
     ok = c.wait(W.in_lr + o, W.in_lr + o + 2, tag) && ok;
     *reinterpret_cast<float4 *>(s_lr + ((W.r0 + (W.lane & 15)) * 2 + (W.right ? 1 : 0)) * 4) = c.value();
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, co
   const int2 *cell_rec = S.cell_rec;
   float *seis_t = S.seis_t;
   const int cell = (blockIdx.x - S.tile0) * blockDim.y + w;
-  constexpr int K = RZ < 10 ? 4 : 2;
+  constexpr int K = RZ < 4 ? 4 : 1;
   Recs<K> rec;
   rec.load(S.cell_ptr, cell_rec, cell, lane, A.sample != 0);
   auto record = [&](int n, const float *p) {  // p^n at this warp's receivers
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, co
     __syncwarp();
     if (n + 1 < nt) halo_out<RZ>(W, 0, (uint32_t)n + 1, smem + n0);
     if (A.stride > 0 && n % A.stride == 0) keep_level<RZ>(A, S, T, W, n, cur);
-    record(n, cur);
+    if (rec.end > rec.beg) record(n, cur);
     f = f_next * fsc;
     if (__syncthreads_or(!ok)) {
       if (tid == 0) atomicOr_system(A.err, 1);
@@ -546,7 +547,7 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
   const int2 *cell_rec = S.cell_rec;
   const float *seis_t = S.seis_t, *sa = S.a + origin + T.z0 * pitch + T.x0;
   const int cell = (blockIdx.x - S.tile0) * blockDim.y + w;
-  constexpr int K = 4;
+  constexpr int K = TIGHT ? 1 : 4;
   Recs<K> rec;
   rec.load(S.cell_ptr, cell_rec, cell, lane, true);
   float rec_a[K], rec_s[K];  // scale * a at the receivers; the record's values, loaded a step ahead
@@ -726,7 +727,7 @@ struct Variant {
 // tallest tile whose four buffers fit 227 KB: TIGHT keeps no halo rows in them.
 const Variant kVariants[] = {
     RBC_RES_VARIANT(1, 8, 2, false, false), RBC_RES_VARIANT(2, 8, 2, false, false),
-    RBC_RES_VARIANT(4, 16, 1, false, true), RBC_RES_VARIANT(7, 15, 1, true, true),
+    RBC_RES_VARIANT(4, 16, 1, false, true), RBC_RES_VARIANT(7, 16, 1, true, true),
     RBC_RES_VARIANT(10, 11, 1, true, true),
 };
 
