@@ -25,11 +25,11 @@ namespace rbc {
 
 namespace {
 
-constexpr int kTY = 8;        // y rows per reverse tile (one warp per field each)
+constexpr int kTY = 8;        // y rows per reverse tile (two per warp)
 #ifndef RBC_FWD3D_ROWS
-#define RBC_FWD3D_ROWS 16
+#define RBC_FWD3D_ROWS 8
 #endif
-constexpr int kTYf = RBC_FWD3D_ROWS;  // y rows per forward tile (one warp each)
+constexpr int kTYf = RBC_FWD3D_ROWS;  // y rows per forward tile (two per warp; two blocks per SM)
 constexpr int kRP = 8;        // forward P ring: 5 live planes + 3 in flight
 constexpr int kRT = 5;        // forward T ring: 1 live plane + 4 in flight
 constexpr int kRPr = 8;       // reverse P ring (two fields): 5 live + 3 in flight
@@ -88,20 +88,35 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
   return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
-// Leapfrog update of 4 consecutive nodes (see rbc_stencil.cuh).  xr: this
-// thread's halo row in shared memory at the centre plane (float4 at xr =
-// x0-4..x0-1, xr+4 = centre, xr+8 = right); rows +-k sit at +-k*kHaloW;
-// zq[0..8]: z queue.
-__device__ __forceinline__ float4 leap4_3d(const float *xr, const float4 *zq, const float4 po, const float4 av) {
-  const float4 lf = lds4(xr), c = lds4(xr + 4), rt = lds4(xr + 8);
-  float4 ym[4], yp[4];
+// Leapfrog update of 4 consecutive nodes in two neighbouring y rows (see
+// rbc_stencil.cuh).  xr: the first row's halo row in shared memory at the centre
+// plane (float4 at xr = x0-4..x0-1, xr+4 = centre, xr+8 = right; rows +-k at
+// +-k*kHaloW); q0 / q1[0..8]: the rows' z queues.  The ten rows of the two y
+// windows are read once: 18 shared-memory reads per two rows with the queues'
+// and the tile's, against 28 row by row.
+__device__ __forceinline__ void leap4_3d2(const float *xr, const float4 *q0, const float4 *q1, const float4 po0,
+                                          const float4 po1, const float4 av0, const float4 av1, float4 &v0,
+                                          float4 &v1) {
+  const float4 c0 = q0[4], c1 = q1[4];
+  float4 ym[4], yp[4];  // rows y - 1 .. y - 4 and y + 2 .. y + 5
 #pragma unroll
   for (int k = 1; k <= 4; ++k) {
     ym[k - 1] = lds4(xr + 4 - k * kHaloW);
-    yp[k - 1] = lds4(xr + 4 + k * kHaloW);
+    yp[k - 1] = lds4(xr + 4 + (k + 1) * kHaloW);
   }
-  const float w[12] = {lf.x, lf.y, lf.z, lf.w, c.x, c.y, c.z, c.w, rt.x, rt.y, rt.z, rt.w};
-  return leap4p<true>(w, zq, ym, yp, po, av);
+  float4 z[4], y[4];
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    z[k - 1] = pair_diff(q0[4 - k], c0, q0[4 + k]);
+    y[k - 1] = pair_diff(ym[k - 1], c0, k == 1 ? c1 : yp[k > 1 ? k - 2 : 0]);
+  }
+  v0 = leap_fin<false>(c0, po0, av0, lap_shared<true>(lds4(xr), c0, lds4(xr + 8), z, y), nullptr);
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    z[k - 1] = pair_diff(q1[4 - k], c1, q1[4 + k]);
+    y[k - 1] = pair_diff(k == 1 ? c0 : ym[k > 1 ? k - 2 : 0], c1, yp[k - 1]);
+  }
+  v1 = leap_fin<false>(c1, po1, av1, lap_shared<true>(lds4(xr + kHaloW), c1, lds4(xr + kHaloW + 8), z, y), nullptr);
 }
 
 __device__ __forceinline__ void point_sub(float4 &v, int d, float term) {
@@ -179,9 +194,13 @@ constexpr size_t fwd_smem() {
 }
 static_assert(kRP >= 8, "the P ring must hold a tile's first 8 planes");
 
-// TY rows per tile (one consumer warp each) plus one producer warp.
+// TY rows per tile (two per consumer warp) plus one producer warp.  Per step on
+// 580 x 580 x 380: one row per warp and 16-row tiles 402 us; the x padding left
+// out of the copies and launches that overlap 390; two rows per warp 369; tiles
+// of 8 rows, two blocks per SM, 366 (191 x 150 x 133: 19.3 / 18.3 / 16.9 / 15.6;
+// floor of the larger grid at the copy rate: 302).
 template <int TY>
-__global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_constant__ CUtensorMap tm_cur,
+__global__ void __launch_bounds__(32 * (TY / 2 + 1), TY <= 8 ? 2 : 1) k_fwd3d_tma(const __grid_constant__ CUtensorMap tm_cur,
                                                                const __grid_constant__ CUtensorMap tm_a,
                                                                const __grid_constant__ CUtensorMap tm_old,
                                                                const StepArgs A) {
@@ -200,19 +219,20 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
   const int nthr = blockDim.x * blockDim.y;
   const int gx = (L.NX + kTileX - 1) / kTileX, gy = (L.NY + TY - 1) / TY;
   const int ntiles = gx * gy * ((L.NZ + A.zc - 1) / A.zc);
+  if (tid == 0) {
+    *abort_blk = 0;
+    for (int s = 0; s < kRP; ++s) mbar_init(&fullP[s], 1), mbar_init(&emptyP[s], TY / 2);
+    for (int s = 0; s < kRT; ++s) mbar_init(&fullT[s], 1), mbar_init(&emptyT[s], TY / 2);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  griddep_wait();
   if (A.sample) {
     const int nrec = A.info->nrec;
     for (int r = blockIdx.x * nthr + tid; r < nrec; r += gridDim.x * nthr)
       A.seis_t[(long long)A.n * nrec + r] = A.cur[A.rec_off[r]];
   }
-  if (tid == 0) {
-    *abort_blk = 0;
-    for (int s = 0; s < kRP; ++s) mbar_init(&fullP[s], 1), mbar_init(&emptyP[s], TY);
-    for (int s = 0; s < kRT; ++s) mbar_init(&fullT[s], 1), mbar_init(&emptyT[s], TY);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  if (w == TY) {
+  if (w == TY / 2) {
     // ---- producer (one lane): P planes and T tiles in the order they are consumed
     if (lane == 0) {
       const uint32_t pbytes = sizeof(float) * kPStage, tbytes = sizeof(float) * 2 * kTTile;
@@ -252,6 +272,9 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
           if (ok) issueT(T.zb + r, tx, ty);
         }
       }
+      // stay until the consumers have released the last planes, so that a wait of theirs that gives up is reported
+      // and no copy outlives the block
+      for (int k = max(0, gp - kRP); ok && k < gp; ++k) ok = mbar_wait_ab(&emptyP[k % kRP], (k / kRP) & 1, abort_blk);
       if (*abort_blk) {
         flag_error(A.err, 1);
         // let every issued copy land before the block's shared memory is released
@@ -262,28 +285,29 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
     }
     return;
   }
-  // ---- consumers: one row of the tile per warp, a float4 of x per lane
+  // ---- consumers: two rows of the tile per warp, a float4 of x per lane
   const int src = A.info->src_off;
   const float fsrc = A.wav[A.n] * A.info->src_fwd;
-  const int rowc = (w + 4) * kHaloW + lane * 4;
+  const int rowc = (2 * w + 4) * kHaloW + lane * 4;
   int gp = 0, gt = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const Tile3 T = tile_of(t, gx, gy, A.zc, L.NZ);
-    const int x0 = T.bx * kTileX + lane * 4, y = T.by * TY + w;
-    const bool xok = x0 < L.NX4, yok = y < L.NY;
+    const int x0 = T.bx * kTileX + lane * 4, y = T.by * TY + 2 * w;
+    const bool xok = x0 < L.NX4, yok = y < L.NY, yok1 = y + 1 < L.NY;
     const int col = L.origin + y * L.pitch + x0;
     const int nplanes = T.ze - T.zb;
-    float4 q[9];
+    float4 q[9], q1[9];
     bool ok = true;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       ok = ok && mbar_wait_ab(&fullP[(gp + j) % kRP], ((gp + j) / kRP) & 1, abort_blk);
       q[j] = lds4(sp + ((gp + j) % kRP) * kPStage + rowc + 4);
+      q1[j] = lds4(sp + ((gp + j) % kRP) * kPStage + rowc + kHaloW + 4);
     }
     ok = __all_sync(0xffffffffu, ok);  // keep the warp's decision uniform
     if (lane == 0)
       for (int j = 0; j < 4; ++j) mbar_arrive(&emptyP[(gp + j) % kRP]);
-#pragma unroll 4  // the z queue's shifts become register renames within an unrolled group
+#pragma unroll 3  // the z queue's shifts become register renames within an unrolled group
     for (int r = 0; ok && r < nplanes; ++r) {
       const int z = T.zb + r;
       const int top = gp + r + 8, cen = gp + r + 4, tk = gt + r;
@@ -292,14 +316,18 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       q[8] = lds4(sp + (top % kRP) * kPStage + rowc + 4);
+      q1[8] = lds4(sp + (top % kRP) * kPStage + rowc + kHaloW + 4);
       if (xok && yok) {
-        const float *tt = st + (tk % kRT) * 2 * kTTile + w * 128 + lane * 4;
-        const float4 av = lds4(tt), po = lds4(tt + kTTile);
-        float4 v = leap4_3d(sp + (cen % kRP) * kPStage + rowc, q, po, av);
+        const float *tt = st + (tk % kRT) * 2 * kTTile + 2 * w * 128 + lane * 4;
+        const float4 av = lds4(tt), po = lds4(tt + kTTile), av1 = lds4(tt + 128), po1 = lds4(tt + kTTile + 128);
+        float4 v, v1;
+        leap4_3d2(sp + (cen % kRP) * kPStage + rowc, q, q1, po, po1, av, av1, v, v1);
         const int o = col + z * L.plane;
-        const int d = src - o;
+        const int d = src - o, d1 = d - L.pitch;
         if ((unsigned)d < 4u) point_sub(v, d, cmp(av, d) * fsrc);
+        if ((unsigned)d1 < 4u) point_sub(v1, d1, cmp(av1, d1) * fsrc);
         st4(A.nxt + o, v);
+        if (yok1) st4(A.nxt + o + L.pitch, v1);
       }
       __syncwarp();
       if (lane == 0) {
@@ -307,7 +335,7 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
         mbar_arrive(&emptyT[tk % kRT]);
       }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) q[k] = q[k + 1];
+      for (int k = 0; k < 8; ++k) q[k] = q[k + 1], q1[k] = q1[k + 1];
     }
     if (!ok) break;
     __syncwarp();
@@ -316,20 +344,29 @@ __global__ void __launch_bounds__(32 * (TY + 1)) k_fwd3d_tma(const __grid_consta
     gp += nplanes + 8;
     gt += nplanes;
   }
+  griddep_launch();
 }
 
 // ------------------------------------------------------------- reverse ----
-// 2 x kTY consumer warps: warps 0..kTY-1 advance p^R and accumulate the
-// imaging integrals (reading pbar at the centre plane from the pbar ring),
-// warps kTY..2kTY-1 advance pbar and then add the record at the receivers of
-// their own row of the tile; the last warp produces.  P stage: the p^R and
+// Three groups of kTY / 2 consumer warps, two rows of the tile per warp: the
+// first advance p^R, the second advance pbar and then add the record at the
+// receivers of their rows, the third accumulate the imaging integrals from the
+// centre plane of both rings; the last warp produces.  (The integrals in the
+// p^R warps made those the slowest: 941 -> 878 us per step on 580 x 580 x
+// 380.)  What bounds it is the warps' own row work, 0.88 us per plane of a tile
+// whether the fields come from L2 or from DRAM (floor 0.71 us): before, one row
+// per warp and the grid's x padding read with it, 956 us.  The plane loop is
+// unrolled by 3: by 4 the p^R and pbar warps, at different places of the loop,
+// no longer fit the instruction cache (1234 us), by 1 the queues' shifts cost
+// 929.  P stage: the p^R and
 // pbar halo planes; T stage: a, p^R and pbar tiles overwritten in place, and
 // the num/den tiles where the tile meets the image box.
+constexpr int kRevW = 3 * kTY / 2;  // consumer warps
 constexpr size_t kRevSmem =
     sizeof(float) * (2 * kRPr * kPStage + kRTr * 5 * kTTile) + 16 * (kRPr + kRTr) + 16;
 static_assert(kRPr >= 8, "the P ring must hold a tile's first 8 planes");
 
-__global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_constant__ CUtensorMap tm_rc,
+__global__ void __launch_bounds__(32 * (kRevW + 1)) k_rev3d_tma(const __grid_constant__ CUtensorMap tm_rc,
                                                                    const __grid_constant__ CUtensorMap tm_bc,
                                                                    const __grid_constant__ CUtensorMap tm_a,
                                                                    const __grid_constant__ CUtensorMap tm_rn,
@@ -353,12 +390,13 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
   const bool do_r = A.do_r != 0, do_b = A.do_b != 0;
   if (tid == 0) {
     *abort_blk = 0;
-    for (int s = 0; s < kRPr; ++s) mbar_init(&fullP[s], 1), mbar_init(&emptyP[s], 2 * kTY);
-    for (int s = 0; s < kRTr; ++s) mbar_init(&fullT[s], 1), mbar_init(&emptyT[s], 2 * kTY);
+    for (int s = 0; s < kRPr; ++s) mbar_init(&fullP[s], 1), mbar_init(&emptyP[s], kRevW);
+    for (int s = 0; s < kRTr; ++s) mbar_init(&fullT[s], 1), mbar_init(&emptyT[s], kRevW);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (w == 2 * kTY) {
+  griddep_wait();
+  if (w == kRevW) {
     if (lane == 0) {
       const uint32_t pbytes = 2 * sizeof(float) * kPStage;
       int gp = 0, gt = 0;
@@ -401,6 +439,7 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
           if (ok) issueT(T.zb + r, tx, ty, tile_img);
         }
       }
+      for (int k = max(0, gp - kRPr); ok && k < gp; ++k) ok = mbar_wait_ab(&emptyP[k % kRPr], (k / kRPr) & 1, abort_blk);
       if (*abort_blk) {
         flag_error(A.err, 1);
         for (int k = max(0, gp - kRPr); k < gp; ++k) mbar_wait(&fullP[k % kRPr], (k / kRPr) & 1);
@@ -409,8 +448,64 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
     }
     return;
   }
-  const bool is_r = w < kTY;                // p^R group, else pbar group
-  const int row = is_r ? w : w - kTY;
+  if (w >= kTY) {
+    // ---- imaging warps ----
+    const int row = 2 * (w - kTY);
+    const int rowc = (row + 4) * kHaloW + lane * 4;
+    int gp = 0, gt = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const Tile3 T = tile_of(t, gx, gy, A.zc, L.NZ);
+      const int x0 = T.bx * kTileX + lane * 4, y = T.by * kTY + row;
+      const bool img_x = x0 < L.NX4 && x0 + 3 >= A.ix0 && x0 < A.ix1;
+      const bool img0 = img_x && y < L.NY && y >= A.iy0 && y < A.iy1;
+      const bool img1 = img_x && y + 1 < L.NY && y + 1 >= A.iy0 && y + 1 < A.iy1;
+      const int col = L.origin + y * L.pitch + x0;
+      const int nplanes = T.ze - T.zb;
+      bool ok = true;
+      // every plane is released once it has landed: the first four and the last four are not used here
+      auto pass = [&](int k) {
+        ok = __all_sync(0xffffffffu, mbar_wait_ab(&fullP[k % kRPr], (k / kRPr) & 1, abort_blk));
+        if (ok && lane == 0) mbar_arrive(&emptyP[k % kRPr]);
+      };
+      for (int j = 0; ok && j < 4; ++j) pass(gp + j);
+      for (int r = 0; ok && r < nplanes; ++r) {
+        const int z = T.zb + r;
+        const int cen = gp + r + 4, tk = gt + r;
+        ok = mbar_wait_ab(&fullP[cen % kRPr], (cen / kRPr) & 1, abort_blk) &&
+             mbar_wait_ab(&fullT[tk % kRTr], (tk / kRTr) & 1, abort_blk);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (z >= A.iz0 && z < A.iz1) {
+          const int o = col + z * L.plane;
+          const float *tt = st + (tk % kRTr) * 5 * kTTile + row * 128 + lane * 4;
+          const int cs = (cen % kRPr) * kPStage + rowc + 4;
+          if (img0) {
+            const float4 c = lds4(spr + cs), b = lds4(spb + cs);
+            st4(A.num + o, add4(lds4(tt + 3 * kTTile), masked_prod(c, b, x0, A.ix0, A.ix1)));
+            st4(A.den + o, add4(lds4(tt + 4 * kTTile), masked_prod(c, c, x0, A.ix0, A.ix1)));
+          }
+          if (img1) {
+            const float4 c = lds4(spr + cs + kHaloW), b = lds4(spb + cs + kHaloW);
+            st4(A.num + o + L.pitch, add4(lds4(tt + 3 * kTTile + 128), masked_prod(c, b, x0, A.ix0, A.ix1)));
+            st4(A.den + o + L.pitch, add4(lds4(tt + 4 * kTTile + 128), masked_prod(c, c, x0, A.ix0, A.ix1)));
+          }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&emptyP[cen % kRPr]);
+          mbar_arrive(&emptyT[tk % kRTr]);
+        }
+      }
+      for (int j = nplanes + 4; ok && j < nplanes + 8; ++j) pass(gp + j);
+      if (!ok) break;
+      gp += nplanes + 8;
+      gt += nplanes;
+    }
+    griddep_launch();
+    return;
+  }
+  const bool is_r = w < kTY / 2;            // p^R group, else pbar group
+  const int row = 2 * (is_r ? w : w - kTY / 2);
   const bool upd = is_r ? do_r : do_b;
   float *nxt = is_r ? A.rn : A.bn;
   const float *sp = is_r ? spr : spb;
@@ -422,20 +517,21 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const Tile3 T = tile_of(t, gx, gy, A.zc, L.NZ);
     const int x0 = T.bx * kTileX + lane * 4, y = T.by * kTY + row;
-    const bool xok = x0 < L.NX4, yok = y < L.NY;
-    const bool img_xy = is_r && xok && yok && y >= A.iy0 && y < A.iy1 && x0 + 3 >= A.ix0 && x0 < A.ix1;
+    const bool xok = x0 < L.NX4, yok = y < L.NY, yok1 = y + 1 < L.NY;
     const int col = L.origin + y * L.pitch + x0;
     const int nplanes = T.ze - T.zb;
-    float4 q[9];
+    float4 q[9], q1[9];
     bool ok = true;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       ok = ok && mbar_wait_ab(&fullP[(gp + j) % kRPr], ((gp + j) / kRPr) & 1, abort_blk);
       q[j] = lds4(sp + ((gp + j) % kRPr) * kPStage + rowc + 4);
+      q1[j] = lds4(sp + ((gp + j) % kRPr) * kPStage + rowc + kHaloW + 4);
     }
     ok = __all_sync(0xffffffffu, ok);  // keep the warp's decision uniform
     if (lane == 0)
       for (int j = 0; j < 4; ++j) mbar_arrive(&emptyP[(gp + j) % kRPr]);
+#pragma unroll 3
     for (int r = 0; ok && r < nplanes; ++r) {
       const int z = T.zb + r;
       const int top = gp + r + 8, cen = gp + r + 4, tk = gt + r;
@@ -444,21 +540,20 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       q[8] = lds4(sp + (top % kRPr) * kPStage + rowc + 4);
+      q1[8] = lds4(sp + (top % kRPr) * kPStage + rowc + kHaloW + 4);
       if (xok && yok) {
         const int o = col + z * L.plane;
         const float *tt = st + (tk % kRTr) * 5 * kTTile + row * 128 + lane * 4;
-        const float4 av = lds4(tt);
         const int cs = (cen % kRPr) * kPStage + rowc;
         if (upd) {
-          float4 v = leap4_3d(sp + cs, q, lds4(tt + tslot * kTTile), av);
-          const int d = src - o;
+          const float4 av = lds4(tt), av1 = lds4(tt + 128);
+          float4 v, v1;
+          leap4_3d2(sp + cs, q, q1, lds4(tt + tslot * kTTile), lds4(tt + tslot * kTTile + 128), av, av1, v, v1);
+          const int d = src - o, d1 = d - L.pitch;
           if ((unsigned)d < 4u) point_sub(v, d, cmp(av, d) * fsrc);
+          if ((unsigned)d1 < 4u) point_sub(v1, d1, cmp(av1, d1) * fsrc);
           st4(nxt + o, v);
-        }
-        if (img_xy && z >= A.iz0 && z < A.iz1) {
-          const float4 b = lds4(spb + cs + 4);  // pbar_n at this node
-          st4(A.num + o, add4(lds4(tt + 3 * kTTile), masked_prod(q[4], b, x0, A.ix0, A.ix1)));
-          st4(A.den + o, add4(lds4(tt + 4 * kTTile), masked_prod(q[4], q[4], x0, A.ix0, A.ix1)));
+          if (yok1) st4(nxt + o + L.pitch, v1);
         }
       }
       __syncwarp();
@@ -467,7 +562,7 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
         mbar_arrive(&emptyT[tk % kRTr]);
       }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) q[k] = q[k + 1];
+      for (int k = 0; k < 8; ++k) q[k] = q[k + 1], q1[k] = q1[k + 1];
     }
     if (!ok) break;
     __syncwarp();
@@ -475,11 +570,11 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
       for (int j = nplanes + 4; j < nplanes + 8; ++j) mbar_arrive(&emptyP[(gp + j) % kRPr]);
     gp += nplanes + 8;
     gt += nplanes;
-    // Eq. 2 source term at this warp's receivers (its row of the tile), after
+    // Eq. 2 source term at this warp's receivers (its rows of the tile), after
     // the warp's own stores of pbar_{n-1}
     if (!is_r && do_b) {
       const int cell = t * kTY + row;
-      const int beg = A.tile_ptr[cell], end = A.tile_ptr[cell + 1];
+      const int beg = A.tile_ptr[cell], end = A.tile_ptr[cell + 2];  // both rows
       if (end > beg) {
         __threadfence();
         __syncwarp();
@@ -493,6 +588,7 @@ __global__ void __launch_bounds__(32 * (2 * kTY + 1)) k_rev3d_tma(const __grid_c
       }
     }
   }
+  griddep_launch();
 }
 
 // ----------------------------------------------------------- host side ----
@@ -513,7 +609,9 @@ bool make_map(CUtensorMap *m, const Lay &L, const float *buf, int box_x, int box
   auto fn = encode_fn();
   if (!fn) return false;
   const float *base = buf + 0;  // buffer start (tensor coordinate 0 = padded -32, -4, -4)
-  cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)(L.NZ + 2 * kHaloR)};
+  // the columns past the grid are left outside the map: TMA fills them with
+  // zeros instead of reading the row's padding
+  cuuint64_t dims[3] = {(cuuint64_t)(kHaloX + L.NX4), (cuuint64_t)L.rows, (cuuint64_t)(L.NZ + 2 * kHaloR)};
   cuuint64_t strides[2] = {(cuuint64_t)L.pitch * sizeof(float), (cuuint64_t)L.plane * sizeof(float)};
   cuuint32_t box[3] = {(cuuint32_t)box_x, (cuuint32_t)box_y, 1};
   cuuint32_t estr[3] = {1, 1, 1};
@@ -542,21 +640,25 @@ void *tmap_encode_fn() { return reinterpret_cast<void *>(encode_fn()); }
 
 int tile_rows_3d() { return kTY; }
 
-// z planes per tile of the 3-D kernels for this grid: with one persistent
-// block per SM, the busiest block streams ceil(tiles / SMs) tiles of zc + 8
-// planes each (8 halo planes per tile), so take the chunking that minimises
-// that product (on 580 x 580 x 380: 95 planes forward, 190 reverse).
+// z planes per tile of the 3-D kernels for this grid: the busiest of the
+// persistent blocks (two per SM forward, one reverse) streams ceil(tiles /
+// blocks) tiles of zc + 8 planes each (8 halo planes per tile), so take the
+// chunking that minimises that product (on 580 x 580 x 380: 95 planes forward,
+// 190 reverse; on 191 x 150 x 133: 17 and 34).  Chunks go down to 4 planes: a
+// small grid has too few tiles otherwise (60 x 60 x 50: 5.3 us forward and 8.7
+// reverse against 12.4 and 15.4 with chunks of at least 16).
 int zc_for_3d(const Lay &L, bool fwd) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms < 1) sms = 1;
+  const int slots = fwd ? 2 * sms : sms;
   const long long per = (long long)cdiv(L.NX, kTileX) * cdiv(L.NY, fwd ? RBC_FWD3D_ROWS : kTY);
   int best = k3dZC;
   long long best_cost = -1;
-  for (int c = 1; c <= cdiv(L.NZ, 16); ++c) {
+  for (int c = 1; c <= cdiv(L.NZ, 4); ++c) {
     const int zc = cdiv(L.NZ, c);
-    const long long cost = ((per * c + sms - 1) / sms) * (zc + 8);
+    const long long cost = ((per * c + slots - 1) / slots) * (zc + 8);
     if (best_cost < 0 || cost < best_cost) best_cost = cost, best = zc;
   }
   return best;
@@ -577,8 +679,8 @@ bool launch_fwd3d(const StepArgs &A, cudaStream_t s) {
   if (!make_map(&mc, A.L, A.cur, kHaloW, TY + 8) || !make_map(&ma, A.L, A.a, kTileX, TY) ||
       !make_map(&mo, A.L, A.nxt, kTileX, TY))
     return false;
-  k_fwd3d_tma<TY><<<persistent_grid(A.L, A.zc, TY, (const void *)k_fwd3d_tma<TY>, 32 * (TY + 1), smem),
-                    dim3(32, TY + 1), smem, s>>>(mc, ma, mo, A);
+  launch_pdl(k_fwd3d_tma<TY>, dim3(persistent_grid(A.L, A.zc, TY, (const void *)k_fwd3d_tma<TY>, 32 * (TY / 2 + 1), smem)),
+             dim3(32, TY / 2 + 1), smem, s, mc, ma, mo, A);
   return true;
 }
 
@@ -594,8 +696,9 @@ bool launch_rev3d(const RevArgs &A, cudaStream_t s) {
       !make_map(&mbn, A.L, A.bn, kTileX, kTY) || !make_map(&mnum, A.L, A.num, kTileX, kTY) ||
       !make_map(&mden, A.L, A.den, kTileX, kTY))
     return false;
-  k_rev3d_tma<<<persistent_grid(A.L, A.zc, kTY, (const void *)k_rev3d_tma, 32 * (2 * kTY + 1), kRevSmem),
-                dim3(32, 2 * kTY + 1), kRevSmem, s>>>(mr, mb, ma, mrn, mbn, mnum, mden, A);
+  launch_pdl(k_rev3d_tma,
+             dim3(persistent_grid(A.L, A.zc, kTY, (const void *)k_rev3d_tma, 32 * (kRevW + 1), kRevSmem)),
+             dim3(32, kRevW + 1), kRevSmem, s, mr, mb, ma, mrn, mbn, mnum, mden, A);
   return true;
 }
 

@@ -100,8 +100,10 @@ __device__ __forceinline__ float4 sub4(const float4 a, const float4 b) {
 }
 
 // h^2 Laplacian at four consecutive nodes: x window (lf, c, rt); z[k-1] =
-// D_k[row] - D_k[row - k].
-__device__ __forceinline__ float4 lap_shared(const float4 lf, const float4 c, const float4 rt, const float4 *z) {
+// D_k[row] - D_k[row - k] (3-D: y[k-1] along the third axis).
+template <bool kThreeD = false>
+__device__ __forceinline__ float4 lap_shared(const float4 lf, const float4 c, const float4 rt, const float4 *z,
+                                             const float4 *y = nullptr) {
   const float w[12] = {lf.x, lf.y, lf.z, lf.w, c.x, c.y, c.z, c.w, rt.x, rt.y, rt.z, rt.w};
   float d1[5], d3[7];
   float2 d2[3], d4[4];
@@ -123,13 +125,21 @@ __device__ __forceinline__ float4 lap_shared(const float4 lf, const float4 c, co
     s[2] = make_float2(d3[2 * j + 3] - d3[2 * j], d3[2 * j + 4] - d3[2 * j + 1]);
     s[3] = sub2(d4[j + 2], d4[j]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = __fadd2_rn(s[k], half2of(z[k], j));
+    for (int k = 0; k < 4; ++k) {
+      s[k] = __fadd2_rn(s[k], half2of(z[k], j));
+      if (kThreeD) s[k] = __fadd2_rn(s[k], half2of(y[k], j));
+    }
     float2 lap = __fmul2_rn(make_float2(kC4, kC4), s[3]);
     lap = __ffma2_rn(make_float2(kC3, kC3), s[2], lap);
     lap = __ffma2_rn(make_float2(kC2, kC2), s[1], lap);
     out[j] = __ffma2_rn(make_float2(kC1, kC1), s[0], lap);
   }
   return make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
+}
+
+// (m - p) + (q - p) for the neighbours m, q of p on either side
+__device__ __forceinline__ float4 pair_diff(const float4 m, const float4 p, const float4 q) {
+  return sub4(sub4(q, p), sub4(p, m));
 }
 
 // (2 p - p_old) + a lap; *inc (kInc) = a lap, rounded by itself as in leap4p_inc.
