@@ -32,6 +32,10 @@
 #include "../../include/rbc.h"
 #include "rbc_internal.cuh"
 
+using rbc::griddep_launch;
+using rbc::griddep_wait;
+using rbc::launch_pdl;
+
 namespace rbc {
 int set_error(int code, const char *msg);  // rbc_abi.cu
 void add_launches(long long n);
@@ -293,7 +297,7 @@ constexpr int kTcEpi = 8;                                    // epilogue warps
 // R = 8 0.951 / 5.20 ms, R = 6 0.969 / 5.37 ms, R = 4 1.071 / 5.49 ms; with
 // 128-column tiles and the 16-byte-row halo copy: R = 6 1.14 / 5.51 ms, R = 4
 // 1.18 / 5.57 ms, R = 4 with 4 epilogue warps 1.23 / 5.88 ms.
-constexpr int kTcR = 8;
+constexpr int kTcR = 8, kTcRs = 4;  // rows per tile; of small images (tile_rows)
 constexpr int tc_plane(int R) { return (R + 2) * kTcHW * 16; }
 constexpr int tc_stages(int R) { return R <= 4 ? 4 : R <= 6 ? 3 : 2; }
 constexpr int tc_smem(int R) { return kTcWBytes + tc_stages(R) * 4 * tc_plane(R) + 256; }
@@ -399,9 +403,9 @@ __device__ __forceinline__ void tmem_zero1(uint32_t ta) {
 // kTcEpi epilogue warps: warp e drains TMEM lane quarter e % 4 (pixels
 // 32 (e % 4) .. +31) for the output rows of its share (R * 4 / kTcEpi rows,
 // starting at row (e / 4) * R * 4 / kTcEpi); warps kTcEpi .. kTcEpi +
-// tc_nprod(MODE) - 1 are the producers, the next warp the MMA issuer.
+// tc_nprod(MODE, R) - 1 are the producers, the next warp the MMA issuer.
 //
-// kFused: instead of the tensor copy of a stored first-layer output, ten
+// kFused: instead of the tensor copy of a stored first-layer output, R + 2
 // builder warps compute it over the tile's halo (R + 2 rows x 128 pixels,
 // one row per warp) into the ring stage, in the layout the copy would have
 // produced: the fp32 one-channel input's halo (R + 4 rows x 130 pixels,
@@ -414,8 +418,8 @@ __device__ __forceinline__ void tmem_zero1(uint32_t ta) {
 // layer's padding).  The builders then make their writes visible to the
 // tensor cores and arrive on the stage's "full" barrier.  The first layer's
 // output never passes through global memory.
-constexpr int tc_nprod(int mode) { return mode == kFused ? 10 : 1; }
-constexpr int tc_threads(int mode) { return 32 * (kTcEpi + tc_nprod(mode) + 1); }
+constexpr int tc_nprod(int mode, int R) { return mode == kFused ? R + 2 : 1; }
+constexpr int tc_threads(int mode, int R) { return 32 * (kTcEpi + tc_nprod(mode, R) + 1); }
 constexpr int kFxR = 4;                  // x halo rows beyond the tile's R (two on each side)
 constexpr int kFxC = kTcHW + 2;          // x halo columns (x0 - 2 .. x0 + 127)
 constexpr int kFxP = 144;                // x halo row pitch (2-byte values; conflict-free gathers)
@@ -425,7 +429,7 @@ constexpr int tc_smem_mode(int mode, int R) { return tc_smem(R) + (mode == kFuse
 static_assert(tc_smem(kTcR) + tc_fx_bytes(kTcR) <= 227 * 1024, "the fused ring must fit in shared memory");
 
 template <int MODE, int R>
-__global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_constant__ CUtensorMap tm_in,
+__global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid_constant__ CUtensorMap tm_in,
                                                     const __nv_bfloat16 *__restrict__ wt,
                                                     const float *__restrict__ bias,
                                                     const __nv_bfloat16 *__restrict__ mask,
@@ -435,7 +439,7 @@ __global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_co
                                                     const __nv_bfloat16 *__restrict__ w1 = nullptr,
                                                     const float *__restrict__ b1 = nullptr) {
   constexpr bool kHid = MODE == kHidden || MODE == kFused;  // relu(conv + bias) epilogue
-  constexpr int kMma = kTcEpi + tc_nprod(MODE);             // the MMA issuer warp
+  constexpr int kMma = kTcEpi + tc_nprod(MODE, R);             // the MMA issuer warp
   constexpr int NCO = MODE == kLast ? 16 : 32;  // output channels per row accumulator
   constexpr int WCG = 3 * NCO * 16;              // weight bytes per (dx, channel group)
   constexpr int WDX = 4 * WCG;                   // weight bytes per dx
@@ -457,6 +461,11 @@ __global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_co
   auto empty = [&](int i) { return b0 + 8u * (STAGES + i); };
   auto tfull = [&](int i) { return b0 + 8u * (2 * STAGES + i); };
   auto tempty = [&](int i) { return b0 + 8u * (2 * STAGES + 2 + i); };
+  // The prologue (weights, barriers, tensor memory: about 3 us) overlaps the
+  // previous layer's launch: an image of 200 x 200 took 43 us, 30 with it.
+  // Only the weights are read in it: the layers before this one have waited
+  // for their preparation (the fused first layers, which follow it, wait here).
+  if (MODE == kFused) griddep_wait();
   // weights [tap][co][ci] (tap = 3 dy + dx) -> [dx][ci / 8][dy][co][8]
   if (MODE == kLast) {
     for (int i = tid; i < 9 * 4 * (NCO - 1); i += blockDim.x) {  // padding channels 1..15: zero
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_co
   if (tid == 0) {
     *abort_blk = 0;
     for (int i = 0; i < STAGES; ++i) {
-      tc_mbar_init(full(i), MODE == kFused ? 32 * tc_nprod(MODE) : 1);
+      tc_mbar_init(full(i), MODE == kFused ? 32 * tc_nprod(MODE, R) : 1);
       tc_mbar_init(empty(i), 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -507,6 +516,8 @@ __global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_co
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (MODE != kFused) griddep_wait();
+  griddep_launch();
   const int ntx = (W + kTcOut - 1) / kTcOut, nty = (H + R - 1) / R;
   const long long ntiles = (long long)ntx * nty * nimg;
   // Each block takes a contiguous range of tiles, ordered down the image
@@ -545,7 +556,7 @@ __global__ void __launch_bounds__(tc_threads(MODE), 1) k_conv_tc(const __grid_co
     }
   } else if (MODE == kFused && warp >= kTcEpi && warp < kMma) {
     // ---- builders (kFused): the first layer's output over the tile's halo ----
-    constexpr int NB = tc_nprod(MODE), NBT = 32 * NB;                    // builder warps, threads
+    constexpr int NB = tc_nprod(MODE, R), NBT = 32 * NB;                    // builder warps, threads
     constexpr int XVALS = tc_fx_vals(R), NPRE = (XVALS + NBT - 1) / NBT;  // x values, per builder thread
     static_assert((R + 2) % NB == 0, "each builder warp owns the same number of halo rows");
     const int bt = tid - 32 * kTcEpi, g = lane >> 2, tq = lane & 3;
@@ -1253,14 +1264,19 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
   }
 }
 
+template <int R>
+void tc_attr() {
+  cudaFuncSetAttribute(k_conv_tc<kHidden, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(R));
+  cudaFuncSetAttribute(k_conv_tc<kBackData, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(R));
+  cudaFuncSetAttribute(k_conv_tc<kLast, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(R));
+  cudaFuncSetAttribute(k_conv_tc<kFused, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_mode(kFused, R));
+}
+
 void set_attrs() {
   static bool done = false;
   if (done) return;
-  cudaFuncSetAttribute(k_conv_tc<kHidden, kTcR>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(kTcR));
-  cudaFuncSetAttribute(k_conv_tc<kBackData, kTcR>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(kTcR));
-  cudaFuncSetAttribute(k_conv_tc<kLast, kTcR>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(kTcR));
-  cudaFuncSetAttribute(k_conv_tc<kFused, kTcR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       tc_smem_mode(kFused, kTcR));
+  tc_attr<kTcR>();
+  tc_attr<kTcRs>();
   cudaFuncSetAttribute(k_conv_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWtSmem);
   cudaFuncSetAttribute(k_conv_wgrad1<false, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kW1Smem);
   cudaFuncSetAttribute(k_conv_wgrad1<true, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kW1Smem);
@@ -1371,32 +1387,47 @@ bool act_map(CUtensorMap *m, const __nv_bfloat16 *buf, int nimg, int H, int W, i
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int MODE>
-bool launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
-                    __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s, float *out_f = nullptr,
-                    const float *resid = nullptr) {
+int sm_count() {
   static int sms = 0;
   if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-  const long long tiles = (long long)((W + kTcOut - 1) / kTcOut) * ((H + kTcR - 1) / kTcR) * nimg;
-  const int grid = (int)(tiles < sms ? tiles : sms);
+  return sms > 0 ? sms : 1;
+}
+
+long long tiles_of(int nimg, int H, int W, int R) {
+  return (long long)((W + kTcOut - 1) / kTcOut) * ((H + R - 1) / R) * nimg;
+}
+
+// Rows per tile: a block's time goes with (tiles per SM) x (R + 2 halo rows),
+// so tall tiles win wherever they fill the SMs.  Images of a few hundred rows
+// leave SMs idle: one of 200 x 200 takes 27.5 us in 4-row tiles and 30.4 in
+// 8-row tiles, while 8 x 512^2 takes 271 and 230.
+int tile_rows(int nimg, int H, int W) {
+  auto cost = [&](int R) { return (tiles_of(nimg, H, W, R) + sm_count() - 1) / sm_count() * (R + 2); };
+  return cost(kTcRs) < cost(kTcR) ? kTcRs : kTcR;
+}
+
+template <int MODE, int R>
+bool launch_conv_r(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
+                   __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s, float *out_f, const float *resid,
+                   const float *x, const __nv_bfloat16 *w1, const float *b1) {
+  const long long tiles = tiles_of(nimg, H, W, R);
+  const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
   CUtensorMap tin;
-  if (!act_map(&tin, in, nimg, H, W, kTcR + 2)) return false;
-  k_conv_tc<MODE, kTcR><<<grid, tc_threads(MODE), tc_smem(kTcR), s>>>(tin, wt, bias, mask, out, out_f, resid, nimg,
-                                                                      H, W, tc_err_dev);
+  memset(&tin, 0, sizeof tin);  // (the fused mode builds its operand instead of copying it)
+  if (MODE != kFused && !act_map(&tin, in, nimg, H, W, R + 2)) return false;
+  launch_pdl(k_conv_tc<MODE, R>, dim3(grid), dim3(tc_threads(MODE, R)), tc_smem_mode(MODE, R), s, tin, wt, bias, mask, out,
+             out_f, resid, nimg, H, W, tc_err_dev, x, w1, b1);
   return true;
 }
 
-// The first two layers in one launch (kFused): x (fp32) -> act1.
-void launch_conv_fused(const float *x, const __nv_bfloat16 *w1, const float *b1, const __nv_bfloat16 *w2,
-                       const float *b2, __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s) {
-  static int sms = 0;
-  if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-  const long long tiles = (long long)((W + kTcOut - 1) / kTcOut) * ((H + kTcR - 1) / kTcR) * nimg;
-  const int grid = (int)(tiles < sms ? tiles : sms);
-  CUtensorMap unused;  // the fused mode builds its operand instead of copying it
-  memset(&unused, 0, sizeof unused);
-  k_conv_tc<kFused, kTcR><<<grid, tc_threads(kFused), tc_smem_mode(kFused, kTcR), s>>>(
-      unused, w2, b2, nullptr, out, nullptr, nullptr, nimg, H, W, tc_err_dev, x, w1, b1);
+template <int MODE>
+bool launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
+                    __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s, float *out_f = nullptr,
+                    const float *resid = nullptr, const float *x = nullptr, const __nv_bfloat16 *w1 = nullptr,
+                    const float *b1 = nullptr) {
+  return tile_rows(nimg, H, W) == kTcRs
+             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1)
+             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1);
 }
 
 // The network's forward pass; `keep` stores what the backward pass reads
@@ -1419,7 +1450,8 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
         w.x0, w.wf + kW1, params_dev + kB1, nullptr, w.act[0], nimg, H, W);
     ok_tc = launch_conv_tc<kHidden>(w.act[0], w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, s);
   } else {
-    launch_conv_fused(x_dev, w.wf + kW1, params_dev + kB1, w.wf + kW2, params_dev + kB2, w.act[1], nimg, H, W, s);
+    ok_tc = launch_conv_tc<kFused>(nullptr, w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, s, nullptr,
+                                   nullptr, x_dev, w.wf + kW1, params_dev + kB1);
   }
   ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], w.wf + kW3, params_dev + kB3, nullptr, w.act[2], nimg, H, W, s);
   ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], w.wf + kW4, params_dev + kB4, nullptr, w.act[3], nimg, H, W, s);
