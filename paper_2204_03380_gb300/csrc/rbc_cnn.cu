@@ -804,81 +804,75 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t *r, const void *smem_row) {
 // Weight and bias gradients of the 32 -> 32 layers on the 5th-generation
 // tensor cores:
 //   dW[dy][dx][co][ci] = sum_p dz[co][p] x[ci][p + (dy - 1, dx - 1)],   db[co] = sum_p dz[co][p].
-// Re-indexed by q = p + (dy - 1) rows, the taps split between the operands:
-//   dW[dy][dx][co][ci] = sum_q x[ci][q + (0, dx - 1)] dz[co][q - (dy - 1, 0)],
-// so that one MMA per 16 pixels q of a row (K = 16) computes all nine taps,
-// D[32 dx + ci][32 (2 - dy) + co] (M = 128, N = 96; fp32 in tensor memory).
-// Both operands are MN-major (channels contiguous) in a pixel-major layout
-// with the 64-byte swizzle: a pixel's 32 channels form one 64-byte row, and
-// the swizzle is a function of the shared-memory address, so a descriptor
-// may start at any pixel.  A = x: its 32-row M blocks start one pixel apart
-// (leading byte offset 64), block j holding the tap dx = j (block 3 is read
-// but not used); B = dz: its 32-column N blocks start one staged row apart,
-// block i holding the tap dy = 2 - i; a K step of 8 pixels is 512 bytes.
-// Tiles of 4 rows x 128 pixels: x is staged over the tile's rows and pixels
-// x0 - 1 .. x0 + 130, dz over rows y0 - 1 .. y0 + 4 and pixels x0 .. x0 + 127,
-// in two stages: the 512 threads load tile k + 1 into registers (16 bytes
-// per chunk, consecutive lanes on consecutive pixels of a channel-group plane,
-// so the loads coalesce; zero outside the image) while tile k is multiplied,
-// and store the chunks into their swizzled places once tile k - 1's MMAs have
-// released the stage.  (cp.async copies into the swizzled places do not
-// coalesce: about 30 L2 requests per warp instruction against 4 for linear
-// destinations, measured; and a tensor copy with the 64-byte swizzle pads a
-// box whose rows are the planar layout's 16 bytes.)  One thread issues a
-// tile's 32 MMAs into the accumulator the block keeps over all its tiles;
-// meanwhile the block's threads sum dz over the tile's own rows for db (one
-// pixel each).  At the end warps 0-2 read the accumulator
-// (lane 32 dx + ci) and add it to dW.  Every wait is bounded; a block that
-// gives up flags the error word.
-constexpr int kWtR = 4, kWtC = 128, kWtXP = kWtC + 4;       // rows, pixels per row, staged x pixels per row
-constexpr int kWtXB = kWtR * kWtXP * 64;                    // staged x bytes
-constexpr int kWtZB = (kWtR + 2) * kWtC * 64;               // staged dz bytes
-constexpr int kWtStage = kWtXB + kWtZB;
-constexpr size_t kWtSmem = 2 * (size_t)kWtStage + 1024;
-static_assert(kWtXB % 1024 == 0 && kWtStage % 1024 == 0, "staged regions start on the swizzle period");
-static_assert(kWtSmem <= 227 * 1024, "two stages must fit in shared memory");
-// kind::f16, fp32 accumulator, bf16 A and B, both MN-major, N = 96, M = 128
+// Tiles of kWtR rows x kWtC pixels of x; two tensor copies stage its rows (with
+// a pixel on either side) and dz's (with a row on either side) as they lie in
+// memory, [row][channel group][pixel][8 channels].  That is the MN-major
+// operand layout without a swizzle: 8 pixels of a group are a core matrix
+// (pixels K, channels MN; 128 contiguous bytes), the next 8 pixels follow, and the
+// channel groups of consecutive rows are equally far apart, so one operand may
+// span several rows.  An MMA takes four dz rows (M = 4 x 32 channels) against two
+// x rows (N = 2 x 32) over 16 pixels (K); the three horizontal taps move x's start by a
+// pixel and have accumulators of their own:
+//   D_dx[32 j + co][32 i + ci] = sum dz[co][row y - 1 + j][px] x[ci][row y + i][px + dx - 1],
+// the tap dy = 2 + i - j for j - i in 0..2; the two other row pairs are not used.
+// (x on M and dz on N reads x's unaligned starts twice as often.)
+// Three stages: warp 4 copies, one thread of warp 5 issues the MMAs, warps 0-3 (one
+// channel group each) sum dz over the tile's own rows for db.  At the end warps 0-3 add
+// the two row pairs of each tap in shared memory and the block adds
+// them to dW, once.  Bound by the operands' shared-memory reads (6 KB per MMA, 66
+// cycles; x's starts are not on 128 bytes) and DRAM together: 8 x 512^2 takes
+// 49 us (268 MB: 5.5 TB/s) where staging through registers into swizzled
+// pixel-major rows, with two block barriers a tile, took 95.
+// Every wait is bounded; a block that gives up flags the error word.
+constexpr int kWtR = 8, kWtC = 64, kWtXP = kWtC + 2;        // x rows, pixels per row, staged x pixels per row
+constexpr int kWtXRow = 4 * kWtXP * 16, kWtZRow = 4 * kWtC * 16;  // bytes of a staged x, dz row
+constexpr int kWtXB = kWtR * kWtXRow, kWtZB = (kWtR + 2) * kWtZRow;  // staged x, dz bytes
+constexpr int kWtStage = kWtXB + kWtZB, kWtStages = 3;
+constexpr size_t kWtSmem = kWtStages * (size_t)kWtStage + 1024;
+static_assert(kWtXB % 128 == 0 && kWtZB % 128 == 0, "the copies land on 128 bytes");
+static_assert(kWtSmem <= 227 * 1024, "the stages must fit in shared memory");
+static_assert(9 * 32 * 33 * 4 <= kWtStages * kWtStage, "the taps' sums reuse the stages");
+// kind::f16, fp32 accumulator, bf16 A and B, both MN-major, N = 64, M = 128
 constexpr uint32_t kWtIdesc =
-    (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((96u >> 3) << 17) | ((128u >> 4) << 24);
+    (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr int kWtThreads = 192;
 
-// 64-byte swizzle of a byte offset from a 1024-byte-aligned base: the 16-byte
-// chunk index (bits 4-5) XOR bits 7-8.
-__device__ __forceinline__ uint32_t swz64(uint32_t off) { return off ^ (((off >> 7) & 3u) << 4); }
-__device__ __forceinline__ uint64_t umma_desc_sw64(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  // start, leading (MN block) and stride (K block) byte offsets in 16-byte
-  // units, descriptor version 1, layout type 4 (64-byte swizzle), base offset 0
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46) | (4ull << 61);
+__device__ __forceinline__ void wt_copy(uint32_t dst, const CUtensorMap *tm, int c0, int y, int img, uint32_t bar) {
+  // coordinates (8-byte element along the row, group 0, y, image)
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+      "%5}], [%6];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(0), "r"(y), "r"(img), "r"(bar)
+      : "memory");
 }
 
-constexpr int kWtThreads = 512;
-constexpr int kWtXC = 4 * kWtR * kWtXP, kWtZC = 4 * (kWtR + 2) * kWtC;  // 16-byte chunks of a tile's x and dz
-constexpr int kWtPre = (kWtXC + kWtZC + kWtThreads - 1) / kWtThreads;   // chunks per thread
-__global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __nv_bfloat16 *__restrict__ x,
-                                                                 const __nv_bfloat16 *__restrict__ dz,
+__global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tm_x,
+                                                                 const __grid_constant__ CUtensorMap tm_z,
                                                                  float *__restrict__ dw, float *__restrict__ db,
                                                                  int nimg, int H, int W, int *err) {
-  extern __shared__ unsigned char s_raw[];
-  __shared__ __align__(8) uint64_t s_bar[2];
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t s_bar[2 * kWtStages + 1];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  __shared__ float s_db[32];
-  const uint32_t raw = (uint32_t)__cvta_generic_to_shared(s_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  unsigned char *gbase = s_raw + (base - raw);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ntx = (W + kWtC - 1) / kWtC, tpi = ntx * ((H + kWtR - 1) / kWtR), ntiles = tpi * nimg;
-  const long long HWp = (long long)H * W;
-  const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&s_bar[0]);
+  const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(s_bar);
+  auto full = [&](int i) { return bar0 + 8u * i; };
+  auto empty = [&](int i) { return bar0 + 8u * (kWtStages + i); };
+  const uint32_t done = bar0 + 8u * (2 * kWtStages);
+  volatile int *abort_blk = &s_abort;
   if (tid == 0) {
     s_abort = 0;
-    tc_mbar_init(bar0, 1);
-    tc_mbar_init(bar0 + 8, 1);
+    for (int i = 0; i < kWtStages; ++i) {
+      tc_mbar_init(full(i), 1);
+      tc_mbar_init(empty(i), 5);  // the MMAs and the four warps that sum dz
+    }
+    tc_mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (tid < 32) s_db[tid] = 0.f;
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
+  if (warp == 5) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(
         (uint32_t)__cvta_generic_to_shared(&s_tmem)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -886,154 +880,135 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __nv_bflo
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
-  auto origin = [&](int tt, int &img, int &y0, int &x0) {
-    img = tt / tpi;
-    const int rem = tt - img * tpi, ty = rem / ntx;
-    y0 = ty * kWtR;
-    x0 = (rem - ty * ntx) * kWtC;
-  };
-  // chunk e of a tile: x chunks [group][row][pixel], then dz chunks [group][row][pixel]
-  // (consecutive lanes read consecutive pixels of one group plane); its
-  // global offset (in 16-byte units, -1 outside the image) and its shared-memory byte offset
-  auto chunk = [&](int e, int img, int y0, int x0, long long &g, uint32_t &o) {
-    int n, r, i, yy, xx;
-    bool ok;
-    if (e < kWtXC) {
-      n = e / (kWtR * kWtXP);
-      const int rem = e - n * (kWtR * kWtXP);
-      r = rem / kWtXP;
-      i = rem - r * kWtXP;
-      yy = y0 + r;
-      xx = x0 - 1 + i;
-      ok = yy < H && xx >= 0 && xx < W;
-      o = swz64((uint32_t)((r * kWtXP + i) * 64 + n * 16));
-    } else {
-      const int e2 = e - kWtXC;
-      n = e2 / ((kWtR + 2) * kWtC);
-      const int rem = e2 - n * ((kWtR + 2) * kWtC);
-      r = rem / kWtC;
-      i = rem - r * kWtC;
-      yy = y0 - 1 + r;
-      xx = x0 + i;
-      ok = yy >= 0 && yy < H && xx < W;
-      o = kWtXB + swz64((uint32_t)((r * kWtC + i) * 64 + n * 16));
-    }
-    g = ok ? ((long long)img * 4 + n) * HWp + (long long)yy * W + xx : -1;
-  };
-  // this thread's chunks of tile tt into registers (loads left in flight)
-  auto load = [&](int tt, uint4 *v) {
-    int img, y0, x0;
-    origin(tt, img, y0, x0);
+  griddep_wait();
+  griddep_launch();
+  float bsum[8];  // warps 0-3: channels 8 warp .. 8 warp + 7
 #pragma unroll
-    for (int j = 0; j < kWtPre; ++j) {
-      const int e = tid + kWtThreads * j;
-      v[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (e < kWtXC + kWtZC) {
-        long long g;
-        uint32_t o;
-        chunk(e, img, y0, x0, g, o);
-        if (g >= 0) v[j] = __ldg(reinterpret_cast<const uint4 *>(e < kWtXC ? x : dz) + g);
+  for (int c = 0; c < 8; ++c) bsum[c] = 0.f;
+  if (warp == 4) {
+    if (lane == 0) {
+      int k = 0;
+      for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
+        const int s = k % kWtStages, u = k / kWtStages;
+        if (u > 0 && !tc_wait(empty(s), (u - 1) & 1, abort_blk)) break;
+        const int img = tt / tpi, rem = tt - img * tpi, ty = rem / ntx;
+        const int y0 = ty * kWtR, x0 = (rem - ty * ntx) * kWtC;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(kWtStage)
+                     : "memory");
+        wt_copy(base + s * kWtStage, &tm_x, 2 * (x0 - 1), y0, img, full(s));
+        wt_copy(base + s * kWtStage + kWtXB, &tm_z, 2 * x0, y0 - 1, img, full(s));
       }
-    }
-  };
-  auto store = [&](int tt, int sb, const uint4 *v) {
-    int img, y0, x0;
-    origin(tt, img, y0, x0);
-    unsigned char *st = gbase + sb * kWtStage;
-#pragma unroll
-    for (int j = 0; j < kWtPre; ++j) {
-      const int e = tid + kWtThreads * j;
-      if (e < kWtXC + kWtZC) {
-        long long g;
-        uint32_t o;
-        chunk(e, img, y0, x0, g, o);
-        *reinterpret_cast<uint4 *>(st + o) = v[j];
-      }
-    }
-  };
-  float bsum[32];
-#pragma unroll
-  for (int c = 0; c < 32; ++c) bsum[c] = 0.f;
-  uint4 v[kWtPre];
-  int k = 0;
-  if ((int)blockIdx.x < ntiles) {
-    load(blockIdx.x, v);
-    store(blockIdx.x, 0, v);
-  }
-  for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
-    const int sb = k & 1, tn = tt + gridDim.x;
-    if (tn < ntiles) load(tn, v);  // in flight while tile k is multiplied
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // this thread's stores, to the tensor cores
-    __syncthreads();                                               // tile k is staged
-    const uint32_t X = base + sb * kWtStage, Z = X + kWtXB;
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t a0 = umma_desc_sw64(X, 64, 512), b0 = umma_desc_sw64(Z, kWtC * 64, 512);
-#pragma unroll
-      for (int r = 0; r < kWtR; ++r)
-#pragma unroll
-        for (int c = 0; c < kWtC / 16; ++c) {
-          const uint64_t ad = a0 + (uint64_t)(((r * kWtXP + 16 * c) * 64) >> 4);
-          const uint64_t bd = b0 + (uint64_t)(((r * kWtC + 16 * c) * 64) >> 4);
-          const uint32_t acc = (k > 0 || r > 0 || c > 0) ? 1u : 0u;
-          asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem), "l"(ad), "l"(bd),
-                       "r"(kWtIdesc), "r"(acc));
+      if (*abort_blk) {  // let the copies in flight land before the block exits
+        for (int i = (k > kWtStages ? k - kWtStages : 0); i < k; ++i) {
+          const long long t0 = clock64();
+          while (!tc_try(full(i % kWtStages), (i / kWtStages) & 1) && clock64() - t0 < kTcWaitCycles) {
+          }
         }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 8 * sb)
-                   : "memory");
-    }
-    // db: dz of the tile's own rows (staged rows 1 .. 4), one pixel per thread
-    static_assert(kWtThreads == kWtR * kWtC, "one pixel of the tile per thread");
-    const unsigned char *zg = gbase + sb * kWtStage + kWtXB;
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      const uint4 q = *reinterpret_cast<const uint4 *>(zg + swz64((uint32_t)((kWtC + tid) * 64 + n * 16)));
-      const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&q);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(h2[e]);
-        bsum[8 * n + 2 * e] += f.x;
-        bsum[8 * n + 2 * e + 1] += f.y;
       }
     }
-    if (tn < ntiles) {
-      // stage sb ^ 1 is free once tile k - 1's MMAs are done (its sums were
-      // read before this iteration's barrier)
-      if (k >= 1 && tid == 0) tc_wait(bar0 + 8 * (sb ^ 1), ((k - 1) >> 1) & 1, &s_abort);
-      __syncthreads();
-      if (s_abort) break;
-      store(tn, sb ^ 1, v);
+  } else if (warp == 5) {
+    if (lane == 0) {
+      int k = 0;
+      for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
+        const int s = k % kWtStages;
+        if (!tc_wait(full(s), (k / kWtStages) & 1, abort_blk)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t X = base + s * kWtStage, Z = X + kWtXB;
+        // leading offset: the next 8 pixels; stride offset: the next channel group
+        const uint64_t a0 = umma_desc(Z, 128, kWtC * 16), b0 = umma_desc(X, 128, kWtXP * 16);
+#pragma unroll
+        for (int r = 0; r < kWtR; r += 2)
+#pragma unroll
+          for (int c = 0; c < kWtC; c += 16)
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              const uint64_t ad = a0 + (uint64_t)((r * kWtZRow + c * 16) >> 4);
+              const uint64_t bd = b0 + (uint64_t)((r * kWtXRow + (c + dx) * 16) >> 4);
+              const uint32_t acc = (k > 0 || r > 0 || c > 0) ? 1u : 0u;
+              asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                           "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + 64 * dx),
+                           "l"(ad), "l"(bd), "r"(kWtIdesc), "r"(acc));
+            }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(s))
+                     : "memory");
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
+                   : "memory");
+      const long long t0 = clock64();  // whatever ended the loop, the MMAs issued finish first
+      while (!tc_try(done, 0)) {
+        if (clock64() - t0 > kTcWaitCycles) {
+          *abort_blk = 1;
+          break;
+        }
+      }
+    }
+  } else {
+    int k = 0;
+    for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
+      const int s = k % kWtStages;
+      const bool got = tc_wait(full(s), (k / kWtStages) & 1, abort_blk);
+      if (__any_sync(0xffffffffu, !got)) break;
+      // dz of the tile's own rows (staged rows 1 .. kWtR), two pixels per thread and row
+      const unsigned char *z = smem + s * kWtStage + kWtXB + kWtZRow + (warp * kWtC + lane) * 16;
+      float t8[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) t8[c] = 0.f;
+#pragma unroll 4
+      for (int r = 0; r < kWtR; ++r) {
+        static_assert(kWtC == 64, "two pixels of a row per lane");
+        const uint4 q[2] = {*reinterpret_cast<const uint4 *>(z + r * kWtZRow),
+                            *reinterpret_cast<const uint4 *>(z + r * kWtZRow + 512)};
+        const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(q);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 f = __bfloat1622float2(h2[e]), g = __bfloat1622float2(h2[4 + e]);
+          t8[2 * e] += f.x + g.x;
+          t8[2 * e + 1] += f.y + g.y;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) tc_arrive(empty(s));
+#pragma unroll
+      for (int c = 0; c < 8; ++c) bsum[c] += t8[c];
     }
   }
-  if (k > 0 && tid == 0 && !s_abort) tc_wait(bar0 + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1, &s_abort);
-  __syncthreads();
+  __syncthreads();  // the MMAs are done, or the block gave up
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool ok = !s_abort;
-  if (ok && k > 0 && warp < 3) {  // lanes 32 dx + ci; column 32 (2 - dy) + co
+  // lane = co, column 64 dx + 32 i + ci; the stages are free
+  float *s_w = reinterpret_cast<float *>(smem);  // [tap][co][33]
 #pragma unroll 1
-    for (int c0 = 0; c0 < 96; c0 += 32) {
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
-      const int dyy = 2 - c0 / 32;
+  for (int i = 0; i < 2; ++i) {
+    if (ok && warp >= i && warp < 3 + i) {
+      const int dyy = 2 + i - warp;
+#pragma unroll 1
+      for (int dx = 0; dx < 3; ++dx) {
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + 64 * dx + 32 * i, v);
+        float *o = s_w + ((3 * dyy + dx) * 32 + lane) * 33;
 #pragma unroll
-      for (int c = 0; c < 32; ++c) atomicAdd(dw + ((3 * dyy + warp) * 32 + c) * 32 + lane, v[c]);
+        for (int c = 0; c < 32; ++c) o[c] = i == 0 ? v[c] : o[c] + v[c];
+      }
+    }
+    __syncthreads();
+  }
+  if (ok) {
+    for (int e = tid; e < 9 * 32 * 32; e += kWtThreads) atomicAdd(dw + e, s_w[(e >> 5) * 33 + (e & 31)]);
+    if (warp < 4) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        float v = bsum[c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) atomicAdd(db + 8 * warp + c, v);
+      }
     }
   }
-#pragma unroll
-  for (int c = 0; c < 32; ++c) {
-    float v = bsum[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) atomicAdd(&s_db[c], v);
-  }
-  __syncthreads();
-  if (ok && tid < 32) atomicAdd(db + tid, s_db[tid]);
   if (!ok && tid == 0) atomicExch(err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
+  if (warp == 5) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
 }
 
 // Weight and bias gradients of the two one-channel end layers, without
@@ -1283,14 +1258,6 @@ void set_attrs() {
   done = true;
 }
 
-// Persistent grid of the tcgen05 weight-gradient kernel: one block per SM (its shared memory).
-int grid_wgrad_tc(int nimg, int H, int W) {
-  static int sms = 0;
-  if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-  const long long tiles = (long long)((W + kWtC - 1) / kWtC) * ((H + kWtR - 1) / kWtR) * nimg;
-  return (int)(tiles < sms ? tiles : sms);
-}
-
 // Persistent grid of the one-channel weight-gradient kernel (attributes set by set_attrs).
 template <bool kFirst, typename TU>
 int grid_wgrad1(int nimg, int H, int W) {
@@ -1387,6 +1354,21 @@ bool act_map(CUtensorMap *m, const __nv_bfloat16 *buf, int nimg, int H, int W, i
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same buffer with its groups before the rows (the weight gradient's
+// operands): dims (2 W elements of a row, group, y, image); box (px pixels, 4
+// groups, by rows, 1).
+bool rows_map(CUtensorMap *m, const __nv_bfloat16 *buf, int nimg, int H, int W, int px, int by) {
+  auto fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(rbc::tmap_encode_fn());
+  if (!fn) return false;
+  cuuint64_t dims[4] = {2 * (cuuint64_t)W, 4, (cuuint64_t)H, (cuuint64_t)nimg};
+  cuuint64_t strides[3] = {(cuuint64_t)W * H * 16, (cuuint64_t)W * 16, (cuuint64_t)W * H * 64};
+  cuuint32_t box[4] = {2 * (cuuint32_t)px, 4, (cuuint32_t)by, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<__nv_bfloat16 *>(buf), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int sm_count() {
   static int sms = 0;
   if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
@@ -1428,6 +1410,17 @@ bool launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const floa
   return tile_rows(nimg, H, W) == kTcRs
              ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1)
              : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1);
+}
+
+// One block per SM (its shared memory), at most one per tile.
+bool launch_wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *dw, float *db, int nimg, int H, int W,
+                  cudaStream_t s) {
+  const long long tiles = (long long)((W + kWtC - 1) / kWtC) * ((H + kWtR - 1) / kWtR) * nimg;
+  const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
+  CUtensorMap tx, tz;
+  if (!rows_map(&tx, x, nimg, H, W, kWtXP, kWtR) || !rows_map(&tz, dz, nimg, H, W, kWtC, kWtR + 2)) return false;
+  launch_pdl(k_conv_wgrad_tc, dim3(grid), dim3(kWtThreads), kWtSmem, s, tx, tz, dw, db, nimg, H, W, tc_err_dev);
+  return true;
 }
 
 // The network's forward pass; `keep` stores what the backward pass reads
@@ -1505,8 +1498,7 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
   const int woff[3] = {kW4, kW3, kW2}, boff[3] = {kB4, kB3, kB2};
   for (int l = 0; l < 3; ++l) {
     const int layer_in = 2 - l;  // act index of this layer's input: act3 (l=0) ... act1
-    k_conv_wgrad_tc<<<grid_wgrad_tc(nimg, H, W), kWtThreads, kWtSmem, s>>>(w.act[layer_in], w.dz[cur], grad_dev + woff[l],
-                                                                     grad_dev + boff[l], nimg, H, W, tc_err_dev);
+    ok_tc = ok_tc && launch_wgrad(w.act[layer_in], w.dz[cur], grad_dev + woff[l], grad_dev + boff[l], nimg, H, W, s);
     ok_tc = ok_tc && launch_conv_tc<kBackData>(w.dz[cur], w.wb + woff[l], nullptr, w.act[layer_in], w.dz[1 - cur], nimg, H, W, s);
     cur = 1 - cur;
   }
