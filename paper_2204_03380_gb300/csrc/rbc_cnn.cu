@@ -50,7 +50,7 @@ constexpr int kW1 = 0, kB1 = kW1 + 9 * C, kW2 = kB1 + C, kB2 = kW2 + 9 * C * C, 
               kNParams = kB5 + 1;
 
 __device__ __forceinline__ void mma16816(float *c, const uint32_t *a, const uint32_t *b) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
 //
 // Per block (one per SM, persistent over tiles), three roles: warp kTcEpi
 // streams each tile's halo (zero-filled outside the image) into a shared-
-// memory ring of tc_stages(R) stages (in the fused first-layer mode, builder
+// memory ring of tc_units(R) half tiles (in the fused first-layer mode, builder
 // warps compute it there instead); the next warp issues the 6 (R + 2)
 // MMAs of a tile into one of two tensor-memory accumulators and commits them
 // to the ring's "empty" and the accumulator's "full" barrier; warps 0 ..
@@ -290,20 +290,38 @@ constexpr int kTcHW = 128;                                   // halo row width (
 constexpr int kTcWBytes = 9 * 4 * 32 * 16;                   // weights, 18432 B
 constexpr long long kTcWaitCycles = 4000000000LL;            // about two seconds
 constexpr int kTcEpi = 8;                                    // epilogue warps
-// Tiles of R output rows: halo planes of R + 2 rows per channel group, a
-// ring of 4 stages for R = 4, 3 for R = 6 and 2 for R = 8 (what fits in
-// 227 KB); R = 8 fills tensor memory with the two accumulator buffers.
-// Measured at 32 x 512^2 with 126-column tiles (inference / training step):
+// Tiles of R output rows: R = 8 fills tensor memory with the two accumulator buffers.
+// Measured with a ring of whole tiles at 32 x 512^2 with 126-column tiles (inference / training step):
 // R = 8 0.951 / 5.20 ms, R = 6 0.969 / 5.37 ms, R = 4 1.071 / 5.49 ms; with
 // 128-column tiles and the 16-byte-row halo copy: R = 6 1.14 / 5.51 ms, R = 4
 // 1.18 / 5.57 ms, R = 4 with 4 epilogue warps 1.23 / 5.88 ms.
 constexpr int kTcR = 8, kTcRs = 4;  // rows per tile; of small images (tile_rows)
-constexpr int tc_plane(int R) { return (R + 2) * kTcHW * 16; }
-constexpr int tc_stages(int R) { return R <= 4 ? 4 : R <= 6 ? 3 : 2; }
-constexpr int tc_smem(int R) { return kTcWBytes + tc_stages(R) * 4 * tc_plane(R) + 256; }
-static_assert(tc_smem(6) <= 227 * 1024, "the R = 6 ring must fit in shared memory");
+// The ring holds units of half a tile's halo (four planes of tc_ur(R) rows of
+// 128 pixels), so that a copy starts when half a tile's MMAs are done.  Three units
+// of five rows: more in flight only crowds L2 when the layer's data do not fit
+// there.  Inference of 8 x 512^2 / 32 x 512^2 / 64 x 400 x 800, us: three units 192 /
+// 681 / 1511, four 190 / 697 / 1602, five 193 / 716 / 1629; two whole tiles 203 / 714 /
+// 1559; seven two-row units 187 / 675 / 1579.
+constexpr int kTcTU = 2;  // units per tile
+constexpr int tc_ur(int R) { return (R + 2) / kTcTU; }
+constexpr int tc_plane(int R) { return tc_ur(R) * kTcHW * 16; }
+constexpr int tc_units(int R) { return R <= 4 ? 6 : 3; }
+constexpr int kTcTail = 512;  // bias, barriers, flags
+constexpr int tc_smem(int R) { return kTcWBytes + tc_units(R) * 4 * tc_plane(R) + kTcTail; }
+static_assert((kTcR + 2) % kTcTU == 0 && (kTcRs + 2) % kTcTU == 0, "a tile is whole units");
 static_assert(2 * 8 * 32 <= 512, "two accumulator buffers must fit in tensor memory");
-static_assert(tc_smem(8) <= 227 * 1024, "the R = 8 ring must fit in shared memory");
+static_assert(128 + 8 * (2 * tc_units(kTcRs) + 4) + 8 <= kTcTail, "bias and barriers fit behind the ring");
+
+// One lane of the warp, by elect.sync, in a warp chosen by a uniform test: the
+// compiler then has what an MMA's issue needs in uniform registers.  A thread
+// chosen by its lane number issued one MMA in 70 - 76 cycles where the
+// operands' reads take 42 - 52 (hidden layer of 8 x 512^2 54 -> 52 us, last layer
+// 45 -> 34; with the ring below 42 and 31).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
+}
 
 __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
   // no swizzle; start, leading (K) and stride (M/N) byte offsets in 16-byte
@@ -392,6 +410,14 @@ __device__ __forceinline__ void tmem_zero1(uint32_t ta) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(ta), "r"(0u) : "memory");
 }
 
+// Store four 8 x 8 bf16 matrices in the fragment layout of an MMA's result; lane 8 j + r gives the address of
+// row r of matrix j.
+__device__ __forceinline__ void stm_x4(uint32_t sa, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(sa), "r"(r0), "r"(r1), "r"(r2),
+               "r"(r3)
+               : "memory");
+}
+
 //   MODE kHidden:   out = relu(conv(in) + bias)                        (32 -> 32)
 //   MODE kBackData: out = conv(in) * (mask > 0)   (weights mirrored and transposed)
 //   MODE kLast:     out_f = resid + conv(in) + bias                    (32 -> 1)
@@ -425,8 +451,8 @@ constexpr int kFxC = kTcHW + 2;          // x halo columns (x0 - 2 .. x0 + 127)
 constexpr int kFxP = 144;                // x halo row pitch (2-byte values; conflict-free gathers)
 constexpr int tc_fx_bytes(int R) { return (R + kFxR) * kFxP * 2; }
 constexpr int tc_fx_vals(int R) { return (R + kFxR) * kFxC; }  // x halo values of a tile
-constexpr int tc_smem_mode(int mode, int R) { return tc_smem(R) + (mode == kFused ? tc_fx_bytes(R) : 0); }
-static_assert(tc_smem(kTcR) + tc_fx_bytes(kTcR) <= 227 * 1024, "the fused ring must fit in shared memory");
+constexpr int tc_smem_mode(int mode, int R) { return tc_smem(R) + (mode == kFused ? 2 * tc_fx_bytes(R) : 0); }
+static_assert(tc_smem_mode(kFused, kTcR) <= 227 * 1024, "the fused ring must fit in shared memory");
 
 template <int MODE, int R>
 __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid_constant__ CUtensorMap tm_in,
@@ -435,7 +461,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
                                                     const __nv_bfloat16 *__restrict__ mask,
                                                     __nv_bfloat16 *__restrict__ out, float *__restrict__ out_f,
                                                     const float *__restrict__ resid, int nimg, int H, int W,
-                                                    int *err, const float *__restrict__ x1 = nullptr,
+                                                    int rev, int *err, const float *__restrict__ x1 = nullptr,
                                                     const __nv_bfloat16 *__restrict__ w1 = nullptr,
                                                     const float *__restrict__ b1 = nullptr) {
   constexpr bool kHid = MODE == kHidden || MODE == kFused;  // relu(conv + bias) epilogue
@@ -445,22 +471,22 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   constexpr int WDX = 4 * WCG;                   // weight bytes per dx
   constexpr int BUF = R * NCO;             // accumulator columns per tile buffer
   constexpr int TCOLS = tmem_cols(2 * BUF);
-  constexpr int PLANE = tc_plane(R), STAGES = tc_stages(R), STAGE = 4 * PLANE;
+  constexpr int PLANE = tc_plane(R), NU = tc_units(R), TU = kTcTU, UR = tc_ur(R), UNIT = 4 * PLANE;
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t s_w = (uint32_t)__cvta_generic_to_shared(smem);
   const uint32_t s_h = s_w + kTcWBytes;  // halo ring
-  unsigned char *tail = smem + kTcWBytes + STAGES * STAGE;
+  unsigned char *tail = smem + kTcWBytes + NU * UNIT;
   float *s_bias = reinterpret_cast<float *>(tail);
-  // barriers: full[STAGES], empty[STAGES], tfull[2], tempty[2]
+  // barriers: full[NU], empty[NU], tfull[2], tempty[2]
   uint64_t *bars = reinterpret_cast<uint64_t *>(tail + 128);
-  uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 4);
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * NU + 4);
   volatile int *abort_blk = reinterpret_cast<volatile int *>(tslot + 1);
   const uint32_t b0 = (uint32_t)__cvta_generic_to_shared(bars);
   auto full = [&](int i) { return b0 + 8u * i; };
-  auto empty = [&](int i) { return b0 + 8u * (STAGES + i); };
-  auto tfull = [&](int i) { return b0 + 8u * (2 * STAGES + i); };
-  auto tempty = [&](int i) { return b0 + 8u * (2 * STAGES + 2 + i); };
+  auto empty = [&](int i) { return b0 + 8u * (NU + i); };
+  auto tfull = [&](int i) { return b0 + 8u * (2 * NU + i); };
+  auto tempty = [&](int i) { return b0 + 8u * (2 * NU + 2 + i); };
   // The prologue (weights, barriers, tensor memory: about 3 us) overlaps the
   // previous layer's launch: an image of 200 x 200 took 43 us, 30 with it.
   // Only the weights are read in it: the layers before this one have waited
@@ -487,8 +513,8 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   if (MODE == kLast && tid == 0) s_bias[0] = bias[0];
   if (tid == 0) {
     *abort_blk = 0;
-    for (int i = 0; i < STAGES; ++i) {
-      tc_mbar_init(full(i), MODE == kFused ? 32 * tc_nprod(MODE, R) : 1);
+    for (int i = 0; i < NU; ++i) {
+      tc_mbar_init(full(i), MODE == kFused ? 32 * UR : 1);
       tc_mbar_init(empty(i), 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -507,7 +533,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);  // (uniform: see elect_one)
   if (warp < 4) {  // every MMA accumulates: both accumulator buffers start at zero
 #pragma unroll 1
     for (int c = 0; c < 2 * BUF; c += 32) tmem_zero32(tmem + ((uint32_t)(warp * 32) << 16) + c);
@@ -518,38 +544,44 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (MODE != kFused) griddep_wait();
   griddep_launch();
-  const int ntx = (W + kTcOut - 1) / kTcOut, nty = (H + R - 1) / R;
-  const long long ntiles = (long long)ntx * nty * nimg;
-  // Each block takes a contiguous range of tiles, ordered down the image
-  // columns (y fastest): a tile's two halo rows are rows of the block's
-  // previous tile, fetched a moment earlier and still in L2, so DRAM reads
-  // each activation row about once instead of 1.5 times.
-  // persistent blocks over the tiles, x fastest (measured against a
-  // contiguous y-fastest range per block, which lost: 1.36 vs 1.27 ms per
-  // 32 x 512^2 inference)
-  auto tile_xy = [&](long long t, int &img, int &y0, int &x0) {
-    img = (int)(t / ((long long)ntx * nty));
-    const int rem = (int)(t % ((long long)ntx * nty));
-    y0 = (rem / ntx) * R;
-    x0 = (rem % ntx) * kTcOut;
+  // (32-bit tile numbers: a tile holds at least 126 pixels of 64 bytes)
+  const int ntx = (W + kTcOut - 1) / kTcOut, tpi = ntx * ((H + R - 1) / R), ntiles = tpi * nimg;
+  // Persistent blocks over the tiles, x fastest (a contiguous y-fastest range per block lost: 1.36
+  // against 1.27 ms per 32 x 512^2 inference).  rev: from the last tile to the
+  // first.  Consecutive layers run in opposite directions, so that a layer begins with what the one
+  // before wrote last and L2 still holds: 8 x 512^2 inference 210 -> 203 us,
+  // training step 808 -> 786.
+  auto tile_xy = [&](int t, int &img, int &y0, int &x0) {
+    if (rev) t = ntiles - 1 - t;
+    img = t / tpi;
+    const int rem = t - img * tpi, ty = rem / ntx;
+    y0 = ty * R;
+    x0 = (rem - ty * ntx) * kTcOut;
   };
   if (MODE != kFused && warp == kTcEpi) {
-    // ---- producer: one TMA copy of the halo per tile ----
+    // ---- producer: one TMA copy per two halo rows ----
     // (one bulk copy per channel group and halo row instead lost by 2.1x)
     if (lane == 0) {
-      int issued = 0;
-      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++issued) {
-        const int s = issued % STAGES, u = issued / STAGES;
-        if (u > 0 && !tc_wait(empty(s), (u - 1) & 1, abort_blk)) break;
+      int q = 0;  // units issued
+      bool go = true;
+      for (int t = blockIdx.x; go && t < ntiles; t += gridDim.x) {
         int img, y0, x0;
         tile_xy(t, img, y0, x0);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(STAGE) : "memory");
-        tc_tma4(s_h + s * STAGE, &tm_in, 2 * (x0 - 1), y0 - 1, img, full(s));
+        for (int uu = 0; uu < TU; ++uu, ++q) {
+          const int s = q % NU, u = q / NU;
+          if (u > 0 && !tc_wait(empty(s), (u - 1) & 1, abort_blk)) {
+            go = false;
+            break;
+          }
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(UNIT)
+                       : "memory");
+          tc_tma4(s_h + s * UNIT, &tm_in, 2 * (x0 - 1), y0 - 1 + UR * uu, img, full(s));
+        }
       }
       if (*abort_blk) {  // let the copies in flight land before the block exits
-        for (int k = (issued > STAGES ? issued - STAGES : 0); k < issued; ++k) {
+        for (int k = (q > NU ? q - NU : 0); k < q; ++k) {
           const long long t0 = clock64();
-          while (!tc_try(full(k % STAGES), (k / STAGES) & 1) && clock64() - t0 < kTcWaitCycles) {
+          while (!tc_try(full(k % NU), (k / NU) & 1) && clock64() - t0 < kTcWaitCycles) {
           }
         }
       }
@@ -558,10 +590,11 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     // ---- builders (kFused): the first layer's output over the tile's halo ----
     constexpr int NB = tc_nprod(MODE, R), NBT = 32 * NB;                    // builder warps, threads
     constexpr int XVALS = tc_fx_vals(R), NPRE = (XVALS + NBT - 1) / NBT;  // x values, per builder thread
-    static_assert((R + 2) % NB == 0, "each builder warp owns the same number of halo rows");
+    static_assert(MODE != kFused || R + 2 == NB, "each builder warp owns a halo row");
     const int bt = tid - 32 * kTcEpi, g = lane >> 2, tq = lane & 3;
     const int bw = warp - kTcEpi;
-    uint16_t *xs = reinterpret_cast<uint16_t *>(smem + tc_smem(R));
+    uint16_t *xs0 = reinterpret_cast<uint16_t *>(smem + tc_smem(R));  // two parked halos
+    constexpr int XS = tc_fx_bytes(R) / 2;
     unsigned char *hs = smem + kTcWBytes;  // generic address of the ring
     const uint16_t *w1u = reinterpret_cast<const uint16_t *>(w1);
     uint32_t bf[4][2];  // B fragments: B[k][co] = w1[tap k][co] for k < 9, zero above
@@ -576,7 +609,6 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     const int o0 = ((2 * tq) / 3) * kFxP + (2 * tq) % 3, o1 = ((2 * tq + 1) / 3) * kFxP + (2 * tq + 1) % 3;
     constexpr int o8 = 2 * kFxP + 2;
     const long long HWp = (long long)H * W;
-    auto bar_b = [] { asm volatile("bar.sync 1, %0;" ::"n"(NBT) : "memory"); };
     // barrier of the builders that returns whether any of them saw the abort
     // flag (one decision for all of them)
     auto bar_b_abort = [&]() -> bool {
@@ -589,7 +621,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     };
     // this thread's share of tile t's x halo (rows y0 - 2 .., columns x0 - 2
     // ..), left in flight as fp32 until park() rounds and stores it
-    auto fetch = [&](long long t, float *v) {
+    auto fetch = [&](int t, float *v) {
       int img, y0, x0;
       tile_xy(t, img, y0, x0);
       const float *src = x1 + (long long)img * HWp;
@@ -601,7 +633,8 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
                                                                                        : 0.f;
       }
     };
-    auto park = [&](const float *v) {
+    auto park = [&](const float *v, int b) {
+      uint16_t *xs = xs0 + b * XS;
 #pragma unroll
       for (int k = 0; k < NPRE; ++k) {
         const int i = bt + NBT * k, r = i / kFxC;
@@ -609,97 +642,115 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
       }
     };
     float v[NPRE];
-    if ((long long)blockIdx.x < ntiles) {
+    if ((int)blockIdx.x < ntiles) {
       fetch(blockIdx.x, v);
-      park(v);
+      park(v, 0);
     }
-    bar_b();
-    int issued = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++issued) {
-      const int s = issued % STAGES, u = issued / STAGES;
-      const long long tn = t + gridDim.x;
+    int k = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
+      const int tn = t + gridDim.x;
       if (tn < ntiles) fetch(tn, v);  // in flight while this tile is built
+      const int q = k * TU + bw / UR, s = q % NU, u = q / NU;
       if (u > 0) tc_wait(empty(s), (u - 1) & 1, abort_blk);
+      // this tile's halo is parked, and every builder is done with the other one
       if (bar_b_abort()) break;
       int img, y0, x0;
       tile_xy(t, img, y0, x0);
-#pragma unroll 1
-      for (int h = bw; h < R + 2; h += NB) {  // halo row h: image row y0 - 1 + h
-        // this lane's 4-byte piece of pixel (h, g) in channel group 0
-        unsigned char *row = hs + s * STAGE + (h * kTcHW + g) * 16 + 4 * tq;
-        if ((unsigned)(y0 - 1 + h) >= (unsigned)H) {  // outside the image: the second layer's zero padding
+      // halo row bw in channel group 0; srow: this lane's 16 bytes of an 8-pixel
+      // block for stmatrix, pixel lane % 8 of group lane / 8
+      unsigned char *row = hs + s * UNIT + (bw % UR) * kTcHW * 16;
+      const uint32_t srow = s_h + s * UNIT + (bw % UR) * kTcHW * 16 + (lane >> 3) * PLANE + (lane & 7) * 16;
+      if ((unsigned)(y0 - 1 + bw) >= (unsigned)H) {  // outside the image: the second layer's zero padding
 #pragma unroll
-          for (int i = 0; i < kTcHW; i += 8)
+        for (int n = 0; n < 4; ++n)
 #pragma unroll
-            for (int n = 0; n < 4; ++n) *reinterpret_cast<uint32_t *>(row + n * PLANE + i * 16) = 0u;
-          continue;
+          for (int i = lane; i < kTcHW; i += 32)
+            *reinterpret_cast<uint4 *>(row + n * PLANE + i * 16) = make_uint4(0u, 0u, 0u, 0u);
+      } else {
+        const uint16_t *xr = xs0 + (k & 1) * XS + bw * kFxP + g;
+#pragma unroll
+        for (int i0 = 0; i0 < kTcHW; i0 += 64) {
+          uint32_t a[4][4];  // 64 pixels' gathers in flight before the first MMA
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint16_t *p0 = xr + i0 + 16 * i, *p1 = p0 + 8;
+            a[i][0] = pack_u16(p0[o0], p0[o1]);
+            a[i][1] = pack_u16(p1[o0], p1[o1]);
+            a[i][2] = tq == 0 ? (uint32_t)p0[o8] : 0u;
+            a[i][3] = tq == 0 ? (uint32_t)p1[o8] : 0u;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float d[4][4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+              d[n][0] = d[n][2] = bs[n].x;
+              d[n][1] = d[n][3] = bs[n].y;
+              mma16816(d[n], a[i], bf[n]);
+            }
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh)  // pixels g (hh = 0) and g + 8
+              stm_x4(srow + (i0 + 16 * i + 8 * hh) * 16, cvt_bf16x2<true>(d[0][2 * hh], d[0][2 * hh + 1]),
+                     cvt_bf16x2<true>(d[1][2 * hh], d[1][2 * hh + 1]), cvt_bf16x2<true>(d[2][2 * hh], d[2][2 * hh + 1]),
+                     cvt_bf16x2<true>(d[3][2 * hh], d[3][2 * hh + 1]));
+          }
         }
-        const uint16_t *xr = xs + h * kFxP + g;
-        const int xg = x0 - 1 + g;  // image column of pixel (h, g)
-#pragma unroll
-        for (int i0 = 0; i0 < kTcHW; i0 += 16) {
-          const uint16_t *p0 = xr + i0, *p1 = p0 + 8;
-          uint32_t a[4];
-          a[0] = pack_u16(p0[o0], p0[o1]);
-          a[1] = pack_u16(p1[o0], p1[o1]);
-          a[2] = tq == 0 ? (uint32_t)p0[o8] : 0u;
-          a[3] = tq == 0 ? (uint32_t)p1[o8] : 0u;
-          float d[4][4];
-#pragma unroll
-          for (int n = 0; n < 4; ++n) {
-            d[n][0] = d[n][2] = bs[n].x;
-            d[n][1] = d[n][3] = bs[n].y;
-            mma16816(d[n], a, bf[n]);
-          }
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {  // pixels g (hh = 0) and g + 8
-            const bool in = (unsigned)(xg + i0 + 8 * hh) < (unsigned)W;
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-              *reinterpret_cast<uint32_t *>(row + n * PLANE + (i0 + 8 * hh) * 16) =
-                  in ? cvt_bf16x2<true>(d[n][2 * hh], d[n][2 * hh + 1]) : 0u;
-          }
+        // columns outside the image: zero
+        const int xw = W - x0 + 1;  // halo pixels from here on lie right of the image
+        if (x0 == 0 || xw < kTcHW) {
+          __syncwarp();
+          if (x0 == 0 && lane < 4) *reinterpret_cast<uint4 *>(row + lane * PLANE) = make_uint4(0u, 0u, 0u, 0u);
+          for (int i = xw + (lane >> 2); i < kTcHW; i += 8)
+            *reinterpret_cast<uint4 *>(row + (lane & 3) * PLANE + i * 16) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_arrive(full(s));
-      bar_b();  // every builder is done with the parked halo
-      if (tn < ntiles) park(v);
-      bar_b();
+      if (tn < ntiles) park(v, (k + 1) & 1);
     }
-  } else if (warp == kMma) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == kMma) {
     // ---- MMA issuer ----
-    if (lane == 0) {
+    if (elect_one()) {
       int k = 0;
-      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
-        const int s = k % STAGES, u = k / STAGES, b = k & 1, ub = k >> 1;
-        if (!tc_wait(full(s), u & 1, abort_blk)) break;
+      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
+        const int b = k & 1, ub = k >> 1;
         if (ub > 0 && !tc_wait(tempty(b), (ub - 1) & 1, abort_blk)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // descriptors differ only in their start-address field: one add per MMA
         // (fully unrolled, the offsets are constants; a single thread issues
         // all of them, so per-MMA arithmetic would bound the tile)
-        const uint64_t a0 = umma_desc(s_h + s * STAGE, PLANE, 128), b0d = umma_desc(s_w, WCG, 128);
+        const uint64_t b0d = umma_desc(s_w, WCG, 128);
         const uint32_t d0 = tmem + b * BUF;
+        bool got = true;
 #pragma unroll
-        for (int h = 0; h < R + 2; ++h) {
-          // output rows h - j for j in [j0, j1] (those inside the tile)
-          const int j0 = h > R - 1 ? h - (R - 1) : 0, j1 = h < 2 ? h : 2;
-          const uint32_t idesc = tc_idesc(NCO * (j1 - j0 + 1));
-          const uint32_t d = d0 + (uint32_t)((R - 1 - h + j0) * NCO);
+        for (int uu = 0; uu < TU; ++uu) {
+          const int q = k * TU + uu, s = q % NU;
+          if (!tc_wait(full(s), (q / NU) & 1, abort_blk)) {
+            got = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t a0 = umma_desc(s_h + s * UNIT, PLANE, 128);
 #pragma unroll
-          for (int dx = 0; dx < 3; ++dx)
+          for (int hh = 0; hh < UR; ++hh) {
+            // output rows h - j for j in [j0, j1] (those inside the tile)
+            const int h = UR * uu + hh, j0 = h > R - 1 ? h - (R - 1) : 0, j1 = h < 2 ? h : 2;
+            const uint32_t idesc = tc_idesc(NCO * (j1 - j0 + 1));
+            const uint32_t d = d0 + (uint32_t)((R - 1 - h + j0) * NCO);
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-              const uint64_t ad = a0 + (uint64_t)((2 * ks * PLANE + (h * kTcHW + dx) * 16) >> 4);
-              const uint64_t bd = b0d + (uint64_t)((dx * WDX + 2 * ks * WCG + j0 * NCO * 16) >> 4);
-              asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                           "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d), "l"(ad),
-                           "l"(bd), "r"(idesc), "r"(1u));
-            }
+            for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+              for (int ks = 0; ks < 2; ++ks) {
+                const uint64_t ad = a0 + (uint64_t)((2 * ks * PLANE + (hh * kTcHW + dx) * 16) >> 4);
+                const uint64_t bd = b0d + (uint64_t)((dx * WDX + 2 * ks * WCG + j0 * NCO * 16) >> 4);
+                asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d), "l"(ad),
+                             "l"(bd), "r"(idesc), "r"(1u));
+              }
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(s))
+                       : "memory");
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(s))
-                     : "memory");
+        if (!got) break;
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull(b))
                      : "memory");
       }
@@ -711,7 +762,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     const uint32_t lanes = (uint32_t)(lq * 32) << 16;
     const long long HWp = (long long)H * W;
     int k = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
       const int b = k & 1, ub = k >> 1;
       int img, y0, x0;
       tile_xy(t, img, y0, x0);
@@ -849,7 +900,7 @@ __device__ __forceinline__ void wt_copy(uint32_t dst, const CUtensorMap *tm, int
 __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tm_x,
                                                                  const __grid_constant__ CUtensorMap tm_z,
                                                                  float *__restrict__ dw, float *__restrict__ db,
-                                                                 int nimg, int H, int W, int *err) {
+                                                                 int nimg, int H, int W, int rev, int *err) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2 * kWtStages + 1];
   __shared__ uint32_t s_tmem;
@@ -879,7 +930,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_co
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
   griddep_wait();
   griddep_launch();
   float bsum[8];  // warps 0-3: channels 8 warp .. 8 warp + 7
@@ -891,7 +942,8 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_co
       for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
         const int s = k % kWtStages, u = k / kWtStages;
         if (u > 0 && !tc_wait(empty(s), (u - 1) & 1, abort_blk)) break;
-        const int img = tt / tpi, rem = tt - img * tpi, ty = rem / ntx;
+        const int ts = rev ? ntiles - 1 - tt : tt;
+        const int img = ts / tpi, rem = ts - img * tpi, ty = rem / ntx;
         const int y0 = ty * kWtR, x0 = (rem - ty * ntx) * kWtC;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(kWtStage)
                      : "memory");
@@ -906,8 +958,8 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_co
         }
       }
     }
-  } else if (warp == 5) {
-    if (lane == 0) {
+  } else if (__shfl_sync(0xffffffffu, warp, 0) == 5) {
+    if (elect_one()) {
       int k = 0;
       for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
         const int s = k % kWtStages;
@@ -1390,26 +1442,26 @@ int tile_rows(int nimg, int H, int W) {
 
 template <int MODE, int R>
 bool launch_conv_r(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
-                   __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s, float *out_f, const float *resid,
+                   __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f, const float *resid,
                    const float *x, const __nv_bfloat16 *w1, const float *b1) {
   const long long tiles = tiles_of(nimg, H, W, R);
   const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
   CUtensorMap tin;
   memset(&tin, 0, sizeof tin);  // (the fused mode builds its operand instead of copying it)
-  if (MODE != kFused && !act_map(&tin, in, nimg, H, W, R + 2)) return false;
+  if (MODE != kFused && !act_map(&tin, in, nimg, H, W, tc_ur(R))) return false;
   launch_pdl(k_conv_tc<MODE, R>, dim3(grid), dim3(tc_threads(MODE, R)), tc_smem_mode(MODE, R), s, tin, wt, bias, mask, out,
-             out_f, resid, nimg, H, W, tc_err_dev, x, w1, b1);
+             out_f, resid, nimg, H, W, rev, tc_err_dev, x, w1, b1);
   return true;
 }
 
 template <int MODE>
 bool launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
-                    __nv_bfloat16 *out, int nimg, int H, int W, cudaStream_t s, float *out_f = nullptr,
+                    __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f = nullptr,
                     const float *resid = nullptr, const float *x = nullptr, const __nv_bfloat16 *w1 = nullptr,
                     const float *b1 = nullptr) {
   return tile_rows(nimg, H, W) == kTcRs
-             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1)
-             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, s, out_f, resid, x, w1, b1);
+             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, resid, x, w1, b1)
+             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, resid, x, w1, b1);
 }
 
 // One block per SM (its shared memory), at most one per tile.
@@ -1419,7 +1471,7 @@ bool launch_wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *dw, fl
   const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
   CUtensorMap tx, tz;
   if (!rows_map(&tx, x, nimg, H, W, kWtXP, kWtR) || !rows_map(&tz, dz, nimg, H, W, kWtC, kWtR + 2)) return false;
-  launch_pdl(k_conv_wgrad_tc, dim3(grid), dim3(kWtThreads), kWtSmem, s, tx, tz, dw, db, nimg, H, W, tc_err_dev);
+  launch_pdl(k_conv_wgrad_tc, dim3(grid), dim3(kWtThreads), kWtSmem, s, tx, tz, dw, db, nimg, H, W, 1, tc_err_dev);
   return true;
 }
 
@@ -1441,14 +1493,14 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
   if (keep) {  // the backward pass reads the first layer's output
     k_conv_1to32<kHidden><<<grid_1to32<kHidden>(nimg, H, W), 256, smem_1to32<kHidden>(), s>>>(
         w.x0, w.wf + kW1, params_dev + kB1, nullptr, w.act[0], nimg, H, W);
-    ok_tc = launch_conv_tc<kHidden>(w.act[0], w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, s);
+    ok_tc = launch_conv_tc<kHidden>(w.act[0], w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, 1, s);
   } else {
-    ok_tc = launch_conv_tc<kFused>(nullptr, w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, s, nullptr,
+    ok_tc = launch_conv_tc<kFused>(nullptr, w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, 1, s, nullptr,
                                    nullptr, x_dev, w.wf + kW1, params_dev + kB1);
   }
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], w.wf + kW3, params_dev + kB3, nullptr, w.act[2], nimg, H, W, s);
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], w.wf + kW4, params_dev + kB4, nullptr, w.act[3], nimg, H, W, s);
-  ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], w.wf + kW5, params_dev + kB5, nullptr, nullptr, nimg, H, W, s,
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], w.wf + kW3, params_dev + kB3, nullptr, w.act[2], nimg, H, W, 0, s);
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], w.wf + kW4, params_dev + kB4, nullptr, w.act[3], nimg, H, W, 1, s);
+  ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], w.wf + kW5, params_dev + kB5, nullptr, nullptr, nimg, H, W, 0, s,
                                          y_dev, x_dev);
   if (!ok_tc) return rbc::set_error(RBC_ECUDA, "rbc_cnn_forward: launch failed");
   rbc::add_launches(keep ? 7 : 5);
@@ -1499,7 +1551,7 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
   for (int l = 0; l < 3; ++l) {
     const int layer_in = 2 - l;  // act index of this layer's input: act3 (l=0) ... act1
     ok_tc = ok_tc && launch_wgrad(w.act[layer_in], w.dz[cur], grad_dev + woff[l], grad_dev + boff[l], nimg, H, W, s);
-    ok_tc = ok_tc && launch_conv_tc<kBackData>(w.dz[cur], w.wb + woff[l], nullptr, w.act[layer_in], w.dz[1 - cur], nimg, H, W, s);
+    ok_tc = ok_tc && launch_conv_tc<kBackData>(w.dz[cur], w.wb + woff[l], nullptr, w.act[layer_in], w.dz[1 - cur], nimg, H, W, 0, s);
     cur = 1 - cur;
   }
   // layer 1
