@@ -362,6 +362,16 @@ int rbc_cnn_infer(const float *params_dev, int nimg, int H, int W,
                   const float *x_dev, float *y_dev, void *ws_dev,
                   void *stream);
 
+/* rbc_cnn_infer on images that are slices of a larger array: image i, row r
+ * starts at x_dev + i x_img + r x_row (strides in values, >= 0; the values of a
+ * row are consecutive), and y_dev likewise.  y_dev's images must not overlap each
+ * other, and overlap x_dev's only where they are the same.
+ * Errors: RBC_EINVAL, RBC_ECUDA. */
+int rbc_cnn_infer_strided(const float *params_dev, int nimg, int H, int W,
+                          const float *x_dev, long long x_img,
+                          long long x_row, float *y_dev, long long y_img,
+                          long long y_row, void *ws_dev, void *stream);
+
 /* grad_dev (param_count fp32) += dL/dparams for the dL/dy in dy_dev, using
  * the activations the preceding rbc_cnn_forward left in ws_dev (same batch,
  * same parameters).  Errors: RBC_EINVAL, RBC_ECUDA. */

@@ -104,10 +104,12 @@ def _load():
     lib.rbc_cnn_workspace_bytes.argtypes = [I, I, I]
     lib.rbc_cnn_forward.argtypes = [P, I, I, I, P, P, P, P]
     lib.rbc_cnn_infer.argtypes = [P, I, I, I, P, P, P, P]
+    lib.rbc_cnn_infer_strided.argtypes = [P, I, I, I, P, C.c_longlong, C.c_longlong, P, C.c_longlong, C.c_longlong, P, P]
     lib.rbc_cnn_backward.argtypes = [P, I, I, I, P, P, P, P]
     lib.rbc_cnn_mse.argtypes = [P, P, C.c_longlong, P, P, P]
     lib.rbc_cnn_adam.argtypes = [P, P, P, P, F, F, F, F, I, P]
-    for name in ("rbc_cnn_forward", "rbc_cnn_infer", "rbc_cnn_backward", "rbc_cnn_mse", "rbc_cnn_adam"):
+    for name in ("rbc_cnn_forward", "rbc_cnn_infer", "rbc_cnn_infer_strided", "rbc_cnn_backward", "rbc_cnn_mse",
+                 "rbc_cnn_adam"):
         getattr(lib, name).restype = I
     lib.rbc_model_static.argtypes = [G, P, P, P, I, P, P, P]
     lib.rbc_model_static.restype = I
@@ -125,8 +127,8 @@ EXPORTED = ("rbc_build_velocity", "rbc_create", "rbc_destroy", "rbc_model", "rbc
             "rbc_image_stack", "rbc_set_snapshots", "rbc_get_panels", "rbc_phase_timing",
             "rbc_model_static", "rbc_fwi_forward", "rbc_fwi_backward", "rbc_batch_create",
             "rbc_batch_destroy", "rbc_batch_rtm", "rbc_batch_info", "rbc_batch_timing",
-            "rbc_cnn_param_count", "rbc_cnn_workspace_bytes", "rbc_cnn_forward", "rbc_cnn_infer", "rbc_cnn_backward",
-            "rbc_cnn_mse", "rbc_cnn_adam", "rbc_inject_fault", "rbc_last_error",
+            "rbc_cnn_param_count", "rbc_cnn_workspace_bytes", "rbc_cnn_forward", "rbc_cnn_infer",
+            "rbc_cnn_infer_strided", "rbc_cnn_backward", "rbc_cnn_mse", "rbc_cnn_adam", "rbc_inject_fault", "rbc_last_error",
             "rbc_launch_count", "rbc_nyquist_stride", "rbc_storage_bytes", "rbc_rtm_storage",
             "rbc_set_coef", "rbc_set_share")
 
@@ -378,6 +380,20 @@ def rbc_cnn_infer(params, x, y, ws, stream=None):
     n, H, W = x.shape
     _check(_lib.rbc_cnn_infer(_dev(params, None, "params"), n, H, W, _dev(x, None, "x"), _dev(y, None, "y"),
                               _u8(ws, "ws"), _stream(stream)))
+
+
+def rbc_cnn_infer_strided(params, x, y, ws, stream=None):
+    """rbc_cnn_infer on views (nimg, H, W) whose rows are contiguous (stride 1
+    along W) and whose images and rows lie any distance apart."""
+    n, H, W = x.shape
+    for t, name in ((x, "x"), (y, "y")):
+        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.float32 and t.stride(2) == 1):
+            raise TypeError(f"{name} must be a float32 CUDA tensor with contiguous rows")
+    if tuple(y.shape) != (n, H, W):
+        raise ValueError(f"y has shape {tuple(y.shape)}, expected {(n, H, W)}")
+    _check(_lib.rbc_cnn_infer_strided(_dev(params, None, "params"), n, H, W, C.c_void_p(x.data_ptr()), x.stride(0),
+                                      x.stride(1), C.c_void_p(y.data_ptr()), y.stride(0), y.stride(1), _u8(ws, "ws"),
+                                      _stream(stream)))
 
 
 def rbc_cnn_backward(params, dy, grad, ws, stream=None):

@@ -454,15 +454,20 @@ constexpr int tc_fx_vals(int R) { return (R + kFxR) * kFxC; }  // x halo values 
 constexpr int tc_smem_mode(int mode, int R) { return tc_smem(R) + (mode == kFused ? 2 * tc_fx_bytes(R) : 0); }
 static_assert(tc_smem_mode(kFused, kTcR) <= 227 * 1024, "the fused ring must fit in shared memory");
 
+// Strides (in values) of the one-channel images: from image to image and from
+// row to row, of the input and of the output.
+struct Img {
+  long long xi, xr, yi, yr;
+};
+
 template <int MODE, int R>
 __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid_constant__ CUtensorMap tm_in,
-                                                    const __nv_bfloat16 *__restrict__ wt,
+                                                    const void *__restrict__ wt_,
                                                     const float *__restrict__ bias,
                                                     const __nv_bfloat16 *__restrict__ mask,
-                                                    __nv_bfloat16 *__restrict__ out, float *__restrict__ out_f,
-                                                    const float *__restrict__ resid, int nimg, int H, int W,
-                                                    int rev, int *err, const float *__restrict__ x1 = nullptr,
-                                                    const __nv_bfloat16 *__restrict__ w1 = nullptr,
+                                                    __nv_bfloat16 *__restrict__ out, float *out_f,
+                                                    const float *xin, const Img st, int nimg, int H, int W,
+                                                    int rev, int *err, const float *__restrict__ w1 = nullptr,
                                                     const float *__restrict__ b1 = nullptr) {
   constexpr bool kHid = MODE == kHidden || MODE == kFused;  // relu(conv + bias) epilogue
   constexpr int kMma = kTcEpi + tc_nprod(MODE, R);             // the MMA issuer warp
@@ -489,24 +494,37 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   auto tempty = [&](int i) { return b0 + 8u * (2 * NU + 2 + i); };
   // The prologue (weights, barriers, tensor memory: about 3 us) overlaps the
   // previous layer's launch: an image of 200 x 200 took 43 us, 30 with it.
-  // Only the weights are read in it: the layers before this one have waited
-  // for their preparation (the fused first layers, which follow it, wait here).
+  // Only the weights are read in it: whatever wrote them comes before the first layer,
+  // which the layers before this one have waited for (the fused first layers wait here).
   if (MODE == kFused) griddep_wait();
-  // weights [tap][co][ci] (tap = 3 dy + dx) -> [dx][ci / 8][dy][co][8]
+  // weights [tap][co][ci] (tap = 3 dy + dx) -> [dx][ci / 8][dy][co][8]; the forward
+  // layers round the fp32 parameters here (a launch of its own for that cost a small
+  // image 4 us), the backward-data pass copies its mirrored bf16 weights
   if (MODE == kLast) {
     for (int i = tid; i < 9 * 4 * (NCO - 1); i += blockDim.x) {  // padding channels 1..15: zero
       const int co = 1 + i % (NCO - 1), r = i / (NCO - 1), j = r & 3, t = r >> 2;
       *reinterpret_cast<uint4 *>(smem + (t % 3) * WDX + j * WCG + (t / 3) * NCO * 16 + co * 16) =
           make_uint4(0u, 0u, 0u, 0u);
     }
-    for (int i = tid; i < 9 * 4; i += blockDim.x) {
-      const int j = i & 3, t = i >> 2;
-      cp_async16(s_w + (t % 3) * WDX + j * WCG + (t / 3) * NCO * 16, wt + t * 32 + j * 8, true);
+    const float *wt = static_cast<const float *>(wt_);
+    for (int i = tid; i < 9 * 32; i += blockDim.x) {
+      const int ci = i & 31, t = i >> 5;
+      *reinterpret_cast<__nv_bfloat16 *>(smem + (t % 3) * WDX + (ci >> 3) * WCG + (t / 3) * NCO * 16 + (ci & 7) * 2) =
+          __float2bfloat16(wt[i]);
     }
-  } else {
+  } else if (MODE == kBackData) {
+    const __nv_bfloat16 *wt = static_cast<const __nv_bfloat16 *>(wt_);
     for (int i = tid; i < 9 * 32 * 4; i += blockDim.x) {
       const int j = i & 3, co = (i >> 2) & 31, t = i >> 7, dy = t / 3, dx = t % 3;
       cp_async16(s_w + dx * WDX + j * WCG + dy * NCO * 16 + co * 16, wt + (t * 32 + co) * 32 + j * 8, true);
+    }
+  } else {
+    const float *wt = static_cast<const float *>(wt_);
+#pragma unroll 8
+    for (int i = tid; i < 9 * 32 * 32; i += tc_threads(MODE, R)) {
+      const int ci = i & 31, co = (i >> 5) & 31, t = i >> 10, dy = t / 3, dx = t % 3;
+      *reinterpret_cast<__nv_bfloat16 *>(smem + dx * WDX + (ci >> 3) * WCG + dy * NCO * 16 + co * 16 + (ci & 7) * 2) =
+          __float2bfloat16(wt[i]);
     }
   }
   if (kHid && tid < 32) s_bias[tid] = bias[tid];
@@ -596,19 +614,18 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     uint16_t *xs0 = reinterpret_cast<uint16_t *>(smem + tc_smem(R));  // two parked halos
     constexpr int XS = tc_fx_bytes(R) / 2;
     unsigned char *hs = smem + kTcWBytes;  // generic address of the ring
-    const uint16_t *w1u = reinterpret_cast<const uint16_t *>(w1);
+    auto w1u = [&](int i) { return __bfloat16_as_ushort(__float2bfloat16(w1[i])); };
     uint32_t bf[4][2];  // B fragments: B[k][co] = w1[tap k][co] for k < 9, zero above
     float2 bs[4];
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
       const int co = 8 * n + g;
-      bf[n][0] = pack_u16(w1u[(2 * tq) * 32 + co], w1u[(2 * tq + 1) * 32 + co]);
-      bf[n][1] = tq == 0 ? pack_u16(w1u[8 * 32 + co], 0) : 0u;
+      bf[n][0] = pack_u16(w1u((2 * tq) * 32 + co), w1u((2 * tq + 1) * 32 + co));
+      bf[n][1] = tq == 0 ? pack_u16(w1u(8 * 32 + co), 0) : 0u;
       bs[n] = make_float2(b1[8 * n + 2 * tq], b1[8 * n + 2 * tq + 1]);
     }
     const int o0 = ((2 * tq) / 3) * kFxP + (2 * tq) % 3, o1 = ((2 * tq + 1) / 3) * kFxP + (2 * tq + 1) % 3;
     constexpr int o8 = 2 * kFxP + 2;
-    const long long HWp = (long long)H * W;
     // barrier of the builders that returns whether any of them saw the abort
     // flag (one decision for all of them)
     auto bar_b_abort = [&]() -> bool {
@@ -624,13 +641,12 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     auto fetch = [&](int t, float *v) {
       int img, y0, x0;
       tile_xy(t, img, y0, x0);
-      const float *src = x1 + (long long)img * HWp;
+      const float *src = xin + img * st.xi;
 #pragma unroll
       for (int k = 0; k < NPRE; ++k) {
         const int i = bt + NBT * k, r = i / kFxC;
         const int yy = y0 - 2 + r, xx = x0 - 2 + (i - r * kFxC);
-        v[k] = (i < XVALS && (unsigned)yy < (unsigned)H && (unsigned)xx < (unsigned)W) ? src[(long long)yy * W + xx]
-                                                                                       : 0.f;
+        v[k] = (i < XVALS && (unsigned)yy < (unsigned)H && (unsigned)xx < (unsigned)W) ? src[yy * st.xr + xx] : 0.f;
       }
     };
     auto park = [&](const float *v, int b) {
@@ -771,7 +787,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
       if (MODE == kLast) {
 #pragma unroll
         for (int i = 0; i < RE; ++i)
-          rs[i] = (y0 + r0 + i < H && xx < W) ? resid[(long long)img * HWp + (long long)(y0 + r0 + i) * W + xx] : 0.f;
+          rs[i] = (y0 + r0 + i < H && xx < W) ? xin[img * st.xi + (y0 + r0 + i) * st.xr + xx] : 0.f;
       }
       uint4 mk[RE][4];  // backward-data: this pixel's masks, loaded while the MMAs run
       if (MODE == kBackData) {
@@ -794,7 +810,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
           const float v0 = tmem_ld1(ta);
           tmem_zero1(ta);  // channel 0 only: the padding channels never leave zero
           const int yy = y0 + rr;
-          if (yy < H && xx < W) out_f[(long long)img * HWp + (long long)yy * W + xx] = rs[rr - r0] + v0 + s_bias[0];
+          if (yy < H && xx < W) out_f[img * st.yi + yy * st.yr + xx] = rs[rr - r0] + v0 + s_bias[0];
         }
       } else {
 #pragma unroll 1
@@ -1441,27 +1457,27 @@ int tile_rows(int nimg, int H, int W) {
 }
 
 template <int MODE, int R>
-bool launch_conv_r(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
-                   __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f, const float *resid,
-                   const float *x, const __nv_bfloat16 *w1, const float *b1) {
+bool launch_conv_r(const __nv_bfloat16 *in, const void *wt, const float *bias, const __nv_bfloat16 *mask,
+                   __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f, const float *x,
+                   const Img &st, const float *w1, const float *b1) {
   const long long tiles = tiles_of(nimg, H, W, R);
   const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
   CUtensorMap tin;
   memset(&tin, 0, sizeof tin);  // (the fused mode builds its operand instead of copying it)
   if (MODE != kFused && !act_map(&tin, in, nimg, H, W, tc_ur(R))) return false;
   launch_pdl(k_conv_tc<MODE, R>, dim3(grid), dim3(tc_threads(MODE, R)), tc_smem_mode(MODE, R), s, tin, wt, bias, mask, out,
-             out_f, resid, nimg, H, W, rev, tc_err_dev, x, w1, b1);
+             out_f, x, st, nimg, H, W, rev, tc_err_dev, w1, b1);
   return true;
 }
 
 template <int MODE>
-bool launch_conv_tc(const __nv_bfloat16 *in, const __nv_bfloat16 *wt, const float *bias, const __nv_bfloat16 *mask,
+bool launch_conv_tc(const __nv_bfloat16 *in, const void *wt, const float *bias, const __nv_bfloat16 *mask,
                     __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f = nullptr,
-                    const float *resid = nullptr, const float *x = nullptr, const __nv_bfloat16 *w1 = nullptr,
+                    const float *x = nullptr, const Img &st = Img(), const float *w1 = nullptr,
                     const float *b1 = nullptr) {
   return tile_rows(nimg, H, W) == kTcRs
-             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, resid, x, w1, b1)
-             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, resid, x, w1, b1);
+             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, x, st, w1, b1)
+             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, x, st, w1, b1);
 }
 
 // One block per SM (its shared memory), at most one per tile.
@@ -1476,38 +1492,42 @@ bool launch_wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *dw, fl
 }
 
 // The network's forward pass; `keep` stores what the backward pass reads
-// (the bf16 input and the first layer's output: two launches for the first
-// two layers); without it the first two layers are one fused launch.
-int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_dev, float *y_dev, void *ws_dev,
-                void *stream, bool keep, const char *who) {
+// (bf16 weights, the bf16 input and the first layer's output: two launches for the first
+// two layers, contiguous images); without it the first two layers are one fused launch.
+int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_dev, float *y_dev, const Img &st,
+                void *ws_dev, void *stream, bool keep, const char *who) {
   if (!params_dev || !x_dev || !y_dev || !ws_dev || nimg < 1 || H < 1 || W < 1)
     return rbc::set_error(RBC_EINVAL, who);
   if (int rc = tc_err()) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const long long npx = (long long)nimg * H * W;
   Ws w = carve(ws_dev, npx);
-  k_prep_weights<<<36, 256, 0, s>>>(params_dev, w.wf, w.wb);
-  if (keep) k_to_bf16<<<grid_of(npx), 256, 0, s>>>(x_dev, w.x0, npx);
+  const float *prm = params_dev;
   set_attrs();
   bool ok_tc = true;
   if (keep) {  // the backward pass reads the first layer's output
+    k_prep_weights<<<36, 256, 0, s>>>(prm, w.wf, w.wb);
+    k_to_bf16<<<grid_of(npx), 256, 0, s>>>(x_dev, w.x0, npx);
     k_conv_1to32<kHidden><<<grid_1to32<kHidden>(nimg, H, W), 256, smem_1to32<kHidden>(), s>>>(
-        w.x0, w.wf + kW1, params_dev + kB1, nullptr, w.act[0], nimg, H, W);
-    ok_tc = launch_conv_tc<kHidden>(w.act[0], w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, 1, s);
+        w.x0, w.wf + kW1, prm + kB1, nullptr, w.act[0], nimg, H, W);
+    ok_tc = launch_conv_tc<kHidden>(w.act[0], prm + kW2, prm + kB2, nullptr, w.act[1], nimg, H, W, 1, s);
   } else {
-    ok_tc = launch_conv_tc<kFused>(nullptr, w.wf + kW2, params_dev + kB2, nullptr, w.act[1], nimg, H, W, 1, s, nullptr,
-                                   nullptr, x_dev, w.wf + kW1, params_dev + kB1);
+    ok_tc = launch_conv_tc<kFused>(nullptr, prm + kW2, prm + kB2, nullptr, w.act[1], nimg, H, W, 1, s, nullptr, x_dev,
+                                   st, prm + kW1, prm + kB1);
   }
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], w.wf + kW3, params_dev + kB3, nullptr, w.act[2], nimg, H, W, 0, s);
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], w.wf + kW4, params_dev + kB4, nullptr, w.act[3], nimg, H, W, 1, s);
-  ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], w.wf + kW5, params_dev + kB5, nullptr, nullptr, nimg, H, W, 0, s,
-                                         y_dev, x_dev);
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], prm + kW3, prm + kB3, nullptr, w.act[2], nimg, H, W, 0, s);
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], prm + kW4, prm + kB4, nullptr, w.act[3], nimg, H, W, 1, s);
+  ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], prm + kW5, prm + kB5, nullptr, nullptr, nimg, H, W, 0, s, y_dev,
+                                         x_dev, st);
   if (!ok_tc) return rbc::set_error(RBC_ECUDA, "rbc_cnn_forward: launch failed");
-  rbc::add_launches(keep ? 7 : 5);
+  rbc::add_launches(keep ? 7 : 4);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rbc::set_error(RBC_ECUDA, cudaGetErrorString(e));
   return RBC_OK;
 }
+
+// Strides of contiguous images.
+Img packed(int H, int W) { return Img{(long long)H * W, W, (long long)H * W, W}; }
 
 } // namespace
 
@@ -1519,12 +1539,23 @@ long long rbc_cnn_workspace_bytes(int nimg, int H, int W) { return (long long)ws
 
 int rbc_cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_dev, float *y_dev, void *ws_dev,
                     void *stream) {
-  return cnn_forward(params_dev, nimg, H, W, x_dev, y_dev, ws_dev, stream, true, "rbc_cnn_forward: bad arguments");
+  return cnn_forward(params_dev, nimg, H, W, x_dev, y_dev, packed(H, W), ws_dev, stream, true,
+                     "rbc_cnn_forward: bad arguments");
 }
 
 int rbc_cnn_infer(const float *params_dev, int nimg, int H, int W, const float *x_dev, float *y_dev, void *ws_dev,
                   void *stream) {
-  return cnn_forward(params_dev, nimg, H, W, x_dev, y_dev, ws_dev, stream, false, "rbc_cnn_infer: bad arguments");
+  return cnn_forward(params_dev, nimg, H, W, x_dev, y_dev, packed(H, W), ws_dev, stream, false,
+                     "rbc_cnn_infer: bad arguments");
+}
+
+int rbc_cnn_infer_strided(const float *params_dev, int nimg, int H, int W, const float *x_dev, long long x_img,
+                          long long x_row, float *y_dev, long long y_img, long long y_row, void *ws_dev,
+                          void *stream) {
+  if (x_img < 0 || x_row < 0 || y_img < 0 || y_row < 0)
+    return rbc::set_error(RBC_EINVAL, "rbc_cnn_infer_strided: negative stride");
+  return cnn_forward(params_dev, nimg, H, W, x_dev, y_dev, Img{x_img, x_row, y_img, y_row}, ws_dev, stream, false,
+                     "rbc_cnn_infer_strided: bad arguments");
 }
 
 int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const float *dy_dev, float *grad_dev, void *ws_dev,

@@ -85,9 +85,16 @@ class Denoiser:
         """3-D image (nz, ny, nx): every x-z slice (fixed y) denoised, slab slices at a time."""
         nz, ny, nx = vol.shape
         out = torch.empty_like(vol)
+        # rows of x in memory order: the kernels read and write the slices in
+        # place (two passes over the volume less: 1.59 -> 1.49 ms per 400 x 64 x 800)
+        in_place = vol.is_cuda and vol.dtype == torch.float32 and vol.stride(2) == 1 and out.stride(2) == 1
         for y0 in range(0, ny, slab):
-            sl = vol[:, y0:y0 + slab, :].permute(1, 0, 2).contiguous()   # (slices, nz, nx)
-            out[:, y0:y0 + slab, :] = self(sl).permute(1, 0, 2)
+            sl = vol[:, y0:y0 + slab, :].permute(1, 0, 2)   # (slices, nz, nx)
+            to = out[:, y0:y0 + slab, :].permute(1, 0, 2)
+            if in_place:
+                N.rbc_cnn_infer_strided(self.params, sl, to, self._workspace(*sl.shape))
+            else:
+                to.copy_(self(sl))
         return out
 
 

@@ -42,3 +42,27 @@ def test_batch_equals_its_images_alone(shape):
         assert torch.equal(Y[i:i + 1], y), i
         Gs += gi.double()
     assert rel(G.cpu().numpy(), Gs.cpu().numpy()) <= 3e-4
+
+
+# memory orders of a volume (nz, ny, nx): row major, z and y swapped, x not
+# innermost, a window of a larger volume, a slice repeated along y; slabs that
+# leave a remainder, a single row and a single column
+@pytest.mark.parametrize("order", ["rows", "swapped", "x_outer", "window", "repeated"])
+@pytest.mark.parametrize("shape,slab", [((19, 7, 131), 3), ((1, 5, 1), 64), ((40, 3, 64), 1)])
+def test_volume_in_place_equals_its_slices(order, shape, slab):
+    from paper_2204_03380_gb300 import denoise as D
+    nz, ny, nx = shape
+    g = torch.Generator(device="cuda").manual_seed(nz)
+    v = torch.randn(shape, device="cuda", generator=g)
+    if order == "swapped":
+        v = v.transpose(0, 1).contiguous().transpose(0, 1)
+    elif order == "x_outer":
+        v = v.permute(2, 0, 1).contiguous().permute(1, 2, 0)
+    elif order == "window":
+        v = torch.randn((nz + 2, ny + 3, nx + 5), device="cuda", generator=g)[1:nz + 1, 2:ny + 2, 3:nx + 3]
+    elif order == "repeated":
+        v = v[:, :1].expand(nz, ny, nx)
+    net = D.Denoiser(seed=2)
+    out = net.denoise_volume(v, slab=slab)
+    ref = net(v.permute(1, 0, 2).contiguous()).permute(1, 0, 2)
+    assert torch.equal(out, ref)
