@@ -61,7 +61,7 @@ enum { kHidden = 0, kLast = 1, kBackData = 2, kFused = 3 };
 
 // The one-channel first layer (1 -> 32 channels, and the last layer's
 // backward-data pass) on the warp-level tensor cores:
-//   wt [tap][32] (bf16);  MODE kHidden: relu(conv + bias);  kBackData: conv * (mask > 0)
+//   wt [tap][32] (bf16);  MODE kHidden: relu(conv + bias);  kBackData: conv where the sign bits are set
 // Per 16 pixels of a row, one m16n8k16 MMA per group of 8 output channels with K = the 9 taps
 // (padded to 16, zero weights): the im2col operand A[pixel][tap] is gathered
 // from the staged halo straight into the A fragments, the weights are the B
@@ -72,11 +72,15 @@ enum { kHidden = 0, kLast = 1, kBackData = 2, kFused = 3 };
 // 8n + 2t, 8n + 2t + 1 of pixels g and g + 8: 4-byte pieces of the pixels'
 // 16-byte channel groups, stored 128 contiguous bytes per warp and group
 // (rounded and clamped at zero by one conversion for the forward layer;
-// masked by a packed compare of the layer's activation for the
-// backward-data pass).  The backward-data pass stages each warp's mask row
-// (8 KB) in shared memory by 16-byte cp.async copies issued before the
-// tile's barrier, so that the copies of the blocks on an SM keep enough bytes
-// in flight without holding registers.
+// masked by the layer's sign bits for the backward-data pass).
+//
+// Sign bits: for every pixel of a layer's output 32 bits of which channels are
+// positive, written beside it in the training forward and read by the backward-data pass in place of
+// the activation (4 bytes per pixel, not 64).  Bit i is channel 2 i, bit 16 + i channel
+// 2 i + 1: a packed comparison of two channels contributes both by one mask.
+// The backward-data kernels of 8 x 512^2 took 39 us (this one) and 80 us (32 -> 32)
+// reading the activation, 23 and 44 with the bits; writing them costs the forward
+// layers nothing that was measured.
 // Tile counts are ints: a tile holds 1024 pixels of 64-byte activations.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
@@ -88,8 +92,6 @@ constexpr int kM1HW = kM1C + 2, kM1HP = (kM1R + 2) * kM1HW;  // halo columns, ha
 // so the A-fragment gathers of a warp (three halo rows) are conflict-free
 constexpr int kM1P = 144;
 constexpr int kM1Pre = (kM1HP + 255) / 256;       // halo values per thread
-constexpr int kM1MaskWords = 4 * kM1C * 4;        // a warp's staged mask row: [group][pixel][4 words]
-template <int MODE> constexpr int smem_1to32() { return MODE == kBackData ? 8 * kM1MaskWords * 4 : 0; }
 __device__ __forceinline__ uint32_t pack_u16(uint16_t lo, uint16_t hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
 // {lo, hi} rounded to bf16 (and clamped at zero for kRelu) in one 4-byte word
 template <bool kRelu>
@@ -100,14 +102,25 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
   return r;
 }
 
+// 0xffff where a half of the pair is positive
+__device__ __forceinline__ uint32_t positive(uint32_t pair) {
+  return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&pair), __float2bfloat162_rn(0.f));
+}
+// 0xffff for the set ones of sign bits i and 16 + i (i a constant)
+__device__ __forceinline__ uint32_t spread(uint32_t bits, int i) {
+  const uint32_t t = bits << (i < 8 ? 7 - i : 15 - i);  // to the top of bytes 0 and 2, or 1 and 3
+  uint32_t r;  // selectors 8 + k replicate byte k's top bit
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(t), "r"(i < 8 ? 0xaa88u : 0xbb99u));
+  return r;
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__restrict__ in,
                                                         const __nv_bfloat16 *__restrict__ wt,
                                                         const float *__restrict__ bias,
-                                                        const __nv_bfloat16 *__restrict__ mask,
+                                                        uint32_t *__restrict__ bits,
                                                         __nv_bfloat16 *__restrict__ out, int nimg, int H, int W) {
   __shared__ __align__(16) uint16_t s_x[2][(kM1R + 2) * kM1P];
-  extern __shared__ __align__(16) uint32_t s_m[];  // kBackData: the warps' mask rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int ntx = (W + kM1C - 1) / kM1C, tpi = ntx * ((H + kM1R - 1) / kM1R), ntiles = tpi * nimg;
   const long long HWp = (long long)H * W;
@@ -149,11 +162,23 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
       if (i < kM1HP) s_x[b][r * kM1P + (i - r * kM1HW)] = v[k];
     }
   };
+  // kBackData: sign bits of this warp's row, pixels lane, lane + 32, ..
+  auto fetch_bits = [&](int img, int y0, int x0, uint32_t *m) {
+    if constexpr (MODE == kBackData) {
+#pragma unroll
+      for (int k = 0; k < kM1C / 32; ++k) {
+        const int xx = x0 + lane + 32 * k;
+        m[k] = (y0 + warp < H && xx < W) ? bits[img * HWp + (long long)(y0 + warp) * W + xx] : 0u;
+      }
+    }
+  };
   uint16_t v[kM1Pre];
+  uint32_t sb[kM1C / 32] = {}, sb_n[kM1C / 32] = {};
   int img = 0, y0 = 0, x0 = 0;
   if ((int)blockIdx.x < ntiles) {
     origin(blockIdx.x, img, y0, x0);
     fetch(img, y0, x0, v);
+    fetch_bits(img, y0, x0, sb);
     park(v, 0);
   }
   uint32_t *o32 = reinterpret_cast<uint32_t *>(out);
@@ -164,26 +189,12 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
     if (tn < ntiles) {  // in flight during this tile
       origin(tn, img_n, y0_n, x0_n);
       fetch(img_n, y0_n, x0_n, v);
+      fetch_bits(img_n, y0_n, x0_n, sb_n);
     }
     const int y = y0 + warp;
     const int nx = min(kM1C, W - x0);  // columns of the tile inside the image
-    uint32_t *sm = s_m + warp * kM1MaskWords;
-    if (MODE == kBackData && y < H) {
-      __syncwarp();  // the warp's reads of its previous mask row are done
-      const uint4 *m16 = reinterpret_cast<const uint4 *>(mask) + ((long long)img * 4 * HWp + (long long)y * W + x0);
-#pragma unroll
-      for (int k = 0; k < 4 * kM1C / 32; ++k) {
-        const int c = lane + 32 * k, n = c / kM1C, px = c % kM1C;
-        if (px < nx) cp_async16((uint32_t)__cvta_generic_to_shared(sm + 4 * c), m16 + n * HWp + px, true);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    }
     __syncthreads();  // s_x[b] holds tile tt
     if (y < H) {
-      if (MODE == kBackData) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncwarp();
-      }
       const uint16_t *sr = s_x[b] + warp * kM1P + g;
       // 4-byte piece t of pixel (y, x0 + g) in each channel group
       uint32_t *orow[4];
@@ -208,24 +219,33 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
 #pragma unroll
         for (int h = 0; h < 2; ++h) {  // pixels g (h = 0) and g + 8
           const int px = 16 * sg + 8 * h;
-          if (px + g >= nx) continue;
+          const bool in = px + g < nx;
+          uint32_t w = 0;  // this pixel's sign bits (kBackData: moved down by t)
+          if (MODE == kBackData) w = __shfl_sync(0xffffffffu, sb[sg >> 1], (16 * (sg & 1) + 8 * h) | g) >> t;
 #pragma unroll
           for (int n = 0; n < 4; ++n) {
             uint32_t r;
             if (MODE == kHidden) {
               r = cvt_bf16x2<true>(d[n][2 * h], d[n][2 * h + 1]);
+              w |= positive(r) & (0x00010001u << (4 * n));
             } else {
-              __nv_bfloat162 m2;
-              *reinterpret_cast<uint32_t *>(&m2) = sm[(n * kM1C + px + g) * 4 + t];
-              r = cvt_bf16x2<false>(d[n][2 * h], d[n][2 * h + 1]) & __hgt2_mask(m2, __float2bfloat162_rn(0.f));
+              r = cvt_bf16x2<false>(d[n][2 * h], d[n][2 * h + 1]) & spread(w, 4 * n);
             }
-            orow[n][px * 4] = r;
+            if (in) orow[n][px * 4] = r;
+          }
+          if (MODE == kHidden) {
+            w <<= t;
+            w |= __shfl_xor_sync(0xffffffffu, w, 1);
+            w |= __shfl_xor_sync(0xffffffffu, w, 2);
+            if (in && t == 0) bits[img * HWp + (long long)y * W + x0 + px + g] = w;
           }
         }
       }
     }
     if (tn < ntiles) {  // read two tiles on, after the next barrier
       park(v, b ^ 1);
+#pragma unroll
+      for (int k = 0; k < kM1C / 32; ++k) sb[k] = sb_n[k];
       img = img_n;
       y0 = y0_n;
       x0 = x0_n;
@@ -274,8 +294,8 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
 // to the ring's "empty" and the accumulator's "full" barrier; warps 0 ..
 // kTcEpi - 1 (two per tensor-memory lane quarter, one pixel per thread, half
 // of the rows each) drain the other accumulator with tcgen05.ld, apply the
-// epilogue (the backward-data pass reads its ReLU mask from global memory,
-// issued before the accumulator wait) and store.  Copies of the next tiles,
+// epilogue (the backward-data pass reads the sign bits of the layer below a
+// tile ahead) and store.  Copies of the next tiles,
 // MMAs of tile k and the epilogue of tile k-1 overlap.  Every wait is bounded; a
 // block that gives up flags the error word and stops.
 // A tile is kTcOut = 126 output columns: its halo row is then 128 pixels of
@@ -419,7 +439,7 @@ __device__ __forceinline__ void stm_x4(uint32_t sa, uint32_t r0, uint32_t r1, ui
 }
 
 //   MODE kHidden:   out = relu(conv(in) + bias)                        (32 -> 32)
-//   MODE kBackData: out = conv(in) * (mask > 0)   (weights mirrored and transposed)
+//   MODE kBackData: out = conv(in) where the sign bits are set   (weights mirrored and transposed)
 //   MODE kLast:     out_f = resid + conv(in) + bias                    (32 -> 1)
 //   MODE kFused:    out = relu(conv(a1) + bias) with a1 = relu(conv1(x1) + b1)
 //                   computed in the block (the first two layers, for inference)
@@ -464,7 +484,7 @@ template <int MODE, int R>
 __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid_constant__ CUtensorMap tm_in,
                                                     const void *__restrict__ wt_,
                                                     const float *__restrict__ bias,
-                                                    const __nv_bfloat16 *__restrict__ mask,
+                                                    uint32_t *__restrict__ bits,
                                                     __nv_bfloat16 *__restrict__ out, float *out_f,
                                                     const float *xin, const Img st, int nimg, int H, int W,
                                                     int rev, int *err, const float *__restrict__ w1 = nullptr,
@@ -777,28 +797,33 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     const int lq = warp & 3, r0 = (warp >> 2) * RE;
     const uint32_t lanes = (uint32_t)(lq * 32) << 16;
     const long long HWp = (long long)H * W;
+    // backward-data: this pixel's sign bits in the rows of a tile, loaded a tile ahead
+    auto load_bits = [&](int t, uint32_t *m) {
+      int img, y0, x0;
+      tile_xy(t, img, y0, x0);
+      const int px = lq * 32 + lane, xx = px < kTcOut ? x0 + px : W;
+#pragma unroll
+      for (int i = 0; i < RE; ++i)
+        m[i] = (y0 + r0 + i < H && xx < W) ? bits[img * HWp + (long long)(y0 + r0 + i) * W + xx] : 0u;
+    };
+    uint32_t sb[RE] = {}, sb_n[RE] = {};
+    if (MODE == kBackData && (int)blockIdx.x < ntiles) load_bits(blockIdx.x, sb_n);
     int k = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
       const int b = k & 1, ub = k >> 1;
       int img, y0, x0;
       tile_xy(t, img, y0, x0);
+      if (MODE == kBackData) {
+#pragma unroll
+        for (int i = 0; i < RE; ++i) sb[i] = sb_n[i];
+        if (t + gridDim.x < ntiles) load_bits(t + gridDim.x, sb_n);
+      }
       const int px = lq * 32 + lane, xx = px < kTcOut ? x0 + px : W;  // MMA rows 126, 127: no pixel
       float rs[RE];     // last layer: this pixel's residual input, loaded while the MMAs run
       if (MODE == kLast) {
 #pragma unroll
         for (int i = 0; i < RE; ++i)
           rs[i] = (y0 + r0 + i < H && xx < W) ? xin[img * st.xi + (y0 + r0 + i) * st.xr + xx] : 0.f;
-      }
-      uint4 mk[RE][4];  // backward-data: this pixel's masks, loaded while the MMAs run
-      if (MODE == kBackData) {
-#pragma unroll
-        for (int i = 0; i < RE; ++i)
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            mk[i][q] = (y0 + r0 + i < H && xx < W)
-                           ? reinterpret_cast<const uint4 *>(mask)[((long long)img * 4 + q) * HWp +
-                                                                  (long long)(y0 + r0 + i) * W + xx]
-                           : make_uint4(0u, 0u, 0u, 0u);
       }
       const bool ok = tc_wait(tfull(b), ub & 1, abort_blk);
       if (__any_sync(0xffffffffu, !ok)) break;
@@ -813,41 +838,39 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
           if (yy < H && xx < W) out_f[img * st.yi + yy * st.yr + xx] = rs[rr - r0] + v0 + s_bias[0];
         }
       } else {
-#pragma unroll 1
-      for (int rr = r0; rr < r0 + RE; ++rr) {
-        float v[32];
-        const uint32_t ta = tmem + lanes + b * BUF + (R - 1 - rr) * NCO;
-        tmem_ld32(ta, v);
-        tmem_zero32(ta);  // the next tile in this buffer accumulates from zero
-        const int yy = y0 + rr;
-        if (yy < H && xx < W) {
-          const long long pix = (long long)yy * W + xx;
-          if (kHid) {
+#pragma unroll(MODE == kBackData ? RE : 1)
+        for (int i = 0; i < RE; ++i) {
+          const int rr = r0 + i;
+          float v[32];
+          const uint32_t ta = tmem + lanes + b * BUF + (R - 1 - rr) * NCO;
+          tmem_ld32(ta, v);
+          tmem_zero32(ta);  // the next tile in this buffer accumulates from zero
+          const int yy = y0 + rr;
+          if (yy < H && xx < W) {
+            const long long pix = (long long)yy * W + xx;
+            if (kHid) {
 #pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] = fmaxf(v[c] + s_bias[c], 0.f);
-          } else {
+              for (int c = 0; c < 32; ++c) v[c] = fmaxf(v[c] + s_bias[c], 0.f);
+            }
+            uint32_t w = 0;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              const uint4 m4 = mk[rr - r0][q];
-              const __nv_bfloat162 *m2 = reinterpret_cast<const __nv_bfloat162 *>(&m4);
+              uint32_t pk[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                const float2 mf = __bfloat1622float2(m2[e]);
-                v[q * 8 + 2 * e] = mf.x > 0.f ? v[q * 8 + 2 * e] : 0.f;
-                v[q * 8 + 2 * e + 1] = mf.y > 0.f ? v[q * 8 + 2 * e + 1] : 0.f;
+                pk[e] = cvt_bf16x2<false>(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
+                if (MODE == kBackData) pk[e] &= spread(sb[i], 4 * q + e);
+              }
+              reinterpret_cast<uint4 *>(out)[((long long)img * 4 + q) * HWp + pix] =
+                  make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              if (MODE == kHidden && bits) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w |= positive(pk[e]) & (0x00010001u << (4 * q + e));
               }
             }
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 pk;
-            __nv_bfloat162 *p2 = reinterpret_cast<__nv_bfloat162 *>(&pk);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) p2[e] = __floats2bfloat162_rn(v[q * 8 + 2 * e], v[q * 8 + 2 * e + 1]);
-            reinterpret_cast<uint4 *>(out)[((long long)img * 4 + q) * HWp + pix] = pk;
+            if (MODE == kHidden && bits) bits[img * HWp + pix] = w;
           }
         }
-      }
       }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1347,9 +1370,7 @@ int grid_1to32(int nimg, int H, int W) {
   if (!slots) {
     int sms = 152, per = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-    if (smem_1to32<MODE>() > 48 * 1024)
-      cudaFuncSetAttribute(k_conv_1to32<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_1to32<MODE>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_conv_1to32<MODE>, 256, smem_1to32<MODE>());
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_conv_1to32<MODE>, 256, 0);
     slots = sms * (per > 0 ? per : 1);
   }
   const long long tiles = (long long)((W + kM1C - 1) / kM1C) * ((H + kM1R - 1) / kM1R) * nimg;
@@ -1364,27 +1385,34 @@ int grid_of(long long n) {
 
 // Workspace layout (bytes): bf16 weights fwd, bf16 weights bwd, x (bf16),
 // four hidden activations (bf16, 32 ch), two 32-channel gradient buffers
-// (bf16) and the last-layer output gradient (bf16).
+// (bf16), the last-layer output gradient (bf16) and the activations' sign bits.
 struct Ws {
   __nv_bfloat16 *wf, *wb, *x0, *act[4], *dz[2], *dy1;
+  uint32_t *bits[4];
+  size_t bytes;
 };
 
-size_t ws_bytes(long long npx) {
-  return sizeof(__nv_bfloat16) * (2 * (size_t)kNParams + 256 + (size_t)npx * (1 + 4 * C + 2 * C + 1)) + 1024;
-}
-
 Ws carve(void *ws, long long npx) {
-  auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  char *p = static_cast<char *>(ws);
+  size_t at = 0;
+  auto take = [&](size_t b) {
+    char *p = static_cast<char *>(ws) + at;
+    at += (b + 255) / 256 * 256;
+    return reinterpret_cast<__nv_bfloat16 *>(p);
+  };
+  const size_t n = (size_t)npx;
   Ws w;
-  w.wf = reinterpret_cast<__nv_bfloat16 *>(p); p += al(sizeof(__nv_bfloat16) * kNParams);
-  w.wb = reinterpret_cast<__nv_bfloat16 *>(p); p += al(sizeof(__nv_bfloat16) * kNParams);
-  w.x0 = reinterpret_cast<__nv_bfloat16 *>(p); p += al(sizeof(__nv_bfloat16) * npx);
-  for (int l = 0; l < 4; ++l) { w.act[l] = reinterpret_cast<__nv_bfloat16 *>(p); p += al(sizeof(__nv_bfloat16) * npx * C); }
-  for (int l = 0; l < 2; ++l) { w.dz[l] = reinterpret_cast<__nv_bfloat16 *>(p); p += al(sizeof(__nv_bfloat16) * npx * C); }
-  w.dy1 = reinterpret_cast<__nv_bfloat16 *>(p);
+  w.wf = take(2 * kNParams);
+  w.wb = take(2 * kNParams);
+  w.x0 = take(2 * n);
+  for (int l = 0; l < 4; ++l) w.act[l] = take(2 * n * C);
+  for (int l = 0; l < 2; ++l) w.dz[l] = take(2 * n * C);
+  w.dy1 = take(2 * n);
+  for (int l = 0; l < 4; ++l) w.bits[l] = reinterpret_cast<uint32_t *>(take(4 * n));
+  w.bytes = at;
   return w;
 }
+
+size_t ws_bytes(long long npx) { return carve(nullptr, npx).bytes; }
 
 // Error word of the tensor-core kernels' bounded waits (mapped host memory,
 // read at the next call).
@@ -1457,7 +1485,7 @@ int tile_rows(int nimg, int H, int W) {
 }
 
 template <int MODE, int R>
-bool launch_conv_r(const __nv_bfloat16 *in, const void *wt, const float *bias, const __nv_bfloat16 *mask,
+bool launch_conv_r(const __nv_bfloat16 *in, const void *wt, const float *bias, uint32_t *bits,
                    __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f, const float *x,
                    const Img &st, const float *w1, const float *b1) {
   const long long tiles = tiles_of(nimg, H, W, R);
@@ -1465,19 +1493,19 @@ bool launch_conv_r(const __nv_bfloat16 *in, const void *wt, const float *bias, c
   CUtensorMap tin;
   memset(&tin, 0, sizeof tin);  // (the fused mode builds its operand instead of copying it)
   if (MODE != kFused && !act_map(&tin, in, nimg, H, W, tc_ur(R))) return false;
-  launch_pdl(k_conv_tc<MODE, R>, dim3(grid), dim3(tc_threads(MODE, R)), tc_smem_mode(MODE, R), s, tin, wt, bias, mask, out,
+  launch_pdl(k_conv_tc<MODE, R>, dim3(grid), dim3(tc_threads(MODE, R)), tc_smem_mode(MODE, R), s, tin, wt, bias, bits, out,
              out_f, x, st, nimg, H, W, rev, tc_err_dev, w1, b1);
   return true;
 }
 
 template <int MODE>
-bool launch_conv_tc(const __nv_bfloat16 *in, const void *wt, const float *bias, const __nv_bfloat16 *mask,
+bool launch_conv_tc(const __nv_bfloat16 *in, const void *wt, const float *bias, uint32_t *bits,
                     __nv_bfloat16 *out, int nimg, int H, int W, int rev, cudaStream_t s, float *out_f = nullptr,
                     const float *x = nullptr, const Img &st = Img(), const float *w1 = nullptr,
                     const float *b1 = nullptr) {
   return tile_rows(nimg, H, W) == kTcRs
-             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, x, st, w1, b1)
-             : launch_conv_r<MODE, kTcR>(in, wt, bias, mask, out, nimg, H, W, rev, s, out_f, x, st, w1, b1);
+             ? launch_conv_r<MODE, kTcRs>(in, wt, bias, bits, out, nimg, H, W, rev, s, out_f, x, st, w1, b1)
+             : launch_conv_r<MODE, kTcR>(in, wt, bias, bits, out, nimg, H, W, rev, s, out_f, x, st, w1, b1);
 }
 
 // One block per SM (its shared memory), at most one per tile.
@@ -1508,15 +1536,17 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
   if (keep) {  // the backward pass reads the first layer's output
     k_prep_weights<<<36, 256, 0, s>>>(prm, w.wf, w.wb);
     k_to_bf16<<<grid_of(npx), 256, 0, s>>>(x_dev, w.x0, npx);
-    k_conv_1to32<kHidden><<<grid_1to32<kHidden>(nimg, H, W), 256, smem_1to32<kHidden>(), s>>>(
-        w.x0, w.wf + kW1, prm + kB1, nullptr, w.act[0], nimg, H, W);
-    ok_tc = launch_conv_tc<kHidden>(w.act[0], prm + kW2, prm + kB2, nullptr, w.act[1], nimg, H, W, 1, s);
+    k_conv_1to32<kHidden><<<grid_1to32<kHidden>(nimg, H, W), 256, 0, s>>>(
+        w.x0, w.wf + kW1, prm + kB1, w.bits[0], w.act[0], nimg, H, W);
+    ok_tc = launch_conv_tc<kHidden>(w.act[0], prm + kW2, prm + kB2, w.bits[1], w.act[1], nimg, H, W, 1, s);
   } else {
     ok_tc = launch_conv_tc<kFused>(nullptr, prm + kW2, prm + kB2, nullptr, w.act[1], nimg, H, W, 1, s, nullptr, x_dev,
                                    st, prm + kW1, prm + kB1);
   }
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], prm + kW3, prm + kB3, nullptr, w.act[2], nimg, H, W, 0, s);
-  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], prm + kW4, prm + kB4, nullptr, w.act[3], nimg, H, W, 1, s);
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[1], prm + kW3, prm + kB3, keep ? w.bits[2] : nullptr, w.act[2], nimg,
+                                           H, W, 0, s);
+  ok_tc = ok_tc && launch_conv_tc<kHidden>(w.act[2], prm + kW4, prm + kB4, keep ? w.bits[3] : nullptr, w.act[3], nimg,
+                                           H, W, 1, s);
   ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], prm + kW5, prm + kB5, nullptr, nullptr, nimg, H, W, 0, s, y_dev,
                                          x_dev, st);
   if (!ok_tc) return rbc::set_error(RBC_ECUDA, "rbc_cnn_forward: launch failed");
@@ -1573,8 +1603,8 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
       dy_dev, w.act[3], grad_dev + kW5, grad_dev + kB5, nimg, H, W);
   k_to_bf16<<<grid_of(npx), 256, 0, s>>>(dy_dev, w.dy1, npx);
   set_attrs();
-  k_conv_1to32<kBackData><<<grid_1to32<kBackData>(nimg, H, W), 256, smem_1to32<kBackData>(), s>>>(
-      w.dy1, w.wb + kW5, nullptr, w.act[3], w.dz[0], nimg, H, W);
+  k_conv_1to32<kBackData><<<grid_1to32<kBackData>(nimg, H, W), 256, 0, s>>>(
+      w.dy1, w.wb + kW5, nullptr, w.bits[3], w.dz[0], nimg, H, W);
   // layers 4, 3, 2: dW from dz; dz below = conv^T(dz) masked
   int cur = 0;
   bool ok_tc = true;
@@ -1582,7 +1612,8 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
   for (int l = 0; l < 3; ++l) {
     const int layer_in = 2 - l;  // act index of this layer's input: act3 (l=0) ... act1
     ok_tc = ok_tc && launch_wgrad(w.act[layer_in], w.dz[cur], grad_dev + woff[l], grad_dev + boff[l], nimg, H, W, s);
-    ok_tc = ok_tc && launch_conv_tc<kBackData>(w.dz[cur], w.wb + woff[l], nullptr, w.act[layer_in], w.dz[1 - cur], nimg, H, W, 0, s);
+    ok_tc = ok_tc && launch_conv_tc<kBackData>(w.dz[cur], w.wb + woff[l], nullptr, w.bits[layer_in], w.dz[1 - cur],
+                                               nimg, H, W, 0, s);
     cur = 1 - cur;
   }
   // layer 1
