@@ -115,7 +115,7 @@ __device__ __forceinline__ uint32_t spread(uint32_t bits, int i) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__restrict__ in,
+__global__ void __launch_bounds__(256, 3) k_conv_1to32(const float *__restrict__ in, __nv_bfloat16 *__restrict__ in16,
                                                         const __nv_bfloat16 *__restrict__ wt,
                                                         const float *__restrict__ bias,
                                                         uint32_t *__restrict__ bits,
@@ -125,6 +125,8 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
   const int ntx = (W + kM1C - 1) / kM1C, tpi = ntx * ((H + kM1R - 1) / kM1R), ntiles = tpi * nimg;
   const long long HWp = (long long)H * W;
   const uint16_t *win = reinterpret_cast<const uint16_t *>(wt);
+  griddep_wait();
+  griddep_launch();
   // B fragments: B[k][co] = w[tap k][co] for k < 9, zero above
   uint32_t bf[4][2];
   float2 bs[4];
@@ -144,22 +146,27 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
     y0 = ty * kM1R;
     x0 = (rem - ty * ntx) * kM1C;
   };
-  const uint16_t *xin = reinterpret_cast<const uint16_t *>(in);
-  auto fetch = [&](int img, int y0, int x0, uint16_t *v) {
-    const uint16_t *src = xin + (long long)img * HWp;
+  auto fetch = [&](int img, int y0, int x0, float *v) {
+    const float *src = in + (long long)img * HWp;
 #pragma unroll
     for (int k = 0; k < kM1Pre; ++k) {
       const int i = tid + 256 * k, r = i / kM1HW;
       const int yy = y0 + r - 1, xx = x0 + (i - r * kM1HW) - 1;
       v[k] = (i < kM1HP && (unsigned)yy < (unsigned)H && (unsigned)xx < (unsigned)W) ? src[(long long)yy * W + xx]
-                                                                                      : (uint16_t)0;
+                                                                                      : 0.f;
     }
   };
-  auto park = [&](const uint16_t *v, int b) {
+  // rounded to bf16; the forward layer also writes the tile's own pixels to in16
+  auto park = [&](const float *v, int b, int img, int y0, int x0) {
 #pragma unroll
     for (int k = 0; k < kM1Pre; ++k) {
-      const int i = tid + 256 * k, r = i / kM1HW;
-      if (i < kM1HP) s_x[b][r * kM1P + (i - r * kM1HW)] = v[k];
+      const int i = tid + 256 * k, r = i / kM1HW, c = i - r * kM1HW;
+      if (i < kM1HP) {
+        const __nv_bfloat16 h = __float2bfloat16(v[k]);
+        s_x[b][r * kM1P + c] = __bfloat16_as_ushort(h);
+        if (MODE == kHidden && r >= 1 && r <= kM1R && c >= 1 && c <= kM1C && y0 + r - 1 < H && x0 + c - 1 < W)
+          in16[img * HWp + (long long)(y0 + r - 1) * W + x0 + c - 1] = h;
+      }
     }
   };
   // kBackData: sign bits of this warp's row, pixels lane, lane + 32, ..
@@ -172,14 +179,14 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
       }
     }
   };
-  uint16_t v[kM1Pre];
+  float v[kM1Pre];
   uint32_t sb[kM1C / 32] = {}, sb_n[kM1C / 32] = {};
   int img = 0, y0 = 0, x0 = 0;
   if ((int)blockIdx.x < ntiles) {
     origin(blockIdx.x, img, y0, x0);
     fetch(img, y0, x0, v);
     fetch_bits(img, y0, x0, sb);
-    park(v, 0);
+    park(v, 0, img, y0, x0);
   }
   uint32_t *o32 = reinterpret_cast<uint32_t *>(out);
   int b = 0;
@@ -243,7 +250,7 @@ __global__ void __launch_bounds__(256, 3) k_conv_1to32(const __nv_bfloat16 *__re
       }
     }
     if (tn < ntiles) {  // read two tiles on, after the next barrier
-      park(v, b ^ 1);
+      park(v, b ^ 1, img_n, y0_n, x0_n);
 #pragma unroll
       for (int k = 0; k < kM1C / 32; ++k) sb[k] = sb_n[k];
       img = img_n;
@@ -1144,6 +1151,8 @@ __global__ void __launch_bounds__(128) k_conv_wgrad1(const TU *__restrict__ u, c
   const int ntx = (W + kW1C - 1) / kW1C, tpi = ntx * ((H + kW1R - 1) / kW1R), ntiles = tpi * nimg;
   const long long HWp = (long long)H * W;
   for (int i = tid; i < kW1Red; i += 128) s_red[i] = 0.f;
+  griddep_wait();
+  griddep_launch();
   // halo offsets of this lane's A rows: tap g, and tap 8 (g = 0); the last
   // layer reads u at q - off(tap), the mirrored tap
   const int tg = kFirst ? g : 8 - g;
@@ -1280,6 +1289,8 @@ __global__ void k_prep_weights(const float *__restrict__ prm, __nv_bfloat16 *__r
   // [8 - t][ci][co] (only layers 2..5 are needed backwards)
   const int offs[5] = {kW1, kW2, kW3, kW4, kW5};
   const int cin[5] = {1, C, C, C, C}, cout[5] = {C, C, C, C, 1};
+  griddep_wait();
+  griddep_launch();
   for (int l = 0; l < 5; ++l) {
     const int n = 9 * cin[l] * cout[l];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1291,15 +1302,13 @@ __global__ void k_prep_weights(const float *__restrict__ prm, __nv_bfloat16 *__r
   }
 }
 
-__global__ void k_to_bf16(const float *__restrict__ x, __nv_bfloat16 *__restrict__ y, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16(x[i]);
-}
-
 // loss = mean((y - t)^2) (fp64 accumulate); dy = 2 (y - t) / n
 __global__ void k_mse(const float *__restrict__ y, const float *__restrict__ t, long long n, float *__restrict__ dy,
                       double *loss) {
+  griddep_wait();
+  griddep_launch();
   double acc = 0.0;
+#pragma unroll 4
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float d = y[i] - t[i];
     if (dy) dy[i] = 2.f * d / (float)n;
@@ -1320,6 +1329,8 @@ __global__ void k_mse(const float *__restrict__ y, const float *__restrict__ t, 
 // Adam (Kingma & Ba 2015) with bias correction.
 __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
                        int n, float lr, float b1, float b2, float eps, float c1, float c2) {
+  griddep_wait();
+  griddep_launch();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -1385,9 +1396,9 @@ int grid_of(long long n) {
 
 // Workspace layout (bytes): bf16 weights fwd, bf16 weights bwd, x (bf16),
 // four hidden activations (bf16, 32 ch), two 32-channel gradient buffers
-// (bf16), the last-layer output gradient (bf16) and the activations' sign bits.
+// (bf16) and the activations' sign bits.
 struct Ws {
-  __nv_bfloat16 *wf, *wb, *x0, *act[4], *dz[2], *dy1;
+  __nv_bfloat16 *wf, *wb, *x0, *act[4], *dz[2];
   uint32_t *bits[4];
   size_t bytes;
 };
@@ -1406,7 +1417,6 @@ Ws carve(void *ws, long long npx) {
   w.x0 = take(2 * n);
   for (int l = 0; l < 4; ++l) w.act[l] = take(2 * n * C);
   for (int l = 0; l < 2; ++l) w.dz[l] = take(2 * n * C);
-  w.dy1 = take(2 * n);
   for (int l = 0; l < 4; ++l) w.bits[l] = reinterpret_cast<uint32_t *>(take(4 * n));
   w.bytes = at;
   return w;
@@ -1534,10 +1544,9 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
   set_attrs();
   bool ok_tc = true;
   if (keep) {  // the backward pass reads the first layer's output
-    k_prep_weights<<<36, 256, 0, s>>>(prm, w.wf, w.wb);
-    k_to_bf16<<<grid_of(npx), 256, 0, s>>>(x_dev, w.x0, npx);
-    k_conv_1to32<kHidden><<<grid_1to32<kHidden>(nimg, H, W), 256, 0, s>>>(
-        w.x0, w.wf + kW1, prm + kB1, w.bits[0], w.act[0], nimg, H, W);
+    launch_pdl(k_prep_weights, dim3(36), dim3(256), 0, s, prm, w.wf, w.wb);
+    launch_pdl(k_conv_1to32<kHidden>, dim3(grid_1to32<kHidden>(nimg, H, W)), dim3(256), 0, s, x_dev, w.x0, w.wf + kW1,
+               prm + kB1, w.bits[0], w.act[0], nimg, H, W);
     ok_tc = launch_conv_tc<kHidden>(w.act[0], prm + kW2, prm + kB2, w.bits[1], w.act[1], nimg, H, W, 1, s);
   } else {
     ok_tc = launch_conv_tc<kFused>(nullptr, prm + kW2, prm + kB2, nullptr, w.act[1], nimg, H, W, 1, s, nullptr, x_dev,
@@ -1550,7 +1559,7 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
   ok_tc = ok_tc && launch_conv_tc<kLast>(w.act[3], prm + kW5, prm + kB5, nullptr, nullptr, nimg, H, W, 0, s, y_dev,
                                          x_dev, st);
   if (!ok_tc) return rbc::set_error(RBC_ECUDA, "rbc_cnn_forward: launch failed");
-  rbc::add_launches(keep ? 7 : 4);
+  rbc::add_launches(keep ? 6 : 4);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rbc::set_error(RBC_ECUDA, cudaGetErrorString(e));
   return RBC_OK;
@@ -1599,12 +1608,10 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
   Ws w = carve(ws_dev, npx);  // activations from the preceding rbc_cnn_forward
 
   // layer 5: dW5, db5 from dy; dz4 = conv^T(dy) masked by act4 > 0
-  k_conv_wgrad1<false, float><<<grid_wgrad1<false, float>(nimg, H, W), 128, kW1Smem, s>>>(
-      dy_dev, w.act[3], grad_dev + kW5, grad_dev + kB5, nimg, H, W);
-  k_to_bf16<<<grid_of(npx), 256, 0, s>>>(dy_dev, w.dy1, npx);
-  set_attrs();
-  k_conv_1to32<kBackData><<<grid_1to32<kBackData>(nimg, H, W), 256, 0, s>>>(
-      w.dy1, w.wb + kW5, nullptr, w.bits[3], w.dz[0], nimg, H, W);
+  launch_pdl(k_conv_wgrad1<false, float>, dim3(grid_wgrad1<false, float>(nimg, H, W)), dim3(128), kW1Smem, s, dy_dev,
+             w.act[3], grad_dev + kW5, grad_dev + kB5, nimg, H, W);
+  launch_pdl(k_conv_1to32<kBackData>, dim3(grid_1to32<kBackData>(nimg, H, W)), dim3(256), 0, s, dy_dev, nullptr,
+             w.wb + kW5, nullptr, w.bits[3], w.dz[0], nimg, H, W);
   // layers 4, 3, 2: dW from dz; dz below = conv^T(dz) masked
   int cur = 0;
   bool ok_tc = true;
@@ -1617,10 +1624,10 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
     cur = 1 - cur;
   }
   // layer 1
-  k_conv_wgrad1<true, __nv_bfloat16><<<grid_wgrad1<true, __nv_bfloat16>(nimg, H, W), 128, kW1Smem, s>>>(
-      w.x0, w.dz[cur], grad_dev + kW1, grad_dev + kB1, nimg, H, W);
+  launch_pdl(k_conv_wgrad1<true, __nv_bfloat16>, dim3(grid_wgrad1<true, __nv_bfloat16>(nimg, H, W)), dim3(128), kW1Smem,
+             s, w.x0, w.dz[cur], grad_dev + kW1, grad_dev + kB1, nimg, H, W);
   if (!ok_tc) return rbc::set_error(RBC_ECUDA, "rbc_cnn_backward: launch failed");
-  rbc::add_launches(10);
+  rbc::add_launches(9);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rbc::set_error(RBC_ECUDA, cudaGetErrorString(e));
   return RBC_OK;
@@ -1628,7 +1635,9 @@ int rbc_cnn_backward(const float *params_dev, int nimg, int H, int W, const floa
 
 int rbc_cnn_mse(const float *y_dev, const float *t_dev, long long n, float *dy_dev, double *loss_dev, void *stream) {
   if (!y_dev || !t_dev || !loss_dev || n < 1) return rbc::set_error(RBC_EINVAL, "rbc_cnn_mse: bad arguments");
-  k_mse<<<grid_of(n), 256, 0, (cudaStream_t)stream>>>(y_dev, t_dev, n, dy_dev, loss_dev);
+  // four blocks per SM: each adds its sum to one double, and 2432 such adds took 20 us
+  const int most = 4 * sm_count(), grid = grid_of(n) < most ? grid_of(n) : most;
+  launch_pdl(k_mse, dim3(grid), dim3(256), 0, (cudaStream_t)stream, y_dev, t_dev, n, dy_dev, loss_dev);
   rbc::add_launches(1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rbc::set_error(RBC_ECUDA, cudaGetErrorString(e));
@@ -1640,8 +1649,8 @@ int rbc_cnn_adam(float *params_dev, const float *grad_dev, float *m_dev, float *
   if (!params_dev || !grad_dev || !m_dev || !v_dev || step < 1) return rbc::set_error(RBC_EINVAL, "rbc_cnn_adam: bad arguments");
   // bias corrections formed in fp64: 1 - b2^step cancels badly in fp32 at small steps
   const float c1 = (float)(1.0 - pow((double)b1, (double)step)), c2 = (float)(1.0 - pow((double)b2, (double)step));
-  k_adam<<<grid_of(kNParams), 256, 0, (cudaStream_t)stream>>>(params_dev, grad_dev, m_dev, v_dev, kNParams, lr, b1, b2,
-                                                              eps, c1, c2);
+  launch_pdl(k_adam, dim3(grid_of(kNParams)), dim3(256), 0, (cudaStream_t)stream, params_dev, grad_dev, m_dev, v_dev,
+             kNParams, lr, b1, b2, eps, c1, c2);
   rbc::add_launches(1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return rbc::set_error(RBC_ECUDA, cudaGetErrorString(e));
