@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (MODE != kFused) griddep_wait();
   griddep_launch();
-  // (32-bit tile numbers: a tile holds at least 126 pixels of 64 bytes)
+  // (32-bit tile numbers: a tile holds at least one pixel of some 400 bytes of workspace)
   const int ntx = (W + kTcOut - 1) / kTcOut, tpi = ntx * ((H + R - 1) / R), ntiles = tpi * nimg;
   // Persistent blocks over the tiles, x fastest (a contiguous y-fastest range per block lost: 1.36
   // against 1.27 ms per 32 x 512^2 inference).  rev: from the last tile to the

@@ -303,8 +303,8 @@ __device__ __forceinline__ void keep_level(const ResArgs &A, const ResShot &S, c
 }
 
 // ------------------------------------------------------------- forward ----
-template <int RZ, int MAXW, int MINB>
-__global__ void __launch_bounds__(32 * MAXW, MINB) k_res_fwd(const ResArgs A, const int H) {
+template <int RZ, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const int H) {
   extern __shared__ __align__(16) float smem[];
   const int fl = buf_floats<false>(H), h4 = 4 * kTileX;
   float *s_a = smem + 2 * fl;
@@ -500,8 +500,8 @@ constexpr int tm_cols(int rz, int warps) {
 
 // MODE 0: imaging integrals (Eq. 3); 1: FWI gradient; 2: RTM with wavefield storage (Algorithm 2: only pbar is
 // stepped, and the integrals are formed at the kept levels, with p^n read from the store)
-template <int RZ, int MAXW, int MINB, bool TIGHT, bool TM, int MODE>
-__global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, const int H) {
+template <int RZ, int MAXW, bool TIGHT, bool TM, int MODE>
+__global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const int H) {
   constexpr bool kGrad = MODE == 1, kStore = MODE == 2;
   constexpr int NB = kStore ? 2 : 4, B0 = kStore ? 0 : 2, FB = kStore ? 0 : 1;  // buffers; pbar's first, its exchange field
   extern __shared__ __align__(16) float smem[];
@@ -709,26 +709,27 @@ __global__ void __launch_bounds__(32 * MAXW, MINB) k_res_rev(const ResArgs A, co
 inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 
 struct Variant {
-  int rz, maxw, minb;
+  int rz, maxw;
   bool tight, tm;
   const void *fn[4];  // forward, imaging, FWI gradient, storage
 };
-#define RBC_RES_VARIANT(RZ, MAXW, MINB, TIGHT, TM)                                                                 \
-  {RZ, MAXW, MINB, TIGHT, TM,                                                                                      \
-   {(const void *)k_res_fwd<RZ, MAXW, MINB>, (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 0>,                \
-    (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 1>, (const void *)k_res_rev<RZ, MAXW, MINB, TIGHT, TM, 2>}}
-// Rows per warp, most warps per block, blocks per SM, layout.  res_plan takes
+#define RBC_RES_VARIANT(RZ, MAXW, TIGHT, TM)                                                                 \
+  {RZ, MAXW, TIGHT, TM,                                                                                      \
+   {(const void *)k_res_fwd<RZ, MAXW>, (const void *)k_res_rev<RZ, MAXW, TIGHT, TM, 0>,                \
+    (const void *)k_res_rev<RZ, MAXW, TIGHT, TM, 1>, (const void *)k_res_rev<RZ, MAXW, TIGHT, TM, 2>}}
+// Rows per warp, most warps per block, layout; one block per SM.  res_plan takes
 // the first that holds the grid: with few rows per warp a step is short (300 x
-// 300 forward: 1.6 / 1.9 / 2.5 / 2.8 / 3.1 us with 1 / 2 / 4 / 7 / 10 rows).
-// One or two rows per warp run 8 warps (two blocks to an SM); the others,
-// whose kernels allocate tensor memory and so run one block per SM, as few
-// warps as fit, which spreads the grid over the SMs (1500 x 800 forward +
-// reverse: 9.3 us with 10 warps of 7 rows, 11.2 with 15).  The last is the
+// 300 forward: 1.6 / 1.9 / 2.5 / 2.8 / 3.1 us with 1 / 2 / 4 / 7 / 10 rows),
+// and as few warps as fit, which spreads the grid over the SMs (1500 x 800 forward +
+// reverse: 9.3 us with 10 warps of 7 rows, 11.2 with 15), but eight at least with
+// one or two rows (300 x 300: 1.52 us with 8, 1.72 with 6).  Blocks of 8 warps, two to
+// an SM, left some SMs two and some one: forward / RTM step of 400 x 400 1.79 / 5.40 us against
+// 1.58 / 4.71 now, 700 x 500 2.05 / 5.74 against 1.90 / 5.54.  The last is the
 // tallest tile whose four buffers fit 227 KB: TIGHT keeps no halo rows in them.
 const Variant kVariants[] = {
-    RBC_RES_VARIANT(1, 8, 2, false, false), RBC_RES_VARIANT(2, 8, 2, false, false),
-    RBC_RES_VARIANT(4, 16, 1, false, true), RBC_RES_VARIANT(7, 16, 1, true, true),
-    RBC_RES_VARIANT(10, 11, 1, true, true),
+    RBC_RES_VARIANT(1, 16, false, false), RBC_RES_VARIANT(2, 16, false, false),
+    RBC_RES_VARIANT(4, 16, false, true), RBC_RES_VARIANT(7, 16, true, true),
+    RBC_RES_VARIANT(10, 11, true, true),
 };
 
 size_t res_smem(int dir, int H, const Variant &V) {
@@ -737,11 +738,11 @@ size_t res_smem(int dir, int H, const Variant &V) {
   if (dir == kResFwd) rows = 2 * (H + 8) + H;
   else rows = V.tight ? nb * H + 4 : nb * (H + 8) + (V.tm ? 0 : H);
   const size_t need = sizeof(float) * (rows * kTileX + 8 * (size_t)H) + (dir != kResFwd && V.tm ? 16 : 0);
-  // The forward kernels allocate no tensor memory: more than half an SM's shared
+  // Kernels that allocate no tensor memory: more than half an SM's shared
   // memory keeps a second block off it.  Loops in flight together otherwise land
   // on the same SMs while others idle (four shots of 300 x 300 at once: 3.6 -> 2.4 us a step;
   // one shot of 2301 x 751: 3.64 -> 3.42).
-  return V.minb == 1 && dir == kResFwd ? std::max(need, (size_t)116 * 1024) : need;
+  return dir == kResFwd || !V.tm ? std::max(need, (size_t)116 * 1024) : need;
 }
 
 } // namespace
@@ -765,10 +766,9 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
     const Variant &V = kVariants[v];
     int nzmax = 1;
     for (int s = 0; s < nshots; ++s) nzmax = std::max(nzmax, L[s].NZ);
-    // one or two rows per warp: the tallest tiles (two blocks to an SM); more: the lowest that fit (one)
+    // the lowest tiles that fit; with one or two rows per warp at least eight warps
     const int top = std::min(V.maxw, std::max(cdiv(nzmax, V.rz), cdiv(4, V.rz)));
-    for (int i = 1; best_v < 0 && i <= top; ++i) {
-      const int nw = V.rz < 4 ? top + 1 - i : i;
+    for (int nw = V.rz < 4 && force_w <= 0 ? std::min(8, top) : 1; best_v < 0 && nw <= top; ++nw) {
       if (force_v >= 0 && (v != force_v || (force_w > 0 && nw != force_w))) continue;
       const int H = nw * V.rz;
       if (H < 4) continue;
@@ -776,8 +776,7 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
       if (sm > (size_t)maxsm) continue;
       long long blocks = 0;
       for (int s = 0; s < nshots; ++s) blocks += (long long)cdiv(L[s].NX, kTileX) * cdiv(L[s].NZ, H);
-      // (more blocks than the variant's registers allow: no need to ask the runtime)
-      if (blocks * share > (long long)(V.maxw * V.minb / nw) * sms) continue;
+      if (blocks * share > sms) continue;  // (one block per SM: no need to ask the runtime)
       int per = 1 << 20;
       for (int f = dir == kResStore ? 3 : dir; f <= (dir == kResRev ? 2 : dir == kResStore ? 3 : 0); ++f) {
         const void *fn = V.fn[f];
@@ -863,9 +862,9 @@ std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
   double best_us = 1e30;
   for (int v = 0; v < (int)(sizeof kVariants / sizeof kVariants[0]); ++v) {
     const Variant &V = kVariants[v];
-    const int cap = V.minb * sms;
+    const int cap = sms;
     int hmax = V.maxw * V.rz;
-    while (hmax > V.rz && res_smem(kResRev, hmax, V) > 227 * 1024 / V.minb) hmax -= V.rz;
+    while (hmax > V.rz && res_smem(kResRev, hmax, V) > 227 * 1024) hmax -= V.rz;
     std::vector<int> tiles(nshots);
     bool fits = true;
     for (int i = 0; i < nshots; ++i) {
