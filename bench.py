@@ -216,17 +216,17 @@ def load_workload(W, args):
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the stencil
 # kernels from ncu captures (profiles/), recorded with a hash of the kernel
 # sources they were taken on: a capture of older sources reads as null.
-#   k_rev2d_tile on the 2-D survey grid, warm L2 as in the time loop (one-pass
-#   metrics capture, mean of three launches): the shot's fields stay in L2.
+#   k_res_rev on the 2-D survey grid: one launch of a short record, divided by its
+#   steps (the fields are on the chip; what remains is records and their last values).
 #   3-D kernels: captured on the 380 x 380 x 280 grid as a multiple of their
 #   algorithmic bytes; the traffic of their tiles grows in proportion to the
 #   nodes, so a full 580 x 580 x 380 launch gets that multiple of its own.
-_SRC2 = ["rbc_kernels.cu", "rbc_tile2d.cuh", "rbc_stencil.cuh", "rbc_internal.cuh"]
+_SRC2 = ["rbc_resident.cu", "rbc_stencil.cuh", "rbc_internal.cuh"]
 _SRC3 = ["rbc_kernels3d.cu", "rbc_stencil.cuh", "rbc_internal.cuh"]
 TRAFFIC = {
-    "k_rev2d_tile": {"sources": _SRC2, "sha1": "f860ce948d6f75a4", "bytes_per_launch": 1.02e6, "ratio": None},
-    "k_rev3d_tma": {"sources": _SRC3, "sha1": "b0ea2b88596cbbf5", "bytes_per_launch": None, "ratio": 1.122},
-    "k_fwd3d_tma": {"sources": _SRC3, "sha1": "b0ea2b88596cbbf5", "bytes_per_launch": None, "ratio": 1.087},
+    "k_res_rev": {"sources": _SRC2, "sha1": "cc91d41be50bd9e8", "bytes_per_launch": 1.0e4, "ratio": None},
+    "k_rev3d_tma": {"sources": _SRC3, "sha1": "3b21a33f400b3d11", "bytes_per_launch": None, "ratio": 1.118},
+    "k_fwd3d_tma": {"sources": _SRC3, "sha1": "3b21a33f400b3d11", "bytes_per_launch": None, "ratio": 1.090},
 }
 
 
@@ -249,7 +249,7 @@ def kernel_traffic(kernel, algorithmic_bytes):
 
 
 def reverse_traffic(ndim, algorithmic_bytes):
-    return kernel_traffic("k_rev2d_tile" if ndim == 2 else "k_rev3d_tma", algorithmic_bytes)
+    return kernel_traffic("k_res_rev" if ndim == 2 else "k_rev3d_tma", algorithmic_bytes)
 
 
 def measured_peaks():
@@ -426,11 +426,11 @@ def run_batch(args, rank, world):
                                                                          max(s["width"] for s in inp["shots"])],
                       "nt": w.nt, "autotuned": info, "s_per_shot": el / args.steps / len(shots),
                       "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB write)"},
-           "roofline": {"bound": "hbm", "kernel": "k_rev2d_batch (fused reverse pass, all shots)",
+           "roofline": {"bound": "hbm", "kernel": "k_res_rev (fused reverse pass, all shots, per time step)",
                         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                         "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s",
                         "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_s * 1e6,
-                        "forward_kernel": {"kernel": "k_fwd2d_batch", "launch_us": fwd_s * 1e6,
+                        "forward_kernel": {"kernel": "k_res_fwd", "launch_us": fwd_s * 1e6,
                                            "achieved": 16 * sum(npads) / fwd_s / 1e9}},
            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(out), flush=True)
@@ -726,8 +726,8 @@ def run_fwi(args, rank, world):
     value = upd * args.steps / el / 1e9
     nint = w.nx * w.nz
     rev_bytes = 28 * w.npad + 8 * nint        # gradient mode: num += pbar x increment
-    # shots run concurrently (one stream each): launch time = phase time per
-    # launch of one shot's loop, i.e. the launches of all shots share the phase
+    # shots run concurrently (one stream each): time per step = phase time per
+    # step of one shot's loop, i.e. the steps of all shots share the phase
     rev_launch_s = t_b / (len(srcs) * (w.nt + 1))
     fwd_launch_s = t_f / (len(srcs) * w.nt)
     peaks = measured_peaks()
@@ -772,12 +772,12 @@ def run_fwi(args, rank, world):
                       "s_per_gradient": t_grad, "forward_phase_s": t_f, "backward_phase_s": t_b,
                       "shot_streams": shot_streams(g, len(srcs)), "misfit": float(J.detach()),
                       "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB write)"},
-           "roofline": {"bound": "hbm", "kernel": "k_rev2d_tile<2, 4, 7, true> (reconstruction + exact adjoint + gradient; "
-                                                  "shots on concurrent streams: backward phase / launches)",
+           "roofline": {"bound": "hbm", "kernel": "k_res_rev in gradient mode (reconstruction + exact adjoint + gradient; "
+                                                  "shots on concurrent streams: backward phase / time steps)",
                         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                         "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
                         "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_launch_s * 1e6,
-                        "forward_kernel": {"kernel": "k_fwd2d", "launch_us": fwd_launch_s * 1e6,
+                        "forward_kernel": {"kernel": "k_res_fwd", "launch_us": fwd_launch_s * 1e6,
                                            "achieved": 16 * w.npad / fwd_launch_s / 1e9}},
            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(out), flush=True)
@@ -1033,21 +1033,21 @@ def main():
     rev_launch_s = phases["rev_ms"] / 1e3 / max(phases["rev_launches"], 1)
     achieved = rev_bytes_per_launch(w) / rev_launch_s / 1e9
     fwd_launch_s = phases["fwd_ms"] / 1e3 / max(phases["fwd_launches"], 1)
-    kname = "k_rev2d_tile" if w.ndim == 2 else "k_rev3d_tma"
+    kname = "k_res_rev" if w.ndim == 2 else "k_rev3d_tma"
     roofline = {"bound": "hbm", "kernel": f"{kname} (fused reverse pass)", "achieved": achieved, "peak": peak,
                 "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s",
                 "traffic": (reverse_traffic(w.ndim, rev_bytes_per_launch(w))
                             if w.ndim == 3 or tuple(w.padded) == (871, 2421) else None),
-                "traffic_source": ("ncu dram bytes of k_rev2d_tile on this grid, warm L2" if w.ndim == 2 else
+                "traffic_source": ("ncu dram bytes of k_res_rev's loop on this grid, per step" if w.ndim == 2 else
                                    "ncu dram bytes of k_rev3d_tma on 380x380x280, scaled by the algorithmic bytes"),
                 "bytes_per_launch": rev_bytes_per_launch(w), "launch_us": rev_launch_s * 1e6,
-                "forward_kernel": {"kernel": "k_fwd2d" if w.ndim == 2 else "k_fwd3d_tma",
+                "forward_kernel": {"kernel": "k_res_fwd" if w.ndim == 2 else "k_fwd3d_tma",
                                    "achieved": fwd_bytes_per_launch(w) / fwd_launch_s / 1e9,
                                    "launch_us": fwd_launch_s * 1e6,
                                    "bytes_per_launch": fwd_bytes_per_launch(w)},
-                "note": ("one shot's working set (about 56 MB) is L2-resident during its time loop, "
-                         "so achieved can exceed the HBM copy bandwidth") if w.ndim == 2 else
+                "note": ("one launch per time loop, the fields on the chip: bytes and time are per time step, "
+                         "the kernel is bound by fp32 issue, not by HBM") if w.ndim == 2 else
                         "working set of 4 GB: DRAM-bound"}
 
     if storage:
@@ -1055,7 +1055,7 @@ def main():
         fb, rb = storage_phase_bytes(w, stride)
         fwd_s, rev_s = phases["fwd_ms"] / 1e3 / nshots_ph, phases["rev_ms"] / 1e3 / nshots_ph
         achieved = (fb + rb) / (fwd_s + rev_s) / 1e9
-        roofline = {"bound": "hbm", "kernel": "k_fwd2d/k_fwd3d_tma steps + store/image kernels (whole phases)",
+        roofline = {"bound": "hbm", "kernel": "k_res_fwd/k_res_rev loops or k_fwd3d_tma steps + store/image kernels (whole phases)",
                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": roofline["peak_source"], "traffic": None,
                     "forward_phase": {"bytes": fb, "s": fwd_s, "GB/s": fb / fwd_s / 1e9},
