@@ -21,8 +21,8 @@
 // 0.69 us for every ten-row warp on a scheduler (143 clocks per row; 59 packed
 // operations take 118), so a survey tile (11 warps) 2.9 us, and the exchange
 // adds 0.5 us; on small grids the fixed part and the exchange are all there
-// is.  Measured (us per step; before, one launch per step): survey forward 3.6
-// (6.1), forward + reverse 11.2 (18.8); 300 x 300 forward 1.5 (2.7), forward +
+// is.  Measured (us per step; before, one launch per step): survey forward 3.4
+// (6.1), forward + reverse 10.9 (18.8); 300 x 300 forward 1.5 (2.7), forward +
 // reverse 4.5 (6.7).  Tensor memory for a and the sums: 8 us per reverse step
 // against 12.4 with the sums in registers (spilled) and a read from L2 twice.
 // Tried and not kept: a warp-to-warp order (mbarriers) instead of the block

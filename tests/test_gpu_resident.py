@@ -13,7 +13,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 # (kernel variant by rows per warp: 1, 2, 4, 7, 10; warps per block), None: the plan's own choice
-TILES = [None, "0,4", "0,8", "1,3", "1,8", "2,1", "2,3", "3,2", "4,2"]
+TILES = [None, "0,4", "0,8", "0,16", "1,3", "1,8", "1,16", "2,1", "2,3", "3,2", "4,2"]
 GRIDS = [("ragged", 150, 37, 9, 301), ("narrow", 1, 30, 4, 200), ("flat", 261, 1, 4, 150), ("edge", 120, 24, 4, 250)]
 
 
@@ -82,6 +82,35 @@ def test_a_shared_device_gives_the_same_results():
             R.rbc_set_share(ctx, 0)
     finally:
         R.rbc_destroy(ctx)
+
+
+def test_loops_of_several_streams_that_do_not_fit_together():
+    # three loops of 114 blocks and two of a few, each on its own stream, queued at once and twice over: on 152 SMs
+    # the large ones have to follow one another, whichever of them the small ones run beside (a cooperative launch
+    # starts as a whole or not at all, so that none of them waits half resident)
+    import paper_2204_03380_gb300 as R
+    runs = []
+    for k, (n, nt) in enumerate([(280, 700), (280, 300), (40, 900), (280, 500), (90, 200)]):
+        w, v, src, rec, wav = case_2d(f"flight{k}", n, n, 10, nt, seed=k)
+        g, a, _ = gpu_build(R, torch, w, v)
+        wt = torch.tensor(np.asarray(wav, np.float32), device="cuda")
+        runs.append((R.rbc_create(g, a), src, wt, rec, [torch.zeros((len(rec), nt + 1), device="cuda") for _ in range(3)],
+                     torch.cuda.Stream()))
+    try:
+        for c, src, wt, rec, out, _ in runs:
+            R.rbc_model(c, src, wt, rec, out[0])
+        torch.cuda.synchronize()
+        for i in (1, 2):
+            for c, src, wt, rec, out, s in runs:
+                R.rbc_model(c, src, wt, rec, out[i], stream=s)
+        torch.cuda.synchronize()
+        for c, src, wt, rec, out, _ in runs:
+            R.rbc_model(c, src, wt, rec, torch.empty_like(out[0]))   # (an earlier wait that ran out would be reported)
+            assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    finally:
+        torch.cuda.synchronize()
+        for r in runs:
+            R.rbc_destroy(r[0])
 
 
 def test_a_capturing_stream_is_refused():
