@@ -19,8 +19,8 @@
 // (mma.sync m16n8k16, the 9 taps padded to K = 16): as its own kernel in the
 // training forward (its output is kept for the backward pass), inside the
 // second layer's kernel for inference.  The weight gradients of
-// the 32 -> 32 layers run on tcgen05 too (one MMA per 16 pixels covers all
-// nine taps); those of the one-channel end layers on mma.sync with the taps
+// the 32 -> 32 layers run on tcgen05 too (four rows of one operand against two
+// of the other per MMA); those of the one-channel end layers on mma.sync with the taps
 // on M.  Persistent blocks add their sums to the fp32 gradient once each.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -465,10 +465,12 @@ __device__ __forceinline__ void stm_x4(uint32_t sa, uint32_t r0, uint32_t r1, ui
 // prefetched a tile ahead into registers, rounded to bf16) is parked in
 // shared memory, and each 16 pixels of a halo row are one m16n8k16 MMA per 8
 // channels as in k_conv_1to32 (taps padded to K = 16, bias as the
-// accumulator's start, relu and rounding in one conversion), stored as
-// 4-byte pieces of the pixels' 16-byte channel groups at constant offsets
-// from the row's base; outside the image the stage holds zeros (the second
-// layer's padding).  The builders then make their writes visible to the
+// accumulator's start, relu and rounding in one conversion), stored by
+// stmatrix as rows of 16 bytes (a pixel's channel group); 64 pixels' operands are
+// gathered ahead, and two parked halos leave one barrier per tile.  Outside
+// the image the stage holds zeros (the second
+// layer's padding).  These warps bound the fused layers: mma.sync and tcgen05
+// take turns on the tensor pipe (32 x 512^2: 235 us; 175 without the mma.sync).  The builders then make their writes visible to the
 // tensor cores and arrive on the stage's "full" barrier.  The first layer's
 // output never passes through global memory.
 constexpr int tc_nprod(int mode, int R) { return mode == kFused ? R + 2 : 1; }
@@ -912,13 +914,11 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t *r, const void *smem_row) {
 // pixel and have accumulators of their own:
 //   D_dx[32 j + co][32 i + ci] = sum dz[co][row y - 1 + j][px] x[ci][row y + i][px + dx - 1],
 // the tap dy = 2 + i - j for j - i in 0..2; the two other row pairs are not used.
-// (x on M and dz on N reads x's unaligned starts twice as often.)
 // Three stages: warp 4 copies, one thread of warp 5 issues the MMAs, warps 0-3 (one
 // channel group each) sum dz over the tile's own rows for db.  At the end warps 0-3 add
 // the two row pairs of each tap in shared memory and the block adds
-// them to dW, once.  Bound by the operands' shared-memory reads (6 KB per MMA, 66
-// cycles; x's starts are not on 128 bytes) and DRAM together: 8 x 512^2 takes
-// 49 us (268 MB: 5.5 TB/s) where staging through registers into swizzled
+// them to dW, once.  Bound by DRAM and, close behind, the operands' shared-memory reads
+// (6 KB per MMA, 48 cycles): 8 x 512^2 takes 46 us (268 MB: 5.8 TB/s) where staging through registers into swizzled
 // pixel-major rows, with two block barriers a tile, took 95.
 // Every wait is bounded; a block that gives up flags the error word.
 constexpr int kWtR = 8, kWtC = 64, kWtXP = kWtC + 2;        // x rows, pixels per row, staged x pixels per row
