@@ -447,6 +447,14 @@ __device__ __forceinline__ void tm_st4(uint32_t ta, const float4 v) {
                "f"(v.w)
                : "memory");
 }
+// st4 to shared memory where `on`, as one predicated store: the lanes of a warp do not part at it, so that the
+// whole-warp (.sync.aligned) accesses of the next row need no __syncwarp (one per row cost the survey's reverse
+// loop 3 %).  Not ordered against other shared-memory accesses by itself: every reader of the row is behind a
+// __syncwarp or __syncthreads, and the thread's own earlier load of the place feeds the stored value.
+__device__ __forceinline__ void st4_if(bool on, float *p, const float4 v) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %0, 0;\n@q st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n}" ::"r"((uint32_t)on),
+               "r"((uint32_t)__cvta_generic_to_shared(p)), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+}
 // Wait for this thread's tensor-memory loads; the loaded values are used after it only.
 __device__ __forceinline__ void tm_wait(float4 &a) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(a.x), "+f"(a.y), "+f"(a.z), "+f"(a.w)::"memory");
@@ -455,6 +463,7 @@ __device__ __forceinline__ void tm_tie(float4 &a) { asm volatile("" : "+f"(a.x),
 
 // Large tiles: a and the sums in tensor memory, used as a thread-private store
 // (a warp reaches the 32 lanes of its quarter; 12 columns per row: a, num, den).
+// Its accesses are the whole warp's: the lanes are together before a sweep and do not part in its rows.
 template <int RZ, int MODE>
 struct KeepTm {
   static constexpr bool kGrad = MODE == 1;
@@ -613,7 +622,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
                            }
                          }
                          keep.add(j, kGrad ? inc : c, cb);
-                         if (xok) st4(smem + rn0 + own + j * kTileX, v);
+                         st4_if(xok, smem + rn0 + own + j * kTileX, v);
                        });
       keep.flush();
     } else if (kStore) {
@@ -652,12 +661,14 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
       float *bc = smem + bc0, *bn = smem + bn0;
       if (t > 0)  // level nt is zero everywhere
         ok = halo_in<RZ, TIGHT>(W, FB, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
+      else
+        __syncwarp();
       sweep<RZ, TIGHT>(W, smem, bc0, bn0, bc + W.r0 * kTileX - 4 * kTileX,
                        TIGHT && last ? s_x : bc + (W.r0 + RZ) * kTileX, top, qa, lofs, lstep, rofs, rstep,
                        [&](int j) { keep.pre_a(j); },
                        [&](int j, const float4 c, const float4 po, const float4 lap) {
                          const float4 v = leap_fin<false>(c, po, keep.a(j), lap, nullptr);
-                         if (xok) st4(bn + own + j * kTileX, v);
+                         st4_if(xok, bn + own + j * kTileX, v);
                        });
       __syncwarp();
       if (rec.end > rec.beg) {
@@ -685,6 +696,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
   for (int j = 0; j < RZ; ++j) {
     const int z = T.z0 + W.r0 + j;
     float4 n4, d4;
+    __syncwarp();  // (the row before ended with lanes that had nothing to write)
     keep.sums(j, n4, d4);
     if (!ok || W.r0 + j >= W.rows || z < S.iz0 || z >= S.iz1) continue;
 #pragma unroll
