@@ -136,8 +136,8 @@ int rbc_set_coef(rbc_ctx *ctx, const float *a_dev, int check, void *stream);
  * the same time on their own streams (1 at creation): its 2-D time loops then
  * take that share of the device each, so that the contexts' loops run side by
  * side instead of one after the other.  Results do not depend on it.
- * Synchronises the device when the number changes.
- * Errors: RBC_EINVAL (NULL, contexts < 1), RBC_ENOMEM, RBC_ECUDA.
+ * Applies to the calls that follow; allocates nothing and waits for nothing.
+ * Errors: RBC_EINVAL (NULL, contexts < 1).
  */
 int rbc_set_share(rbc_ctx *ctx, int contexts);
 
@@ -471,7 +471,10 @@ int rbc_model_static(const rbc_grid *g, const float *a_dev,
  * and the next call on the context returns RBC_ETIMEOUT (the results of the
  * faulted call are invalid).  Nothing faults, traps or hangs.  mode 0
  * clears a pending request.  With ctx = NULL the request applies to the next
- * 3-D rbc_model_static call instead (reported by the call after it).
+ * 3-D rbc_model_static call instead (reported by the call after it).  mode 3
+ * (ctx = NULL): the next rbc_create or rbc_batch_create of a 2-D grid finds no
+ * memory for the tables of its one-launch time loops and, as it would then,
+ * steps with one launch per step instead; mode 0 or 1 with NULL clears it.
  * Errors: RBC_EINVAL, RBC_ENOTSUP (2-D context).
  */
 int rbc_inject_fault(rbc_ctx *ctx, int mode);

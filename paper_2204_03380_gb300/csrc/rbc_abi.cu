@@ -3,11 +3,13 @@
 // per-shot tables, and the time loops of Algorithms 1 and 3 issued either as
 // plain launches or as one captured CUDA graph per context and loop kind.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -129,10 +131,9 @@ struct rbc_ctx {
   int fault = 0;  // rbc_inject_fault: applies to the next call only
   // 2-D grids that fit on the chip: the whole time loop as one launch
   // (rbc_resident.cu), by kResFwd .. kResStore (variant -1: one launch per step)
-  ResPlan res[3];
-  ResTile *res_tiles[3] = {nullptr, nullptr, nullptr};
-  unsigned long long *res_ll = nullptr;
-  char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, receiver cells
+  std::map<int, std::array<ResPlan, 3>> res;  // the plans of every share seen (host tables)
+  unsigned long long *res_ll = nullptr;       // room for the exchange words of any of them (null: no resident loops)
+  char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, tiles, receiver cells
   size_t res_blob_cap = 0;
   int share = 1;             // contexts in flight at once (rbc_set_share)
 };
@@ -241,21 +242,34 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
   return RBC_OK;
 }
 
-// Whether this call's loop (kResFwd ..) runs as one resident launch.
-bool resident(const rbc_ctx *c, int dir) {
-  return c->res[dir].variant >= 0 && c->snap.empty() && (dir != kResFwd || c->levels_per_launch == 1);
+// The plan of a resident loop (kResFwd ..) for the context's share of the device; null: one launch per step.
+const ResPlan *res_plan_of(rbc_ctx *c, int dir) {
+  if (!c->res_ll) return nullptr;
+  auto it = c->res.find(c->share);
+  if (it == c->res.end()) {
+    if (c->res.size() >= 8) c->res.clear();
+    it = c->res.emplace(c->share, std::array<ResPlan, 3>()).first;
+    for (int d = 0; d < 3; ++d) res_plan(&c->L, 1, d, c->share, &it->second[d]);
+  }
+  return it->second[dir].variant >= 0 ? &it->second[dir] : nullptr;
+}
+
+// The same for this call: null also with snapshots, or where the forward loop advances two levels per launch.
+const ResPlan *resident(rbc_ctx *c, int dir) {
+  return c->snap.empty() && (dir != kResFwd || c->levels_per_launch == 1) ? res_plan_of(c, dir) : nullptr;
 }
 
 // Tables of a resident loop (one copy to the device) and its launch.  The
 // receivers are sorted by the warp that owns their rows; num / den are the
 // reverse loop's outputs.
-int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, int reinject, int sample, int grad,
-                 int overwrite, int dense, float *num, float *den, cudaStream_t s, int stride = 0) {
-  const ResPlan &P = c->res[dir];
+int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec, const int *rec, int reinject,
+                 int sample, int grad, int overwrite, int dense, float *num, float *den, cudaStream_t s,
+                 int stride = 0) {
   const Lay &L = c->L;
   const int cells = P.blocks * P.warps;
   auto up = [](size_t n) { return (n + 63) / 64 * 64; };
-  const size_t o_shot = 64, o_ptr = o_shot + up(sizeof(ResShot)), o_rec = o_ptr + up(sizeof(int) * (cells + 1)),
+  const size_t tb = sizeof(ResTile) * P.tiles.size(), o_shot = 64, o_tile = o_shot + up(sizeof(ResShot)),
+               o_ptr = o_tile + up(tb), o_rec = o_ptr + up(sizeof(int) * (cells + 1)),
                need = o_rec + up(sizeof(int2) * nrec);
   static_assert(sizeof(ShotInfo) <= 64, "the shot's info precedes its table");
   if (need > c->res_blob_cap) {
@@ -268,6 +282,7 @@ int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, 
   std::vector<char> blob(need, 0);
   const ShotInfo info = shot_info(c, src, nrec, reinject);
   std::memcpy(blob.data(), &info, sizeof info);
+  std::memcpy(blob.data() + o_tile, P.tiles.data(), tb);
   int *ptr = reinterpret_cast<int *>(blob.data() + o_ptr);
   int2 *cr = reinterpret_cast<int2 *>(blob.data() + o_rec);
   res_cells(P, L, cells, nrec, rec, 0, ptr, cr);
@@ -289,7 +304,7 @@ int run_resident(rbc_ctx *c, int dir, const int *src, int nrec, const int *rec, 
   std::memcpy(blob.data() + o_shot, &S, sizeof S);
   CK(cudaMemcpyAsync(c->res_blob, blob.data(), need, cudaMemcpyHostToDevice, s));
   ResArgs A{};
-  A.tiles = c->res_tiles[dir];
+  A.tiles = reinterpret_cast<const ResTile *>(c->res_blob + o_tile);
   A.shots = reinterpret_cast<const ResShot *>(c->res_blob + o_shot);
   A.ll = c->res_ll;
   A.wav = c->wav;
@@ -484,24 +499,17 @@ int enqueue_reverse(rbc_ctx *c, cudaStream_t s) {
   return RBC_OK;
 }
 
-// Plans and tables of the resident loops of a 2-D context.
-int create_resident(rbc_ctx *c) {
-  if (c->L.ndim != 2) return RBC_OK;
-  size_t ll = 0;
-  cudaFree(c->res_ll);
-  c->res_ll = nullptr;
-  for (int dir = 0; dir < 3; ++dir) {
-    cudaFree(c->res_tiles[dir]);
-    c->res_tiles[dir] = nullptr;
-    ResPlan &P = c->res[dir];
-    if (!res_plan(&c->L, 1, dir, c->share, &P)) continue;
-    const size_t tb = sizeof(ResTile) * P.tiles.size();
-    CK(cudaMalloc(&c->res_tiles[dir], tb));
-    CK(cudaMemcpy(c->res_tiles[dir], P.tiles.data(), tb, cudaMemcpyHostToDevice));
-    ll = std::max(ll, res_ll_bytes(P, dir));
+// Room for the exchange words of a 2-D context's resident loops, whatever its share; where there is none the
+// context steps with one launch per step.
+void create_resident(rbc_ctx *c) {
+  if (c->L.ndim != 2) return;
+  int nf = 0;
+  for (int dir = 0; dir < 3; ++dir)
+    if (res_plan(&c->L, 1, dir, 1, &c->res[1][dir])) nf = std::max(nf, dir == kResRev ? 2 : 1);
+  if (nf && res_malloc((void **)&c->res_ll, res_ll_bound(c->L, nf)) != cudaSuccess) {
+    c->res_ll = nullptr;
+    cudaGetLastError();
   }
-  if (ll) CK(cudaMalloc(&c->res_ll, ll));
-  return RBC_OK;
 }
 
 typedef int (*enqueue_fn)(rbc_ctx *, cudaStream_t, int);
@@ -689,12 +697,12 @@ int run_loop(rbc_ctx *c, int kind, enqueue_fn fn, cudaStream_t s) {
 
 // Algorithm 1 with the record at the receivers (time-major, in c->seis_t).
 int run_model(rbc_ctx *c, const int *src, int nrec, const int *rec, const float *wavelet, cudaStream_t s) {
-  const bool res = resident(c, 0);
+  const ResPlan *res = resident(c, kResFwd);
   int rc = res ? check_nodes(c, src, nrec, rec) : upload_shot(c, src, nrec, rec, 1, s);
   if (rc) return rc;
   if (res && ((rc = check_capture(s)) || (rc = ensure_receivers(c, std::max(nrec, 1))))) return rc;
   CK(cudaMemcpyAsync(c->wav, wavelet, sizeof(float) * c->g.nt, cudaMemcpyDeviceToDevice, s));
-  if (res) return run_resident(c, 0, src, nrec, rec, 1, 1, 0, 0, 0, nullptr, nullptr, s);
+  if (res) return run_resident(c, *res, kResFwd, src, nrec, rec, 1, 1, 0, 0, 0, nullptr, nullptr, s);
   return run_loop(c, 0, enq_model, s);
 }
 
@@ -807,11 +815,7 @@ int rbc_create(const rbc_grid *g, const float *a_dev, rbc_ctx **out) {
   }
   launch_copy_in(L, a_dev, c->a, 0);
   ++g_launches;
-  rc = create_resident(c);
-  if (rc) {
-    rbc_destroy(c);
-    return rc;
-  }
+  create_resident(c);
   rc = ensure_receivers(c, 64);
   if (rc) {
     rbc_destroy(c);
@@ -853,10 +857,8 @@ int rbc_set_coef(rbc_ctx *c, const float *a_dev, int check, void *stream) {
 
 int rbc_set_share(rbc_ctx *c, int contexts) {
   if (!c || contexts < 1) return fail(RBC_EINVAL, "ctx is NULL or contexts < 1");
-  if (contexts == c->share) return RBC_OK;
-  CK(cudaDeviceSynchronize());
   c->share = contexts;
-  return create_resident(c);
+  return RBC_OK;
 }
 
 int rbc_destroy(rbc_ctx *c) {
@@ -872,7 +874,6 @@ int rbc_destroy(rbc_ctx *c) {
   cudaFree(c->tile_ptr);
   cudaFree(c->seis_t);
   cudaFree(c->dmax);
-  for (ResTile *t : c->res_tiles) cudaFree(t);
   cudaFree(c->res_ll);
   cudaFree(c->res_blob);
   if (c->cap) cudaStreamDestroy(c->cap);
@@ -911,7 +912,7 @@ int rbc_rtm_shot(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int 
   int rc = check_device_error(c);
   if (rc) return rc;
   const int rein = flags & RBC_REINJECT_SOURCE, ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
-  const bool resf = resident(c, 0), resr = resident(c, 1);
+  const ResPlan *resf = resident(c, kResFwd), *resr = resident(c, kResRev);
   rc = check_nodes(c, src_host, nrec, rec_host);
   if (rc) return rc;
   if ((resf || resr) && (rc = check_capture(s))) return rc;
@@ -923,11 +924,11 @@ int rbc_rtm_shot(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int 
     ++g_launches;
   }
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = resf ? run_resident(c, 0, src_host, 0, nullptr, rein, 0, 0, 0, 0, nullptr, nullptr, s)
+  rc = resf ? run_resident(c, *resf, kResFwd, src_host, 0, nullptr, rein, 0, 0, 0, 0, nullptr, nullptr, s)
             : run_loop(c, 1, enq_rtm_fwd, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = resr ? run_resident(c, 1, src_host, nrec, rec_host, rein, 0, 0, ow, 1, num_dev, den_dev, s)
+  rc = resr ? run_resident(c, *resr, kResRev, src_host, nrec, rec_host, rein, 0, 0, ow, 1, num_dev, den_dev, s)
             : run_loop(c, 2, enq_rtm_rev, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
@@ -979,7 +980,8 @@ int rbc_rtm_storage(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
   if (rc) return rc;
   // both loops resident, or both by steps (the forward step path keeps a level with a launch of its own, whatever
   // the temporal-blocking option)
-  const bool res = c->res[kResFwd].variant >= 0 && c->res[kResStore].variant >= 0 && c->snap.empty();
+  const ResPlan *resf = res_plan_of(c, kResFwd), *ress = res_plan_of(c, kResStore);
+  const bool res = resf && ress && c->snap.empty();
   rc = check_nodes(c, src_host, nrec, rec_host);
   if (rc) return rc;
   if (res && (rc = check_capture(s))) return rc;
@@ -1000,11 +1002,11 @@ int rbc_rtm_storage(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
   }
   if (c->timing && (rc = record_event(c, s))) return rc;
   const int ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
-  rc = res ? run_resident(c, kResFwd, src_host, 0, nullptr, 0, 0, 0, 0, 0, nullptr, nullptr, s, stride)
+  rc = res ? run_resident(c, *resf, kResFwd, src_host, 0, nullptr, 0, 0, 0, 0, 0, nullptr, nullptr, s, stride)
            : run_loop(c, 4, enq_store_fwd, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
-  rc = res ? run_resident(c, kResStore, src_host, nrec, rec_host, 0, 0, 0, ow, 1, num_dev, den_dev, s, stride)
+  rc = res ? run_resident(c, *ress, kResStore, src_host, nrec, rec_host, 0, 0, 0, ow, 1, num_dev, den_dev, s, stride)
            : run_loop(c, 5, enq_store_rev, s);
   if (rc) return rc;
   if (c->timing && (rc = record_event(c, s))) return rc;
@@ -1084,7 +1086,7 @@ int rbc_fwi_backward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, 
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
-  const bool res = resident(c, 1);
+  const ResPlan *res = resident(c, kResRev);
   rc = res ? check_nodes(c, src_host, nrec, rec_host) : upload_shot(c, src_host, nrec, rec_host, 1, s);
   if (rc) return rc;
   if (res && ((rc = check_capture(s)) || (rc = ensure_receivers(c, std::max(nrec, 1))))) return rc;
@@ -1098,7 +1100,7 @@ int rbc_fwi_backward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, 
   // adjoint record: row m = -resid[.][m-1] / h^(2-d), injected as + h^(2-d) a row
   launch_fwi_adjoint_source(resid_dev, c->seis_t, nrec, nt, -1.0f, s);
   ++g_launches;
-  rc = res ? run_resident(c, 1, src_host, nrec, rec_host, 1, 0, 1, 1, 0, c->num, nullptr, s)
+  rc = res ? run_resident(c, *res, kResRev, src_host, nrec, rec_host, 1, 0, 1, 1, 0, c->num, nullptr, s)
            : run_loop(c, 3, enq_fwi_adj, s);
   if (rc) return rc;
   launch_fwi_finalize(c->L, c->num, c->a, grad_dev, c->g.nb, c->g.nx, c->g.nz, c->g.dt, c->g.h, s);
@@ -1157,7 +1159,9 @@ int rbc_phase_timing(rbc_ctx *c, int enable, double *out) {
 }
 
 int rbc_inject_fault(rbc_ctx *c, int mode) {
-  if (mode != 0 && mode != 1) return fail(RBC_EINVAL, "unknown fault mode %d", mode);
+  if (mode != 0 && mode != 1 && !(mode == 3 && !c)) return fail(RBC_EINVAL, "unknown fault mode %d", mode);
+  if (!c) res_fail_alloc(mode == 3);
+  if (mode == 3) return RBC_OK;
   if (!c) {  // the next 3-D rbc_model_static call
     static_inject_fault(mode);
     return RBC_OK;

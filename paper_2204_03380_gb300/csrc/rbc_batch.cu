@@ -879,32 +879,37 @@ int enq_rev(rbc_batch *b, int g, cudaStream_t s) {
   return RBC_OK;
 }
 
+void drop_res(rbc_batch *b) {
+  for (rbc_batch::Res &r : b->res) cudaFree(r.tiles[0]), cudaFree(r.tiles[1]);
+  b->res.clear();
+}
+
 // Groups, plans and tables of the resident loops; a batch whose shots do not
-// all fit keeps none.
-int create_res(rbc_batch *b) {
-  if (getenv("RBC_BATCH_TILES")) return RBC_OK;  // names the kernels of the step path
+// all fit, or whose tables find no memory, keeps none.
+void create_res(rbc_batch *b) {
+  if (getenv("RBC_BATCH_TILES")) return;  // names the kernels of the step path
   size_t ll = 0;
+  bool ok = true;
   for (const std::vector<int> &g : res_groups(b->L.data(), b->nshots)) {
-    rbc_batch::Res r;
+    b->res.emplace_back();
+    rbc_batch::Res &r = b->res.back();
     r.shots = g;
     std::vector<Lay> L;
     for (int i : g) L.push_back(b->L[i]);
-    for (int dir = 0; dir < 2; ++dir) {
-      if (!res_plan(L.data(), (int)L.size(), dir, 1, &r.plan[dir])) {
-        for (rbc_batch::Res &q : b->res) cudaFree(q.tiles[0]), cudaFree(q.tiles[1]);
-        cudaFree(r.tiles[0]);
-        b->res.clear();
-        return RBC_OK;
-      }
+    for (int dir = 0; ok && dir < 2; ++dir) {
+      if (!(ok = res_plan(L.data(), (int)L.size(), dir, 1, &r.plan[dir]))) break;
       const size_t tb = sizeof(ResTile) * r.plan[dir].tiles.size();
-      BCK(cudaMalloc(&r.tiles[dir], tb));
-      BCK(cudaMemcpy(r.tiles[dir], r.plan[dir].tiles.data(), tb, cudaMemcpyHostToDevice));
+      ok = res_malloc((void **)&r.tiles[dir], tb) == cudaSuccess &&
+           cudaMemcpy(r.tiles[dir], r.plan[dir].tiles.data(), tb, cudaMemcpyHostToDevice) == cudaSuccess;
       ll = std::max(ll, res_ll_bytes(r.plan[dir], dir));
     }
-    b->res.push_back(r);
+    if (!ok) break;
   }
-  if (ll) BCK(cudaMalloc(&b->res_ll, ll));
-  return RBC_OK;
+  if (ok && ll && res_malloc((void **)&b->res_ll, ll) != cudaSuccess) b->res_ll = nullptr, ok = false;
+  if (!ok) {
+    drop_res(b);
+    cudaGetLastError();
+  }
 }
 
 // The call's tables: every shot's ShotInfo, then per group the forward and
@@ -1081,10 +1086,7 @@ int rbc_batch_create(const rbc_grid *g, int nshots, const int *nx_host, const fl
       return bfail(RBC_ECFL, "rbc_batch_create: shot %d is unstable (max (v dt/h)^2 = %g)", s, am);
     }
   }
-  if (int rc = create_res(b)) {
-    rbc_batch_destroy(b);
-    return rc;
-  }
+  create_res(b);
   const int nf = b->res.empty() ? 7 : 5;  // the resident loops keep the receiver wavefield on the chip
   total *= nf;
   if (cudaMalloc(&b->arena, sizeof(float) * total) != cudaSuccess || cudaMemset(b->arena, 0, sizeof(float) * total) ||
@@ -1172,7 +1174,7 @@ int rbc_batch_destroy(rbc_batch *b) {
   cudaFree(b->d_tile_rec);
   cudaFree(b->d_seis_t);
   cudaFree(b->d_wav);
-  for (rbc_batch::Res &r : b->res) cudaFree(r.tiles[0]), cudaFree(r.tiles[1]);
+  drop_res(b);
   cudaFree(b->res_ll);
   cudaFree(b->res_blob);
   if (b->cap) cudaStreamDestroy(b->cap);

@@ -33,6 +33,7 @@
 // against 3.4: the wait is not what bounds a step); 16 warps of 7 rows instead
 // of 11 of 10 (the same).
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -837,6 +838,26 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
 size_t res_ll_bytes(const ResPlan &P, int dir) {
   return sizeof(u64) * (size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H);
 }
+
+size_t res_ll_bound(const Lay &L, int nf) {
+  int dev = 0, sms = 0, hmax = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (const Variant &V : kVariants) hmax = std::max(hmax, V.maxw * V.rz);
+  const long long gx = cdiv(L.NX, kTileX), blocks = std::min((long long)sms, gx * cdiv(L.NZ, 4));
+  // ll_words(H) per block, and blocks * H <= gx * (NZ + H - 1)
+  return sizeof(u64) * nf * 2 * (size_t)(blocks * 2 * kEdge + 8 * gx * (L.NZ + hmax - 1));
+}
+
+namespace {
+std::atomic<bool> g_fail_alloc{false};
+}
+
+cudaError_t res_malloc(void **p, size_t bytes) {
+  return g_fail_alloc.exchange(false) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+
+void res_fail_alloc(bool on) { g_fail_alloc = on; }
 
 void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc) {
   const int t = (z / P.H) * cdiv(L.NX, kTileX) + x / kTileX, r = z % P.H;

@@ -66,6 +66,12 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out);
 // indices, or none when a shot does not fit.
 std::vector<std::vector<int>> res_groups(const Lay *L, int nshots);
 size_t res_ll_bytes(const ResPlan &P, int dir);
+// At least res_ll_bytes of any plan of this grid alone, for loops of nf fields.
+size_t res_ll_bound(const Lay &L, int nf);
+// cudaMalloc for the loops' own tables, without which a context or batch takes the step path; res_fail_alloc(true)
+// makes the next one fail (rbc_inject_fault).
+cudaError_t res_malloc(void **p, size_t bytes);
+void res_fail_alloc(bool on);
 // The (tile, warp) cell that owns a node, within its shot's tiles, and the
 // node's place in the tile.
 void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc);

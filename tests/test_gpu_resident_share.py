@@ -1,0 +1,82 @@
+"""Contexts that share the device: rbc_set_share, and contexts or batches
+whose loops' tables find no memory."""
+import numpy as np
+import pytest
+
+from rtm_cases import case_2d, gpu_build
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(R, name, nx, nz, nb, nt, seed=0):
+    w, v, src, rec, wav = case_2d(name, nx, nz, nb, nt, seed=seed)
+    g, a, _ = gpu_build(R, torch, w, v)
+    wt = torch.tensor(np.asarray(wav, np.float32), device="cuda")
+    return R.rbc_create(g, a), g, a, src, rec, wt, torch.zeros((len(rec), nt + 1), device="cuda")
+
+
+def test_a_change_of_share_waits_for_nothing_and_allocates_nothing():
+    import paper_2204_03380_gb300 as R
+    long, _, _, src, rec, wt, out = _ctx(R, "long", 300, 300, 50, 30000)   # some 50 ms
+    other, _, _, src2, rec2, wt2, out2 = _ctx(R, "other", 400, 300, 50, 60)
+    try:
+        R.rbc_model(long, src, wt, rec, out)
+        for n in (2, 5, 3):   # (kernels are loaded at their first launch)
+            R.rbc_set_share(other, n)
+            R.rbc_model(other, src2, wt2, rec2, out2)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        R.rbc_model(long, src, wt, rec, out)
+        done = torch.cuda.Event()
+        done.record()
+        for n in (2, 5, 1, 3):
+            R.rbc_set_share(other, n)
+        assert not done.query()                       # the loop is still running: nothing waited for it
+        R.rbc_model(other, src2, wt2, rec2, out2)     # with tables of another share
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+    finally:
+        torch.cuda.synchronize()
+        R.rbc_destroy(long)
+        R.rbc_destroy(other)
+
+
+def test_a_context_whose_tables_find_no_memory_steps():
+    import paper_2204_03380_gb300 as R
+    runs = []
+    for mode in (0, 3):
+        R.rbc_inject_fault(None, mode)
+        ctx, _, _, src, rec, wt, out = _ctx(R, "nomem", 150, 60, 10, 120)
+        try:
+            for n in (1, 4):
+                R.rbc_set_share(ctx, n)
+                R.rbc_launch_count(True)
+                R.rbc_model(ctx, src, wt, rec, out)
+                torch.cuda.synchronize()
+                assert (R.rbc_launch_count() > 120) == (mode == 3)
+        finally:
+            R.rbc_destroy(ctx)
+        runs.append(out.cpu())
+    assert torch.equal(*runs) and float(runs[0].abs().max()) > 0
+
+
+def test_a_batch_whose_tables_find_no_memory_steps():
+    import paper_2204_03380_gb300 as R
+    c0, g, a, src, rec, wt, seis = _ctx(R, "bnomem", 150, 60, 10, 120)
+    R.rbc_model(c0, src, wt, rec, seis)
+    R.rbc_destroy(c0)
+    imgs = []
+    for mode in (0, 3):
+        R.rbc_inject_fault(None, mode)
+        b = R.rbc_batch_create(g, [150], [a])
+        try:
+            img = torch.zeros(g.interior, device="cuda")
+            R.rbc_launch_count(True)
+            R.rbc_batch_rtm(b, [dict(src=src, rec=rec, seis=seis, off_x=0)], wt, R.RBC_REINJECT_SOURCE, 1e-2, img)
+            torch.cuda.synchronize()
+            assert (R.rbc_launch_count() > 120) == (mode == 3)
+        finally:
+            R.rbc_batch_destroy(b)
+        imgs.append(img)
+    assert float((imgs[0] - imgs[1]).norm()) <= 1e-5 * float(imgs[0].norm()) and float(imgs[0].norm()) > 0
