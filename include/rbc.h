@@ -133,9 +133,11 @@ int rbc_set_coef(rbc_ctx *ctx, const float *a_dev, int check, void *stream);
 
 /*
  * rbc_set_share -- tell a context that `contexts` contexts of its kind run at
- * the same time on their own streams (1 at creation): its 2-D time loops then
- * take that share of the device each, so that the contexts' loops run side by
- * side instead of one after the other.  Results do not depend on it.
+ * the same time on their own streams: its 2-D time loops are then planned for
+ * the time of all of them -- side by side on a part of the device each, one
+ * after the other, or by one launch per step, whichever is through first.
+ * Results do not depend on it.  Until it is called, a context counts those
+ * that were called on other streams since its own last call.
  * Applies to the calls that follow; allocates nothing and waits for nothing.
  * Errors: RBC_EINVAL (NULL, contexts < 1).
  */

@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -131,11 +132,14 @@ struct rbc_ctx {
   int fault = 0;  // rbc_inject_fault: applies to the next call only
   // 2-D grids that fit on the chip: the whole time loop as one launch
   // (rbc_resident.cu), by kResFwd .. kResStore (variant -1: one launch per step)
-  std::map<int, std::array<ResPlan, 3>> res;  // the plans of every share seen (host tables)
+  std::map<int, std::array<ResPlan, 3>> res;  // the plans, by `loops` (host tables)
   unsigned long long *res_ll = nullptr;       // room for the exchange words of any of them (null: no resident loops)
   char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, tiles, receiver cells
   size_t res_blob_cap = 0;
-  int share = 1;             // contexts in flight at once (rbc_set_share)
+  int share = 0;             // contexts in flight at once as the caller says (rbc_set_share; 0: counted)
+  int loops = 1;             // contexts in flight with this call
+  unsigned long long called = 0, on_stream = 0;  // this context's last counted call (0: none yet) and its stream
+  unsigned long long born = 0;                   // calls counted before its creation
 };
 
 namespace {
@@ -242,14 +246,62 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
   return RBC_OK;
 }
 
-// The plan of a resident loop (kResFwd ..) for the context's share of the device; null: one launch per step.
+// The 2-D contexts with resident loops that are alive, and the number of their calls so far.
+struct Flight {
+  std::mutex m;
+  std::vector<rbc_ctx *> live;
+  unsigned long long calls = 0;
+};
+Flight &flight() {
+  static Flight *f = new Flight();  // (outlives contexts destroyed at exit)
+  return *f;
+}
+
+// Contexts whose loops may run beside this call's, itself included: those called on other streams since its own last
+// call.  A program that runs k contexts on k streams calls the others in between; one that uses its contexts in turn
+// on one stream, or one context at a time, is counted as one.  At its first call (on a stream of the caller's making)
+// contexts that have not been called yet count too, so that a first round of calls runs side by side as well.
+// Nothing but the plan depends on the count.
+int count_loops(rbc_ctx *c, cudaStream_t s) {
+  unsigned long long id = 0;
+  if (!c->res_ll || cudaStreamGetId(s, &id) != cudaSuccess) return 1;
+  Flight &f = flight();
+  std::lock_guard<std::mutex> lock(f.m);
+  std::vector<unsigned long long> seen(1, id);
+  int n = 1;
+  for (const rbc_ctx *x : f.live) {
+    if (x == c || x->dev != c->dev) continue;
+    if (!x->called) {
+      n += !c->called && s != nullptr && s != cudaStreamLegacy;
+    } else if (x->called > std::max(c->called, c->born) &&
+               std::find(seen.begin(), seen.end(), x->on_stream) == seen.end()) {
+      seen.push_back(x->on_stream);
+      ++n;
+    }
+  }
+  c->called = ++f.calls;
+  c->on_stream = id;
+  return n;
+}
+
+// At the start of a call that runs a loop.  (On a capturing stream, where the call is refused further on, nothing is
+// asked of the runtime that would end the capture.)
+void begin_loops(rbc_ctx *c, cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  c->loops = 1;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return;
+  const int n = count_loops(c, s);
+  c->loops = c->share ? c->share : n;
+}
+
+// The plan of a resident loop (kResFwd ..) beside the loops in flight; null: one launch per step.
 const ResPlan *res_plan_of(rbc_ctx *c, int dir) {
   if (!c->res_ll) return nullptr;
-  auto it = c->res.find(c->share);
+  auto it = c->res.find(c->loops);
   if (it == c->res.end()) {
     if (c->res.size() >= 8) c->res.clear();
-    it = c->res.emplace(c->share, std::array<ResPlan, 3>()).first;
-    for (int d = 0; d < 3; ++d) res_plan(&c->L, 1, d, c->share, &it->second[d]);
+    it = c->res.emplace(c->loops, std::array<ResPlan, 3>()).first;
+    for (int d = 0; d < 3; ++d) res_plan_shared(&c->L, d, c->loops, &it->second[d]);
   }
   return it->second[dir].variant >= 0 ? &it->second[dir] : nullptr;
 }
@@ -272,12 +324,14 @@ int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec
                o_ptr = o_tile + up(tb), o_rec = o_ptr + up(sizeof(int) * (cells + 1)),
                need = o_rec + up(sizeof(int2) * nrec);
   static_assert(sizeof(ShotInfo) <= 64, "the shot's info precedes its table");
+  // room for any plan's tables and as many receivers as the record has: grows with the receivers only
+  const size_t most = std::max(need, (size_t)(32 << 10) + sizeof(int2) * c->rec_cap);
   if (need > c->res_blob_cap) {
     cudaFree(c->res_blob);  // waits for the work that reads it
     c->res_blob = nullptr;
     c->res_blob_cap = 0;
-    CK(cudaMalloc(&c->res_blob, 2 * need));
-    c->res_blob_cap = 2 * need;
+    CK(cudaMalloc(&c->res_blob, most));
+    c->res_blob_cap = most;
   }
   std::vector<char> blob(need, 0);
   const ShotInfo info = shot_info(c, src, nrec, reinject);
@@ -697,6 +751,7 @@ int run_loop(rbc_ctx *c, int kind, enqueue_fn fn, cudaStream_t s) {
 
 // Algorithm 1 with the record at the receivers (time-major, in c->seis_t).
 int run_model(rbc_ctx *c, const int *src, int nrec, const int *rec, const float *wavelet, cudaStream_t s) {
+  begin_loops(c, s);
   const ResPlan *res = resident(c, kResFwd);
   int rc = res ? check_nodes(c, src, nrec, rec) : upload_shot(c, src, nrec, rec, 1, s);
   if (rc) return rc;
@@ -816,15 +871,16 @@ int rbc_create(const rbc_grid *g, const float *a_dev, rbc_ctx **out) {
   launch_copy_in(L, a_dev, c->a, 0);
   ++g_launches;
   create_resident(c);
-  rc = ensure_receivers(c, 64);
-  if (rc) {
-    rbc_destroy(c);
-    return rc;
-  }
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     rbc_destroy(c);
     return fail(RBC_ECUDA, "create: %s", cudaGetErrorString(e));
+  }
+  if (c->res_ll) {
+    Flight &f = flight();
+    std::lock_guard<std::mutex> lock(f.m);
+    c->born = f.calls;
+    f.live.push_back(c);
   }
   *out = c;
   return RBC_OK;
@@ -863,6 +919,11 @@ int rbc_set_share(rbc_ctx *c, int contexts) {
 
 int rbc_destroy(rbc_ctx *c) {
   if (!c) return RBC_OK;
+  {
+    Flight &f = flight();
+    std::lock_guard<std::mutex> lock(f.m);
+    f.live.erase(std::remove(f.live.begin(), f.live.end(), c), f.live.end());
+  }
   cudaDeviceSynchronize();
   const int pending = check_device_error(c);
   drop_graphs(c);
@@ -912,6 +973,7 @@ int rbc_rtm_shot(rbc_ctx *c, const int *src_host, const float *wavelet_dev, int 
   int rc = check_device_error(c);
   if (rc) return rc;
   const int rein = flags & RBC_REINJECT_SOURCE, ow = (flags & RBC_ZERO_FIRST) ? 1 : 0;
+  begin_loops(c, s);
   const ResPlan *resf = resident(c, kResFwd), *resr = resident(c, kResRev);
   rc = check_nodes(c, src_host, nrec, rec_host);
   if (rc) return rc;
@@ -980,6 +1042,7 @@ int rbc_rtm_storage(rbc_ctx *c, const int *src_host, const float *wavelet_dev, i
   if (rc) return rc;
   // both loops resident, or both by steps (the forward step path keeps a level with a launch of its own, whatever
   // the temporal-blocking option)
+  begin_loops(c, s);
   const ResPlan *resf = res_plan_of(c, kResFwd), *ress = res_plan_of(c, kResStore);
   const bool res = resf && ress && c->snap.empty();
   rc = check_nodes(c, src_host, nrec, rec_host);
@@ -1086,6 +1149,7 @@ int rbc_fwi_backward(rbc_ctx *c, const int *src_host, const float *wavelet_dev, 
   cudaStream_t s = (cudaStream_t)stream;
   int rc = check_device_error(c);
   if (rc) return rc;
+  begin_loops(c, s);
   const ResPlan *res = resident(c, kResRev);
   rc = res ? check_nodes(c, src_host, nrec, rec_host) : upload_shot(c, src_host, nrec, rec_host, 1, s);
   if (rc) return rc;

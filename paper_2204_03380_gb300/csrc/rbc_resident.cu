@@ -835,6 +835,37 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
   return true;
 }
 
+// Several loops of a grid at a time, each on its own stream.  Side by side each has fewer blocks, taller tiles and a
+// longer step; loops that do not fit together follow one another; and with one launch per step the loops fill each
+// other's gaps.  The way that is through first is taken, by these estimates of a step of all k loops (us; measured
+// forward and forward + reverse for 1 to 6 loops of 200 x 200 to 2421 x 871): resident 1.5 + 0.075 r, reverse 2.6 +
+// 0.15 r, with r the rows on the fullest of an SM's four schedulers; by launches 2.3 + 0.2 k + 1.3 M or 2.3 k M,
+// reverse 3.9 + 0.3 k + 3.3 M or 5.5 k M (6.7 where the fields leave L2), for M million nodes.  Steps are taken where
+// they are a fifth quicker: a context's first call by steps makes its graphs (5 us per step).
+// Four loops of 400 x 400 take 2.42 / 6.52 us so (forward / both), 6.09 / 17.77 with the whole device each and
+// 3.45 / 9.47 by launches; three of 1100 x 700 6.6 / 18.5 in turn, 7.3 / 22.6 as two and one, 5.4 / 17.4 by launches; two of
+// 2421 x 871 7.05 / 21.3 in turn, 8.8 / 36.4 by launches.
+bool res_plan_shared(const Lay *L, int dir, int loops, ResPlan *out) {
+  if (loops == 1) return res_plan(L, 1, dir, 1, out);
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  out->variant = -1;
+  const double m = 1e-6 * L->NX * L->NZ, km = loops * m;
+  const bool rev = dir == kResRev;
+  const double steps = rev ? std::max(3.9 + 0.3 * loops + 3.3 * m, (km > 3.3 ? 6.7 : 5.5) * km)
+                           : std::max(2.3 + 0.2 * loops + 1.3 * m, 2.3 * km);
+  double best = 1.25 * steps;
+  for (int j = 1; j <= std::min(loops, sms); ++j) {
+    ResPlan P;
+    if (!res_plan(L, 1, dir, j, &P)) break;
+    const int r = P.rz * cdiv(P.warps, 4);
+    const double t = cdiv(loops, sms / P.blocks) * (rev ? 2.6 + 0.15 * r : 1.5 + 0.075 * r);
+    if (t < 0.98 * best) best = t, *out = P;  // (with nothing in it, the shorter steps)
+  }
+  return out->variant >= 0;
+}
+
 size_t res_ll_bytes(const ResPlan &P, int dir) {
   return sizeof(u64) * (size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H);
 }

@@ -62,6 +62,9 @@ struct ResPlan {
 // they do not fit on this device at once); share: the device is shared by that
 // many such loops.
 bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out);
+// Plan for one of `loops` loops of a grid that run at a time: chosen for the time of all of them; false where one
+// launch per step is through sooner.
+bool res_plan_shared(const Lay *L, int dir, int loops, ResPlan *out);
 // Shots of a batch sorted into groups whose loops run at once: groups of shot
 // indices, or none when a shot does not fit.
 std::vector<std::vector<int>> res_groups(const Lay *L, int nshots);

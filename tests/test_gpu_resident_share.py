@@ -80,3 +80,53 @@ def test_a_batch_whose_tables_find_no_memory_steps():
             R.rbc_batch_destroy(b)
         imgs.append(img)
     assert float((imgs[0] - imgs[1]).norm()) <= 1e-5 * float(imgs[0].norm()) and float(imgs[0].norm()) > 0
+
+
+@pytest.mark.parametrize("nx,nz,nb,share", [(300, 300, 50, 40), (1000, 600, 50, 2), (1000, 600, 50, 3), (2301, 751, 60, 2)])
+def test_any_share_gives_the_same_record(nx, nz, nb, share):
+    # side by side, in turn, or by launches
+    import paper_2204_03380_gb300 as R
+    ctx, _, _, src, rec, wt, out = _ctx(R, "many", nx, nz, nb, 60)
+    try:
+        recs = []
+        for n in (1, share, 1):
+            R.rbc_set_share(ctx, n)
+            R.rbc_model(ctx, src, wt, rec, out)
+            recs.append(out.cpu())
+        assert torch.equal(recs[0], recs[1]) and torch.equal(recs[0], recs[2]) and float(recs[0].abs().max()) > 0
+    finally:
+        R.rbc_destroy(ctx)
+
+
+def test_contexts_on_streams_of_their_own_run_side_by_side():
+    # four contexts of 400 x 400 padded nodes, no rbc_set_share: with the whole device for each loop they would take
+    # four times as long as one; side by side they take some 1.5 times (one launch per step: 2.2 times)
+    import paper_2204_03380_gb300 as R
+    runs = [_ctx(R, f"own{k}", 300, 300, 50, 4000, seed=k) for k in range(4)]
+    streams = [torch.cuda.Stream() for _ in runs]
+    try:
+        def timed(n):
+            t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            main = torch.cuda.current_stream()
+            t[0].record(main)
+            for (ctx, _, _, src, rec, wt, out), s in zip(runs[:n], streams):
+                s.wait_event(t[0])
+                R.rbc_model(ctx, src, wt, rec, out, stream=s)
+                main.wait_stream(s)
+            t[1].record(main)
+            torch.cuda.synchronize()
+            return t[0].elapsed_time(t[1])
+
+        first = [None] * len(runs)
+        timed(4)
+        for k, r in enumerate(runs):
+            first[k] = r[-1].clone()
+        together = min(timed(4) for _ in range(3))
+        alone = min(timed(1) for _ in range(4))   # (the first of these still counts the others)
+        assert together < 0.6 * 4 * alone, (together, alone)
+        for k, r in enumerate(runs):
+            assert torch.equal(r[-1], first[k])
+    finally:
+        torch.cuda.synchronize()
+        for r in runs:
+            R.rbc_destroy(r[0])
