@@ -25,7 +25,10 @@
  * a PyTorch CUDA tensor).  Pointers named *_host are host memory.  No call
  * allocates memory visible to the caller; an rbc_ctx owns its internal
  * wavefields.  Calls that take a `stream` (a cudaStream_t; NULL = legacy
- * default stream) are asynchronous on it unless stated.
+ * default stream) are asynchronous on it unless stated.  A 2-D time loop that
+ * fits on the chip keeps all or most of the device's SMs for a launch of some
+ * two milliseconds at a time (or the whole loop, if shorter): a kernel that is
+ * queued on another stream meanwhile may have to wait for the launch's end.
  *
  * Errors.  Every call returns RBC_OK (0) or a positive error code, never
  * throws, and leaves a thread-local message for rbc_last_error().  On an
@@ -302,7 +305,7 @@ int rbc_batch_destroy(rbc_batch *b);
  * (+=, shots may overlap).  shots: nshots descriptors (host); flags must be
  * RBC_REINJECT_SOURCE.  When every shot fits on the chip (about 2.1 M padded
  * nodes), the shots run in groups that fill it, one launch per phase and
- * group.  Otherwise they run in groups of consecutive shots whose
+ * group (a few for long records).  Otherwise they run in groups of consecutive shots whose
  * seven fields fit an L2 budget (environment RBC_BATCH_L2MB, megabytes,
  * default 96; 0 = one group), each group's forward then reverse phase, so
  * that a group's fields stay in L2 through its time loops.  Each phase of

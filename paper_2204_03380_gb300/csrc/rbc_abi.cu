@@ -345,6 +345,10 @@ int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec
   S.a = c->a;
   S.p[0] = c->p[0];
   S.p[1] = c->p[1];
+  S.q[0] = c->q[0];
+  S.q[1] = c->q[1];
+  S.cnum = c->num;
+  S.cden = c->den;
   S.info = reinterpret_cast<const ShotInfo *>(c->res_blob);
   S.seis_t = c->seis_t;
   S.cell_ptr = reinterpret_cast<const int *>(c->res_blob + o_ptr);
@@ -370,8 +374,10 @@ int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec
   A.store = c->store;
   A.stride = stride;
   A.err = c->err_dev;
-  CK(res_launch(P, dir, A, s));
-  ++g_launches;
+  long long launches = 0;
+  const cudaError_t e = res_launch(P, dir, A, s, &launches);
+  g_launches += launches;
+  CK(e);
   return RBC_OK;
 }
 

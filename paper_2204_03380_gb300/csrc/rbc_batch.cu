@@ -960,6 +960,10 @@ int upload_res(rbc_batch *b, const rbc_shot *shots, cudaStream_t s, std::vector<
         S.a = H.a;
         S.p[0] = H.p0;
         S.p[1] = H.p1;
+        S.q[0] = H.q0;
+        S.q[1] = H.q1;
+        S.cnum = H.num;
+        S.cden = H.den;
         S.info = reinterpret_cast<const ShotInfo *>(b->res_blob) + i;
         S.seis_t = const_cast<float *>(H.seis_t);
         S.cell_ptr = reinterpret_cast<const int *>(b->res_blob + o_ptr[i]);
@@ -989,8 +993,7 @@ int run_res(rbc_batch *b, int dir, int g, size_t o_shots, cudaStream_t s, long l
   A.nt = b->g.nt;
   A.overwrite = 1;  // num / den in the pitched layout: k_batch_max and k_batch_image read them
   A.err = b->err_dev;
-  BCK(res_launch(b->res[g].plan[dir], dir, A, s));
-  ++*launches;
+  BCK(res_launch(b->res[g].plan[dir], dir, A, s, launches));
   return RBC_OK;
 }
 
@@ -1087,7 +1090,10 @@ int rbc_batch_create(const rbc_grid *g, int nshots, const int *nx_host, const fl
     }
   }
   create_res(b);
-  const int nf = b->res.empty() ? 7 : 5;  // the resident loops keep the receiver wavefield on the chip
+  // resident loops of one part keep the receiver wavefield on the chip
+  bool parts = false;
+  for (const rbc_batch::Res &r : b->res) parts = parts || res_parts(r.plan[1], g->nt + 1) > 1;
+  const int nf = b->res.empty() || parts ? 7 : 5;
   total *= nf;
   if (cudaMalloc(&b->arena, sizeof(float) * total) != cudaSuccess || cudaMemset(b->arena, 0, sizeof(float) * total) ||
       cudaMalloc(&b->ds, sizeof(BShot) * nshots) != cudaSuccess ||

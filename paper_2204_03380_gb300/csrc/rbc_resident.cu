@@ -4,8 +4,9 @@
 // 16 bytes per node, fused reverse 60) and pays a launch's latency.  A grid of
 // up to about 2.1 M padded nodes (the 2421 x 871 survey grid, at 7 fields) has
 // room on the chip: 152 SMs hold 34 MB of shared memory and 39 MB of tensor
-// memory.  Here one cooperative launch runs a whole loop.  Each block keeps a
-// tile of 128 columns x H rows for all its steps: the two levels of each field
+// memory.  Here one cooperative launch runs a whole loop, or a part of it of
+// some two milliseconds (res_plan).  Each block keeps a
+// tile of 128 columns x H rows for all the launch's steps: the two levels of each field
 // in shared memory; a and the imaging sums in registers and shared memory
 // (tiles of one or two rows per warp) or in tensor memory, which serves as a
 // thread-private store (32 lanes of a quarter x 512 columns; no MMA runs) and
@@ -303,6 +304,11 @@ __device__ __forceinline__ void keep_level(const ResArgs &A, const ResShot &S, c
   }
 }
 
+// Whether an earlier part gave up waiting (its words never came: no use waiting for them in this one).  A block barrier.
+__device__ __forceinline__ bool given_up(const ResArgs &A, int tid) {
+  return __syncthreads_or(A.t0 > 0 && tid == 0 && *(volatile const int *)A.err != 0);
+}
+
 // ------------------------------------------------------------- forward ----
 template <int RZ, int MAXW>
 __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const int H) {
@@ -316,10 +322,16 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
   const int origin = S.L.origin, pitch = S.L.pitch, NX4 = S.L.NX4;
   const Place W = place_of<RZ>(A, T, w, lane, H, 1);
   for (int i = tid; i < (2 * fl + H * kTileX + 8 * H) / 4; i += nthr) *reinterpret_cast<float4 *>(smem + 4 * i) = zero4();
-  __syncthreads();
+  if (given_up(A, tid)) return;
   for (int i = tid; i < T.rows * 32; i += nthr) {
-    const int r = i >> 5, x = T.x0 + 4 * (i & 31);
-    if (x < NX4) *reinterpret_cast<float4 *>(s_a + 4 * i) = ldg4(S.a + origin + (T.z0 + r) * pitch + x);
+    const int r = i >> 5, x = T.x0 + 4 * (i & 31), o = origin + (T.z0 + r) * pitch + x;
+    if (x < NX4) {
+      *reinterpret_cast<float4 *>(s_a + 4 * i) = ldg4(S.a + o);
+      if (A.t0 > 0) {  // the part before left its last two levels
+        st4(smem + h4 + 4 * i, ld4(S.p[0] + o));
+        st4(smem + fl + h4 + 4 * i, ld4(S.p[1] + o));
+      }
+    }
   }
   const int x0 = T.x0 + 4 * lane;
   const bool xok = x0 < NX4;
@@ -352,8 +364,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
   __syncthreads();
   const int nt = A.nt;
   bool ok = true;
-  float f = has_src ? A.wav[0] * fsc : 0.f, f_next = 0.f;
-  for (int n = 0; n < nt; ++n) {
+  float f = has_src ? A.wav[A.t0] * fsc : 0.f, f_next = 0.f;
+  for (int n = A.t0; n < A.t1; ++n) {
     if (has_src && n + 1 < nt) f_next = A.wav[n + 1];  // in flight during this step
     const int c0 = (n & 1 ? fl : 0) + h4, n0 = (n & 1 ? 0 : fl) + h4;
     float *cur = smem + c0, *np = smem + n0 + W.r0 * kTileX + 4 * lane;
@@ -379,9 +391,11 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
       return;
     }
   }
-  record(nt, smem + (nt & 1 ? fl : 0) + h4);
-  if (A.stride > 0 && nt % A.stride == 0) keep_level<RZ>(A, S, T, W, nt, smem + (nt & 1 ? fl : 0) + h4);
-  // the last two levels, for the reverse loop and rbc_get_panels
+  if (A.t1 == nt) {
+    record(nt, smem + (nt & 1 ? fl : 0) + h4);
+    if (A.stride > 0 && nt % A.stride == 0) keep_level<RZ>(A, S, T, W, nt, smem + (nt & 1 ? fl : 0) + h4);
+  }
+  // the last two levels, for the next part, or the reverse loop and rbc_get_panels
   for (int j = 0; j < RZ; ++j) {
     const int r = W.r0 + j;
     if (r < W.rows && xok) {
@@ -529,6 +543,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
   const Place W = place_of<RZ>(A, T, w, lane, H, kStore ? 1 : 2);
   const int nt = A.nt;
   constexpr int TC = tm_cols(RZ, MAXW);
+  if (given_up(A, tid)) return;
   if (TM && w == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
         (uint32_t)__cvta_generic_to_shared(s_tm)), "r"(TC));
@@ -545,6 +560,10 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
       if (!kStore) {
         st4(smem + h4 + 4 * i, ld4(S.p[0] + o));
         st4(smem + fl + h4 + 4 * i, ld4(S.p[1] + o));
+      }
+      if (A.t0 > 0) {  // left by the part before
+        st4(smem + B0 * fl + h4 + 4 * i, ld4(S.q[0] + o));
+        st4(smem + (B0 + 1) * fl + h4 + 4 * i, ld4(S.q[1] + o));
       }
       if (!TM) st4(s_x + 4 * i, ldg4(S.a + o));
     }
@@ -569,7 +588,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
 #pragma unroll
   for (int i = 0; i < K; ++i)
     rec_a[i] = rec.id[i] >= 0 ? rsc * __ldg(sa + (rec.loc[i] / kTileX) * pitch + rec.loc[i] % kTileX) : 0.f;
-  load_s(kGrad ? A.nt + 1 : A.nt);
+  load_s((kGrad ? nt + 1 : nt) - A.t0);
   const int row0 = origin + (T.z0 + W.r0) * pitch;
   const bool has_src = src >= row0 + T.x0 && src < row0 + T.x0 + RZ * pitch;
   const int lstep = lane == 0 ? 8 : kTileX, rstep = lane == 31 ? 8 : kTileX;
@@ -584,20 +603,31 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
     keep.ta = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * RZ * 12);
 #pragma unroll 1
     for (int j = 0; j < RZ; ++j) {
-      const float4 av = W.r0 + j < T.rows && xok ? ldg4(S.a + row0 + j * pitch + x0) : zero4();
+      const bool in = W.r0 + j < T.rows && xok, sums = in && A.t0 > 0;
+      const int o = row0 + j * pitch + x0;
+      const float4 av = in ? ldg4(S.a + o) : zero4();
+      const float4 n4 = sums ? ld4(S.cnum + o) : zero4(), d4 = sums && !kGrad ? ld4(S.cden + o) : zero4();
       __syncwarp();
       tm_st4(keep.ta + 12 * j, av);
-      tm_st4(keep.ta + 12 * j + 4, zero4());
-      tm_st4(keep.ta + 12 * j + 8, zero4());
+      tm_st4(keep.ta + 12 * j + 4, n4);
+      tm_st4(keep.ta + 12 * j + 8, d4);
     }
     keep.flush();
   } else {
     keep.init(s_x, W);
+    if (A.t0 > 0) {
+#pragma unroll
+      for (int j = 0; j < RZ; ++j)
+        if (W.r0 + j < T.rows && xok) {
+          keep.num[j] = ld4(S.cnum + row0 + j * pitch + x0);
+          if constexpr (!kGrad) keep.den[j] = ld4(S.cden + row0 + j * pitch + x0);
+        }
+    }
   }
   __syncthreads();
   bool ok = true;
-  float f_next = 0.f;
-  for (int t = 0; t <= nt; ++t) {
+  float f_next = has_src && A.t0 > 0 ? A.wav[nt - A.t0] : 0.f;
+  for (int t = A.t0; t < A.t1; ++t) {
     const float f = f_next * fsc;
     if (has_src && t < nt) f_next = A.wav[nt - 1 - t];  // in flight during this step
     // p^R level n; pbar level n (FWI: adjoint level n + 1)
@@ -699,7 +729,23 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
     float4 n4, d4;
     __syncwarp();  // (the row before ended with lanes that had nothing to write)
     keep.sums(j, n4, d4);
-    if (!ok || W.r0 + j >= W.rows || z < S.iz0 || z >= S.iz1) continue;
+    if (!ok || W.r0 + j >= W.rows) continue;
+    if (A.t1 <= nt) {  // another part follows
+      if (xok) {
+        const int o = row0 + j * pitch + x0;
+        const float *b = smem + h4 + own + j * kTileX;
+        if (!kStore) {
+          st4(S.p[0] + o, lds4(b));
+          st4(S.p[1] + o, lds4(b + fl));
+        }
+        st4(S.q[0] + o, lds4(b + B0 * fl));
+        st4(S.q[1] + o, lds4(b + (B0 + 1) * fl));
+        st4(S.cnum + o, n4);
+        if (!kGrad) st4(S.cden + o, d4);
+      }
+      continue;
+    }
+    if (z < S.iz0 || z >= S.iz1) continue;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int x = x0 + e;
@@ -811,6 +857,13 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
   out->warps = best_w;
   out->H = best_w * V.rz;
   out->smem = res_smem(dir, out->H, V);
+  // A loop holds its SMs: a kernel on another stream that needs them starts where a part ends, so a part takes some
+  // two milliseconds, by the estimates of res_plan_shared.  (A denoiser call beside a survey shot waited 15 ms, a
+  // whole loop; 1.8 ms with such parts.)  A part costs 5 us on 300 x 300 (reverse 7) and 11 on 2421 x 871, for the
+  // fields to global memory and back; the survey's reverse loop gains 3 % by them.
+  const int r = V.rz * cdiv(best_w, 4);
+  const char *est = getenv("RBC_RES_STEPS");
+  out->steps = est && atoi(est) > 0 ? atoi(est) : (int)(2000 / (dir == kResRev ? 2.6 + 0.15 * r : 1.5 + 0.075 * r));
   out->tiles.clear();
   out->tile0.assign(1, 0);
   for (int s = 0; s < nshots; ++s) {
@@ -954,11 +1007,10 @@ std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
   return best;
 }
 
-cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s) {
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches) {
   const Variant &V = kVariants[P.variant];
   const void *fn = V.fn[dir == kResStore ? 3 : dir == kResRev && A.grad ? 2 : dir];
   cudaError_t e = cudaMemsetAsync(A.ll, 0, res_ll_bytes(P, dir), s);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.blocks);
   cfg.blockDim = dim3(32, P.warps);
@@ -972,7 +1024,14 @@ cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t
   ResArgs a = A;
   int H = P.H;
   void *args[2] = {&a, &H};
-  return cudaLaunchKernelExC(&cfg, fn, args);
+  const int n = dir == kResFwd ? A.nt : A.nt + 1, parts = res_parts(P, n);
+  for (int k = 0; k < parts && e == cudaSuccess; ++k) {
+    a.t0 = (int)((long long)n * k / parts);
+    a.t1 = (int)((long long)n * (k + 1) / parts);
+    e = cudaLaunchKernelExC(&cfg, fn, args);
+    if (e == cudaSuccess) ++*launches;
+  }
+  return e;
 }
 
 } // namespace rbc

@@ -23,6 +23,8 @@ struct ResShot {
   Lay L;
   const float *a;
   float *p[2];              // level m in p[m & 1]: written by the forward loop, read by the reverse loop
+  float *q[2];              // pbar's level m in q[m & 1], sums in cnum / cden (pitched): what a reverse loop of several
+  float *cnum, *cden;       // parts leaves for the next part (unused with one part)
   const ShotInfo *info;
   float *seis_t;            // [levels][nrec] time-major record
   const int *cell_ptr;      // receivers of each (tile, warp) of this shot's tile range (CSR)
@@ -38,6 +40,7 @@ struct ResArgs {
   unsigned long long *ll;   // halo exchange words, zeroed before the launch
   const float *wav;         // f[0..nt-1]
   int nt;
+  int t0, t1;               // this part's steps (res_launch)
   int sample;               // forward: record every level at the receivers
   int grad;                 // reverse: 1 = FWI gradient (num += mu p_tt), 0 = imaging integrals
   int overwrite;            // reverse: outputs are set, not added to
@@ -53,6 +56,7 @@ struct ResPlan {
   int variant = -1;         // index into the kernel variants, -1: does not fit
   int rz = 0, warps = 0, H = 0;
   int blocks = 0;
+  int steps = 1;            // most steps of one launch (a longer loop runs in parts)
   size_t smem = 0;
   std::vector<ResTile> tiles;
   std::vector<int> tile0;   // first tile of each shot, then the tile count
@@ -81,6 +85,8 @@ void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc)
 // Receiver cells of one shot (its tiles * warps cells): CSR pointers and
 // {place in the tile, receiver}, positions offset by `base`.
 void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *rec, int base, int *ptr, int2 *out);
-cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s);
+// Parts of a loop of n steps (forward: nt; reverse: nt + 1).
+inline int res_parts(const ResPlan &P, int n) { return (n + P.steps - 1) / P.steps; }
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches);
 
 } // namespace rbc

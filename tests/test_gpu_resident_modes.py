@@ -127,3 +127,72 @@ def test_the_step_path_of_a_batch_is_tuned_and_matches(l2mb, groups, monkeypatch
     monkeypatch.setattr(R, "rbc_batch_info", lambda b: seen.append(info(b)) or seen[-1])
     tb.test_batch_matches_single_shots_and_oracle(None, l2mb, groups, monkeypatch)
     assert any(t > 0 for t in seen[0]["tune_us"].values())   # the tuner timed its candidates
+
+
+@pytest.mark.parametrize("case", [c for c in CASES if c[5] in (None, "0,4", "1,16", "2,5", "2,16", "3,9", "4,11")],
+                         ids=lambda c: f"{c[0]}-{c[5]}")
+def test_a_loop_in_parts_gives_the_same_bits(case, monkeypatch):
+    # fields, sums, receivers, the source and the exchange words carried from part to part: every step a part of its
+    # own, and parts that cut the record unevenly
+    import paper_2204_03380_gb300 as R
+    *dims, tile = case
+    w, v, src, rec, wav = _case(*dims)
+    rec = np.unique(rec, axis=0)   # (a repeated receiver's adds have no fixed order)
+    _env(monkeypatch, tile)
+    wt = torch.tensor(np.asarray(wav, np.float32), device="cuda")
+    outs, counts = [], []
+    for steps in (None, "1", "23"):
+        monkeypatch.delenv("RBC_RES_STEPS", raising=False)
+        if steps:
+            monkeypatch.setenv("RBC_RES_STEPS", steps)
+        g, a, _ = gpu_build(R, torch, w, v)
+        seis = torch.zeros((len(rec), w.nt + 1), device="cuda")
+        z = [torch.ones(g.interior, device="cuda") for _ in range(5)]
+        store = torch.empty(R.rbc_storage_bytes(g, 3) // 4, device="cuda")
+        panels = [torch.empty(g.padded, device="cuda") for _ in range(4)]
+        misfit, resid = torch.zeros(1, dtype=torch.float64, device="cuda"), torch.empty_like(seis)
+        R.rbc_launch_count(True)
+        ctx = R.rbc_create(g, a)
+        try:
+            R.rbc_model(ctx, src, wt, rec, seis)
+            R.rbc_get_panels(ctx, *panels[:2])
+            R.rbc_rtm_shot(ctx, src, wt, rec, seis, R.RBC_REINJECT_SOURCE, *z[:2])     # += onto ones
+            R.rbc_rtm_storage(ctx, src, wt, rec, seis, 3, store, R.RBC_ZERO_FIRST, *z[2:4])
+            R.rbc_get_panels(ctx, *panels[2:])                                             # the forward loop's, kept
+            R.rbc_fwi_forward(ctx, src, wt, rec, torch.zeros_like(seis), resid, misfit)
+            R.rbc_fwi_backward(ctx, src, wt, rec, resid, None, z[4])
+            torch.cuda.synchronize()
+        finally:
+            R.rbc_destroy(ctx)
+        counts.append(R.rbc_launch_count())
+        outs.append([t.cpu() for t in [seis, store, resid, *z, *panels]])
+    assert counts[0] < 40 and counts[1] > 6 * w.nt > counts[2] > counts[0]
+    for o in outs[1:]:
+        for k, (x, y) in enumerate(zip(outs[0], o)):
+            assert torch.equal(x, y), k
+    assert all(float(x.abs().max()) > 0 for x in outs[0])
+
+
+def test_a_batch_in_parts_gives_the_same_bits(monkeypatch):
+    import paper_2204_03380_gb300 as R
+    w, v, src, rec, wav = _case("bparts", 150, 37, 9, 201)
+    rec = np.unique(rec, axis=0)
+    wt = torch.tensor(np.asarray(wav, np.float32), device="cuda")
+    g, a, _ = gpu_build(R, torch, w, v)
+    seis = torch.randn((len(rec), w.nt + 1), generator=torch.Generator().manual_seed(1)).cuda()
+    imgs = []
+    for steps in (None, "1", "23"):
+        if steps:
+            monkeypatch.setenv("RBC_RES_STEPS", steps)
+        b = R.rbc_batch_create(g, [150, 150], [a, a])
+        try:
+            for _ in range(2):
+                img = torch.zeros((w.nz, 300), device="cuda")
+                R.rbc_batch_rtm(b, [dict(src=src, rec=rec, seis=seis, off_x=150 * k) for k in range(2)], wt,
+                                R.RBC_REINJECT_SOURCE, 1e-2, img)
+                torch.cuda.synchronize()
+                imgs.append(img)
+        finally:
+            R.rbc_batch_destroy(b)
+    assert all(torch.equal(imgs[0], i) for i in imgs) and float(imgs[0].abs().max()) > 0
+    assert torch.equal(imgs[0][:, :150], imgs[0][:, 150:])

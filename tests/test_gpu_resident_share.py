@@ -130,3 +130,30 @@ def test_contexts_on_streams_of_their_own_run_side_by_side():
         torch.cuda.synchronize()
         for r in runs:
             R.rbc_destroy(r[0])
+
+
+def test_a_kernel_on_another_stream_runs_before_a_long_loop_ends():
+    # the loop takes every SM's shared memory for some 40 ms in all, and the denoiser's kernels need most of an SM's
+    import paper_2204_03380_gb300 as R
+    from paper_2204_03380_gb300.denoise import Denoiser
+    ctx, _, _, src, rec, wt, out = _ctx(R, "survey", 2301, 751, 60, 12000)
+    net, x = Denoiser(seed=1), torch.randn((1, 200, 200), device="cuda")
+    loop, side = torch.cuda.Stream(), torch.cuda.Stream()
+    try:
+        ref = net(x)
+        R.rbc_model(ctx, src, wt, rec, out, stream=loop)
+        torch.cuda.synchronize()
+        R.rbc_model(ctx, src, wt, rec, out, stream=loop)
+        done = torch.cuda.Event()
+        done.record(loop)
+        with torch.cuda.stream(side):
+            y = net(x)
+            ready = torch.cuda.Event()
+            ready.record(side)
+        ready.synchronize()
+        assert not done.query()
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref)
+    finally:
+        torch.cuda.synchronize()
+        R.rbc_destroy(ctx)
