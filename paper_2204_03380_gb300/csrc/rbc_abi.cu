@@ -563,10 +563,11 @@ int enqueue_reverse(rbc_ctx *c, cudaStream_t s) {
 // context steps with one launch per step.
 void create_resident(rbc_ctx *c) {
   if (c->L.ndim != 2) return;
-  int nf = 0;
+  size_t ll = 0;
   for (int dir = 0; dir < 3; ++dir)
-    if (res_plan(&c->L, 1, dir, 1, &c->res[1][dir])) nf = std::max(nf, dir == kResRev ? 2 : 1);
-  if (nf && res_malloc((void **)&c->res_ll, res_ll_bound(c->L, nf)) != cudaSuccess) {
+    if (res_plan(&c->L, 1, dir, 1, &c->res[1][dir]))
+      ll = std::max({ll, res_ll_bytes(c->res[1][dir], dir), res_ll_bound(c->L, dir == kResRev ? 2 : 1)});
+  if (ll && res_malloc((void **)&c->res_ll, ll) != cudaSuccess) {
     c->res_ll = nullptr;
     cudaGetLastError();
   }

@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
   const int nt = A.nt;
   bool ok = true;
   float f = has_src ? A.wav[A.t0] * fsc : 0.f, f_next = 0.f;
+  int keep = A.stride > 0 ? (A.t0 + A.stride - 1) / A.stride * A.stride : -1;  // the next level kept
   for (int n = A.t0; n < A.t1; ++n) {
     if (has_src && n + 1 < nt) f_next = A.wav[n + 1];  // in flight during this step
     const int c0 = (n & 1 ? fl : 0) + h4, n0 = (n & 1 ? 0 : fl) + h4;
@@ -383,7 +384,10 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
                      });
     __syncwarp();
     if (n + 1 < nt) halo_out<RZ>(W, 0, (uint32_t)n + 1, smem + n0);
-    if (A.stride > 0 && n % A.stride == 0) keep_level<RZ>(A, S, T, W, n, cur);
+    if (n == keep) {
+      keep_level<RZ>(A, S, T, W, n, cur);
+      keep += A.stride;
+    }
     if (rec.end > rec.beg) record(n, cur);
     f = f_next * fsc;
     if (__syncthreads_or(!ok)) {
@@ -393,7 +397,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
   }
   if (A.t1 == nt) {
     record(nt, smem + (nt & 1 ? fl : 0) + h4);
-    if (A.stride > 0 && nt % A.stride == 0) keep_level<RZ>(A, S, T, W, nt, smem + (nt & 1 ? fl : 0) + h4);
+    if (nt == keep) keep_level<RZ>(A, S, T, W, nt, smem + (nt & 1 ? fl : 0) + h4);
   }
   // the last two levels, for the next part, or the reverse loop and rbc_get_panels
   for (int j = 0; j < RZ; ++j) {
@@ -627,7 +631,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
   __syncthreads();
   bool ok = true;
   float f_next = has_src && A.t0 > 0 ? A.wav[nt - A.t0] : 0.f;
-  for (int t = A.t0; t < A.t1; ++t) {
+#pragma unroll 1
+  for (int t = A.t0; t != A.t1; ++t) {
     const float f = f_next * fsc;
     if (has_src && t < nt) f_next = A.wav[nt - 1 - t];  // in flight during this step
     // p^R level n; pbar level n (FWI: adjoint level n + 1)
@@ -690,10 +695,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
     if (!kStore && t < nt) halo_out<RZ>(W, 0, (uint32_t)t + 1, smem + rn0);
     if (do_b) {
       float *bc = smem + bc0, *bn = smem + bn0;
-      if (t > 0)  // level nt is zero everywhere
-        ok = halo_in<RZ, TIGHT>(W, FB, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
-      else
-        __syncwarp();
+      // (level nt is zero everywhere, as the words are before the first)
+      ok = halo_in<RZ, TIGHT>(W, FB, (uint32_t)t, s_lr, bc - h4, TIGHT ? s_x : bc + H * kTileX, qa) && ok;
       sweep<RZ, TIGHT>(W, smem, bc0, bn0, bc + W.r0 * kTileX - 4 * kTileX,
                        TIGHT && last ? s_x : bc + (W.r0 + RZ) * kTileX, top, qa, lofs, lstep, rofs, rstep,
                        [&](int j) { keep.pre_a(j); },
@@ -928,7 +931,7 @@ size_t res_ll_bound(const Lay &L, int nf) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   for (const Variant &V : kVariants) hmax = std::max(hmax, V.maxw * V.rz);
-  const long long gx = cdiv(L.NX, kTileX), blocks = std::min((long long)sms, gx * cdiv(L.NZ, 4));
+  const long long gx = cdiv(L.NX, kTileX), blocks = std::min((long long)sms / 2, gx * cdiv(L.NZ, 4));
   // ll_words(H) per block, and blocks * H <= gx * (NZ + H - 1)
   return sizeof(u64) * nf * 2 * (size_t)(blocks * 2 * kEdge + 8 * gx * (L.NZ + hmax - 1));
 }

@@ -73,7 +73,7 @@ bool res_plan_shared(const Lay *L, int dir, int loops, ResPlan *out);
 // indices, or none when a shot does not fit.
 std::vector<std::vector<int>> res_groups(const Lay *L, int nshots);
 size_t res_ll_bytes(const ResPlan &P, int dir);
-// At least res_ll_bytes of any plan of this grid alone, for loops of nf fields.
+// At least res_ll_bytes of any plan of this grid on half of the device or less, for loops of nf fields.
 size_t res_ll_bound(const Lay &L, int nf);
 // cudaMalloc for the loops' own tables, without which a context or batch takes the step path; res_fail_alloc(true)
 // makes the next one fail (rbc_inject_fault).
