@@ -1208,10 +1208,13 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     if (st != cudaStreamCaptureStatusNone) return bfail(RBC_ECUDA, "rbc_batch_rtm: the stream is capturing");
   }
   const int nt = b->g.nt;
-  // receiver tables of every shot (counting sort by reverse tile)
+  // checks, and for the step path the receiver tables of every shot (counting sort by reverse tile; the resident
+  // loops have cells of their own, upload_res)
+  const bool steps = b->res.empty();
   std::vector<int> off, ptr, order;
   std::vector<int> rec_base(b->nshots), ptr_base(b->nshots);
   long long seis_total = 0;
+  int nrec_total = 0;
   std::vector<long long> seis_base(b->nshots);
   for (int i = 0; i < b->nshots; ++i) {
     const rbc_shot &sh = shots[i];
@@ -1222,13 +1225,19 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
       return bfail(RBC_EINVAL, "rbc_batch_rtm: shot %d has a bad receiver list", i);
     auto inside = [&](const int *r) { return r[0] >= 0 && r[0] < L.NX && r[1] == 0 && r[2] >= 0 && r[2] < L.NZ; };
     if (!inside(sh.src)) return bfail(RBC_EINVAL, "rbc_batch_rtm: shot %d source outside its grid", i);
+    for (int r = 0; r < sh.nrec; ++r)
+      if (!inside(sh.rec_host + 3 * r))
+        return bfail(RBC_EINVAL, "rbc_batch_rtm: shot %d receiver %d outside its grid", i, r);
+    seis_base[i] = seis_total;
+    seis_total += (long long)(nt + 1) * sh.nrec;
+    nrec_total += sh.nrec;
+    if (!steps) continue;
     const int gx = cdiv(L.NX, kTileX), gz = cdiv(L.NZ, rev_tile_rows(b));
     rec_base[i] = (int)off.size();
     ptr_base[i] = (int)ptr.size();
     std::vector<int> cnt(gx * gz + 1, 0), tile(sh.nrec);
     for (int r = 0; r < sh.nrec; ++r) {
       const int *q = sh.rec_host + 3 * r;
-      if (!inside(q)) return bfail(RBC_EINVAL, "rbc_batch_rtm: shot %d receiver %d outside its grid", i, r);
       off.push_back(lay_off(L, q[0], 0, q[2]));
       tile[r] = (q[2] / rev_tile_rows(b)) * gx + q[0] / kTileX;
       cnt[tile[r] + 1]++;
@@ -1239,12 +1248,10 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     const int obase = (int)order.size();
     for (int t = 0; t <= gx * gz; ++t) ptr.push_back(obase + cnt[t]);
     order.insert(order.end(), ord.begin(), ord.end());
-    seis_base[i] = seis_total;
-    seis_total += (long long)(nt + 1) * sh.nrec;
   }
   // grow the capacity buffers (invalidates the graphs)
-  const int nr = std::max(1, (int)off.size()), np = std::max(1, (int)ptr.size());
-  if (nr > b->rec_cap || np > b->tile_cap || !b->d_seis_t || !b->d_rec_off) {
+  const int nr = std::max(1, nrec_total), np = std::max(1, (int)ptr.size());
+  if (nr > b->rec_cap || !b->d_seis_t || (steps && (np > b->tile_cap || !b->d_rec_off))) {
     drop_graphs(b);
     cudaFree(b->d_rec_off);
     cudaFree(b->d_tile_rec);
@@ -1254,18 +1261,22 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     b->d_seis_t = nullptr;
     b->rec_cap = std::max(nr, b->rec_cap);
     b->tile_cap = std::max(np, b->tile_cap);
-    BCK(cudaMalloc(&b->d_rec_off, sizeof(int) * b->rec_cap));
-    BCK(cudaMalloc(&b->d_tile_rec, sizeof(int) * b->rec_cap));
-    BCK(cudaMalloc(&b->d_tile_ptr, sizeof(int) * b->tile_cap));
+    if (steps) {
+      BCK(cudaMalloc(&b->d_rec_off, sizeof(int) * b->rec_cap));
+      BCK(cudaMalloc(&b->d_tile_rec, sizeof(int) * b->rec_cap));
+      BCK(cudaMalloc(&b->d_tile_ptr, sizeof(int) * b->tile_cap));
+    }
     BCK(cudaMalloc(&b->d_seis_t, sizeof(float) * (size_t)b->rec_cap * (nt + 1)));
   }
   for (int i = 0; i < b->nshots; ++i) {
     BShot &S = b->hs[i];
     S.src_off = lay_off(b->L[i], shots[i].src[0], 0, shots[i].src[2]);
     S.nrec = shots[i].nrec;
-    S.rec_off = b->d_rec_off + rec_base[i];
-    S.tile_rec = b->d_tile_rec;  // the CSR holds positions in the whole list
-    S.tile_ptr = b->d_tile_ptr + ptr_base[i];
+    if (steps) {
+      S.rec_off = b->d_rec_off + rec_base[i];
+      S.tile_rec = b->d_tile_rec;  // the CSR holds positions in the whole list
+      S.tile_ptr = b->d_tile_ptr + ptr_base[i];
+    }
     S.seis_t = b->d_seis_t + seis_base[i];
     S.off_x = shots[i].off_x;
     S.maxbits = 0;
@@ -1277,7 +1288,7 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     BCK(cudaMemcpyAsync(b->d_rec_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
     BCK(cudaMemcpyAsync(b->d_tile_rec, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, s));
   }
-  BCK(cudaMemcpyAsync(b->d_tile_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, s));
+  if (steps) BCK(cudaMemcpyAsync(b->d_tile_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, s));
   BCK(cudaMemcpyAsync(b->d_wav, wavelet_dev, sizeof(float) * nt, cudaMemcpyDeviceToDevice, s));
   long long launches = 0;
   for (int i = 0; i < b->nshots; ++i)
@@ -1287,9 +1298,9 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     }
   // each group: forward phase then reverse phase (on the chip, or while its fields sit in L2)
   std::vector<size_t> o_shots;
-  if (!b->res.empty())
+  if (!steps)
     if (int rc = upload_res(b, shots, s, &o_shots)) return rc;
-  const int ng = b->res.empty() ? (int)b->grp.size() - 1 : (int)b->res.size();
+  const int ng = steps ? (int)b->grp.size() - 1 : (int)b->res.size();
   for (int g = 0; g < ng; ++g) {
     cudaEvent_t e3[3] = {nullptr, nullptr, nullptr};
     if (b->timing)
@@ -1298,10 +1309,10 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
         b->ev.push_back(e3[k]);
       }
     if (b->timing) BCK(cudaEventRecord(e3[0], s));
-    int rc = b->res.empty() ? run_b(b, 0, g, s, &launches) : run_res(b, 0, g, o_shots[2 * g], s, &launches);
+    int rc = steps ? run_b(b, 0, g, s, &launches) : run_res(b, 0, g, o_shots[2 * g], s, &launches);
     if (rc) return rc;
     if (b->timing) BCK(cudaEventRecord(e3[1], s));
-    rc = b->res.empty() ? run_b(b, 1, g, s, &launches) : run_res(b, 1, g, o_shots[2 * g + 1], s, &launches);
+    rc = steps ? run_b(b, 1, g, s, &launches) : run_res(b, 1, g, o_shots[2 * g + 1], s, &launches);
     if (rc) return rc;
     if (b->timing) BCK(cudaEventRecord(e3[2], s));
   }

@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(tc_threads(MODE, R), 1) k_conv_tc(const __grid
     x0 = (rem - ty * ntx) * kTcOut;
   };
   if (MODE != kFused && warp == kTcEpi) {
-    // ---- producer: one TMA copy per two halo rows ----
+    // ---- producer: one TMA copy per half tile (R / 2 + 1 halo rows) ----
     // (one bulk copy per channel group and halo row instead lost by 2.1x)
     if (lane == 0) {
       int q = 0;  // units issued
@@ -946,7 +946,7 @@ __device__ __forceinline__ void wt_copy(uint32_t dst, const CUtensorMap *tm, int
 __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_constant__ CUtensorMap tm_x,
                                                                  const __grid_constant__ CUtensorMap tm_z,
                                                                  float *__restrict__ dw, float *__restrict__ db,
-                                                                 int nimg, int H, int W, int rev, int *err) {
+                                                                 int nimg, int H, int W, int *err) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar[2 * kWtStages + 1];
   __shared__ uint32_t s_tmem;
@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_conv_wgrad_tc(const __grid_co
       for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x, ++k) {
         const int s = k % kWtStages, u = k / kWtStages;
         if (u > 0 && !tc_wait(empty(s), (u - 1) & 1, abort_blk)) break;
-        const int ts = rev ? ntiles - 1 - tt : tt;
+        const int ts = ntiles - 1 - tt;  // from the last tile, which the kernel before wrote last
         const int img = ts / tpi, rem = ts - img * tpi, ty = rem / ntx;
         const int y0 = ty * kWtR, x0 = (rem - ty * ntx) * kWtC;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(kWtStage)
@@ -1282,22 +1282,22 @@ __global__ void __launch_bounds__(128) k_conv_wgrad1(const TU *__restrict__ u, c
   }
 }
 
-// fp32 master weights -> bf16 compute weights: forward copies and the
-// mirrored / transposed copies for the backward-data pass.
+// fp32 master weights -> bf16 compute weights of the training step: the first
+// layer's as they are (the other forward layers round their own), and layers
+// 2 .. 5 mirrored and transposed for the backward-data pass, [t][co][ci] ->
+// [8 - t][ci][co].
 __global__ void k_prep_weights(const float *__restrict__ prm, __nv_bfloat16 *__restrict__ wf, __nv_bfloat16 *__restrict__ wb) {
-  // forward: same layout as the master; backward: layer l's [t][co][ci] ->
-  // [8 - t][ci][co] (only layers 2..5 are needed backwards)
-  const int offs[5] = {kW1, kW2, kW3, kW4, kW5};
-  const int cin[5] = {1, C, C, C, C}, cout[5] = {C, C, C, C, 1};
+  const int offs[4] = {kW2, kW3, kW4, kW5};
+  const int cout[4] = {C, C, C, 1};
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   griddep_wait();
   griddep_launch();
-  for (int l = 0; l < 5; ++l) {
-    const int n = 9 * cin[l] * cout[l];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      const float v = prm[offs[l] + i];
-      wf[offs[l] + i] = __float2bfloat16(v);
-      const int ci = i % cin[l], co = (i / cin[l]) % cout[l], t = i / (cin[l] * cout[l]);
-      wb[offs[l] + ((8 - t) * cin[l] + ci) * cout[l] + co] = __float2bfloat16(v);
+  for (int i = i0; i < 9 * C; i += step) wf[i] = __float2bfloat16(prm[kW1 + i]);
+  for (int l = 0; l < 4; ++l) {
+    const int n = 9 * C * cout[l];
+    for (int i = i0; i < n; i += step) {
+      const int ci = i % C, co = (i / C) % cout[l], t = i / (C * cout[l]);
+      wb[offs[l] + ((8 - t) * C + ci) * cout[l] + co] = __float2bfloat16(prm[offs[l] + i]);
     }
   }
 }
@@ -1394,7 +1394,7 @@ int grid_of(long long n) {
   return (int)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
 }
 
-// Workspace layout (bytes): bf16 weights fwd, bf16 weights bwd, x (bf16),
+// Workspace layout (bytes): bf16 first-layer weights, bf16 weights bwd, x (bf16),
 // four hidden activations (bf16, 32 ch), two 32-channel gradient buffers
 // (bf16) and the activations' sign bits.
 struct Ws {
@@ -1412,7 +1412,7 @@ Ws carve(void *ws, long long npx) {
   };
   const size_t n = (size_t)npx;
   Ws w;
-  w.wf = take(2 * kNParams);
+  w.wf = take(2 * kNParams);  // (288 of them are used; the activations 56 KB nearer cost a step of 8 x 512^2 3 us)
   w.wb = take(2 * kNParams);
   w.x0 = take(2 * n);
   for (int l = 0; l < 4; ++l) w.act[l] = take(2 * n * C);
@@ -1525,7 +1525,7 @@ bool launch_wgrad(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *dw, fl
   const int grid = (int)(tiles < sm_count() ? tiles : sm_count());
   CUtensorMap tx, tz;
   if (!rows_map(&tx, x, nimg, H, W, kWtXP, kWtR) || !rows_map(&tz, dz, nimg, H, W, kWtC, kWtR + 2)) return false;
-  launch_pdl(k_conv_wgrad_tc, dim3(grid), dim3(kWtThreads), kWtSmem, s, tx, tz, dw, db, nimg, H, W, 1, tc_err_dev);
+  launch_pdl(k_conv_wgrad_tc, dim3(grid), dim3(kWtThreads), kWtSmem, s, tx, tz, dw, db, nimg, H, W, tc_err_dev);
   return true;
 }
 
@@ -1545,7 +1545,7 @@ int cnn_forward(const float *params_dev, int nimg, int H, int W, const float *x_
   bool ok_tc = true;
   if (keep) {  // the backward pass reads the first layer's output
     launch_pdl(k_prep_weights, dim3(36), dim3(256), 0, s, prm, w.wf, w.wb);
-    launch_pdl(k_conv_1to32<kHidden>, dim3(grid_1to32<kHidden>(nimg, H, W)), dim3(256), 0, s, x_dev, w.x0, w.wf + kW1,
+    launch_pdl(k_conv_1to32<kHidden>, dim3(grid_1to32<kHidden>(nimg, H, W)), dim3(256), 0, s, x_dev, w.x0, w.wf,
                prm + kB1, w.bits[0], w.act[0], nimg, H, W);
     ok_tc = launch_conv_tc<kHidden>(w.act[0], prm + kW2, prm + kB2, w.bits[1], w.act[1], nimg, H, W, 1, s);
   } else {

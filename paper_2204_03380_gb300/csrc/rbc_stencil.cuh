@@ -24,10 +24,8 @@ __device__ __forceinline__ float2 sum_diff2(const float2 m, const float2 p, cons
 }
 
 // w[0..11]: x window x0-4 .. x0+7 (centre at w[4..7]); zq[0..8]: z window
-// (zq[4] = centre); ym[k-1] / yp[k-1]: y neighbours at distance k (3-D only).
-template <bool kThreeD>
-__device__ __forceinline__ float4 leap4p(const float *w, const float4 *zq, const float4 *ym, const float4 *yp,
-                                         const float4 po, const float4 av) {
+// (zq[4] = centre).
+__device__ __forceinline__ float4 leap4p(const float *w, const float4 *zq, const float4 po, const float4 av) {
   float2 out[2];
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
@@ -40,7 +38,6 @@ __device__ __forceinline__ float4 leap4p(const float *w, const float4 *zq, const
       const float2 xp = make_float2(w[4 + 2 * j + k], w[5 + 2 * j + k]);
       float2 t = sum_diff2(xm, xp, np);
       t = __fadd2_rn(t, sum_diff2(half2of(zq[4 - k], j), half2of(zq[4 + k], j), np));
-      if (kThreeD) t = __fadd2_rn(t, sum_diff2(half2of(ym[k - 1], j), half2of(yp[k - 1], j), np));
       s[k] = t;
     }
     float2 lap = __fmul2_rn(make_float2(kC4, kC4), s[4]);
@@ -84,8 +81,8 @@ __device__ __forceinline__ float4 leap4p_inc(const float *w, const float4 *zq, c
   return make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
 }
 
-// ---- the 2-D update with shared differences (resident loops) ----
-// The same roundings as leap4p<false>, bit for bit, with fewer operations: with
+// ---- the update with shared differences (resident 2-D loops, 3-D steps) ----
+// The same roundings as leap4p, bit for bit, with fewer operations: with
 // D_k[i] = p_{i+k} - p_i, the term (p_{-k} - p) + (p_{+k} - p) is D_k[i] -
 // D_k[i-k] (rounding is symmetric in the sign), and every D_k serves two
 // nodes: along x within the float4, along z by a march down the rows.  59

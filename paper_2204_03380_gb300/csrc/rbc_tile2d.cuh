@@ -37,7 +37,7 @@ __device__ __forceinline__ float4 shfl_dn4(float4 v) {
 __device__ __forceinline__ float4 leap4_2d(const float4 lf, const float4 c, const float4 rt, const float4 *zq,
                                            const float4 po, const float4 av) {
   const float w[12] = {lf.x, lf.y, lf.z, lf.w, c.x, c.y, c.z, c.w, rt.x, rt.y, rt.z, rt.w};
-  return leap4p<false>(w, zq, nullptr, nullptr, po, av);
+  return leap4p(w, zq, po, av);
 }
 
 // Subtract a point term from component (src - o) of v when the source node
