@@ -140,7 +140,8 @@ int rbc_set_coef(rbc_ctx *ctx, const float *a_dev, int check, void *stream);
  * the time of all of them -- side by side on a part of the device each, one
  * after the other, or by one launch per step, whichever is through first.
  * Results do not depend on it.  Until it is called, a context counts those
- * that were called on other streams since its own last call.
+ * contexts and batches that were called on other streams since its own last
+ * call; a batch always does.
  * Applies to the calls that follow; allocates nothing and waits for nothing.
  * Errors: RBC_EINVAL (NULL, contexts < 1).
  */

@@ -10,7 +10,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
-#include <mutex>
 #include <string>
 #include <vector>
 
@@ -134,12 +133,12 @@ struct rbc_ctx {
   // (rbc_resident.cu), by kResFwd .. kResStore (variant -1: one launch per step)
   std::map<int, std::array<ResPlan, 3>> res;  // the plans, by `loops` (host tables)
   unsigned long long *res_ll = nullptr;       // room for the exchange words of any of them (null: no resident loops)
+  size_t res_ll_cap = 0;
   char *res_blob = nullptr;  // this call's tables: ShotInfo, ResShot, tiles, receiver cells
   size_t res_blob_cap = 0;
   int share = 0;             // contexts in flight at once as the caller says (rbc_set_share; 0: counted)
   int loops = 1;             // contexts in flight with this call
-  unsigned long long called = 0, on_stream = 0;  // this context's last counted call (0: none yet) and its stream
-  unsigned long long born = 0;                   // calls counted before its creation
+  LoopUser user;
 };
 
 namespace {
@@ -246,51 +245,13 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
   return RBC_OK;
 }
 
-// The 2-D contexts with resident loops that are alive, and the number of their calls so far.
-struct Flight {
-  std::mutex m;
-  std::vector<rbc_ctx *> live;
-  unsigned long long calls = 0;
-};
-Flight &flight() {
-  static Flight *f = new Flight();  // (outlives contexts destroyed at exit)
-  return *f;
-}
-
-// Contexts whose loops may run beside this call's, itself included: those called on other streams since its own last
-// call.  A program that runs k contexts on k streams calls the others in between; one that uses its contexts in turn
-// on one stream, or one context at a time, is counted as one.  At its first call (on a stream of the caller's making)
-// contexts that have not been called yet count too, so that a first round of calls runs side by side as well.
-// Nothing but the plan depends on the count.
-int count_loops(rbc_ctx *c, cudaStream_t s) {
-  unsigned long long id = 0;
-  if (!c->res_ll || cudaStreamGetId(s, &id) != cudaSuccess) return 1;
-  Flight &f = flight();
-  std::lock_guard<std::mutex> lock(f.m);
-  std::vector<unsigned long long> seen(1, id);
-  int n = 1;
-  for (const rbc_ctx *x : f.live) {
-    if (x == c || x->dev != c->dev) continue;
-    if (!x->called) {
-      n += !c->called && s != nullptr && s != cudaStreamLegacy;
-    } else if (x->called > std::max(c->called, c->born) &&
-               std::find(seen.begin(), seen.end(), x->on_stream) == seen.end()) {
-      seen.push_back(x->on_stream);
-      ++n;
-    }
-  }
-  c->called = ++f.calls;
-  c->on_stream = id;
-  return n;
-}
-
 // At the start of a call that runs a loop.  (On a capturing stream, where the call is refused further on, nothing is
 // asked of the runtime that would end the capture.)
 void begin_loops(rbc_ctx *c, cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   c->loops = 1;
   if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return;
-  const int n = count_loops(c, s);
+  const int n = c->res_ll ? flight_count(&c->user, s) : 1;
   c->loops = c->share ? c->share : n;
 }
 
@@ -301,7 +262,10 @@ const ResPlan *res_plan_of(rbc_ctx *c, int dir) {
   if (it == c->res.end()) {
     if (c->res.size() >= 8) c->res.clear();
     it = c->res.emplace(c->loops, std::array<ResPlan, 3>()).first;
-    for (int d = 0; d < 3; ++d) res_plan_shared(&c->L, d, c->loops, &it->second[d]);
+    for (int d = 0; d < 3; ++d)
+      if (res_plan_shared(&c->L, 1, d, c->loops, true, &it->second[d]) &&
+          res_ll_bytes(it->second[d], d) > c->res_ll_cap)  // (a tile shape forced since the context's creation)
+        it->second[d].variant = -1;
   }
   return it->second[dir].variant >= 0 ? &it->second[dir] : nullptr;
 }
@@ -566,11 +530,12 @@ void create_resident(rbc_ctx *c) {
   size_t ll = 0;
   for (int dir = 0; dir < 3; ++dir)
     if (res_plan(&c->L, 1, dir, 1, &c->res[1][dir]))
-      ll = std::max({ll, res_ll_bytes(c->res[1][dir], dir), res_ll_bound(c->L, dir == kResRev ? 2 : 1)});
+      ll = std::max({ll, res_ll_bytes(c->res[1][dir], dir), res_ll_bound(&c->L, 1, dir == kResRev ? 2 : 1)});
   if (ll && res_malloc((void **)&c->res_ll, ll) != cudaSuccess) {
     c->res_ll = nullptr;
     cudaGetLastError();
   }
+  c->res_ll_cap = ll;
 }
 
 typedef int (*enqueue_fn)(rbc_ctx *, cudaStream_t, int);
@@ -883,12 +848,7 @@ int rbc_create(const rbc_grid *g, const float *a_dev, rbc_ctx **out) {
     rbc_destroy(c);
     return fail(RBC_ECUDA, "create: %s", cudaGetErrorString(e));
   }
-  if (c->res_ll) {
-    Flight &f = flight();
-    std::lock_guard<std::mutex> lock(f.m);
-    c->born = f.calls;
-    f.live.push_back(c);
-  }
+  if (c->res_ll) flight_add(&c->user);
   *out = c;
   return RBC_OK;
 }
@@ -926,11 +886,7 @@ int rbc_set_share(rbc_ctx *c, int contexts) {
 
 int rbc_destroy(rbc_ctx *c) {
   if (!c) return RBC_OK;
-  {
-    Flight &f = flight();
-    std::lock_guard<std::mutex> lock(f.m);
-    f.live.erase(std::remove(f.live.begin(), f.live.end(), c), f.live.end());
-  }
+  flight_remove(&c->user);
   cudaDeviceSynchronize();
   const int pending = check_device_error(c);
   drop_graphs(c);

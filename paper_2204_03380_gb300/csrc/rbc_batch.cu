@@ -24,6 +24,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <vector>
 
 #include "../../include/rbc.h"
@@ -621,7 +622,10 @@ struct rbc_batch {
     ResTile *tiles[2] = {nullptr, nullptr};
   };
   std::vector<Res> res;
+  std::map<int, std::vector<Res>> res_beside;    // the same groups, planned beside other loops in flight (by their number)
+  LoopUser user;
   unsigned long long *res_ll = nullptr;
+  size_t res_ll_cap = 0;
   char *res_blob = nullptr;                      // the call's tables of all groups
   size_t res_blob_cap = 0;
 };
@@ -879,9 +883,35 @@ int enq_rev(rbc_batch *b, int g, cudaStream_t s) {
   return RBC_OK;
 }
 
-void drop_res(rbc_batch *b) {
-  for (rbc_batch::Res &r : b->res) cudaFree(r.tiles[0]), cudaFree(r.tiles[1]);
-  b->res.clear();
+void drop_res(std::vector<rbc_batch::Res> *res) {
+  for (rbc_batch::Res &r : *res) cudaFree(r.tiles[0]), cudaFree(r.tiles[1]);
+  res->clear();
+}
+
+std::vector<Lay> group_layouts(const rbc_batch *b, const std::vector<int> &g) {
+  std::vector<Lay> L;
+  for (int i : g) L.push_back(b->L[i]);
+  return L;
+}
+
+// The groups with plans for `loops` loops in flight, and their tables (copied on s); false where one has none.
+bool plan_groups(rbc_batch *b, const std::vector<std::vector<int>> &groups, int loops, std::vector<rbc_batch::Res> *out,
+                 size_t *ll, cudaStream_t s) {
+  for (const std::vector<int> &g : groups) {
+    out->emplace_back();
+    rbc_batch::Res &r = out->back();
+    r.shots = g;
+    const std::vector<Lay> L = group_layouts(b, g);
+    for (int dir = 0; dir < 2; ++dir) {
+      if (!res_plan_shared(L.data(), (int)L.size(), dir, loops, false, &r.plan[dir])) return false;
+      const size_t tb = sizeof(ResTile) * r.plan[dir].tiles.size();
+      if (res_malloc((void **)&r.tiles[dir], tb) != cudaSuccess ||
+          cudaMemcpyAsync(r.tiles[dir], r.plan[dir].tiles.data(), tb, cudaMemcpyHostToDevice, s) != cudaSuccess)
+        return false;
+      *ll = std::max({*ll, res_ll_bytes(r.plan[dir], dir), res_ll_bound(L.data(), (int)L.size(), dir + 1)});
+    }
+  }
+  return true;
 }
 
 // Groups, plans and tables of the resident loops; a batch whose shots do not
@@ -889,43 +919,56 @@ void drop_res(rbc_batch *b) {
 void create_res(rbc_batch *b) {
   if (getenv("RBC_BATCH_TILES")) return;  // names the kernels of the step path
   size_t ll = 0;
-  bool ok = true;
-  for (const std::vector<int> &g : res_groups(b->L.data(), b->nshots)) {
-    b->res.emplace_back();
-    rbc_batch::Res &r = b->res.back();
-    r.shots = g;
-    std::vector<Lay> L;
-    for (int i : g) L.push_back(b->L[i]);
-    for (int dir = 0; ok && dir < 2; ++dir) {
-      if (!(ok = res_plan(L.data(), (int)L.size(), dir, 1, &r.plan[dir]))) break;
-      const size_t tb = sizeof(ResTile) * r.plan[dir].tiles.size();
-      ok = res_malloc((void **)&r.tiles[dir], tb) == cudaSuccess &&
-           cudaMemcpy(r.tiles[dir], r.plan[dir].tiles.data(), tb, cudaMemcpyHostToDevice) == cudaSuccess;
-      ll = std::max(ll, res_ll_bytes(r.plan[dir], dir));
-    }
-    if (!ok) break;
-  }
-  if (ok && ll && res_malloc((void **)&b->res_ll, ll) != cudaSuccess) b->res_ll = nullptr, ok = false;
-  if (!ok) {
-    drop_res(b);
+  if (!plan_groups(b, res_groups(b->L.data(), b->nshots), 1, &b->res, &ll, 0) ||
+      (ll && res_malloc((void **)&b->res_ll, ll) != cudaSuccess)) {
+    b->res_ll = nullptr;
+    drop_res(&b->res);
     cudaGetLastError();
   }
+  b->res_ll_cap = ll;
+}
+
+// The groups to run with `loops` loops in flight.  A batch of one group is planned beside the others (four batches of
+// one shot of 300 x 300: 6.1 us per step of all, 17.1 with the whole device each); several groups fill the device, and
+// a smaller last one gains nothing beside full ones (200 shots of 96 x 96, two batches: 33.6 us, 44.1 planned beside).
+const std::vector<rbc_batch::Res> &groups_for(rbc_batch *b, int loops, cudaStream_t s) {
+  if (loops == 1 || b->res.size() > 1) return b->res;
+  auto it = b->res_beside.find(loops);
+  if (it != b->res_beside.end()) return it->second.empty() ? b->res : it->second;
+  if (b->res_beside.size() >= 8) return b->res;
+  std::vector<rbc_batch::Res> &out = b->res_beside[loops];
+  std::vector<std::vector<int>> groups;
+  for (const rbc_batch::Res &r : b->res) groups.push_back(r.shots);
+  size_t ll = 0;
+  bool ok = plan_groups(b, groups, loops, &out, &ll, s);
+  for (rbc_batch::Res &r : out) {
+    for (int dir = 0; ok && dir < 2; ++dir)  // (a tile shape forced since the batch's creation)
+      ok = res_ll_bytes(r.plan[dir], dir) <= b->res_ll_cap;
+    if (!b->hs[0].q0) r.plan[1].steps = b->g.nt + 1;  // no fields to hand pbar from part to part in
+  }
+  if (!ok) {
+    drop_res(&out);
+    cudaGetLastError();
+    return b->res;
+  }
+  return out;
 }
 
 // The call's tables: every shot's ShotInfo, then per group the forward and
 // reverse ResShot arrays, then the reverse receiver cells of every shot.
-int upload_res(rbc_batch *b, const rbc_shot *shots, cudaStream_t s, std::vector<size_t> *o_shots) {
+int upload_res(rbc_batch *b, const std::vector<rbc_batch::Res> &res, const rbc_shot *shots, cudaStream_t s,
+               std::vector<size_t> *o_shots) {
   auto up = [](size_t n) { return (n + 63) / 64 * 64; };
   size_t need = up(sizeof(ShotInfo) * b->nshots);
   o_shots->clear();
-  for (const rbc_batch::Res &r : b->res)
+  for (const rbc_batch::Res &r : res)
     for (int dir = 0; dir < 2; ++dir) {
       o_shots->push_back(need);
       need += up(sizeof(ResShot) * r.shots.size());
     }
   std::vector<size_t> o_ptr(b->nshots), o_rec(b->nshots);
   std::vector<int> cells(b->nshots);
-  for (const rbc_batch::Res &r : b->res)
+  for (const rbc_batch::Res &r : res)
     for (size_t k = 0; k < r.shots.size(); ++k) {
       const int i = r.shots[k];
       cells[i] = (r.plan[1].tile0[k + 1] - r.plan[1].tile0[k]) * r.plan[1].warps;
@@ -950,7 +993,7 @@ int upload_res(rbc_batch *b, const rbc_shot *shots, cudaStream_t s, std::vector<
     std::memcpy(blob.data() + sizeof(ShotInfo) * i, &info, sizeof info);
   }
   size_t n = 0;
-  for (const rbc_batch::Res &r : b->res)
+  for (const rbc_batch::Res &r : res)
     for (int dir = 0; dir < 2; ++dir, ++n)
       for (size_t k = 0; k < r.shots.size(); ++k) {
         const int i = r.shots[k];
@@ -984,16 +1027,16 @@ int upload_res(rbc_batch *b, const rbc_shot *shots, cudaStream_t s, std::vector<
   return RBC_OK;
 }
 
-int run_res(rbc_batch *b, int dir, int g, size_t o_shots, cudaStream_t s, long long *launches) {
+int run_res(rbc_batch *b, const rbc_batch::Res &r, int dir, size_t o_shots, cudaStream_t s, long long *launches) {
   ResArgs A{};
-  A.tiles = b->res[g].tiles[dir];
+  A.tiles = r.tiles[dir];
   A.shots = reinterpret_cast<const ResShot *>(b->res_blob + o_shots);
   A.ll = b->res_ll;
   A.wav = b->d_wav;
   A.nt = b->g.nt;
   A.overwrite = 1;  // num / den in the pitched layout: k_batch_max and k_batch_image read them
   A.err = b->err_dev;
-  BCK(res_launch(b->res[g].plan[dir], dir, A, s, launches));
+  BCK(res_launch(r.plan[dir], dir, A, s, launches));
   return RBC_OK;
 }
 
@@ -1162,12 +1205,20 @@ int rbc_batch_create(const rbc_grid *g, int nshots, const int *nx_host, const fl
     rbc_batch_destroy(b);
     return rc;
   }
+  if (!b->res.empty()) {
+    if (cudaDeviceSynchronize() != cudaSuccess) {  // the coefficients and tables are in place for any stream
+      rbc_batch_destroy(b);
+      return bfail(RBC_ECUDA, "rbc_batch_create: %s", cudaGetErrorString(cudaGetLastError()));
+    }
+    flight_add(&b->user);
+  }
   *out = b;
   return RBC_OK;
 }
 
 int rbc_batch_destroy(rbc_batch *b) {
   if (!b) return RBC_OK;
+  flight_remove(&b->user);
   cudaDeviceSynchronize();
   drop_graphs(b);
   cudaFree(b->arena);
@@ -1180,7 +1231,8 @@ int rbc_batch_destroy(rbc_batch *b) {
   cudaFree(b->d_tile_rec);
   cudaFree(b->d_seis_t);
   cudaFree(b->d_wav);
-  drop_res(b);
+  drop_res(&b->res);
+  for (auto &r : b->res_beside) drop_res(&r.second);
   cudaFree(b->res_ll);
   cudaFree(b->res_blob);
   if (b->cap) cudaStreamDestroy(b->cap);
@@ -1298,9 +1350,10 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
     }
   // each group: forward phase then reverse phase (on the chip, or while its fields sit in L2)
   std::vector<size_t> o_shots;
+  const std::vector<rbc_batch::Res> &res = steps ? b->res : groups_for(b, flight_count(&b->user, s), s);
   if (!steps)
-    if (int rc = upload_res(b, shots, s, &o_shots)) return rc;
-  const int ng = steps ? (int)b->grp.size() - 1 : (int)b->res.size();
+    if (int rc = upload_res(b, res, shots, s, &o_shots)) return rc;
+  const int ng = steps ? (int)b->grp.size() - 1 : (int)res.size();
   for (int g = 0; g < ng; ++g) {
     cudaEvent_t e3[3] = {nullptr, nullptr, nullptr};
     if (b->timing)
@@ -1309,10 +1362,10 @@ int rbc_batch_rtm(rbc_batch *b, const rbc_shot *shots, const float *wavelet_dev,
         b->ev.push_back(e3[k]);
       }
     if (b->timing) BCK(cudaEventRecord(e3[0], s));
-    int rc = steps ? run_b(b, 0, g, s, &launches) : run_res(b, 0, g, o_shots[2 * g], s, &launches);
+    int rc = steps ? run_b(b, 0, g, s, &launches) : run_res(b, res[g], 0, o_shots[2 * g], s, &launches);
     if (rc) return rc;
     if (b->timing) BCK(cudaEventRecord(e3[1], s));
-    rc = steps ? run_b(b, 1, g, s, &launches) : run_res(b, 1, g, o_shots[2 * g + 1], s, &launches);
+    rc = steps ? run_b(b, 1, g, s, &launches) : run_res(b, res[g], 1, o_shots[2 * g + 1], s, &launches);
     if (rc) return rc;
     if (b->timing) BCK(cudaEventRecord(e3[2], s));
   }

@@ -38,6 +38,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <type_traits>
 
 #include "rbc_resident.cuh"
@@ -901,20 +902,22 @@ bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out) {
 // Four loops of 400 x 400 take 2.42 / 6.52 us so (forward / both), 6.09 / 17.77 with the whole device each and
 // 3.45 / 9.47 by launches; three of 1100 x 700 6.6 / 18.5 in turn, 7.3 / 22.6 as two and one, 5.4 / 17.4 by launches; two of
 // 2421 x 871 7.05 / 21.3 in turn, 8.8 / 36.4 by launches.
-bool res_plan_shared(const Lay *L, int dir, int loops, ResPlan *out) {
-  if (loops == 1) return res_plan(L, 1, dir, 1, out);
+bool res_plan_shared(const Lay *L, int nshots, int dir, int loops, bool steps, ResPlan *out) {
+  if (loops == 1) return res_plan(L, nshots, dir, 1, out);
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   out->variant = -1;
-  const double m = 1e-6 * L->NX * L->NZ, km = loops * m;
   const bool rev = dir == kResRev;
-  const double steps = rev ? std::max(3.9 + 0.3 * loops + 3.3 * m, (km > 3.3 ? 6.7 : 5.5) * km)
-                           : std::max(2.3 + 0.2 * loops + 1.3 * m, 2.3 * km);
-  double best = 1.25 * steps;
+  double best = 1e30;
+  if (steps) {
+    const double m = 1e-6 * L->NX * L->NZ, km = loops * m;
+    best = 1.25 * (rev ? std::max(3.9 + 0.3 * loops + 3.3 * m, (km > 3.3 ? 6.7 : 5.5) * km)
+                       : std::max(2.3 + 0.2 * loops + 1.3 * m, 2.3 * km));
+  }
   for (int j = 1; j <= std::min(loops, sms); ++j) {
     ResPlan P;
-    if (!res_plan(L, 1, dir, j, &P)) break;
+    if (!res_plan(L, nshots, dir, j, &P)) break;
     const int r = P.rz * cdiv(P.warps, 4);
     const double t = cdiv(loops, sms / P.blocks) * (rev ? 2.6 + 0.15 * r : 1.5 + 0.075 * r);
     if (t < 0.98 * best) best = t, *out = P;  // (with nothing in it, the shorter steps)
@@ -926,14 +929,73 @@ size_t res_ll_bytes(const ResPlan &P, int dir) {
   return sizeof(u64) * (size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H);
 }
 
-size_t res_ll_bound(const Lay &L, int nf) {
+size_t res_ll_bound(const Lay *L, int nshots, int nf) {
   int dev = 0, sms = 0, hmax = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   for (const Variant &V : kVariants) hmax = std::max(hmax, V.maxw * V.rz);
-  const long long gx = cdiv(L.NX, kTileX), blocks = std::min((long long)sms / 2, gx * cdiv(L.NZ, 4));
-  // ll_words(H) per block, and blocks * H <= gx * (NZ + H - 1)
-  return sizeof(u64) * nf * 2 * (size_t)(blocks * 2 * kEdge + 8 * gx * (L.NZ + hmax - 1));
+  // ll_words(H) per block; a shot's blocks * H <= gx * (NZ + H - 1)
+  long long blocks = 0, rows = 0;
+  for (int s = 0; s < nshots; ++s) {
+    const long long gx = cdiv(L[s].NX, kTileX);
+    blocks += gx * cdiv(L[s].NZ, 4);
+    rows += gx * (L[s].NZ + hmax - 1);
+  }
+  return sizeof(u64) * nf * 2 * (size_t)(std::min((long long)sms / 2, blocks) * 2 * kEdge + 8 * rows);
+}
+
+namespace {
+// The contexts and batches with resident loops that are alive, and the number of their calls so far.
+struct Flight {
+  std::mutex m;
+  std::vector<LoopUser *> live;
+  unsigned long long calls = 0;
+};
+Flight &flight() {
+  static Flight *f = new Flight();  // (outlives what is destroyed at exit)
+  return *f;
+}
+}
+
+void flight_add(LoopUser *u) {
+  Flight &f = flight();
+  std::lock_guard<std::mutex> lock(f.m);
+  cudaGetDevice(&u->dev);
+  u->born = f.calls;
+  f.live.push_back(u);
+}
+
+void flight_remove(LoopUser *u) {
+  Flight &f = flight();
+  std::lock_guard<std::mutex> lock(f.m);
+  f.live.erase(std::remove(f.live.begin(), f.live.end(), u), f.live.end());
+}
+
+// Users whose loops may run beside this call's, itself included: those called on other streams since its own last
+// call.  A program that runs k contexts on k streams calls the others in between; one that uses its contexts in turn
+// on one stream, or one context at a time, is counted as one.  At its first call (on a stream of the caller's making)
+// users that have not been called yet count too, so that a first round of calls runs side by side as well.
+// Nothing but the plan depends on the count.
+int flight_count(LoopUser *u, cudaStream_t s) {
+  unsigned long long id = 0;
+  if (cudaStreamGetId(s, &id) != cudaSuccess) return 1;
+  Flight &f = flight();
+  std::lock_guard<std::mutex> lock(f.m);
+  std::vector<unsigned long long> seen(1, id);
+  int n = 1;
+  for (const LoopUser *x : f.live) {
+    if (x == u || x->dev != u->dev) continue;
+    if (!x->called) {
+      n += !u->called && s != nullptr && s != cudaStreamLegacy;
+    } else if (x->called > std::max(u->called, u->born) &&
+               std::find(seen.begin(), seen.end(), x->on_stream) == seen.end()) {
+      seen.push_back(x->on_stream);
+      ++n;
+    }
+  }
+  u->called = ++f.calls;
+  u->on_stream = id;
+  return n;
 }
 
 namespace {

@@ -66,15 +66,24 @@ struct ResPlan {
 // they do not fit on this device at once); share: the device is shared by that
 // many such loops.
 bool res_plan(const Lay *L, int nshots, int dir, int share, ResPlan *out);
-// Plan for one of `loops` loops of a grid that run at a time: chosen for the time of all of them; false where one
-// launch per step is through sooner.
-bool res_plan_shared(const Lay *L, int dir, int loops, ResPlan *out);
+// Plan for one of `loops` such loops that run at a time: chosen for the time of all of them; false where it does not
+// fit or (steps) one launch per step is through sooner.
+bool res_plan_shared(const Lay *L, int nshots, int dir, int loops, bool steps, ResPlan *out);
+// A context or batch whose loops may run beside others', and the number of them in flight with a call of it.
+struct LoopUser {
+  int dev = 0;
+  unsigned long long called = 0, on_stream = 0;  // its last counted call (0: none yet) and that call's stream
+  unsigned long long born = 0;                   // calls counted before it was added
+};
+void flight_add(LoopUser *u);
+void flight_remove(LoopUser *u);
+int flight_count(LoopUser *u, cudaStream_t s);
 // Shots of a batch sorted into groups whose loops run at once: groups of shot
 // indices, or none when a shot does not fit.
 std::vector<std::vector<int>> res_groups(const Lay *L, int nshots);
 size_t res_ll_bytes(const ResPlan &P, int dir);
-// At least res_ll_bytes of any plan of this grid on half of the device or less, for loops of nf fields.
-size_t res_ll_bound(const Lay &L, int nf);
+// At least res_ll_bytes of any plan of these grids on half of the device or less, for loops of nf fields.
+size_t res_ll_bound(const Lay *L, int nshots, int nf);
 // cudaMalloc for the loops' own tables, without which a context or batch takes the step path; res_fail_alloc(true)
 // makes the next one fail (rbc_inject_fault).
 cudaError_t res_malloc(void **p, size_t bytes);
