@@ -216,12 +216,12 @@ def load_workload(W, args):
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the stencil
 # kernels from ncu captures (profiles/), recorded with a hash of the kernel
 # sources they were taken on: a capture of older sources reads as null.
-#   k_res_rev on the 2-D survey grid: one launch of a short record, divided by its
-#   steps (the fields are on the chip; what remains is records and their last values).
+#   k_res_rev on the 2-D survey grid: the launches of one loop, divided by its steps (the
+#   fields are on the chip; what remains is records and what one part of the loop leaves the next).
 #   3-D kernels: captured on the 380 x 380 x 280 grid as a multiple of their
 #   algorithmic bytes; the traffic of their tiles grows in proportion to the
 #   nodes, so a full 580 x 580 x 380 launch gets that multiple of its own.
-_SRC2 = ["rbc_resident.cu", "rbc_stencil.cuh", "rbc_internal.cuh"]
+_SRC2 = ["rbc_resident.cu", "rbc_resident.cuh", "rbc_tile2d.cuh", "rbc_stencil.cuh", "rbc_internal.cuh"]
 _SRC3 = ["rbc_kernels3d.cu", "rbc_stencil.cuh", "rbc_internal.cuh"]
 TRAFFIC = {
     "k_res_rev": {"sources": _SRC2, "sha1": "cc91d41be50bd9e8", "bytes_per_launch": 1.0e4, "ratio": None},
@@ -248,8 +248,29 @@ def kernel_traffic(kernel, algorithmic_bytes):
     return t["bytes_per_launch"] if t["bytes_per_launch"] else t["ratio"] * algorithmic_bytes
 
 
-def reverse_traffic(ndim, algorithmic_bytes):
-    return kernel_traffic("k_res_rev" if ndim == 2 else "k_rev3d_tma", algorithmic_bytes)
+# Packed fp32 operations of the resident 2-D loops per four nodes and field (rbc_stencil.cuh), each two cycles of a
+# scheduler's FMA pipe per warp.
+PACKED_OPS = 59
+
+
+def issue_roofline(nodes, fields, step_s, sms, sm_mhz):
+    """Roofline of a resident 2-D loop: its packed fp32 operations per second
+    against what the SMs' schedulers issue at the clock it ran at."""
+    achieved = nodes / 4 * PACKED_OPS * fields / step_s / 1e9
+    peak = sms * 4 * 32 / 2 * sm_mhz * 1e6 / 1e9
+    return {"bound": "fp32 issue", "achieved": achieved, "peak": peak, "unit": "G packed fp32 op/s",
+            "frac": achieved / peak, "peak_source": f"{sms} SMs x 4 schedulers x 16 lanes per cycle at {sm_mhz:.0f} MHz",
+            "traffic": None, "launch_us": step_s * 1e6}
+
+
+def resident_loops(launches, loops, nt):
+    """(forward, reverse): whether the loops of `loops` 2-D shots of nt steps
+    ran on the chip, from the launches they took.  A loop by steps is nt
+    launches or more (its forward half that with two levels per launch); a
+    resident one, even in parts, far fewer, and up to eight serve a shot's
+    records and images."""
+    per = max(0.0, launches / loops - 8) / nt
+    return per < 0.25 or 0.75 < per < 1.4, per < 0.75
 
 
 def measured_peaks():
@@ -397,7 +418,21 @@ def run_batch(args, rank, world):
     rev_bytes = sum(28 * p + 16 * q for p, q in zip(npads, nints))
     rev_s = phases["rev_ms"] / 1e3 / max(phases["rev_launches"], 1)
     fwd_s = phases["fwd_ms"] / 1e3 / max(phases["fwd_launches"], 1)
-    achieved = rev_bytes / rev_s / 1e9
+    on_chip = launches < args.steps * w.nt
+    if on_chip:
+        sms = torch.cuda.get_device_properties(local).multi_processor_count
+        mhz = clocks.get("sm_mhz") or 2070.0
+        roofline = dict(issue_roofline(sum(npads), 2, rev_s, sms, mhz),
+                        kernel="k_res_rev (fused reverse pass, all shots, per time step)",
+                        forward_kernel=dict(issue_roofline(sum(npads), 1, fwd_s, sms, mhz), kernel="k_res_fwd"))
+    else:
+        achieved = rev_bytes / rev_s / 1e9
+        roofline = {"bound": "hbm", "kernel": "the batch's reverse kernel (all shots, per time step)",
+                    "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+                    "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s",
+                    "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_s * 1e6,
+                    "forward_kernel": {"kernel": "the batch's forward kernel", "launch_us": fwd_s * 1e6,
+                                       "achieved": 16 * sum(npads) / fwd_s / 1e9}}
     if rank != 0:
         return
     cpu = None
@@ -424,14 +459,9 @@ def run_batch(args, rank, world):
            "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
            "config": {"workload": w.name, "shots": len(shots), "widths": [min(s["width"] for s in inp["shots"]),
                                                                          max(s["width"] for s in inp["shots"])],
-                      "nt": w.nt, "autotuned": info, "s_per_shot": el / args.steps / len(shots),
+                      "nt": w.nt, "autotuned": None if on_chip else info, "s_per_shot": el / args.steps / len(shots),
                       "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB write)"},
-           "roofline": {"bound": "hbm", "kernel": "k_res_rev (fused reverse pass, all shots, per time step)",
-                        "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                        "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s",
-                        "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_s * 1e6,
-                        "forward_kernel": {"kernel": "k_res_fwd", "launch_us": fwd_s * 1e6,
-                                           "achieved": 16 * sum(npads) / fwd_s / 1e9}},
+           "roofline": roofline,
            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(out), flush=True)
     if dist is not None:
@@ -732,7 +762,21 @@ def run_fwi(args, rank, world):
     fwd_launch_s = t_f / (len(srcs) * w.nt)
     peaks = measured_peaks()
     peak = peaks["hbm_gbs"] if peaks else 6800.0
-    achieved = rev_bytes / rev_launch_s / 1e9
+    res_f, res_r = resident_loops(launches, len(srcs) * args.steps, w.nt)
+    what = "gradient mode (reconstruction + exact adjoint + gradient; shots on concurrent streams: backward phase / time steps)"
+    if res_f and res_r:
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        mhz = clocks.get("sm_mhz") or 2070.0
+        roofline = dict(issue_roofline(w.npad, 2, rev_launch_s, sms, mhz), kernel="k_res_rev in " + what,
+                        forward_kernel=dict(issue_roofline(w.npad, 1, fwd_launch_s, sms, mhz), kernel="k_res_fwd"))
+    else:
+        achieved = rev_bytes / rev_launch_s / 1e9
+        roofline = {"bound": "hbm", "kernel": ("k_res_rev in " if res_r else "k_rev2d_tile in ") + what,
+                    "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+                    "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
+                    "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_launch_s * 1e6,
+                    "forward_kernel": {"kernel": "k_res_fwd" if res_f else "k_fwd2d", "launch_us": fwd_launch_s * 1e6,
+                                       "achieved": 16 * w.npad / fwd_launch_s / 1e9}}
     # end to end: observed records from pinned host memory, gradient and misfit read back
     e2e = None
     if not args.no_e2e:
@@ -772,13 +816,7 @@ def run_fwi(args, rank, world):
                       "s_per_gradient": t_grad, "forward_phase_s": t_f, "backward_phase_s": t_b,
                       "shot_streams": shot_streams(g, len(srcs)), "misfit": float(J.detach()),
                       "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB write)"},
-           "roofline": {"bound": "hbm", "kernel": "k_res_rev in gradient mode (reconstruction + exact adjoint + gradient; "
-                                                  "shots on concurrent streams: backward phase / time steps)",
-                        "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                        "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
-                        "traffic": None, "bytes_per_launch": rev_bytes, "launch_us": rev_launch_s * 1e6,
-                        "forward_kernel": {"kernel": "k_res_fwd", "launch_us": fwd_launch_s * 1e6,
-                                           "achieved": 16 * w.npad / fwd_launch_s / 1e9}},
+           "roofline": roofline,
            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(out), flush=True)
 
@@ -1031,24 +1069,30 @@ def main():
     peaks = measured_peaks()
     peak = peaks["hbm_gbs"] if peaks else 6800.0
     rev_launch_s = phases["rev_ms"] / 1e3 / max(phases["rev_launches"], 1)
-    achieved = rev_bytes_per_launch(w) / rev_launch_s / 1e9
     fwd_launch_s = phases["fwd_ms"] / 1e3 / max(phases["fwd_launches"], 1)
-    kname = "k_res_rev" if w.ndim == 2 else "k_rev3d_tma"
-    roofline = {"bound": "hbm", "kernel": f"{kname} (fused reverse pass)", "achieved": achieved, "peak": peak,
-                "unit": "GB/s", "frac": achieved / peak,
+    res_f, res_r = resident_loops(launches, args.steps * B, w.nt) if w.ndim == 2 else (False, False)
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
+    mhz = clocks.get("sm_mhz") or 2070.0
+
+    def phase_roofline(kernel, on_chip, fields, nbytes, launch_s, traffic):
+        if on_chip:
+            return dict(issue_roofline(w.npad, fields, launch_s, sms, mhz), kernel=kernel, traffic=traffic,
+                        note="one launch per part of a time loop, the fields on the chip: time and traffic are per "
+                             "time step")
+        ach = nbytes / launch_s / 1e9
+        return {"kernel": kernel, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s",
-                "traffic": (reverse_traffic(w.ndim, rev_bytes_per_launch(w))
-                            if w.ndim == 3 or tuple(w.padded) == (871, 2421) else None),
-                "traffic_source": ("ncu dram bytes of k_res_rev's loop on this grid, per step" if w.ndim == 2 else
-                                   "ncu dram bytes of k_rev3d_tma on 380x380x280, scaled by the algorithmic bytes"),
-                "bytes_per_launch": rev_bytes_per_launch(w), "launch_us": rev_launch_s * 1e6,
-                "forward_kernel": {"kernel": "k_res_fwd" if w.ndim == 2 else "k_fwd3d_tma",
-                                   "achieved": fwd_bytes_per_launch(w) / fwd_launch_s / 1e9,
-                                   "launch_us": fwd_launch_s * 1e6,
-                                   "bytes_per_launch": fwd_bytes_per_launch(w)},
-                "note": ("one launch per time loop, the fields on the chip: bytes and time are per time step, "
-                         "the kernel is bound by fp32 issue, not by HBM") if w.ndim == 2 else
-                        "working set of 4 GB: DRAM-bound"}
+                "traffic": traffic, "bytes_per_launch": nbytes, "launch_us": launch_s * 1e6}
+
+    kr = "k_rev3d_tma" if w.ndim == 3 else "k_res_rev" if res_r else "k_rev2d_tile"
+    kf = "k_fwd3d_tma" if w.ndim == 3 else "k_res_fwd" if res_f else "k_fwd2d"
+    captured = w.ndim == 3 or res_r and tuple(w.padded) == (871, 2421)
+    roofline = phase_roofline(f"{kr} (fused reverse pass)", res_r, 2, rev_bytes_per_launch(w), rev_launch_s,
+                              kernel_traffic(kr, rev_bytes_per_launch(w)) if captured else None)
+    if captured:
+        roofline["traffic_source"] = ("ncu dram bytes of k_res_rev's loop on this grid, per step" if w.ndim == 2 else
+                                      "ncu dram bytes of k_rev3d_tma on 380x380x280, scaled by the algorithmic bytes")
+    roofline["forward_kernel"] = phase_roofline(kf, res_f, 1, fwd_bytes_per_launch(w), fwd_launch_s, None)
 
     if storage:
         nshots_ph = max(phases["shots"], 1)
@@ -1057,9 +1101,13 @@ def main():
         achieved = (fb + rb) / (fwd_s + rev_s) / 1e9
         roofline = {"bound": "hbm", "kernel": "k_res_fwd/k_res_rev loops or k_fwd3d_tma steps + store/image kernels (whole phases)",
                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                    "peak_source": roofline["peak_source"], "traffic": None,
+                    "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback 6.8 TB/s", "traffic": None,
                     "forward_phase": {"bytes": fb, "s": fwd_s, "GB/s": fb / fwd_s / 1e9},
                     "reverse_phase": {"bytes": rb, "s": rev_s, "GB/s": rb / rev_s / 1e9}}
+        if w.ndim == 2 and launches < args.steps * B * w.nt:
+            roofline = dict(issue_roofline(w.npad, 2, (fwd_s + rev_s) / w.nt, sms, mhz),
+                            kernel="k_res_fwd and k_res_rev in storage mode (a step of both phases)",
+                            forward_phase={"s": fwd_s}, reverse_phase={"s": rev_s})
     if rank != 0:
         R.rbc_destroy(ctx)
         if dist is not None:
