@@ -725,6 +725,7 @@ int run_loop(rbc_ctx *c, int kind, enqueue_fn fn, cudaStream_t s) {
 int run_model(rbc_ctx *c, const int *src, int nrec, const int *rec, const float *wavelet, cudaStream_t s) {
   begin_loops(c, s);
   const ResPlan *res = resident(c, kResFwd);
+  if (res && res_many_receivers(*res, nrec)) res = nullptr;
   int rc = res ? check_nodes(c, src, nrec, rec) : upload_shot(c, src, nrec, rec, 1, s);
   if (rc) return rc;
   if (res && ((rc = check_capture(s)) || (rc = ensure_receivers(c, std::max(nrec, 1))))) return rc;

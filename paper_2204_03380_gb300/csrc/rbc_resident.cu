@@ -265,6 +265,7 @@ __device__ __forceinline__ void sweep(const Place &W, const float *smem, int c0,
 
 // This warp's receivers: the first K * 32 in registers (node's place in the
 // tile, receiver), the rest read from the table at every step.
+constexpr int rec_regs(int rz) { return rz < 4 ? 4 : 1; }  // K of the forward loop
 template <int K>
 struct Recs {
   int beg, end, loc[K], id[K];
@@ -342,7 +343,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
   const int2 *cell_rec = S.cell_rec;
   float *seis_t = S.seis_t;
   const int cell = (blockIdx.x - S.tile0) * blockDim.y + w;
-  constexpr int K = RZ < 4 ? 4 : 1;
+  constexpr int K = rec_regs(RZ);
   Recs<K> rec;
   rec.load(S.cell_ptr, cell_rec, cell, lane, A.sample != 0);
   auto record = [&](int n, const float *p) {  // p^n at this warp's receivers
@@ -923,6 +924,14 @@ bool res_plan_shared(const Lay *L, int nshots, int dir, int loops, bool steps, R
     if (t < 0.98 * best) best = t, *out = P;  // (with nothing in it, the shorter steps)
   }
   return out->variant >= 0;
+}
+
+// A warp records what its registers do not hold in turns of 32, each a table read from L2 behind its sweep: a step of
+// 1100 x 700 takes 2.4 us with 1100 receivers, 6.0 with 86 k (22 more per warp), 10.3 with 193 k (90 more) and 35 with
+// every node; by launches, whose blocks hide the reads behind one another, 3.7, 6.4, 10.0 and 30.  (2421 x 871: 9.4
+// against 10.3 with 132 k receivers, 26.9 against 24.1 with 528 k.)
+bool res_many_receivers(const ResPlan &P, int nrec) {
+  return nrec > (64 + 32LL * rec_regs(P.rz)) * P.blocks * P.warps;
 }
 
 size_t res_ll_bytes(const ResPlan &P, int dir) {

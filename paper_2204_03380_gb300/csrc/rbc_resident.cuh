@@ -94,6 +94,8 @@ void res_cell(const ResPlan &P, const Lay &L, int x, int z, int *cell, int *loc)
 // Receiver cells of one shot (its tiles * warps cells): CSR pointers and
 // {place in the tile, receiver}, positions offset by `base`.
 void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *rec, int base, int *ptr, int2 *out);
+// Whether a forward loop that records nrec receivers is through sooner by launches.
+bool res_many_receivers(const ResPlan &P, int nrec);
 // Parts of a loop of n steps (forward: nt; reverse: nt + 1).
 inline int res_parts(const ResPlan &P, int n) { return (n + P.steps - 1) / P.steps; }
 cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches);

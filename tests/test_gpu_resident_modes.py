@@ -196,3 +196,28 @@ def test_a_batch_in_parts_gives_the_same_bits(monkeypatch):
             R.rbc_batch_destroy(b)
     assert all(torch.equal(imgs[0], i) for i in imgs) and float(imgs[0].abs().max()) > 0
     assert torch.equal(imgs[0][:, :150], imgs[0][:, 150:])
+
+
+@pytest.mark.parametrize("tile,every,steps", [("2,9", 1, True), ("2,9", 4, False), ("0,8", 1, False)])
+def test_records_of_most_nodes_match_whichever_path_takes_them(tile, every, steps, monkeypatch):
+    # more receivers than a warp's turns are worth go by launches: 4 rows per warp hold 32 and take 64 more
+    import paper_2204_03380_gb300 as R
+    w, v, src, _, wav = _case("dense", 120, 215, 9, 60)
+    X, Z = np.meshgrid(np.arange(0, w.nx + 2 * w.nb, every), np.arange(w.nz + 2 * w.nb))
+    rec = np.stack([X.ravel(), 0 * X.ravel(), Z.ravel()], 1).astype(np.int32)
+    wt = torch.tensor(np.asarray(wav, np.float32), device="cuda")
+    out = []
+    for t in ("step", tile):
+        _env(monkeypatch, t)
+        g, a, _ = gpu_build(R, torch, w, v)
+        seis = torch.zeros((len(rec), w.nt + 1), device="cuda")
+        ctx = R.rbc_create(g, a)
+        try:
+            R.rbc_launch_count(True)
+            R.rbc_model(ctx, src, wt, rec, seis)
+            torch.cuda.synchronize()
+            assert (R.rbc_launch_count() > w.nt) == (steps or t == "step")
+        finally:
+            R.rbc_destroy(ctx)
+        out.append(seis.cpu())
+    assert torch.equal(*out) and float(out[0].abs().max()) > 0
