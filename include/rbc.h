@@ -370,7 +370,7 @@ int rbc_cnn_infer(const float *params_dev, int nimg, int H, int W,
 
 /* rbc_cnn_infer on images that are slices of a larger array: image i, row r
  * starts at x_dev + i x_img + r x_row (strides in values, >= 0; the values of a
- * row are consecutive), and y_dev likewise.  y_dev's images must not overlap each
+ * row are consecutive), and y_dev likewise (here 4-byte alignment will do).  y_dev's images must not overlap each
  * other, and overlap x_dev's only where they are the same.
  * Errors: RBC_EINVAL, RBC_ECUDA. */
 int rbc_cnn_infer_strided(const float *params_dev, int nimg, int H, int W,

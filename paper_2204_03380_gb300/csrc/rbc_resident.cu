@@ -22,10 +22,13 @@
 // 0.69 us for every ten-row warp on a scheduler (143 clocks per row; 59 packed
 // operations take 118), so a survey tile (11 warps) 2.9 us, and the exchange
 // adds 0.5 us; on small grids the fixed part and the exchange are all there
-// is.  Measured (us per step; before, one launch per step): survey forward 3.4
-// (6.1), forward + reverse 10.9 (18.8); 300 x 300 forward 1.5 (2.7), forward +
-// reverse 4.5 (6.7).  Tensor memory for a and the sums: 8 us per reverse step
+// is.  Measured (us per step; before, one launch per step): survey forward 3.5
+// (6.1), forward + reverse 10.5 (18.8); 300 x 300 forward 1.5 (2.7), forward +
+// reverse 4.4 (6.7).  Tensor memory for a and the sums: 8 us per reverse step
 // against 12.4 with the sums in registers (spilled) and a read from L2 twice.
+// Reverse kernels of 16 warps have 128 registers a thread and still spill some:
+// 156 bytes stored (7 rows per warp, imaging), 124 (7, gradient), 68 (2,
+// imaging), 28 and 12 (4); ten rows of 11 warps, with 162 registers, none.
 // Tried and not kept: a warp-to-warp order (mbarriers) instead of the block
 // barrier at each step -- the warps drift apart and their unrolled rows no
 // longer fit the instruction cache (18 us per reverse step); the same with the
@@ -802,11 +805,11 @@ size_t res_smem(int dir, int H, const Variant &V) {
   if (dir == kResFwd) rows = 2 * (H + 8) + H;
   else rows = V.tight ? nb * H + 4 : nb * (H + 8) + (V.tm ? 0 : H);
   const size_t need = sizeof(float) * (rows * kTileX + 8 * (size_t)H) + (dir != kResFwd && V.tm ? 16 : 0);
-  // Kernels that allocate no tensor memory: more than half an SM's shared
-  // memory keeps a second block off it.  Loops in flight together otherwise land
+  // More than half an SM's shared memory keeps a second loop's block off it.  Loops in flight together otherwise land
   // on the same SMs while others idle (four shots of 300 x 300 at once: 3.6 -> 2.4 us a step;
-  // one shot of 2301 x 751: 3.64 -> 3.42).
-  return dir == kResFwd || !V.tm ? std::max(need, (size_t)116 * 1024) : need;
+  // one shot of 2301 x 751: 3.64 -> 3.42), and two loops whose blocks share SMs could each hold tensor memory that
+  // the other waits for.
+  return std::max(need, (size_t)116 * 1024);
 }
 
 } // namespace
@@ -1039,9 +1042,10 @@ void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *r
 // step by rows per warp, measured on grids that fill the device (us).
 std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
   const double step_us[] = {4.4, 5.5, 7.3, 9.4, 11.0};
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, maxsm = 0;
   std::vector<std::vector<int>> best;
   if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return best;
   std::vector<int> order(nshots);
@@ -1055,7 +1059,7 @@ std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
     const Variant &V = kVariants[v];
     const int cap = sms;
     int hmax = V.maxw * V.rz;
-    while (hmax > V.rz && res_smem(kResRev, hmax, V) > 227 * 1024) hmax -= V.rz;
+    while (hmax > V.rz && res_smem(kResRev, hmax, V) > (size_t)maxsm) hmax -= V.rz;
     std::vector<int> tiles(nshots);
     bool fits = true;
     for (int i = 0; i < nshots; ++i) {

@@ -52,7 +52,7 @@ def _pool(grid, a, n, device):
     while len(pool) < n:
         pool.append((N.rbc_create(grid, a), torch.cuda.Stream(device)))
     for ctx, _ in pool[:n]:
-        N.rbc_set_share(ctx, n)   # (nothing to do unless the number of shots in flight changed)
+        N.rbc_set_share(ctx, n)   # (a number for the plans of the calls that follow)
     return pool[:n]
 
 

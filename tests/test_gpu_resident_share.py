@@ -197,3 +197,34 @@ def test_batches_on_streams_of_their_own_run_side_by_side():
         torch.cuda.synchronize()
         for b in batches:
             R.rbc_batch_destroy(b)
+
+
+def test_loops_with_tensor_memory_in_flight_together(monkeypatch):
+    # reverse loops of low tiles, whose fields take little of an SM: 4, 7 and 10 rows per warp hold 256, 512 and 512
+    # tensor-memory columns, which must not meet on an SM
+    import paper_2204_03380_gb300 as R
+    runs = []
+    for k, tile in enumerate(("2,3", "3,2", "4,1", "2,5")):
+        monkeypatch.setenv("RBC_RES_TILE", tile)
+        ctx, g, _, src, rec, wt, seis = _ctx(R, f"tm{k}", 500, 250, 20, 300, seed=k)
+        num = [torch.empty(g.interior, device="cuda") for _ in range(3)]
+        runs.append((ctx, src, wt, rec, seis, num, torch.cuda.Stream()))
+    flags = R.RBC_REINJECT_SOURCE | R.RBC_ZERO_FIRST
+    R.rbc_launch_count(True)
+    try:
+        for n in range(2):   # one by one, then in flight together and several times over
+            for _ in range(1 + 3 * n):
+                for ctx, src, wt, rec, seis, num, s in runs:
+                    R.rbc_set_share(ctx, 1)
+                    if n == 0:
+                        R.rbc_model(ctx, src, wt, rec, seis)
+                    R.rbc_rtm_shot(ctx, src, wt, rec, seis, flags, num[n], num[2], stream=s if n else None)
+            torch.cuda.synchronize()
+        assert R.rbc_launch_count() < 300
+        for ctx, src, wt, rec, seis, num, _ in runs:
+            assert torch.equal(*num[:2]) and float(num[0].abs().max()) > 0
+            R.rbc_model(ctx, src, wt, rec, seis)   # (an earlier wait that ran out would be reported)
+    finally:
+        torch.cuda.synchronize()
+        for r in runs:
+            R.rbc_destroy(r[0])
