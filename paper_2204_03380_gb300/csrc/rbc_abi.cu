@@ -129,8 +129,8 @@ struct rbc_ctx {
   int *err_host = nullptr;
   int *err_dev = nullptr;
   int fault = 0;  // rbc_inject_fault: applies to the next call only
-  // 2-D grids that fit on the chip: the whole time loop as one launch
-  // (rbc_resident.cu), by kResFwd .. kResStore (variant -1: one launch per step)
+  // 2-D grids that fit on the chip: a time loop as one launch or a few
+  // (rbc_resident.cu), planned by kResFwd .. kResStore (variant -1: one launch per step)
   std::map<int, std::array<ResPlan, 3>> res;  // the plans, by `loops` (host tables)
   unsigned long long *res_ll = nullptr;       // room for the exchange words of any of them (null: no resident loops)
   size_t res_ll_cap = 0;
