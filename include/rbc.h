@@ -477,11 +477,15 @@ int rbc_model_static(const rbc_grid *g, const float *a_dev,
  * and the next call on the context returns RBC_ETIMEOUT (the results of the
  * faulted call are invalid).  Nothing faults, traps or hangs.  mode 0
  * clears a pending request.  With ctx = NULL the request applies to the next
- * 3-D rbc_model_static call instead (reported by the call after it).  mode 3
+ * 3-D rbc_model_static call instead (reported by the call after it).  mode 2
+ * (2-D contexts): the first part of the next call's first resident loop is not
+ * launched (where the loop has several), so that the blocks of the second wait
+ * for edges that were never sent, give up after some seconds and report it the
+ * same way; the parts after it return at once.  mode 3
  * (ctx = NULL): the next rbc_create or rbc_batch_create of a 2-D grid finds no
  * memory for the tables of its one-launch time loops and, as it would then,
  * steps with one launch per step instead; mode 0 or 1 with NULL clears it.
- * Errors: RBC_EINVAL, RBC_ENOTSUP (2-D context).
+ * Errors: RBC_EINVAL, RBC_ENOTSUP (mode 1 on a 2-D context, 2 on a 3-D one).
  */
 int rbc_inject_fault(rbc_ctx *ctx, int mode);
 

@@ -250,8 +250,13 @@ int upload_shot(rbc_ctx *c, const int *src, int nrec, const int *rec, int reinje
 void begin_loops(rbc_ctx *c, cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   c->loops = 1;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return;
-  const int n = c->res_ll ? flight_count(&c->user, s) : 1;
+  if (!c->res_ll) return;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (st != cudaStreamCaptureStatusNone) return;
+  const int n = flight_count(&c->user, s);
   c->loops = c->share ? c->share : n;
 }
 
@@ -260,7 +265,7 @@ const ResPlan *res_plan_of(rbc_ctx *c, int dir) {
   if (!c->res_ll) return nullptr;
   auto it = c->res.find(c->loops);
   if (it == c->res.end()) {
-    if (c->res.size() >= 8) c->res.clear();
+    if (c->res.size() >= 32) c->res.clear();
     it = c->res.emplace(c->loops, std::array<ResPlan, 3>()).first;
     for (int d = 0; d < 3; ++d)
       if (res_plan_shared(&c->L, 1, d, c->loops, true, &it->second[d]) &&
@@ -298,6 +303,7 @@ int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec
     c->res_blob_cap = most;
   }
   std::vector<char> blob(need, 0);
+  const bool withhold = c->fault == 2;
   const ShotInfo info = shot_info(c, src, nrec, reinject);
   std::memcpy(blob.data(), &info, sizeof info);
   std::memcpy(blob.data() + o_tile, P.tiles.data(), tb);
@@ -339,7 +345,7 @@ int run_resident(rbc_ctx *c, const ResPlan &P, int dir, const int *src, int nrec
   A.stride = stride;
   A.err = c->err_dev;
   long long launches = 0;
-  const cudaError_t e = res_launch(P, dir, A, s, &launches);
+  const cudaError_t e = res_launch(P, dir, A, s, &launches, withhold);
   g_launches += launches;
   CK(e);
   return RBC_OK;
@@ -1187,7 +1193,7 @@ int rbc_phase_timing(rbc_ctx *c, int enable, double *out) {
 }
 
 int rbc_inject_fault(rbc_ctx *c, int mode) {
-  if (mode != 0 && mode != 1 && !(mode == 3 && !c)) return fail(RBC_EINVAL, "unknown fault mode %d", mode);
+  if (mode != 0 && mode != 1 && !(mode == 2 && c) && !(mode == 3 && !c)) return fail(RBC_EINVAL, "unknown fault mode %d", mode);
   if (!c) res_fail_alloc(mode == 3);
   if (mode == 3) return RBC_OK;
   if (!c) {  // the next 3-D rbc_model_static call
@@ -1195,6 +1201,7 @@ int rbc_inject_fault(rbc_ctx *c, int mode) {
     return RBC_OK;
   }
   if (mode == 1 && c->L.ndim != 3) return fail(RBC_ENOTSUP, "fault mode 1 needs a 3-D context");
+  if (mode == 2 && c->L.ndim != 2) return fail(RBC_ENOTSUP, "fault mode 2 needs a 2-D context");
   c->fault = mode;
   return RBC_OK;
 }

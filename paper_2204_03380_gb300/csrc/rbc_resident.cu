@@ -311,7 +311,12 @@ __device__ __forceinline__ void keep_level(const ResArgs &A, const ResShot &S, c
 
 // Whether an earlier part gave up waiting (its words never came: no use waiting for them in this one).  A block barrier.
 __device__ __forceinline__ bool given_up(const ResArgs &A, int tid) {
-  return __syncthreads_or(A.t0 > 0 && tid == 0 && *(volatile const int *)A.err != 0);
+  return __syncthreads_or(A.t0 > 0 && tid == 0 && *(volatile const int *)A.gave_up != 0);
+}
+
+__device__ __forceinline__ void give_up(const ResArgs &A) {
+  *(volatile int *)A.gave_up = 1;
+  atomicOr_system(A.err, 1);  // reported by the next call, which clears it: later parts go by the mark above
 }
 
 // ------------------------------------------------------------- forward ----
@@ -396,7 +401,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_fwd(const ResArgs A, const
     if (rec.end > rec.beg) record(n, cur);
     f = f_next * fsc;
     if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicOr_system(A.err, 1);
+      if (tid == 0) give_up(A);
       return;
     }
   }
@@ -726,7 +731,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) k_res_rev(const ResArgs A, const
       if (t < nt) halo_out<RZ>(W, FB, (uint32_t)t + 1, bn);
     }
     if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicOr_system(A.err, 1);
+      if (tid == 0) give_up(A);
       break;
     }
   }
@@ -919,7 +924,7 @@ bool res_plan_shared(const Lay *L, int nshots, int dir, int loops, bool steps, R
     best = 1.25 * (rev ? std::max(3.9 + 0.3 * loops + 3.3 * m, (km > 3.3 ? 6.7 : 5.5) * km)
                        : std::max(2.3 + 0.2 * loops + 1.3 * m, 2.3 * km));
   }
-  for (int j = 1; j <= std::min(loops, sms); ++j) {
+  for (int j = 1; j <= std::min(loops, 16); ++j) {  // (plans for a sixteenth of the device leave room for more)
     ResPlan P;
     if (!res_plan(L, nshots, dir, j, &P)) break;
     const int r = P.rz * cdiv(P.warps, 4);
@@ -938,7 +943,7 @@ bool res_many_receivers(const ResPlan &P, int nrec) {
 }
 
 size_t res_ll_bytes(const ResPlan &P, int dir) {
-  return sizeof(u64) * (size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H);
+  return sizeof(u64) * ((size_t)P.blocks * (dir == kResRev ? 2 : 1) * 2 * ll_words(P.H) + 2);  // (words, then the mark)
 }
 
 size_t res_ll_bound(const Lay *L, int nshots, int nf) {
@@ -953,7 +958,7 @@ size_t res_ll_bound(const Lay *L, int nshots, int nf) {
     blocks += gx * cdiv(L[s].NZ, 4);
     rows += gx * (L[s].NZ + hmax - 1);
   }
-  return sizeof(u64) * nf * 2 * (size_t)(std::min((long long)sms / 2, blocks) * 2 * kEdge + 8 * rows);
+  return sizeof(u64) * (nf * 2 * (size_t)(std::min((long long)sms / 2, blocks) * 2 * kEdge + 8 * rows) + 2);
 }
 
 namespace {
@@ -990,7 +995,10 @@ void flight_remove(LoopUser *u) {
 // Nothing but the plan depends on the count.
 int flight_count(LoopUser *u, cudaStream_t s) {
   unsigned long long id = 0;
-  if (cudaStreamGetId(s, &id) != cudaSuccess) return 1;
+  if (cudaStreamGetId(s, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
   Flight &f = flight();
   std::lock_guard<std::mutex> lock(f.m);
   std::vector<unsigned long long> seen(1, id);
@@ -1085,7 +1093,8 @@ std::vector<std::vector<int>> res_groups(const Lay *L, int nshots) {
   return best;
 }
 
-cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches) {
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches,
+                       bool withhold) {
   const Variant &V = kVariants[P.variant];
   const void *fn = V.fn[dir == kResStore ? 3 : dir == kResRev && A.grad ? 2 : dir];
   cudaError_t e = cudaMemsetAsync(A.ll, 0, res_ll_bytes(P, dir), s);
@@ -1100,10 +1109,11 @@ cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   ResArgs a = A;
+  a.gave_up = reinterpret_cast<int *>(A.ll + res_ll_bytes(P, dir) / sizeof(u64) - 2);
   int H = P.H;
   void *args[2] = {&a, &H};
   const int n = dir == kResFwd ? A.nt : A.nt + 1, parts = res_parts(P, n);
-  for (int k = 0; k < parts && e == cudaSuccess; ++k) {
+  for (int k = withhold && parts > 1 ? 1 : 0; k < parts && e == cudaSuccess; ++k) {
     a.t0 = (int)((long long)n * k / parts);
     a.t1 = (int)((long long)n * (k + 1) / parts);
     e = cudaLaunchKernelExC(&cfg, fn, args);

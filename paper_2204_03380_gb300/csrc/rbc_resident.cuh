@@ -48,6 +48,7 @@ struct ResArgs {
   float *store;             // storage RTM: the kept levels, every `stride` steps (0: none kept)
   int stride;
   int *err;
+  int *gave_up;             // this loop's own mark of a wait that gave up (behind its exchange words), for its later parts
 };
 
 // Tiling of a resident loop over one or several grids: `warps` warps of `rz`
@@ -98,6 +99,8 @@ void res_cells(const ResPlan &P, const Lay &L, int cells, int nrec, const int *r
 bool res_many_receivers(const ResPlan &P, int nrec);
 // Parts of a loop of n steps (forward: nt; reverse: nt + 1).
 inline int res_parts(const ResPlan &P, int n) { return (n + P.steps - 1) / P.steps; }
-cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches);
+// withhold: the first of several parts is not launched (rbc_inject_fault), so that the second waits in vain.
+cudaError_t res_launch(const ResPlan &P, int dir, const ResArgs &A, cudaStream_t s, long long *launches,
+                       bool withhold = false);
 
 } // namespace rbc
