@@ -422,8 +422,9 @@ int rbc_get_panels(rbc_ctx *ctx, float *prev_dev, float *last_dev,
  * the caller's stream.  enable = 1 clears the record and starts timing the
  * forward and reverse phases of every following rbc_rtm_shot on this
  * context; enable = 0 stops, synchronises and writes out[0] = forward ms,
- * out[1] = reverse ms, out[2] = forward stencil launches, out[3] = reverse
- * stencil launches, out[4] = shots timed (out may be NULL).  The phase times
+ * out[1] = reverse ms, out[2] = forward time steps, out[3] = reverse time
+ * steps (a stencil launch each, or a step of a loop that stays on the chip),
+ * out[4] = shots timed (out may be NULL).  The phase times
  * include the few memsets that clear the fields.  Errors: RBC_EINVAL,
  * RBC_ECUDA.
  */
