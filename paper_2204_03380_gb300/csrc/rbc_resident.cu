@@ -27,8 +27,8 @@
 // reverse 4.4 (6.7).  Tensor memory for a and the sums: 8 us per reverse step
 // against 12.4 with the sums in registers (spilled) and a read from L2 twice.
 // Reverse kernels of 16 warps have 128 registers a thread and still spill some:
-// 156 bytes stored (7 rows per warp, imaging), 124 (7, gradient), 68 (2,
-// imaging), 28 and 12 (4); ten rows of 11 warps, with 162 registers, none.
+// 156 bytes stored (7 rows per warp, imaging), 134 (7, gradient), 64 (2,
+// imaging), 28 and 4 (4); ten rows of 11 warps, with 162 registers, none.
 // Tried and not kept: a warp-to-warp order (mbarriers) instead of the block
 // barrier at each step -- the warps drift apart and their unrolled rows no
 // longer fit the instruction cache (18 us per reverse step); the same with the

@@ -228,3 +228,44 @@ def test_loops_with_tensor_memory_in_flight_together(monkeypatch):
         torch.cuda.synchronize()
         for r in runs:
             R.rbc_destroy(r[0])
+
+
+def test_contexts_of_several_host_threads():
+    # every thread makes, uses and destroys contexts of its own on a stream of its own while the others do; the counts
+    # and so the plans change from call to call, the records do not
+    import threading
+
+    import paper_2204_03380_gb300 as R
+    cases = [_ctx(R, f"thr{k}", 120 + 90 * k, 80 + 40 * k, 10, 120, seed=k) for k in range(5)]
+    want = []
+    for ctx, _, _, src, rec, wt, out in cases:
+        R.rbc_model(ctx, src, wt, rec, out)
+        torch.cuda.synchronize()
+        want.append(out.clone())
+        R.rbc_destroy(ctx)
+    errors = []
+
+    def work(k):
+        try:
+            _, g, a, src, rec, wt, _ = cases[k]
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                for _ in range(3):
+                    ctx = R.rbc_create(g, a)
+                    try:
+                        for _ in range(6):
+                            got = torch.zeros_like(want[k])
+                            R.rbc_model(ctx, src, wt, rec, got, stream=s)
+                            s.synchronize()
+                            assert torch.equal(got, want[k])
+                    finally:
+                        R.rbc_destroy(ctx)
+        except BaseException as e:   # reported by the main thread
+            errors.append((k, e))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(cases))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
